@@ -4,6 +4,11 @@ Every step of the path runs in the CUDA kernels behind the C ABI declared in
 include/mdn.h; this module turns torch tensors into pointers and sizes.  There is
 no CPU fallback: if the library is missing or was not built, importing the symbols
 raises.
+
+The per-call entry points hand their arguments to the native module `_native`
+(csrc/py_calls.cpp) first, which checks, allocates and calls in C++; when anything about
+the arguments is not the plain valid case it declines (None) and the Python code below
+does the same work, with the error messages.
 """
 from __future__ import annotations
 
@@ -62,6 +67,17 @@ class MdnError(RuntimeError):
 
 
 _lib = None
+_nat = None
+
+
+def _load_native():
+    """The module of native per-call functions (built in-tree next to libmdn.so); raises if absent."""
+    global _nat
+    if _nat is None:
+        lib()
+        from . import _native
+        _nat = _native
+    return _nat
 
 
 def lib() -> ctypes.CDLL:
@@ -216,8 +232,10 @@ def make_layer_ops(q, v, *, gate_param=None, qk_norm=None, out_norm_gate=None, p
       qk_norm       = dict(d: float32 [H] or None, eps: float)
       out_norm_gate = dict(g: [B,T,H,dv] in q's dtype, w: float32 [dv] or None, eps: float)
       placement     = "fused" (inside the forward's kernels) or "separate" (kernels of their own)"""
-    H, dv = q.shape[2], v.shape[-1]
     ops = MdnLayerOps()
+    if (_nat or _load_native()).fill_layer_ops(ctypes.addressof(ops), q, v, gate_param, qk_norm, out_norm_gate, placement):
+        return ops
+    H, dv = q.shape[2], v.shape[-1]
     if gate_param is not None:
         ops.raw_gates = 1
         ops.decay_a_alpha = _f32_vec("a_alpha", gate_param["a_alpha"], H)
@@ -275,6 +293,15 @@ def chunk_fwd(q, k, v, beta, log_alpha, log_mu, eta=None, *, initial_S=None, ini
     projections x_beta / x_alpha / x_mu / x_eta.
     keep_chunk_states: mdn_chunk_fwd_keep_states; returns (o, final_S, final_M, chunk_states, workspace) where
     chunk_states is the raw uint8 buffer (unpack_chunk_states turns it into float tensors)."""
+    r = (_nat or _load_native()).chunk_fwd(
+        q, k, v, beta, log_alpha, log_mu, eta, initial_S, initial_M, cu_seqlens, scale, o_dtype, _PATHS.get(path),
+        bool(output_final_state), workspace, out, segments, 0 if layer_ops is None else ctypes.addressof(layer_ops),
+        bool(keep_chunk_states))
+    if r is not None:
+        if isinstance(r, int):
+            raise MdnError(r, "mdn_chunk_fwd_keep_states" if keep_chunk_states
+                           else "mdn_chunk_fwd" if layer_ops is None else "mdn_chunk_fwd_fused")
+        return r
     _check_inputs(q, k, v, (("beta", beta), ("log_alpha", log_alpha), ("log_mu", log_mu), ("eta", eta)), "cuda")
     B, T, H, dk = q.shape
     dv = v.shape[-1]
@@ -386,6 +413,9 @@ def bwd_state_chain(q, k, d_o, fwd_workspace, *, v_dim: int, d_final_S=None, d_f
     return adj, dS0, dM0
 
 
+_GRADS = ("dq", "dk", "dv", "dbeta", "dlog_alpha", "dlog_mu", "deta", "d_initial_S", "d_initial_M")
+
+
 def chunk_bwd(q, k, v, beta, log_alpha, log_mu, eta, d_o, *, initial_S=None, initial_M=None, cu_seqlens=None,
               d_final_S=None, d_final_M=None, scale: Optional[float] = None, workspace: Optional[torch.Tensor] = None,
               method: str = "stepwise", saved=None):
@@ -395,6 +425,17 @@ def chunk_bwd(q, k, v, beta, log_alpha, log_mu, eta, d_o, *, initial_S=None, ini
     keep_chunk_states=True) call with the same inputs: mdn_chunk_bwd_saved (method="chunked" only).
     d_o: [B,T,H,dv] (its dtype is taken as the forward's o_dtype).  Returns a dict of float32 tensors
     dq, dk, dv, dbeta, dlog_alpha, dlog_mu, deta (None when eta is None), d_initial_S, d_initial_M."""
+    chunked = method == "chunked"
+    if chunked or method == "stepwise":
+        use_saved = chunked and saved is not None
+        fws, fstates = saved if use_saved else (None, None)
+        r = (_nat or _load_native()).chunk_bwd(
+            q, k, v, beta, log_alpha, log_mu, eta, d_o, initial_S, initial_M, cu_seqlens, d_final_S, d_final_M, scale,
+            workspace, 2 if use_saved else 1 if chunked else 0, fws, fstates)
+        if r is not None:
+            if isinstance(r, int):
+                raise MdnError(r, "mdn_chunk_bwd_saved" if use_saved else "mdn_chunk_bwd_chunked" if chunked else "mdn_chunk_bwd")
+            return dict(zip(_GRADS, r))
     _check_inputs(q, k, v, (("beta", beta), ("log_alpha", log_alpha), ("log_mu", log_mu), ("eta", eta)), "cuda")
     B, T, H, dk = q.shape
     dv = v.shape[-1]
@@ -411,7 +452,6 @@ def chunk_bwd(q, k, v, beta, log_alpha, log_mu, eta, d_o, *, initial_S=None, ini
         _check_state(name, t, (nst, H, dk, dv), "cuda")
     if method not in ("stepwise", "chunked"):
         raise ValueError("method")
-    chunked = method == "chunked"
     if chunked:
         p = make_params(q, v, num_seqs=N, scale=scale, o_dtype=d_o.dtype, path="tensor")
         need = int(lib().mdn_chunk_bwd_saved_workspace_bytes(ctypes.byref(p)) if saved is not None
@@ -496,6 +536,12 @@ def decode_step(q, k, v, beta, log_alpha, log_mu, eta, S, M, *, scale: Optional[
                 layer_ops: Optional[MdnLayerOps] = None) -> torch.Tensor:
     """mdn_decode_step (mdn_decode_step_fused when layer_ops is given): one token per sequence (q, k: [B,1,H,dk];
     v: [B,1,H,dv]; gates [B,1,H]); the fp32 states S, M [B,H,dk,dv] are updated in place.  Returns o [B,1,H,dv]."""
+    r = (_nat or _load_native()).decode_step(q, k, v, beta, log_alpha, log_mu, eta, S, M, scale, o_dtype, out,
+                                            0 if layer_ops is None else ctypes.addressof(layer_ops))
+    if r is not None:
+        if isinstance(r, int):
+            raise MdnError(r, "mdn_decode_step")
+        return r
     _check_inputs(q, k, v, (("beta", beta), ("log_alpha", log_alpha), ("log_mu", log_mu), ("eta", eta)), "cuda")
     B, T, H, dk = q.shape
     dv = v.shape[-1]

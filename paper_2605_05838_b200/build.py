@@ -1,4 +1,5 @@
-"""Builds libmdn.so in-tree with nvcc for sm_100a (cross-compiles without a GPU).
+"""Builds libmdn.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and with g++ the module `_native`
+of the binding's per-call host work on top of it.
 
     python -m paper_2605_05838_b200.build [--force] [--verbose]
 """
@@ -7,6 +8,7 @@ from __future__ import annotations
 import concurrent.futures
 import glob
 import os
+import shutil
 import subprocess
 import sys
 
@@ -14,6 +16,7 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libmdn.so")
+NATIVE = os.path.join(PKG, "_native.so")
 OBJ_DIR = os.path.join(PKG, "build")
 
 # MDN_BUILD_DEBUG=1 in the environment of the BUILD compiles the debug knobs in (-DMDN_DEBUG: precision ablation
@@ -33,6 +36,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     srcs = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
     hdrs = sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + sorted(glob.glob(os.path.join(ROOT, "include", "*.h")))
     if not force and _newer(LIB, srcs + hdrs):
+        build_native(force, verbose)
         write_build_info()
         return LIB
     os.makedirs(OBJ_DIR, exist_ok=True)
@@ -54,8 +58,33 @@ def build(force: bool = False, verbose: bool = False) -> str:
     subprocess.run(["nvcc", "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp] + objs
                    + ["-lcudart", "-lcuda"], check=True)
     os.replace(tmp, LIB)
+    build_native(force, verbose)
     write_build_info()
     return LIB
+
+
+def build_native(force: bool = False, verbose: bool = False) -> str:
+    """csrc/py_calls.cpp -> _native.so, linked to libmdn.so beside it and to torch's libraries (loaded by then)."""
+    import sysconfig
+
+    src = os.path.join(CSRC, "py_calls.cpp")
+    if not force and _newer(NATIVE, [src, os.path.join(ROOT, "include", "mdn.h")]):
+        return NATIVE
+    import torch
+    tdir = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(shutil.which("nvcc"))))
+    tmp = NATIVE + ".tmp.%d" % os.getpid()
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-I", os.path.join(ROOT, "include"), "-I", os.path.join(tdir, "include"),
+           "-I", os.path.join(tdir, "include", "torch", "csrc", "api", "include"), "-I", sysconfig.get_paths()["include"],
+           "-I", os.path.join(cuda, "include"), src, "-o", tmp, "-L", PKG, "-l:libmdn.so", "-L", os.path.join(tdir, "lib"),
+           "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or r.returncode != 0:
+        sys.stderr.write(r.stdout + r.stderr)
+    if r.returncode != 0:
+        raise RuntimeError("g++ failed for " + src)
+    os.replace(tmp, NATIVE)
+    return NATIVE
 
 
 def write_build_info() -> None:

@@ -1,0 +1,60 @@
+"""The native per-call module (csrc/py_calls.cpp): it declines (None) whatever is not the plain valid case, so that the
+Python binding raises its own error, and gives the Python binding's results otherwise.  An int `scale` is one of the
+arguments it declines: the same value as int and as float takes the two routes."""
+import ctypes
+
+import pytest
+import torch
+
+import paper_2605_05838_b200 as mdn
+
+
+def args(B, T, H, dk, dv, dtype, device, seed=0):
+    g = torch.Generator().manual_seed(seed)
+    q, k = (torch.nn.functional.normalize(torch.randn((B, T, H, dk), generator=g), dim=-1).to(dtype) for _ in range(2))
+    v = torch.randn((B, T, H, dv), generator=g).to(dtype)
+    beta = torch.rand((B, T, H), generator=g) * 0.05
+    la, lm = (-0.1 * torch.rand((B, T, H), generator=g) for _ in range(2))
+    eta = 1.0 + 0.1 * torch.randn((B, T, H), generator=g)
+    return [t.to(device) for t in (q, k, v, beta, la, lm, eta)]
+
+
+def test_cpu_tensors_are_declined_and_the_binding_raises():
+    from paper_2605_05838_b200 import build
+    build.build()
+    from paper_2605_05838_b200.binding import _load_native
+    a = args(1, 1, 2, 64, 64, torch.float32, "cpu")
+    S = torch.zeros((1, 2, 64, 64))
+    nat = _load_native()
+    assert nat.decode_step(*a, S, S, None, None, None, 0) is None
+    assert nat.chunk_fwd(*a, None, None, None, None, None, 0, True, None, None, 0, 0, False) is None
+    assert nat.chunk_bwd(*a, a[2], None, None, None, None, None, None, None, 0, None, None) is None
+    ops = mdn.MdnLayerOps()
+    assert nat.fill_layer_ops(ctypes.addressof(ops), a[0], a[2], None, None, None, "fused") is None
+    for call in (lambda: mdn.decode_step(*a, S, S), lambda: mdn.chunk_fwd(*a), lambda: mdn.chunk_bwd(*a, a[2])):
+        with pytest.raises(ValueError):
+            call()
+    with pytest.raises(KeyError):
+        mdn.chunk_fwd(*a, path="nosuch")
+    with pytest.raises(KeyError):
+        mdn.make_layer_ops(a[0], a[2], placement="nosuch")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype,dk,dv,T", [(torch.float32, 64, 128, 1), (torch.float32, 64, 64, 65), (torch.bfloat16, 128, 128, 70)])
+def test_both_routes_give_the_same_bits(dtype, dk, dv, T):
+    a = args(2, T, 3, dk, dv, dtype, "cuda")
+    g = torch.Generator().manual_seed(5)
+    S, M = (torch.randn((2, 3, dk, dv), generator=g).cuda() * 0.1 for _ in range(2))
+    for kw in (dict(), dict(initial_S=S, initial_M=M, o_dtype=torch.float32), dict(output_final_state=False)):
+        for x, y in zip(mdn.chunk_fwd(*a, scale=1, **kw), mdn.chunk_fwd(*a, scale=1.0, **kw)):
+            assert (x is None and y is None) or torch.equal(x, y)
+    if T == 1:
+        S2, M2 = S.clone(), M.clone()
+        o1, o2 = mdn.decode_step(*a, S, M, scale=1), mdn.decode_step(*a, S2, M2, scale=1.0)
+        assert torch.equal(o1, o2) and torch.equal(S, S2) and torch.equal(M, M2)
+    d_o = a[2].clone()
+    g1, g2 = mdn.chunk_bwd(*a, d_o, scale=1), mdn.chunk_bwd(*a, d_o, scale=1.0)
+    assert g1.keys() == g2.keys() and torch.equal(g1["dv"], g2["dv"]) and torch.equal(g1["d_initial_S"], g2["d_initial_S"])
+    with pytest.raises(mdn.MdnError):
+        mdn.chunk_fwd(*a, scale=1.0, segments=2)
