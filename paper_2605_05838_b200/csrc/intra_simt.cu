@@ -1,167 +1,281 @@
-// a2, fp32 SIMT version: per (chunk, head) the intra-chunk system of Eq. 15 and the masked
+// a1 + a2 in fp32: per (chunk, head) the coefficient scan of Eq. 10, the intra-chunk system of Eq. 15 and the masked
 // query-key matrix of Eq. 12.
 //
-//   Gamma[r][i]   = gamma_{r,i}              (i <= r)   built column by column from
-//                   gamma_{r,i} = alpha_r gamma_{r-1,i} + beta_r m_{r,i},  m_{r,i} = mu_r m_{r-1,i}, m_{i,i} = 1
-//   A[r][i]       = alpha_r gamma_{r-1,i} eta_i (k_r . k_i)       (i < r)    = ((P K^T) .* Gamma^-)[r][i]
-//   T             = (I + A)^{-1}             forward substitution, one column per thread
-//   W[r][i]       = scale gamma_{r,i} eta_i (q_r . k_i)           (i <= r)
+//   gamma_{r,i} = alpha_r gamma_{r-1,i} + beta_r m_{r,i},  m_{r,i} = mu_r m_{r-1,i}, m_{i,i} = 1     (thread = column i)
+//   A[r][i]     = alpha_r gamma_{r-1,i} eta_i (k_r . k_i)       (i < r)    = ((P K^T) .* Gamma^-)[r][i]
+//   T           = (I + A)^{-1}             blocked: 16 x 16 diagonal blocks by forward substitution, then
+//                                          T_21 = -T_22 A_21 T_11 at block sizes 16 and 32
+//   W[r][i]     = scale gamma_{r,i} eta_i (q_r . k_i)           (i <= r)
 //
 // Gamma^- is Gamma shifted down one row (the derivation substitutes S_{t-1}); with
 // p_r = alpha_r k_r its entry is alpha_r gamma_{r-1,i}, which the column recurrence
 // produces directly, with no subtraction.  All arithmetic fp32; q, k are widened on load.
-#include "mdn_common.cuh"
+//
+// One 256-thread CTA per (chunk, head).  What bounds it at few chunks is its own latency: the scan and the recurrence
+// of gamma run on three warps while K and Q are on their way, [K; Q] K^T is one register-tiled product that skips the
+// 8 x 16 blocks above the diagonal, and the inverse is seven short parallel steps instead of 64 dependent rows.
+// Two CTAs per SM (93 KB at dk = 128): A, W and T live where K, Q and Gamma were.
+#include "coeff_scan.cuh"
+#include "simt_tile.cuh"
 
 namespace mdn {
+namespace {
 
-constexpr int kIntraThreads = 256;
+struct IntraArgs {
+  ChunkGeom g;
+  const void* q; const void* k;
+  bool in_bf16;
+  float* coef;
+  GateArgs gates;
+  GateParam gp;
+  float scale;
+  float* T; float* W;     // transposed = false: T, W
+  float* TT;              // transposed = true:  T, W^T (in W) and T^T (the exact backward reads those)
+  bool transposed;
+};
 
-template <typename TIn, int DK>
-__device__ __forceinline__ void load_tile_f32(float* dst /*[64][DK+1]*/, const TIn* src, int row_stride, int n,
-                                              int tid) {
-  constexpr int VEC = 16 / sizeof(TIn);
-  constexpr int VPR = DK / VEC;  // vectors per row
-  for (int idx = tid; idx < C * VPR; idx += kIntraThreads) {
-    const int r = idx / VPR, c = (idx % VPR) * VEC;
-    float vals[VEC];
-    if (r < n) {
-      const uint4 raw = __ldg(reinterpret_cast<const uint4*>(src + (size_t)r * row_stride + c));
-      const TIn* e = reinterpret_cast<const TIn*>(&raw);
-#pragma unroll
-      for (int x = 0; x < VEC; ++x) vals[x] = to_f32<TIn>(e[x]);
-    } else {
-#pragma unroll
-      for (int x = 0; x < VEC; ++x) vals[x] = 0.f;
-    }
-#pragma unroll
-    for (int x = 0; x < VEC; ++x) dst[r * (DK + 1) + c + x] = vals[x];
-  }
-}
+template <int DK> struct IntraSmem {   // float offsets
+  static constexpr int LDK = DK + 4, K = 0, Q = K + C * LDK, G = Q + C * LDK, P = G + C * kLT, cv = P + 32 * 36, kFloats = cv + 4 * C;
+  static constexpr size_t bytes(bool bf16) { return (size_t)kFloats * 4 + (bf16 ? (size_t)2 * C * DK * 2 : 0); }
+};
 
-template <typename TOut> __device__ __forceinline__ void store_mat(TOut* dst, int idx, float x);
-template <> __device__ __forceinline__ void store_mat<float>(float* dst, int idx, float x) { dst[idx] = x; }
-template <> __device__ __forceinline__ void store_mat<__nv_bfloat16>(__nv_bfloat16* dst, int idx, float x) {
-  dst[idx] = __float2bfloat16_rn(x);
-}
-
-// TOut = float: T and W fp32.  TOut = bf16: T bf16; W as hi part at Wout and the
-// residual lo part (W - hi, rounded to bf16) at Wout + total_mats*4096.
-template <typename TIn, typename TOut, int DK>
-__global__ void __launch_bounds__(kIntraThreads) intra_simt_kernel(ChunkGeom g, const TIn* __restrict__ q,
-                                                                  const TIn* __restrict__ k,
-                                                                  const float* __restrict__ coef, float scale,
-                                                                  TOut* __restrict__ Tout, TOut* __restrict__ Wout,
-                                                                  size_t w_lo_offset) {
-  extern __shared__ float sm[];
-  const int slot = blockIdx.x / g.H, h = blockIdx.x % g.H;
-  const SlotInfo si = slot_info(g, slot);
+template <int DK>
+__global__ void __launch_bounds__(kSimtThreads, 2) intra_simt_kernel(const IntraArgs a) {
+  extern __shared__ __align__(16) float sm[];
+  using L = IntraSmem<DK>;
+  constexpr int LDK = L::LDK, LP = 36;
+  const int H = a.g.H, slot = blockIdx.x / H, h = blockIdx.x % H;
+  grid_launch_dependents();
+  grid_dependency_wait();
+  const SlotInfo si = slot_info(a.g, slot);
   if (si.seq < 0) return;
-  const int tid = threadIdx.x;
-  constexpr int LD = DK + 1, LM = C + 1;
-  float* Ks = sm;                  // [64][DK+1]
-  float* Qs = Ks + C * LD;         // [64][DK+1]
-  float* Gs = Qs + C * LD;         // [64][65]  gamma, then W
-  float* As = Gs + C * LM;         // [64][65]  alpha_r gamma_{r-1,i}, then A
-  float* Ts = As + C * LM;         // [64][65]
-  float* cv = Ts + C * LM;         // [4][64]   alpha, beta, mu, eta
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  float* Ks = sm + L::K;
+  float* Qs = sm + L::Q;
+  float* Gs = sm + L::G;       // gamma; then T
+  float* Ps = sm + L::P;       // scratch of the inverse
+  float* cv = sm + L::cv;      // alpha, beta, mu, eta
+  float* As = Ks;              // after the product: A, W in the place of K, Q
+  float* Ws = Qs;
+  float* Ts = Gs;
+  uint8_t* raw = reinterpret_cast<uint8_t*>(sm + L::kFloats);
 
-  const size_t tok = (size_t)si.tok0 * g.H + h;
-  load_tile_f32<TIn, DK>(Ks, k + tok * DK, g.H * DK, si.n, tid);
-  load_tile_f32<TIn, DK>(Qs, q + tok * DK, g.H * DK, si.n, tid);
-  const float* cf = coef + ((size_t)slot * g.H + h) * MDN_NUM_COEF * C;
-  {
-    const int which = tid >> 6, r = tid & 63;   // 4 vectors x 64
-    cv[which * C + r] = cf[(kAlpha + which) * C + r];
-  }
-  for (int idx = tid; idx < C * LM; idx += kIntraThreads) { Gs[idx] = 0.f; As[idx] = 0.f; }
-  __syncthreads();
+  const size_t es = a.in_bf16 ? 2 : 4, row0 = ((size_t)si.tok0 * H + h) * DK * es;
+  load_rows<DK>(Ks, raw, static_cast<const uint8_t*>(a.k) + row0, a.in_bf16, (size_t)H * DK, si.n, tid);
+  load_rows<DK>(Qs, raw + C * DK * 2, static_cast<const uint8_t*>(a.q) + row0, a.in_bf16, (size_t)H * DK, si.n, tid);
+  cp_commit();
 
-  if (tid < C) {   // column i of Gamma and of the shifted mask
-    const int i = tid;
-    float m = 1.f, gprev = 0.f;
-    for (int r = i; r < C; ++r) {
-      const float al = cv[0 * C + r], be = cv[1 * C + r], mu = cv[2 * C + r];
-      if (r > i) m *= mu;
-      const float shifted = al * gprev;          // alpha_r gamma_{r-1,i}
-      const float gam = fmaf(be, m, shifted);    // gamma_{r,i}
-      Gs[r * LM + i] = gam;
-      As[r * LM + i] = shifted;
-      gprev = gam;
-    }
-  }
-  __syncthreads();
-
-  for (int idx = tid; idx < C * C; idx += kIntraThreads) {
-    const int r = idx >> 6, i = idx & 63;
-    if (i <= r) {
-      const float* kr = Ks + r * LD;
-      const float* ki = Ks + i * LD;
-      const float* qr = Qs + r * LD;
-      float kk = 0.f, qk = 0.f;
-#pragma unroll 8
-      for (int d = 0; d < DK; ++d) {
-        const float kid = ki[d];
-        kk = fmaf(kr[d], kid, kk);
-        qk = fmaf(qr[d], kid, qk);
+  float* cf = a.coef + ((size_t)slot * H + h) * MDN_NUM_COEF * C;
+  if (a.gates.log_alpha == nullptr) {   // the scan has run: its gate vectors are in the workspace
+    cv[tid] = cf[kAlpha * C + tid];
+    __syncthreads();
+  } else {
+    if (tid < C) {
+      TokenGates tg{1.f, 1.f, 0.f, 0.f};   // exact no-ops past the end of a short chunk
+      if (tid < si.n) {
+        const size_t gi = ((size_t)si.tok0 + tid) * H + h;
+        tg = load_token_gates(a.gp, h, __ldg(a.gates.log_alpha + gi), __ldg(a.gates.log_mu + gi), __ldg(a.gates.beta + gi),
+                              a.gates.eta ? __ldg(a.gates.eta + gi) : 1.f);
       }
-      const float et = cv[3 * C + i];
-      Gs[r * LM + i] = scale * Gs[r * LM + i] * et * qk;         // W
-      As[r * LM + i] = (i < r) ? As[r * LM + i] * et * kk : 0.f;  // A (strictly lower)
+      cv[0 * C + tid] = tg.alpha; cv[1 * C + tid] = tg.beta; cv[2 * C + tid] = tg.mu; cv[3 * C + tid] = tg.eta;
+    }
+    __syncthreads();
+    if (warp == 2) {
+      const float2 a2 = reinterpret_cast<const float2*>(cv)[lane], b2 = reinterpret_cast<const float2*>(cv + C)[lane];
+      const float2 m2 = reinterpret_cast<const float2*>(cv + 2 * C)[lane], e2 = reinterpret_cast<const float2*>(cv + 3 * C)[lane];
+      const float al[2] = {a2.x, a2.y}, be[2] = {b2.x, b2.y}, mu[2] = {m2.x, m2.y}, et[2] = {e2.x, e2.y};
+      const HeadCoefs hc = scan_head(al, mu, be, et, lane);
+      auto put = [&](int which, float x0, float x1) { reinterpret_cast<float2*>(cf + which * C)[lane] = make_float2(x0, x1); };
+      put(kAbar, hc.abar[0], hc.abar[1]);
+      put(kB, hc.b[0], hc.b[1]);
+      put(kAlphaBPrev, hc.ab_prev[0], hc.ab_prev[1]);
+      put(kGS, hc.gs[0], hc.gs[1]);
+      put(kGM, hc.gm[0], hc.gm[1]);
+      put(kMubar, hc.mubar[0], hc.mubar[1]);
+      put(kRk, 1.f, 1.f);
+      put(kRq, 1.f, 1.f);
+      put(kAlpha, al[0], al[1]);
+      put(kBeta, be[0], be[1]);
+      put(kMu, mu[0], mu[1]);
+      put(kEta, et[0], et[1]);
+    }
+  }
+  if (tid < C) {   // column i of Gamma (zero above the diagonal)
+    const int i = tid;
+    float m = 1.f, gam = 0.f;
+#pragma unroll 4
+    for (int rb = 0; rb < C; rb += 4) {
+      const float4 al = lds4(cv + rb), be = lds4(cv + C + rb), mu = lds4(cv + 2 * C + rb);
+      const float a4[4] = {al.x, al.y, al.z, al.w}, b4[4] = {be.x, be.y, be.z, be.w}, m4[4] = {mu.x, mu.y, mu.z, mu.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = rb + u;
+        if (r > i) m *= m4[u];
+        if (r >= i) gam = fmaf(a4[u], gam, b4[u] * m);
+        Gs[r * kLT + i] = r >= i ? gam : 0.f;
+      }
+    }
+  }
+  cp_wait<0>();
+  __syncthreads();
+  if (a.in_bf16) {
+    widen_tile<DK>(Ks, raw, tid);
+    widen_tile<DK>(Qs, raw + C * DK * 2, tid);
+    __syncthreads();
+  }
+
+  // ---- [K; Q] K^T: rows r0 + 16 i (row slots 0..15: K, 16..31: Q), columns jg + 8 jj; block i reaches columns 16 i + 15
+  const int jg = tid & 7, rs = tid >> 3, r0 = rs & 15;
+  const bool w_rows = rs >= 16;
+  float out[4][8];
+  {
+    float2 acc[4][8];
+    zero2(acc);
+    const float* ap = (w_rows ? Qs : Ks) + r0 * LDK;
+    const float* bp = Ks + jg * LDK;
+#pragma unroll 1
+    for (int k = 0; k < DK; k += 4) {
+      float4 av[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) av[i] = lds4(ap + i * 16 * LDK + k);
+#pragma unroll
+      for (int jj = 0; jj < 8; ++jj) {
+        const float4 bv = lds4(bp + jj * 8 * LDK + k);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (jj <= 2 * i + 1) fma4(acc[i][jj], av[i], bv);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int jj = 0; jj < 8; ++jj) out[i][jj] = hsum(acc[i][jj]);
+  }
+  __syncthreads();   // K and Q have been read
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = r0 + 16 * i;
+    const float f = w_rows ? a.scale : cv[r];
+    const float* grow = Gs + (w_rows ? r : max(r - 1, 0)) * kLT;
+    float* dst = (w_rows ? Ws : As) + r * kLT;
+#pragma unroll
+    for (int jj = 0; jj < 8; ++jj) {
+      const int c = jg + 8 * jj;
+      const bool in = w_rows ? c <= r : c < r;
+      dst[c] = in ? f * grow[c] * cv[3 * C + c] * out[i][jj] : 0.f;
+    }
+  }
+  __syncthreads();   // A, W complete; Gamma has been read: T takes its place
+
+  const size_t mat = ((size_t)slot * H + h) * C * C;
+  // step 1: the four diagonal blocks (thread = block, column); the other threads clear the blocks above the diagonal and
+  // write W out
+  if (tid < C) {
+    const int b = tid >> 4, b0 = b * 16, j = tid & 15;
+    float x[16];
+#pragma unroll
+    for (int rr = 0; rr < 16; ++rr) {
+      float acc = (rr == j) ? 1.f : 0.f;
+#pragma unroll
+      for (int m4 = 0; m4 < rr; m4 += 4) {
+        const float4 v4 = lds4(As + (b0 + rr) * kLT + b0 + m4);
+        const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (m4 + e < rr) acc = fmaf(-v[e], x[m4 + e], acc);
+      }
+      x[rr] = acc;
+    }
+#pragma unroll
+    for (int rr = 0; rr < 16; ++rr) Ts[(b0 + rr) * kLT + b0 + j] = x[rr];
+  } else {
+    for (int i = tid - C; i < C * 16; i += kSimtThreads - C) {
+      const int r = i >> 4, c = (i & 15) * 4;
+      if ((c >> 4) > (r >> 4)) *reinterpret_cast<float4*>(Ts + r * kLT + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (!a.transposed) {
+        *reinterpret_cast<float4*>(a.W + mat + i * 4) = lds4(Ws + r * kLT + c);
+      } else {   // row r of W^T
+        *reinterpret_cast<float4*>(a.W + mat + i * 4) = make_float4(Ws[c * kLT + r], Ws[(c + 1) * kLT + r], Ws[(c + 2) * kLT + r], Ws[(c + 3) * kLT + r]);
+      }
     }
   }
   __syncthreads();
-
-  if (tid < C) {   // T = (I + A)^{-1}: column j by forward substitution
-    const int j = tid;
-    for (int r = 0; r < C; ++r) {
-      float acc = (r == j) ? 1.f : 0.f;
-      const float* ar = As + r * LM;
-      for (int i = 0; i < r; ++i) acc = fmaf(-ar[i], Ts[i * LM + j], acc);
-      Ts[r * LM + j] = acc;
+  // step 2: inside each 32 x 32 diagonal block: T_lo = -D_hi (A_lo D_lo); thread = (block, row, two columns)
+  {
+    const int s = tid >> 7, r = (tid >> 3) & 15, c0 = (tid & 7) * 2, R0 = 32 * s + 16, C0 = 32 * s;
+    float2 p = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const float av = As[(R0 + r) * kLT + C0 + k];
+      const float2 d = *reinterpret_cast<const float2*>(Ts + (C0 + k) * kLT + C0 + c0);
+      p = __ffma2_rn(make_float2(av, av), d, p);
     }
+    *reinterpret_cast<float2*>(Ps + (16 * s + r) * LP + c0) = p;
+    __syncthreads();
+    p = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const float tv = -Ts[(R0 + r) * kLT + R0 + k];
+      const float2 d = *reinterpret_cast<const float2*>(Ps + (16 * s + k) * LP + c0);
+      p = __ffma2_rn(make_float2(tv, tv), d, p);
+    }
+    *reinterpret_cast<float2*>(Ts + (R0 + r) * kLT + C0 + c0) = p;
   }
   __syncthreads();
-
-  const size_t mat = ((size_t)slot * g.H + h) * C * C;
-  for (int idx = tid; idx < C * C; idx += kIntraThreads) {
-    const int r = idx >> 6, i = idx & 63;
-    const float t = Ts[r * LM + i], w = Gs[r * LM + i];
-    store_mat<TOut>(Tout + mat, idx, t);
-    store_mat<TOut>(Wout + mat, idx, w);
-    if (sizeof(TOut) == 2) {
-      const float hi = to_f32<TOut>(from_f32<TOut>(w));
-      store_mat<TOut>(Wout + w_lo_offset + mat, idx, w - hi);
-    }
+  // step 3: T[32:64, 0:32] = -T[32:64, 32:64] (A[32:64, 0:32] T[0:32, 0:32]); thread = (row, four columns)
+  {
+    const int r = tid >> 3, c0 = (tid & 7) * 4;
+    auto row_times = [&](const float* row, float sign, const float* b, int ldb) {
+      float2 p0 = make_float2(0.f, 0.f), p1 = p0;
+#pragma unroll 8
+      for (int k = 0; k < 32; ++k) {
+        const float av = sign * row[k];
+        const float4 d = lds4(b + k * ldb + c0);
+        p0 = __ffma2_rn(make_float2(av, av), make_float2(d.x, d.y), p0);
+        p1 = __ffma2_rn(make_float2(av, av), make_float2(d.z, d.w), p1);
+      }
+      return make_float4(p0.x, p0.y, p1.x, p1.y);
+    };
+    const float4 p = row_times(As + (32 + r) * kLT, 1.f, Ts, kLT);
+    *reinterpret_cast<float4*>(Ps + r * LP + c0) = p;
+    __syncthreads();
+    const float4 t = row_times(Ts + (32 + r) * kLT + 32, -1.f, Ps, LP);
+    *reinterpret_cast<float4*>(Ts + (32 + r) * kLT + c0) = t;
+  }
+  __syncthreads();
+  for (int i = tid; i < C * 16; i += kSimtThreads) {
+    const int r = i >> 4, c = (i & 15) * 4;
+    *reinterpret_cast<float4*>(a.T + mat + i * 4) = lds4(Ts + r * kLT + c);
+    if (a.transposed)
+      *reinterpret_cast<float4*>(a.TT + mat + i * 4) = make_float4(Ts[c * kLT + r], Ts[(c + 1) * kLT + r], Ts[(c + 2) * kLT + r], Ts[(c + 3) * kLT + r]);
   }
 }
 
-template <typename TIn, typename TOut, int DK>
-static cudaError_t launch_one(const Plan& pl, const void* q, const void* k) {
-  const size_t smem = (size_t)(2 * C * (DK + 1) + 3 * C * (C + 1) + 4 * C) * sizeof(float);
-  auto kern = intra_simt_kernel<TIn, TOut, DK>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <int DK> cudaError_t launch_one(const Plan& pl, const IntraArgs& a) {
+  const size_t smem = IntraSmem<DK>::bytes(a.in_bf16);
+  const cudaError_t e = cudaFuncSetAttribute(intra_simt_kernel<DK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const size_t n_mats = (size_t)pl.geom.num_slots * pl.p.H;
-  kern<<<(unsigned)n_mats, kIntraThreads, smem, pl.stream>>>(
-      pl.geom, static_cast<const TIn*>(q), static_cast<const TIn*>(k),
-      reinterpret_cast<const float*>(pl.ws + pl.lay.off_coef), pl.p.scale,
-      reinterpret_cast<TOut*>(pl.ws + pl.lay.off_T), reinterpret_cast<TOut*>(pl.ws + pl.lay.off_W),
-      n_mats * C * C);
-  return cudaGetLastError();
+  return launch_pdl(intra_simt_kernel<DK>, dim3((unsigned)pl.geom.num_slots * pl.p.H), dim3(kSimtThreads), smem, pl.stream, a);
 }
 
-cudaError_t launch_intra_simt(const Plan& pl, const void* q, const void* k, int* launches) {
-  const bool in_bf16 = pl.p.io_dtype == MDN_BF16, out_bf16 = pl.lay.mat_dtype == MDN_BF16;
-  cudaError_t e = cudaErrorInvalidValue;
-  if (pl.p.dk == 64) {
-    if (!in_bf16 && !out_bf16) e = launch_one<float, float, 64>(pl, q, k);
-    else if (in_bf16 && !out_bf16) e = launch_one<__nv_bfloat16, float, 64>(pl, q, k);
-    else if (in_bf16 && out_bf16) e = launch_one<__nv_bfloat16, __nv_bfloat16, 64>(pl, q, k);
-  } else if (pl.p.dk == 128) {
-    if (!in_bf16 && !out_bf16) e = launch_one<float, float, 128>(pl, q, k);
-    else if (in_bf16 && !out_bf16) e = launch_one<__nv_bfloat16, float, 128>(pl, q, k);
-    else if (in_bf16 && out_bf16) e = launch_one<__nv_bfloat16, __nv_bfloat16, 128>(pl, q, k);
-  }
+}  // namespace
+
+// gates all NULL: the coefficient vectors are in the workspace; else this kernel runs the scan and writes them.
+// TT != NULL: T goes to its place in the workspace, W^T to W's, T^T to TT (the exact backward's operands).
+cudaError_t launch_intra_simt(const Plan& pl, const void* q, const void* k, const GateArgs& gates, float* TT, int* launches) {
+  IntraArgs a{};
+  a.g = pl.geom;
+  a.q = q; a.k = k;
+  a.in_bf16 = pl.p.io_dtype == MDN_BF16;
+  a.coef = reinterpret_cast<float*>(pl.ws + pl.lay.off_coef);
+  a.gates = gates;
+  a.gp = pl.gp;
+  a.scale = pl.p.scale;
+  a.T = reinterpret_cast<float*>(pl.ws + pl.lay.off_T);
+  a.W = reinterpret_cast<float*>(pl.ws + pl.lay.off_W);
+  a.TT = TT;
+  a.transposed = TT != nullptr;
+  const cudaError_t e = pl.p.dk == 64 ? launch_one<64>(pl, a) : launch_one<128>(pl, a);
   if (e == cudaSuccess) ++*launches;
   return e;
 }

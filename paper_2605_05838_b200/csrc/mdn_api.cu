@@ -89,8 +89,7 @@ static mdn_status make_plan(const mdn_params* p, const int32_t* cu, void* ws, si
   return MDN_OK;
 }
 
-// with_scan = false: only the status word and the chunk map (the tensor path runs the scan inside its
-// intra-chunk kernel).
+// with_scan = false: only the status word and the chunk map (the forward runs the scan inside its intra-chunk kernel).
 static mdn_status run_prep_and_scan(const Plan& pl, const float* beta, const float* log_alpha, const float* log_mu,
                                     const float* eta, int* launches, bool with_scan = true) {
   if (!beta || !log_alpha || !log_mu) return MDN_ERR_INVALID_ARG;
@@ -105,7 +104,7 @@ static mdn_status run_intra(const Plan& pl, const void* q, const void* k, int* l
                             const GateArgs& gates = GateArgs{nullptr, nullptr, nullptr, nullptr}) {
   if (!q || !k || !aligned(q, 16) || !aligned(k, 16)) return MDN_ERR_INVALID_ARG;
   cudaError_t e = pl.p.path == MDN_PATH_TENSOR ? launch_intra_tensor(pl, q, k, gates, launches)
-                                               : launch_intra_simt(pl, q, k, launches);
+                                               : launch_intra_simt(pl, q, k, gates, nullptr, launches);
   if (e != cudaSuccess) t_last_cuda_error = (int)e;
   return e == cudaSuccess ? MDN_OK : MDN_ERR_CUDA;
 }
@@ -164,14 +163,12 @@ static mdn_status run_forward(const Plan& plan, const void* q, const void* k, co
       (final_S && !aligned(final_S, 16)) || (final_M && !aligned(final_M, 16)))
     return MDN_ERR_INVALID_ARG;
   if (!mark_stage(0, pl.stream)) return MDN_ERR_CUDA;
-  // tensor path: the intra-chunk kernel runs the coefficient scan itself (one kernel and one round trip of
-  // the coefficient vectors less); SIMT path: stand-alone scan kernel
-  const bool fused_scan = pl.p.path == MDN_PATH_TENSOR;
-  mdn_status st = run_prep_and_scan(pl, beta, log_alpha, log_mu, eta, &t_last_launches, !fused_scan);
+  // the intra-chunk kernels run the coefficient scan themselves (one kernel and one round trip of the coefficient
+  // vectors less); the stand-alone scan kernel is the stage entry point's
+  mdn_status st = run_prep_and_scan(pl, beta, log_alpha, log_mu, eta, &t_last_launches, false);
   if (st != MDN_OK) return st;
   if (!mark_stage(1, pl.stream)) return MDN_ERR_CUDA;
-  st = fused_scan ? run_intra(pl, q, k, &t_last_launches, GateArgs{beta, log_alpha, log_mu, eta})
-                  : run_intra(pl, q, k, &t_last_launches);
+  st = run_intra(pl, q, k, &t_last_launches, GateArgs{beta, log_alpha, log_mu, eta});
   if (st != MDN_OK) return st;
   if (!mark_stage(2, pl.stream)) return MDN_ERR_CUDA;
   cudaError_t e = pl.p.path == MDN_PATH_TENSOR
@@ -528,14 +525,21 @@ mdn_status mdn_chunk_fwd_fused(const mdn_params* p, const mdn_layer_ops* ops, co
 }
 
 // ---- backward
-static uint64_t bwd_scratch_base(const mdn_ws_layout& lay) { return align_up(lay.off_coef, 256); }
+// The exact backward runs on the fp32 path's workspace (coefficient vectors, T, W as fp32) whatever the call's path;
+// its own scratch follows.
+static mdn_params bwd_params(const mdn_params& p) {
+  mdn_params pe = p;
+  pe.path = MDN_PATH_SIMT;
+  pe.segments = 1;
+  return pe;
+}
 
 size_t mdn_chunk_bwd_workspace_bytes(const mdn_params* p) {
   mdn_ws_layout lay;
-  if (check_params(p) != MDN_OK || make_layout(*p, &lay) != MDN_OK) return 0;
+  if (check_params(p) != MDN_OK || make_layout(bwd_params(*p), &lay) != MDN_OK) return 0;
   BwdScratch bs;
   bwd_scratch_layout(*p, lay.num_slots, &bs);
-  return (size_t)(bwd_scratch_base(lay) + bs.total);   // status word and chunk map, then the backward's scratch
+  return (size_t)(lay.total_bytes + bs.total);
 }
 
 mdn_status mdn_chunk_bwd(const mdn_params* p, const void* q, const void* k, const void* v, const float* beta,
@@ -555,29 +559,16 @@ mdn_status mdn_chunk_bwd(const mdn_params* p, const void* q, const void* k, cons
   if (!aligned(q, 16) || !aligned(k, 16) || !aligned(v, 16) || !aligned(d_o, 16) || !aligned(dq, 16) ||
       !aligned(dk, 16) || !aligned(dv, 16))
     return MDN_ERR_INVALID_ARG;
+  const mdn_params pe = bwd_params(*p);
   Plan pl;
-  pl.p = *p;
-  pl.p.path = MDN_PATH_SIMT;
-  st = make_layout(*p, &pl.lay);
+  st = make_plan(&pe, cu_seqlens, workspace, workspace_bytes, cuda_stream, &pl);
   if (st != MDN_OK) return st;
-  pl.ws = static_cast<char*>(workspace);
-  pl.stream = static_cast<cudaStream_t>(cuda_stream);
-  pl.gp = GateParam{}; pl.qk = QkNorm{}; pl.post = OutPost{};
-  ChunkGeom& g = pl.geom;
-  g.B = p->B; g.T = p->T; g.H = p->H;
-  g.num_seqs = cu_seqlens ? p->num_seqs : p->B;
-  g.chunks_per_seq = (p->T + C - 1) / C;
-  g.num_slots = pl.lay.num_slots;
-  g.cu = cu_seqlens;
-  g.chunk_off = cu_seqlens ? reinterpret_cast<const int32_t*>(pl.ws + pl.lay.off_chunk_off) : nullptr;
-  g.slot_map = cu_seqlens ? reinterpret_cast<const int32_t*>(pl.ws + pl.lay.off_slot_map) : nullptr;
-  if (cudaMemsetAsync(pl.ws + pl.lay.off_status, 0, 4 * sizeof(int32_t), pl.stream) != cudaSuccess) return MDN_ERR_CUDA;
   if (launch_chunk_map(pl, &t_last_launches) != cudaSuccess) return MDN_ERR_CUDA;
   BwdScratch bs;
   bwd_scratch_layout(*p, pl.lay.num_slots, &bs);
   const BwdIo io{q, k, v, beta, log_alpha, log_mu, eta, initial_S, initial_M, d_o, d_final_S, d_final_M,
                  dq, dk, dv, dbeta, dlog_alpha, dlog_mu, deta, d_initial_S, d_initial_M};
-  const cudaError_t e = launch_bwd_stepwise(pl, io, pl.ws + bwd_scratch_base(pl.lay), bs, &t_last_launches);
+  const cudaError_t e = launch_bwd_exact(pl, io, pl.ws + pl.lay.total_bytes, bs, &t_last_launches);
   if (e != cudaSuccess) { t_last_cuda_error = (int)e; return MDN_ERR_CUDA; }
   return MDN_OK;
 }

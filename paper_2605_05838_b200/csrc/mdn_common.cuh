@@ -173,11 +173,14 @@ cudaError_t launch_gate_param(const Plan& pl, const float* x_beta, const float* 
 cudaError_t launch_qk_prep(const Plan& pl, const QkNorm& qk, const void* q, const void* k, void* q_out, void* k_out,
                            int* launches);
 cudaError_t launch_out_norm_gate(const Plan& pl, const OutPost& post, void* o, int* launches);
-cudaError_t launch_intra_simt(const Plan& pl, const void* q, const void* k, int* launches);
+cudaError_t launch_intra_simt(const Plan& pl, const void* q, const void* k, const GateArgs& gates, float* TT, int* launches);
 cudaError_t launch_chain_simt(const Plan& pl, const void* q, const void* k, const void* v,
                               const float* S0, const float* M0, void* o, float* Sf, float* Mf,
                               int* launches);
-
+// ... without the output terms, keeping every chunk's start state [slot][H][2][dk][dv] and V~ [slot][H][64][dv]
+cudaError_t launch_chain_simt_keep(const Plan& pl, const void* k, const void* v, const float* S0, const float* M0,
+                                   float* states, float* vt, int* launches);
+bool simt_narrow_columns(const Plan& pl);   // value columns per CTA of the fp32 chains: 8 or 16
 
 // Tensor-core (tcgen05) path: bf16 q/k/v, dk = dv = 128.
 bool tensor_path_supported(const mdn_params& p);
@@ -200,9 +203,9 @@ cudaError_t launch_seg_combine(const Plan& pl, int G, float* E, const float* Psi
                                const float* PhiM, int* launches);
 
 
-// Backward (bwd_stepwise.cu).  Scratch offsets are relative to the scratch base the API layer places after the
+// Exact backward (bwd_exact.cu).  Scratch offsets are relative to the scratch base the API layer places after the
 // forward's workspace regions.
-struct BwdScratch { uint64_t part_q, part_k, part_g, ck, prev, total; };
+struct BwdScratch { uint64_t tt, states, adj, vt, total; };
 struct BwdIo {
   const void* q; const void* k; const void* v;
   const float* beta; const float* log_alpha; const float* log_mu; const float* eta;
@@ -212,7 +215,7 @@ struct BwdIo {
   float* dS0; float* dM0;
 };
 void bwd_scratch_layout(const mdn_params& p, int num_slots, BwdScratch* s);
-cudaError_t launch_bwd_stepwise(const Plan& pl, const BwdIo& io, char* scratch, const BwdScratch& sl, int* launches);
+cudaError_t launch_bwd_exact(const Plan& pl, const BwdIo& io, char* scratch, const BwdScratch& sl, int* launches);
 
 // Recurrent decode step (one token per sequence, state updated in place).
 cudaError_t launch_decode_step(const mdn_params& p, const void* q, const void* k, const void* v, const float* beta,

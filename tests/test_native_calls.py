@@ -35,8 +35,6 @@ def test_cpu_tensors_are_declined_and_the_binding_raises():
         with pytest.raises(ValueError):
             call()
     with pytest.raises(KeyError):
-        mdn.chunk_fwd(*a, path="nosuch")
-    with pytest.raises(KeyError):
         mdn.make_layer_ops(a[0], a[2], placement="nosuch")
 
 
