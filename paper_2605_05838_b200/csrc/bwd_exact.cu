@@ -9,12 +9,14 @@
 //                                                                         DA = G^- o dA,  dA = -tril(dR V~^T, -1),
 // the coefficient vectors' adjoints as row sums of products that dQ, dK need anyway, and the gate gradients from those
 // by the scans of Eq. 10 in reverse (bwd_gates.cuh).  Five kernels:
-//   status / chunk map;  intra_simt (scan, T, T^T, W^T);  chain_simt without output terms (the states at every chunk's start, V~);
+//   status / chunk map;  intra_simt (scan, T, T^T, W^T dO);  chain_simt without output terms (the states at every chunk's start, V~);
 //   the adjoint chain (dS', dM' at every chunk's end, dR);  the per-chunk kernel (everything else, all chunks in parallel).
 //
 // Why: the serial part of a backward is two walks over the chunks.  The token-by-token form this replaces was serial
 // over tokens (3.4 us per token and chain whatever the GPU's size: 3.4 ms for T = 1023, B H = 16); here 64 tokens cost
 // one chunk step of either chain, and the bulk of the arithmetic (20 of 28 products) is parallel over chunks.
+#include <type_traits>
+
 #include "bwd_gates.cuh"
 #include "simt_tile.cuh"
 
@@ -27,7 +29,8 @@ struct AdjArgs {
   const void* q; const void* k; const void* d_o;
   bool in_bf16, do_bf16;
   int dv;
-  const float* coef; const float* TT; const float* WT;
+  const float* coef; const float* TT;
+  const float* vp;       // W^T dO, [slot][H][64][dv]
   const float* dSf; const float* dMf;
   float scale;
   float* adj;            // [slot][H][2][dk][dv]: dS', dM' at the chunk's end
@@ -35,35 +38,32 @@ struct AdjArgs {
   float* dS0; float* dM0;
 };
 
-template <int DK, int NV> struct AdjSmem {   // float offsets; the K tile is twice buffered for fp32 input, for bf16 the raw
-  static constexpr int LDK = DK + 4;         // staging area is the second buffer
-  static constexpr int Q = 0, TT = Q + C * LDK, WT = TT + C * kLT, D = WT + C * kLT, Dot = D + 2 * NV * LDK, Zt = Dot + NV * kLT,
-                       Wd = Zt + NV * kLT, cv = Wd + 2 * C * NV * 4, K = cv + 2 * kChainCoefs * C;
-  static constexpr size_t bytes(bool bf16) {
-    return (size_t)(K + (bf16 ? 1 : 2) * C * LDK) * 4 + (bf16 ? (size_t)2 * C * DK * 2 : 0);
-  }
+template <int DK, int NV> struct AdjSmem {   // float offsets
+  static constexpr int LDK = DK + 4, LDW = 2 * NV + 4;
+  static constexpr int K = 0, Q = K + 2 * C * LDK, TT = Q + C * LDK, D = TT + C * kLT, Zt = D + 2 * NV * LDK, Wd = Zt + NV * kLT,
+                       cv = Wd + 2 * C * LDW, kFloats = cv + 2 * kChainCoefs * C;
+  static constexpr size_t bytes(bool bf16) { return (size_t)kFloats * 4 + (bf16 ? (size_t)2 * C * DK * 2 : 0); }
 };
 
 // One CTA per (sequence, head, NV value columns), chunks from last to first; the columns of dS', dM' stay in shared
-// memory.  Same structure and products as the forward chain (chain_simt.cu); the two Q terms make its state update
-// twice as long (rows of K, then rows of Q).
+// memory.  The forward chain's structure and tiles (chain_simt.cu) with W^T dO in the place of V; the two Q terms make its
+// state update twice as long (rows of K, then rows of Q).
 template <int DK, int NV>
-__global__ void __launch_bounds__(kSimtThreads, DK == 64 ? 2 : 1) adj_chain_kernel(const AdjArgs a) {
+__global__ void __launch_bounds__(kChainThreads<NV>, 1) adj_chain_kernel(const AdjArgs a) {
   extern __shared__ __align__(16) float sm[];
   using L = AdjSmem<DK, NV>;
-  constexpr int LDK = L::LDK, JT = NV / 8;
-  constexpr int DT = (DK == 64 && NV == 8) ? 2 : 4, JC = NV * DK / (kSimtThreads * DT), JG = NV / JC;
+  constexpr int TH = kChainThreads<NV>, LDK = L::LDK, LDW = L::LDW;
   float* Qs = sm + L::Q;
   float* TTm = sm + L::TT;
-  float* WTm = sm + L::WT;
   float* Ds = sm + L::D;       // [2 NV (columns of dS', then of dM')][LDK]
-  float* Dot = sm + L::Dot;    // dO^T
   float* Zt = sm + L::Zt;      // dV~^T
-  float4* Wd = reinterpret_cast<float4*>(sm + L::Wd);   // [128 rows (K, then Q)][NV]: weights of the update of dS', dM', each twice
-  uint8_t* raw = reinterpret_cast<uint8_t*>(sm + L::K + C * LDK);
+  float* Wd = sm + L::Wd;      // [128 rows (K, then Q)][LDW]: per column the weights of the update of dS', dM'
+  uint8_t* raw = reinterpret_cast<uint8_t*>(sm + L::kFloats);
   uint8_t* rawQ = raw + C * DK * 2;
 
-  const int tid = threadIdx.x, jg = tid & 7, rs = tid >> 3;
+  const int tid = threadIdx.x;
+  const StateTile<NV, 1> st_tile(tid);
+  const TriTile<NV> tri(tid);
   const int H = a.g.H, DV = a.dv, NVB = DV / NV;
   const int vb = blockIdx.x % NVB, h = (blockIdx.x / NVB) % H, seq = blockIdx.x / (NVB * H);
   const int j0 = vb * NV;
@@ -76,33 +76,19 @@ __global__ void __launch_bounds__(kSimtThreads, DK == 64 ? 2 : 1) adj_chain_kern
   auto src_of = [&](const void* p, int c) {
     return static_cast<const void*>(static_cast<const uint8_t*>(p) + ((size_t)(sq.tok0 + c * C) * H + h) * DK * es);
   };
-  auto k_tile = [&](int c) { return sm + L::K + (a.in_bf16 ? 0 : (c & 1) * C * LDK); };
   auto fetch_k = [&](int c) {
-    load_rows<DK>(k_tile(c), raw, src_of(a.k, c), a.in_bf16, (size_t)H * DK, min(C, sq.len - c * C), tid);
+    load_rows<DK, TH>(sm + L::K + (c & 1) * C * LDK, raw, src_of(a.k, c), a.in_bf16, (size_t)H * DK, min(C, sq.len - c * C), tid);
     const float* cf = a.coef + ((size_t)(sq.slot0 + c) * H + h) * MDN_NUM_COEF * C;
     if (tid < kChainCoefs * C / 4) cp16(sm + L::cv + (c & 1) * kChainCoefs * C + tid * 4, cf + tid * 4, true);
   };
   auto mat = [&](int c) { return ((size_t)(sq.slot0 + c) * H + h) * C * C; };
-  float dnext[2][JT];
-  auto load_do = [&](int c) {   // this thread's elements of the chunk's dO: rows rs + 32 i, columns jg + 8 jj
-    const int n = min(C, sq.len - c * C);
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int jj = 0; jj < JT; ++jj) {
-        const int r = rs + 32 * i;
-        dnext[i][jj] = r < n ? load_io(a.d_o, ((size_t)(sq.tok0 + c * C + r) * H + h) * DV + j0 + jg + 8 * jj, a.do_bf16) : 0.f;
-      }
-  };
 
   if (nch > 0) {
     fetch_k(nch - 1);
-    load_mat(WTm, a.WT + mat(nch - 1), tid);
-    load_mat(TTm, a.TT + mat(nch - 1), tid);
+    load_mat<TH>(TTm, a.TT + mat(nch - 1), tid);
     cp_commit();
-    load_do(nch - 1);
   }
-  for (int i = tid; i < 2 * NV * DK; i += kSimtThreads) {
+  for (int i = tid; i < 2 * NV * DK; i += TH) {
     const int jj = i % NV, d = (i / NV) % DK, which = i / (NV * DK);
     const float* src = which ? a.dMf : a.dSf;
     Ds[(which * NV + jj) * LDK + d] = src ? src[st_off + (size_t)d * DV + j0 + jj] : 0.f;
@@ -110,145 +96,70 @@ __global__ void __launch_bounds__(kSimtThreads, DK == 64 ? 2 : 1) adj_chain_kern
 
   for (int c = nch - 1; c >= 0; --c) {
     const int n = min(C, sq.len - c * C);
-    const size_t slot_h = (size_t)(sq.slot0 + c) * H + h;
-    float* Ks = k_tile(c);
+    const size_t slot_h = (size_t)(sq.slot0 + c) * H + h, tok_h = (size_t)(sq.tok0 + c * C) * H + h;
+    float* Ks = sm + L::K + (c & 1) * C * LDK;
     const float* cv = sm + L::cv + (c & 1) * kChainCoefs * C;
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int jj = 0; jj < JT; ++jj) Dot[(jg + 8 * jj) * kLT + rs + 32 * i] = dnext[i][jj];
+    float vp[st_tile.kPairs], dox[16 / tri.SL];
+    st_tile.own([&](int e, int, int r, int j) { vp[e] = __ldg(a.vp + (slot_h * C + r) * DV + j0 + j); });
+    tri.own([&](int e, int r, int j) { dox[e] = r < n ? load_io(a.d_o, (tok_h + (size_t)r * H) * DV + j0 + j, a.do_bf16) : 0.f; });
     cp_wait<0>();
     __syncthreads();   // tiles landed; the previous step's readers are done, its adjoints are written
     if (a.in_bf16) {
-      widen_tile<DK>(Ks, raw, tid);
+      widen_tile<DK, TH>(Ks, raw, tid);
       __syncthreads();
     }
     if (c > 0) fetch_k(c - 1);
-    load_rows<DK>(Qs, rawQ, src_of(a.q, c), a.in_bf16, (size_t)H * DK, n, tid);
+    load_rows<DK, TH>(Qs, rawQ, src_of(a.q, c), a.in_bf16, (size_t)H * DK, n, tid);
     cp_commit();
     {   // the adjoint pair at the chunk's end, [d][j]
       float* dst = a.adj + slot_h * 2 * DK * DV + j0;
-      for (int i = tid; i < 2 * NV * DK; i += kSimtThreads) {
+      for (int i = tid; i < 2 * NV * DK; i += TH) {
         const int j = i % NV, d = (i / NV) % DK, which = i / (NV * DK);
         dst[(size_t)which * DK * DV + (size_t)d * DV + j] = Ds[(which * NV + j) * LDK + d];
       }
     }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {   // weights of the Q rows
-      const int r = rs + 32 * i;
-      const float ws = a.scale * cv[kAbar * C + r], wm = -a.scale * cv[kB * C + r];
-#pragma unroll
-      for (int jj = 0; jj < JT; ++jj) {
-        const float x = dnext[i][jj];
-        Wd[(C + r) * NV + jg + 8 * jj] = make_float4(ws * x, ws * x, wm * x, wm * x);
-      }
-    }
+    tri.own([&](int e, int r, int j) {   // weights of the Q rows
+      *reinterpret_cast<float2*>(Wd + (C + r) * LDW + 2 * j) = make_float2(a.scale * cv[kAbar * C + r] * dox[e], -a.scale * cv[kB * C + r] * dox[e]);
+    });
 
-    // ---- 1: dV~ = W^T dO + g_S.(K dS') - g_M.(K dM'), rows rs + 32 i   (W^T is upper triangular)
-    {
-      float2 acc[2][2 * JT], wv[2][JT];
-      zero2(acc); zero2(wv);
-      dot_tile<2, 2 * JT>(acc, Ks + rs * LDK, 32 * LDK, Ds + jg * LDK, 8 * LDK, 0, DK / 4);
-      dot_tile<2, JT>(wv, WTm + rs * kLT, 32 * kLT, Dot + jg * kLT, 8 * kLT, 8, 16);
-      float2 lo[1][JT];
-#pragma unroll
-      for (int jj = 0; jj < JT; ++jj) lo[0][jj] = wv[0][jj];
-      dot_tile<1, JT>(lo, WTm + rs * kLT, 0, Dot + jg * kLT, 8 * kLT, 0, 8);
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int r = rs + 32 * i;
-        const float gs = cv[kGS * C + r], gm = cv[kGM * C + r];
-#pragma unroll
-        for (int jj = 0; jj < JT; ++jj)
-          Zt[(jg + 8 * jj) * kLT + r] = (i ? hsum(wv[1][jj]) : hsum(lo[0][jj])) + gs * hsum(acc[i][jj]) - gm * hsum(acc[i][JT + jj]);
-      }
-    }
+    // ---- 1: dV~ = W^T dO + g_S.(K dS') - g_M.(K dM')
+    st_tile.template run<DK>(Ks, Ks, Ds, [&](int e, int, int r, int j, float xs, float xm) {
+      Zt[j * kLT + r] = vp[e] + cv[kGS * C + r] * xs - cv[kGM * C + r] * xm;
+    });
     __syncthreads();
-    if (c > 0) load_mat(WTm, a.WT + mat(c - 1), tid);   // W^T has been read
-    cp_commit();
 
     // ---- 2: dR = T^T dV~  (upper triangular)
-    {
-      float2 acc[2][JT];
-      zero2(acc);
-      dot_tile<2, JT>(acc, TTm + rs * kLT, 32 * kLT, Zt + jg * kLT, 8 * kLT, 8, 16);
-      float2 lo[1][JT];
-#pragma unroll
-      for (int jj = 0; jj < JT; ++jj) lo[0][jj] = acc[0][jj];
-      dot_tile<1, JT>(lo, TTm + rs * kLT, 0, Zt + jg * kLT, 8 * kLT, 0, 8);
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int r = rs + 32 * i;
-        const float ws = -cv[kAbar * C + r], wm = cv[kAlphaBPrev * C + r];
-#pragma unroll
-        for (int jj = 0; jj < JT; ++jj) {
-          const float x = i ? hsum(acc[1][jj]) : hsum(lo[0][jj]);
-          const int j = jg + 8 * jj;
-          if (r < n) a.dv_out[((size_t)(sq.tok0 + c * C + r) * H + h) * DV + j0 + j] = x;
-          Wd[r * NV + j] = make_float4(ws * x, ws * x, wm * x, wm * x);
-        }
-      }
-    }
-    cp_wait<1>();   // K of the next step and Q are in
+    tri.template run<false>(TTm, Zt, [&](int r, int j, float x) {
+      if (r < n) a.dv_out[(tok_h + (size_t)r * H) * DV + j0 + j] = x;
+      *reinterpret_cast<float2*>(Wd + r * LDW + 2 * j) = make_float2(-cv[kAbar * C + r] * x, cv[kAlphaBPrev * C + r] * x);
+    });
+    cp_wait<0>();   // Q (and K of the next step) are in
     __syncthreads();
     if (a.in_bf16) {
-      widen_tile<DK>(Qs, rawQ, tid);
+      widen_tile<DK, TH>(Qs, rawQ, tid);
       __syncthreads();
     }
-    if (c > 0) {
-      load_mat(TTm, a.TT + mat(c - 1), tid);   // T^T has been read
-      load_do(c - 1);
-    }
+    if (c > 0) load_mat<TH>(TTm, a.TT + mat(c - 1), tid);   // T^T has been read
     cp_commit();
 
-    // ---- 3: the adjoint pair at the chunk's start, DT key rows x JC columns of both per thread (one owner per entry)
+    // ---- 3: the adjoint pair at the chunk's start (one owner per entry)
     {
-      const int lane = tid & 31, warp = tid >> 5;
-      constexpr int DB = DK / DT / 8;
-      const int d0 = ((warp % DB) * 8 + (lane & 7)) * DT, jq = (warp / DB) * 4 + (lane >> 3);
-      float2 acc[2 * JC][DT / 2];
-      zero2(acc);
-      auto update = [&](const float* kp, const float4* wp) {
-#pragma unroll 4
-        for (int r = 0; r < n; ++r) {
-          float2 kv[DT / 2];
-          if constexpr (DT == 4) {
-            const float4 k4 = lds4(kp + r * LDK);
-            kv[0] = make_float2(k4.x, k4.y); kv[1] = make_float2(k4.z, k4.w);
-          } else {
-            kv[0] = *reinterpret_cast<const float2*>(kp + r * LDK);
-          }
-#pragma unroll
-          for (int jc = 0; jc < JC; ++jc) {
-            const float4 w = wp[r * NV + JG * jc];
-#pragma unroll
-            for (int p = 0; p < DT / 2; ++p) {
-              acc[2 * jc][p] = __ffma2_rn(kv[p], make_float2(w.x, w.y), acc[2 * jc][p]);
-              acc[2 * jc + 1][p] = __ffma2_rn(kv[p], make_float2(w.z, w.w), acc[2 * jc + 1][p]);
-            }
-          }
-        }
-      };
-      update(Ks + d0, Wd + jq);
-      update(Qs + d0, Wd + C * NV + jq);
+      UpdateTile<DK, NV> up(tid);
+      up.add(Ks, Wd, n);
+      up.add(Qs, Wd + C * LDW, n);
       const float aC = cv[kAbar * C + C - 1], bC = cv[kB * C + C - 1], mC = cv[kMubar * C + C - 1];
-#pragma unroll
-      for (int jc = 0; jc < JC; ++jc) {
-        float* sp = Ds + (jq + JG * jc) * LDK + d0;
+      up.finish([&](int d, int j, float ds, float dm) {
+        float* sp = Ds + j * LDK + d;
         float* mp = sp + NV * LDK;
-#pragma unroll
-        for (int p = 0; p < DT / 2; ++p) {
-          const float2 s = *reinterpret_cast<float2*>(sp + 2 * p), m = *reinterpret_cast<float2*>(mp + 2 * p);
-          const float2 ds = acc[2 * jc][p], dm = acc[2 * jc + 1][p];
-          *reinterpret_cast<float2*>(sp + 2 * p) = make_float2(aC * s.x + ds.x, aC * s.y + ds.y);
-          *reinterpret_cast<float2*>(mp + 2 * p) = make_float2(mC * m.x - bC * s.x + dm.x, mC * m.y - bC * s.y + dm.y);
-        }
-      }
+        const float s = *sp, m = *mp;
+        *sp = aC * s + ds;
+        *mp = mC * m - bC * s + dm;
+      });
     }
   }
   cp_wait<0>();
   __syncthreads();
-  for (int i = tid; i < 2 * NV * DK; i += kSimtThreads) {
+  for (int i = tid; i < 2 * NV * DK; i += TH) {
     const int jj = i % NV, d = (i / NV) % DK, which = i / (NV * DK);
     float* dst = which ? a.dM0 : a.dS0;
     if (dst) dst[st_off + (size_t)d * DV + j0 + jj] = Ds[(which * NV + jj) * LDK + d];
@@ -269,22 +180,25 @@ struct ParArgs {
 };
 
 template <int DK, int DV> struct ParSmem {   // float offsets
-  static constexpr int LDK = DK + 4, LDV = DV + 4, LB = 36, kMat = C * kLT;
-  static constexpr int kStages = 3, kStage = DK * LB, kStageArea = kStages * kStage > 2 * kMat ? kStages * kStage : 2 * kMat;
+  static constexpr int LDK = DK + 4, LDV = DV + 4, kMat = C * kLT;
+  static constexpr int kStages = 3, kStage = DK * 32, kStageArea = kStages * kStage > 2 * kMat ? kStages * kStage : 2 * kMat;
   static constexpr int K = 0, Q = K + C * LDK, vec = Q + C * LDK, st = vec + 24 * C, tiles = st + kStageArea,
                        kTiles = 3 * C * LDV > 5 * kMat ? 3 * C * LDV : 5 * kMat, kFloats = tiles + kTiles;
   static_assert(kFloats * 4 <= 232448, "shared memory");
 };
 
-// One 256-thread CTA per (chunk, head).  The six products against states ([64 x dv] times [dv x dk]) stream the states
-// through a three-stage ring of 32-column pieces; dO, dR, V~, K, Q stay in shared memory, dQ and dK in registers (4 rows x dk / 16
-// columns per thread: 12 operand loads feed 64 packed FMAs per four terms).  Bound by the fp32 pipes: 9.5 M
-// multiply-adds per chunk and head at dk = dv = 128.
+// One 256-thread CTA per (chunk, head); its two halves of 128 threads work on different products of the same step, each
+// thread on 8 rows x dk / 16 columns (simt_tile.cuh: the tile that balances operand loads and FMAs):
+//   half 0:  V~ dS'^T (a part of dK, parked in dk),  dO S^T, dO M^T (dQ),   dO V~^T, Q K^T,  DW K
+//   half 1:  V~ dM'^T, dR S^T, dR M^T (dK),                                 dR V~^T, K K^T,  DW^T Q, (DA + DA^T) K
+// The states stream through a three-stage ring (32 value columns of S or M, or 16 of dS' and dM' each); dO, dR, V~, K, Q stay in
+// shared memory, dQ and dK in registers.  Short chunks take tiles of 2 or 4 rows.  Bound by the fp32 pipes and the
+// shared-memory port alike: 9.5 M multiply-adds per chunk and head at dk = dv = 128.
 template <int DK, int DV>
 __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const ParArgs a) {
   extern __shared__ __align__(16) float sm[];
   using L = ParSmem<DK, DV>;
-  constexpr int LDK = L::LDK, LDV = L::LDV, LB = L::LB, E2 = DK / 32, NP = DV / 32;
+  constexpr int LDK = L::LDK, LDV = L::LDV, E2 = DK / 32, NP = DV / 32;
   float* Ks = sm + L::K;
   float* Qs = sm + L::Q;
   float* vec = sm + L::vec;
@@ -308,48 +222,41 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
   if (si.seq < 0) return;
   const int n = si.n;
   const int tid = threadIdx.x, lane = tid & 31;
-  const int dg = (tid & 7) | (((tid >> 5) & 1) << 3), rl = ((tid >> 3) & 3) + 4 * (tid >> 6);   // columns dg.., rows rl + 16 i
+  const bool half1 = tid >= 128;
+  const int dg = tid & 15, rl = (tid >> 4) & 7;   // columns 2 dg + 32 e (+ 1), rows rl + 8 i
   const size_t slot_h = (size_t)slot * H + h, tok_h = (size_t)si.tok0 * H + h;
   const float* fS = a.states + slot_h * 2 * DK * DV;
   const float* aS = a.adj + slot_h * 2 * DK * DV;
   const float scale = a.scale;
 
-  // ---- the ring: piece p = (pass, 32 value columns); key row d of a state lies at ring row (d & 1) dk / 2 + d / 2, so that a
-  // thread's column PAIRS (2 dg + 32 e, + 1) are rows dg + 16 e of either half: conflict-free loads, 8-byte stores
-  auto fetch = [&](int p) {
-    if (p < 6 * NP) {
-      const int pass = p / NP, jb = p % NP;
-      const float* src = (pass < 4 ? fS + (size_t)(pass & 1) * DK * DV : aS + (size_t)(pass & 1) * DK * DV) + jb * 32;
-      float* dst = sm + L::st + (p % L::kStages) * L::kStage;
+  // ---- the ring.  Key row d of a state lies at ring row p(d) = (d & 1) dk / 2 + d / 2, so that a thread's column PAIRS are rows
+  // dg + 16 e of either half; the 16-byte pieces of a row are XOR-swizzled with the row: conflict-free loads
+  auto fetch = [&](int step) {
+    if (step < 4 * NP) {
+      float* dst = sm + L::st + (step % L::kStages) * L::kStage;
+      const bool adj = step < 2 * NP;
+      const float* src = adj ? aS + step * 16 : fS + (step < 3 * NP ? (step - 2 * NP) * 32 : (size_t)DK * DV + (step - 3 * NP) * 32);
 #pragma unroll
       for (int i = 0; i < DK * 8 / kSimtThreads; ++i) {
-        const int idx = tid + i * kSimtThreads, d = idx >> 3, c4 = (idx & 7) * 4;
-        cp16(dst + ((d & 1) * (DK / 2) + (d >> 1)) * LB + c4, src + (size_t)d * DV + c4, true);
+        const int idx = tid + i * kSimtThreads;
+        if (adj) {   // dS' rows, then dM' rows, four pieces each
+          const int which = idx / (DK * 4), d = (idx >> 2) % DK, u = idx & 3, p = (d & 1) * (DK / 2) + (d >> 1);
+          cp16(dst + (which * DK + p) * 16 + ((u ^ (p >> 1)) & 3) * 4, src + (size_t)which * DK * DV + (size_t)d * DV + u * 4, true);
+        } else {
+          const int d = idx >> 3, u = idx & 7, p = (d & 1) * (DK / 2) + (d >> 1);
+          cp16(dst + p * 32 + ((u ^ p) & 7) * 4, src + (size_t)d * DV + u * 4, true);
+        }
       }
     }
     cp_commit();
   };
-  auto load_io_rows = [&](auto width, float* tile, const void* src, bool bf16) {   // 64 rows of one head of an i/o tensor
-    constexpr int D = decltype(width)::value;
-    if (!bf16) { load_rows<D>(tile, nullptr, static_cast<const float*>(src) + tok_h * D, false, (size_t)H * D, n, tid); return; }
-    for (int i = tid; i < C * (D / 8); i += kSimtThreads) {
-      const int r = i / (D / 8), c = (i % (D / 8)) * 8;
-      uint4 u = make_uint4(0u, 0u, 0u, 0u);
-      if (r < n) u = __ldg(reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(src) + (tok_h + (size_t)r * H) * D + c));
-      const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-      float f[8];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) { f[2 * e] = __uint_as_float(w[e] << 16); f[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u); }
-      *reinterpret_cast<float4*>(tile + r * (D + 4) + c) = make_float4(f[0], f[1], f[2], f[3]);
-      *reinterpret_cast<float4*>(tile + r * (D + 4) + c + 4) = make_float4(f[4], f[5], f[6], f[7]);
-    }
-  };
-  load_io_rows(std::integral_constant<int, DV>{}, Do, a.d_o, a.do_bf16);
-  load_io_rows(std::integral_constant<int, DK>{}, Qs, a.q, a.in_bf16);
-  load_io_rows(std::integral_constant<int, DK>{}, Ks, a.k, a.in_bf16);
-  load_rows<DV>(Dr, nullptr, a.dr + tok_h * DV, false, (size_t)H * DV, n, tid);
+  auto head = [&](const void* p, bool bf16, int D) { return static_cast<const void*>(static_cast<const uint8_t*>(p) + tok_h * D * (bf16 ? 2 : 4)); };
   load_rows<DV>(Vt, nullptr, a.vt + slot_h * C * DV, false, DV, C, tid);
+  load_io_rows(Ks, head(a.k, a.in_bf16, DK), a.in_bf16, DK, (size_t)H * DK, n, tid);
   fetch(0);
+  load_io_rows(Do, head(a.d_o, a.do_bf16, DV), a.do_bf16, DV, (size_t)H * DV, n, tid);
+  load_io_rows(Qs, head(a.q, a.in_bf16, DK), a.in_bf16, DK, (size_t)H * DK, n, tid);
+  load_rows<DV>(Dr, nullptr, a.dr + tok_h * DV, false, (size_t)H * DV, n, tid);
   fetch(1);
 
   // ---- vectors: the chain's coefficients, the gates, zeroed adjoints
@@ -386,146 +293,183 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
     }
   }
 
-  float2 dQ[4][E2], dK[4][E2];
-  zero2(dQ); zero2(dK);
-  int p = 0;
-  // one pass: G = A B^T against the next state of the ring;  acc += w.G;  a coefficient vector's adjoint += sign sum_d G o X
-  auto pass = [&](const float* A, float2 (&acc)[4][E2], const float* w, float wf, const float* X, float* dvec, float sign) {
-    float2 G[4][2 * E2];
-    zero2(G);
-#pragma unroll 1
-    for (int jb = 0; jb < NP; ++jb, ++p) {
-      cp_wait<1>();
-      __syncthreads();   // piece p is in; piece p - 1 has been read: its stage takes p + 2
-      fetch(p + 2);
-      dot_tile<4, 2 * E2>(G, A + rl * LDV + jb * 32, 16 * LDV, sm + L::st + (p % L::kStages) * L::kStage + dg * LB, 16 * LB, 0, 8);
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = rl + 16 * i;
-      const float wr = wf * w[r];
-      float s = 0.f;
-#pragma unroll
-      for (int e = 0; e < E2; ++e) {
-        const float2 g = make_float2(hsum(G[i][e]), hsum(G[i][e + E2]));
-        const float2 x = *reinterpret_cast<const float2*>(X + r * LDK + 2 * dg + 32 * e);
-        acc[i][e] = __ffma2_rn(make_float2(wr, wr), g, acc[i][e]);
-        s = fmaf(g.x, x.x, fmaf(g.y, x.y, s));
-      }
-      s += __shfl_xor_sync(0xffffffffu, s, 1);
-      s += __shfl_xor_sync(0xffffffffu, s, 2);
-      s += __shfl_xor_sync(0xffffffffu, s, 4);
-      if ((tid & 7) == 0) atomicAdd(dvec + r, sign * s);
-    }
-  };
-  pass(Do, dQ, V(vAbar), scale, Qs, V(vdAbar), scale);     // dO S^T
-  pass(Do, dQ, V(vB), -scale, Qs, V(vdB), -scale);         // dO M^T
-  pass(Dr, dK, V(vAbar), -1.f, Ks, V(vdAbar), -1.f);       // dR S^T
-  pass(Dr, dK, V(vP), 1.f, Ks, V(vdP), 1.f);               // dR M^T
-  pass(Vt, dK, V(vGS), 1.f, Ks, V(vdGS), 1.f);             // V~ dS'^T
-  pass(Vt, dK, V(vGM), -1.f, Ks, V(vdGM), -1.f);           // V~ dM'^T
-  cp_wait<0>();
-  __syncthreads();   // the ring has been read: gamma, m take its place
-
-  if (tid < C) {          // gamma by the column recurrence of Eq. 10 (thread = column), zero above the diagonal
-    const int i = tid;
-    float m = 1.f, gam = 0.f;
-#pragma unroll 4
-    for (int r = 0; r < C; ++r) {
-      if (r > i) m *= V(vMu)[r];
-      if (r >= i) gam = fmaf(V(vAlpha)[r], gam, V(vBeta)[r] * m);
-      Gam[r * kLT + i] = r >= i ? gam : 0.f;
-    }
-  } else if (tid < 2 * C) {   // m_{r,i} = mu_{i+1} .. mu_r
-    const int i = tid - C;
-    float m = 1.f;
-#pragma unroll 4
-    for (int r = 0; r < C; ++r) {
-      if (r > i) m *= V(vMu)[r];
-      Mm[r * kLT + i] = r >= i ? m : 0.f;
-    }
-  }
-  // ---- the four 64 x 64 products, lower triangle in 16 x 16 blocks: rows rl + 16 i, columns dg + 16 e, e <= i
-  auto product = [&](float (&out)[4][4], const float* A, int lda, const float* B, int ldb, int K) {
-    float2 acc[4][4];
+  auto body = [&](auto rows_tag) {
+    constexpr int R = decltype(rows_tag)::value;   // rows rl + 8 i, i < R, cover the chunk's n tokens
+    float2 acc[R][E2];                             // half 0: dQ, half 1: dK
     zero2(acc);
+    int step = 0;
+    // G = A B^T over the next `steps` stages of the ring (cols = 16 or 32 value columns each); f(i, e, r, column pair of G)
+    auto product = [&](const float* A, int steps, auto cols_tag, auto f, const float* X, float* dvec, float sign) {
+      constexpr int kCols = decltype(cols_tag)::value;
+      float2 G[R][2 * E2];
+      zero2(G);
+      const int swz = kCols == 16 ? (dg >> 1) & 3 : dg & 7;
 #pragma unroll 1
-    for (int k = 0; k < K; k += 4) {
-      float4 av[4];
+      for (int jb = 0; jb < steps; ++jb, ++step) {
+        cp_wait<1>();
+        __syncthreads();   // this step's stage is in; the previous step's has been read and takes step + 2
+        fetch(step + 2);
+        const float* b0 = sm + L::st + (step % L::kStages) * L::kStage + (kCols == 16 && half1 ? DK * 16 : 0) + dg * kCols;
+        const float* a0 = A + rl * LDV + jb * kCols;
+#pragma unroll 2
+        for (int k = 0; k < kCols / 4; ++k) {
+          float4 av[R];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) av[i] = lds4(A + (rl + 16 * i) * lda + k);
+          for (int i = 0; i < R; ++i) av[i] = lds4(a0 + 8 * i * LDV + 4 * k);
+#pragma unroll
+          for (int e = 0; e < 2 * E2; ++e) {
+            const float4 bv = lds4(b0 + 16 * e * kCols + ((k ^ swz) << 2));
+#pragma unroll
+            for (int i = 0; i < R; ++i) fma4(G[i][e], av[i], bv);
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < R; ++i) {   // row sums of G o X are the adjoint of the product's coefficient vector
+        const int r = rl + 8 * i;
+        float s = 0.f;
+#pragma unroll
+        for (int e = 0; e < E2; ++e) {
+          const float2 g = make_float2(hsum(G[i][e]), hsum(G[i][e + E2]));
+          const float2 x = *reinterpret_cast<const float2*>(X + r * LDK + 2 * dg + 32 * e);
+          s = fmaf(g.x, x.x, fmaf(g.y, x.y, s));
+          f(i, e, r, g);
+        }
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        s += __shfl_xor_sync(0xffffffffu, s, 4);
+        s += __shfl_xor_sync(0xffffffffu, s, 8);
+        if (dg == 0) atomicAdd(dvec + r, sign * s);
+      }
+    };
+    auto dk_at = [&](int r, int e) { return reinterpret_cast<float2*>(a.dk + (tok_h + (size_t)r * H) * DK + 2 * dg + 32 * e); };
+    auto add = [&](int i, int e, float w, float2 g) { acc[i][e] = __ffma2_rn(make_float2(w, w), g, acc[i][e]); };
+    product(Vt, 2 * NP, std::integral_constant<int, 16>{},
+            [&](int i, int e, int r, float2 g) {
+              if (half1) add(i, e, -V(vGM)[r], g);
+              else if (r < n) *dk_at(r, e) = make_float2(V(vGS)[r] * g.x, V(vGS)[r] * g.y);
+            },
+            Ks, V(half1 ? vdGM : vdGS), half1 ? -1.f : 1.f);
+    const float* A = half1 ? Dr : Do;
+    const float* X = half1 ? Ks : Qs;
+    const float wA = half1 ? -1.f : scale, wB = half1 ? 1.f : -scale;
+    const float* vb = V(half1 ? vP : vB);
+    product(A, NP, std::integral_constant<int, 32>{}, [&](int i, int e, int r, float2 g) { add(i, e, wA * V(vAbar)[r], g); }, X,
+            V(vdAbar), wA);
+    product(A, NP, std::integral_constant<int, 32>{}, [&](int i, int e, int r, float2 g) { add(i, e, wB * vb[r], g); }, X,
+            V(half1 ? vdP : vdB), wB);
+    cp_wait<0>();
+    __syncthreads();   // the ring has been read: gamma, m take its place
+
+    if (tid < C) {          // gamma by the column recurrence of Eq. 10 (thread = column), zero above the diagonal
+      const int i = tid;
+      float m = 1.f, gam = 0.f;
+#pragma unroll 4
+      for (int r = 0; r < C; ++r) {
+        if (r > i) m *= V(vMu)[r];
+        if (r >= i) gam = fmaf(V(vAlpha)[r], gam, V(vBeta)[r] * m);
+        Gam[r * kLT + i] = r >= i ? gam : 0.f;
+      }
+    } else if (tid >= 128 && tid < 128 + C) {   // m_{r,i} = mu_{i+1} .. mu_r
+      const int i = tid - 128;
+      float m = 1.f;
+#pragma unroll 4
+      for (int r = 0; r < C; ++r) {
+        if (r > i) m *= V(vMu)[r];
+        Mm[r * kLT + i] = r >= i ? m : 0.f;
+      }
+    }
+    // ---- the four 64 x 64 products, lower triangle: rows rl + 8 i, columns dg + 16 e, e <= i / 2
+    auto square = [&](float (&out)[R][4], const float* A, int lda, const float* B, int ldb, int K) {
+      float2 t[R][4];
+      zero2(t);
+#pragma unroll 1
+      for (int k = 0; k < K; k += 4) {
+        float4 av[R];
+#pragma unroll
+        for (int i = 0; i < R; ++i) av[i] = lds4(A + (rl + 8 * i) * lda + k);
+#pragma unroll
+        for (int e = 0; e < (R + 1) / 2; ++e) {
+          const float4 bv = lds4(B + (dg + 16 * e) * ldb + k);
+#pragma unroll
+          for (int i = 2 * e; i < R; ++i) fma4(t[i][e], av[i], bv);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) out[i][e] = hsum(t[i][e]);
+    };
+    float P[R][4], XK[R][4];
+    square(P, A, LDV, Vt, LDV, DV);      // dO V~^T | dR V~^T
+    square(XK, X, LDK, Ks, LDK, DK);     // Q K^T   | K K^T
+    __syncthreads();   // dO, dR, V~ have been read; gamma, m complete
+    // (rows past the tiles' reach: the matrices' rows and columns there are cleared for the gate gradients below)
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const float4 bv = lds4(B + (dg + 16 * e) * ldb + k);
-#pragma unroll
-        for (int i = e; i < 4; ++i) fma4(acc[i][e], av[i], bv);
+        const int r = rl + 8 * i, c = dg + 16 * e;
+        const float et = V(vEta)[c];
+        const float p = i < R ? P[i < R ? i : 0][e] : 0.f, xk = i < R ? XK[i < R ? i : 0][e] : 0.f;
+        if (!half1) {
+          const float dOVt = (r < n && c <= r) ? p : 0.f;
+          const float dw = scale * Gam[r * kLT + c] * et * dOVt;
+          DW[r * kLT + c] = dw;
+          DWT[c * kLT + r] = dw;
+          dGe[r * kLT + c] = scale * dOVt * xk;
+        } else {
+          const float dA = (r < n && c < r) ? -p : 0.f;
+          const float da = (r > 0 ? V(vAlpha)[r] * Gam[(r - 1) * kLT + c] * et : 0.f) * dA;
+          if (c < r) { DAS[r * kLT + c] = da; DAS[c * kLT + r] = da; }
+          else if (c == r) DAS[r * kLT + r] = 0.f;
+          dGm[r * kLT + c] = dA * xk;
+        }
       }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) out[i][e] = hsum(acc[i][e]);
-  };
-  float P1[4][4], P2[4][4], QK[4][4], KK[4][4];
-  product(P1, Do, LDV, Vt, LDV, DV);      // dO V~^T
-  product(P2, Dr, LDV, Vt, LDV, DV);      // dR V~^T
-  product(QK, Qs, LDK, Ks, LDK, DK);
-  product(KK, Ks, LDK, Ks, LDK, DK);
-  __syncthreads();   // dO, dR, V~ have been read; gamma, m complete
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int r = rl + 16 * i, c = dg + 16 * e;
-      const float dOVt = (r < n && c <= r) ? P1[i][e] : 0.f;
-      const float dA = (r < n && c < r) ? -P2[i][e] : 0.f;
-      const float et = V(vEta)[c];
-      const float dw = scale * Gam[r * kLT + c] * et * dOVt;
-      const float da = (r > 0 ? V(vAlpha)[r] * Gam[(r - 1) * kLT + c] * et : 0.f) * dA;
-      DW[r * kLT + c] = dw;
-      DWT[c * kLT + r] = dw;
-      if (c < r) { DAS[r * kLT + c] = da; DAS[c * kLT + r] = da; }
-      else if (c == r) DAS[r * kLT + r] = 0.f;
-      dGe[r * kLT + c] = scale * dOVt * QK[i][e];
-      dGm[r * kLT + c] = dA * KK[i][e];
-    }
-  __syncthreads();
-  // ---- dQ += DW K;  dK += DW^T Q + (DA + DA^T) K
-  auto rows_times = [&](float2 (&acc)[4][E2], const float* A, const float* B) {
+    __syncthreads();
+    // ---- dQ += DW K;  dK += DW^T Q + (DA + DA^T) K
+    auto rows_times = [&](const float* A, const float* B) {
 #pragma unroll 1
-    for (int k = 0; k < n; k += 4) {
-      float4 av[4];
+      for (int k = 0; k < n; k += 4) {
+        float4 av[R];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) av[i] = lds4(A + (rl + 16 * i) * kLT + k);
+        for (int i = 0; i < R; ++i) av[i] = lds4(A + (rl + 8 * i) * kLT + k);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        float2 b[E2];
+        for (int u = 0; u < 4; ++u) {
+          float2 b[E2];
 #pragma unroll
-        for (int e = 0; e < E2; ++e) b[e] = *reinterpret_cast<const float2*>(B + (k + u) * LDK + 2 * dg + 32 * e);
+          for (int e = 0; e < E2; ++e) b[e] = *reinterpret_cast<const float2*>(B + (k + u) * LDK + 2 * dg + 32 * e);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float x = u == 0 ? av[i].x : u == 1 ? av[i].y : u == 2 ? av[i].z : av[i].w;
+          for (int i = 0; i < R; ++i) {
+            const float x = u == 0 ? av[i].x : u == 1 ? av[i].y : u == 2 ? av[i].z : av[i].w;
 #pragma unroll
-          for (int e = 0; e < E2; ++e) acc[i][e] = __ffma2_rn(make_float2(x, x), b[e], acc[i][e]);
+            for (int e = 0; e < E2; ++e) acc[i][e] = __ffma2_rn(make_float2(x, x), b[e], acc[i][e]);
+          }
+        }
+      }
+    };
+    rows_times(half1 ? DWT : DW, half1 ? Qs : Ks);
+    if (half1) rows_times(DAS, Ks);
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int r = rl + 8 * i;
+      if (r < n) {
+#pragma unroll
+        for (int e = 0; e < E2; ++e) {
+          if (!half1) {
+            *reinterpret_cast<float2*>(a.dq + (tok_h + (size_t)r * H) * DK + 2 * dg + 32 * e) = acc[i][e];
+          } else {   // half 0's part has been waiting there
+            float2* at = dk_at(r, e);
+            const float2 x = *at;
+            *at = make_float2(x.x + acc[i][e].x, x.y + acc[i][e].y);
+          }
         }
       }
     }
   };
-  rows_times(dQ, DW, Ks);
-  rows_times(dK, DWT, Qs);
-  rows_times(dK, DAS, Ks);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = rl + 16 * i;
-    if (r < n) {
-#pragma unroll
-      for (int e = 0; e < E2; ++e) {
-        const size_t at = (tok_h + (size_t)r * H) * DK + 2 * dg + 32 * e;
-        *reinterpret_cast<float2*>(a.dq + at) = dQ[i][e];
-        *reinterpret_cast<float2*>(a.dk + at) = dK[i][e];
-      }
-    }
-  }
+  if (n > 32) body(std::integral_constant<int, 8>{});
+  else if (n > 16) body(std::integral_constant<int, 4>{});
+  else body(std::integral_constant<int, 2>{});
   __syncthreads();   // DW, DW^T, DA have been read: the gate gradients' work matrices take their places
   gate_gradients(vec, GateMats{Gam, Mm, dGe, dGm, DW, DWT}, DAS, n, tok_h, H, a.gates);
 }
@@ -534,7 +478,7 @@ template <int DK, int NV> cudaError_t launch_adj(const Plan& pl, const AdjArgs& 
   const size_t smem = AdjSmem<DK, NV>::bytes(a.in_bf16);
   const cudaError_t e = cudaFuncSetAttribute(adj_chain_kernel<DK, NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(adj_chain_kernel<DK, NV>, dim3((unsigned)pl.geom.num_seqs * pl.p.H * (a.dv / NV)), dim3(kSimtThreads), smem,
+  return launch_pdl(adj_chain_kernel<DK, NV>, dim3((unsigned)pl.geom.num_seqs * pl.p.H * (a.dv / NV)), dim3(kChainThreads<NV>), smem,
                     pl.stream, a);
 }
 template <int DK, int DV> cudaError_t launch_par(const Plan& pl, const ParArgs& a) {
@@ -554,6 +498,7 @@ void bwd_scratch_layout(const mdn_params& p, int num_slots, BwdScratch* s) {
   s->states = take(mats * 2 * p.dk * p.dv);
   s->adj = take(mats * 2 * p.dk * p.dv);
   s->vt = take(mats * C * p.dv);
+  s->vp = take(mats * C * p.dv);
   s->total = off;
 }
 
@@ -562,7 +507,8 @@ cudaError_t launch_bwd_exact(const Plan& pl, const BwdIo& io, char* scratch, con
   float* states = reinterpret_cast<float*>(scratch + sl.states);
   float* adj = reinterpret_cast<float*>(scratch + sl.adj);
   float* vt = reinterpret_cast<float*>(scratch + sl.vt);
-  cudaError_t e = launch_intra_simt(pl, io.q, io.k, GateArgs{io.beta, io.log_alpha, io.log_mu, io.eta}, tt, launches);
+  float* vp = reinterpret_cast<float*>(scratch + sl.vp);
+  cudaError_t e = launch_intra_simt(pl, io.q, io.k, GateArgs{io.beta, io.log_alpha, io.log_mu, io.eta}, IntraBwd{io.d_o, tt, vp}, launches);
   if (e != cudaSuccess) return e;
   e = launch_chain_simt_keep(pl, io.k, io.v, io.S0, io.M0, states, vt, launches);
   if (e != cudaSuccess) return e;
@@ -573,7 +519,7 @@ cudaError_t launch_bwd_exact(const Plan& pl, const BwdIo& io, char* scratch, con
   a.q = io.q; a.k = io.k; a.d_o = io.d_o;
   a.in_bf16 = in_bf16; a.do_bf16 = do_bf16;
   a.dv = pl.p.dv;
-  a.coef = coef; a.TT = tt; a.WT = reinterpret_cast<const float*>(pl.ws + pl.lay.off_W);
+  a.coef = coef; a.TT = tt; a.vp = vp;
   a.dSf = io.dSf; a.dMf = io.dMf;
   a.scale = pl.p.scale;
   a.adj = adj; a.dv_out = io.dv;

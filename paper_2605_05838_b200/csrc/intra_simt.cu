@@ -15,6 +15,8 @@
 // of gamma run on three warps while K and Q are on their way, [K; Q] K^T is one register-tiled product that skips the
 // 8 x 16 blocks above the diagonal, and the inverse is seven short parallel steps instead of 64 dependent rows.
 // Two CTAs per SM (93 KB at dk = 128): A, W and T live where K, Q and Gamma were.
+#include <type_traits>
+
 #include "coeff_scan.cuh"
 #include "simt_tile.cuh"
 
@@ -29,14 +31,17 @@ struct IntraArgs {
   GateArgs gates;
   GateParam gp;
   float scale;
-  float* T; float* W;     // transposed = false: T, W
-  float* TT;              // transposed = true:  T, W^T (in W) and T^T (the exact backward reads those)
-  bool transposed;
+  float* T; float* W;
+  IntraBwd bwd;           // set for the exact backward: T, T^T and W^T dO leave instead of T and W
+  int dv;
+  bool do_bf16;
 };
 
 template <int DK> struct IntraSmem {   // float offsets
   static constexpr int LDK = DK + 4, K = 0, Q = K + C * LDK, G = Q + C * LDK, P = G + C * kLT, cv = P + 32 * 36, kFloats = cv + 4 * C;
-  static constexpr size_t bytes(bool bf16) { return (size_t)kFloats * 4 + (bf16 ? (size_t)2 * C * DK * 2 : 0); }
+  static constexpr size_t bytes(bool bf16, int dv_bwd) {   // dv_bwd: dv for the exact backward (the dO tile), else 0
+    return (size_t)kFloats * 4 + (bf16 ? (size_t)2 * C * DK * 2 : 0) + (dv_bwd ? (size_t)C * (dv_bwd + 4) * 4 : 0);
+  }
 };
 
 template <int DK>
@@ -63,6 +68,11 @@ __global__ void __launch_bounds__(kSimtThreads, 2) intra_simt_kernel(const Intra
   const size_t es = a.in_bf16 ? 2 : 4, row0 = ((size_t)si.tok0 * H + h) * DK * es;
   load_rows<DK>(Ks, raw, static_cast<const uint8_t*>(a.k) + row0, a.in_bf16, (size_t)H * DK, si.n, tid);
   load_rows<DK>(Qs, raw + C * DK * 2, static_cast<const uint8_t*>(a.q) + row0, a.in_bf16, (size_t)H * DK, si.n, tid);
+  const int LDV = a.dv + 4;
+  float* Do = reinterpret_cast<float*>(raw + (a.in_bf16 ? 2 * C * DK * 2 : 0));
+  if (a.bwd.TT != nullptr)
+    load_io_rows(Do, static_cast<const uint8_t*>(a.bwd.d_o) + ((size_t)si.tok0 * H + h) * a.dv * (a.do_bf16 ? 2 : 4), a.do_bf16, a.dv,
+                 (size_t)H * a.dv, si.n, tid);
   cp_commit();
 
   float* cf = a.coef + ((size_t)slot * H + h) * MDN_NUM_COEF * C;
@@ -168,6 +178,33 @@ __global__ void __launch_bounds__(kSimtThreads, 2) intra_simt_kernel(const Intra
   __syncthreads();   // A, W complete; Gamma has been read: T takes its place
 
   const size_t mat = ((size_t)slot * H + h) * C * C;
+  if (a.bwd.TT != nullptr) {   // W^T dO: eight rows per warp (W read as it lies: its row r is the update by dO's row r)
+    const int i0 = warp * 8;
+    float* dst = a.bwd.vp + (((size_t)slot * H + h) * C + i0) * a.dv;
+    auto columns = [&](auto width) {
+      constexpr int W2 = decltype(width)::value;   // float2 column pairs per lane
+      float2 acc[8][W2];
+      zero2(acc);
+#pragma unroll 2
+      for (int r = i0; r < si.n; ++r) {
+        const float4 wa = lds4(Ws + r * kLT + i0), wb = lds4(Ws + r * kLT + i0 + 4);
+        const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+        float2 d[W2];
+#pragma unroll
+        for (int e = 0; e < W2; ++e) d[e] = *reinterpret_cast<const float2*>(Do + r * LDV + 2 * lane + 64 * e);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+          for (int e = 0; e < W2; ++e) acc[i][e] = __ffma2_rn(make_float2(w[i], w[i]), d[e], acc[i][e]);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int e = 0; e < W2; ++e) *reinterpret_cast<float2*>(dst + (size_t)i * a.dv + 2 * lane + 64 * e) = acc[i][e];
+    };
+    if (a.dv == 64) columns(std::integral_constant<int, 1>{});
+    else columns(std::integral_constant<int, 2>{});
+  }
   // step 1: the four diagonal blocks (thread = block, column); the other threads clear the blocks above the diagonal and
   // write W out
   if (tid < C) {
@@ -192,11 +229,7 @@ __global__ void __launch_bounds__(kSimtThreads, 2) intra_simt_kernel(const Intra
     for (int i = tid - C; i < C * 16; i += kSimtThreads - C) {
       const int r = i >> 4, c = (i & 15) * 4;
       if ((c >> 4) > (r >> 4)) *reinterpret_cast<float4*>(Ts + r * kLT + c) = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (!a.transposed) {
-        *reinterpret_cast<float4*>(a.W + mat + i * 4) = lds4(Ws + r * kLT + c);
-      } else {   // row r of W^T
-        *reinterpret_cast<float4*>(a.W + mat + i * 4) = make_float4(Ws[c * kLT + r], Ws[(c + 1) * kLT + r], Ws[(c + 2) * kLT + r], Ws[(c + 3) * kLT + r]);
-      }
+      if (a.bwd.TT == nullptr) *reinterpret_cast<float4*>(a.W + mat + i * 4) = lds4(Ws + r * kLT + c);
     }
   }
   __syncthreads();
@@ -246,13 +279,13 @@ __global__ void __launch_bounds__(kSimtThreads, 2) intra_simt_kernel(const Intra
   for (int i = tid; i < C * 16; i += kSimtThreads) {
     const int r = i >> 4, c = (i & 15) * 4;
     *reinterpret_cast<float4*>(a.T + mat + i * 4) = lds4(Ts + r * kLT + c);
-    if (a.transposed)
-      *reinterpret_cast<float4*>(a.TT + mat + i * 4) = make_float4(Ts[c * kLT + r], Ts[(c + 1) * kLT + r], Ts[(c + 2) * kLT + r], Ts[(c + 3) * kLT + r]);
+    if (a.bwd.TT != nullptr)
+      *reinterpret_cast<float4*>(a.bwd.TT + mat + i * 4) = make_float4(Ts[c * kLT + r], Ts[(c + 1) * kLT + r], Ts[(c + 2) * kLT + r], Ts[(c + 3) * kLT + r]);
   }
 }
 
 template <int DK> cudaError_t launch_one(const Plan& pl, const IntraArgs& a) {
-  const size_t smem = IntraSmem<DK>::bytes(a.in_bf16);
+  const size_t smem = IntraSmem<DK>::bytes(a.in_bf16, a.bwd.TT ? a.dv : 0);
   const cudaError_t e = cudaFuncSetAttribute(intra_simt_kernel<DK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   return launch_pdl(intra_simt_kernel<DK>, dim3((unsigned)pl.geom.num_slots * pl.p.H), dim3(kSimtThreads), smem, pl.stream, a);
@@ -261,8 +294,8 @@ template <int DK> cudaError_t launch_one(const Plan& pl, const IntraArgs& a) {
 }  // namespace
 
 // gates all NULL: the coefficient vectors are in the workspace; else this kernel runs the scan and writes them.
-// TT != NULL: T goes to its place in the workspace, W^T to W's, T^T to TT (the exact backward's operands).
-cudaError_t launch_intra_simt(const Plan& pl, const void* q, const void* k, const GateArgs& gates, float* TT, int* launches) {
+// bwd: the exact backward's extra operands (W is then not written).
+cudaError_t launch_intra_simt(const Plan& pl, const void* q, const void* k, const GateArgs& gates, const IntraBwd& bwd, int* launches) {
   IntraArgs a{};
   a.g = pl.geom;
   a.q = q; a.k = k;
@@ -273,8 +306,9 @@ cudaError_t launch_intra_simt(const Plan& pl, const void* q, const void* k, cons
   a.scale = pl.p.scale;
   a.T = reinterpret_cast<float*>(pl.ws + pl.lay.off_T);
   a.W = reinterpret_cast<float*>(pl.ws + pl.lay.off_W);
-  a.TT = TT;
-  a.transposed = TT != nullptr;
+  a.bwd = bwd;
+  a.dv = pl.p.dv;
+  a.do_bf16 = pl.p.o_dtype == MDN_BF16;
   const cudaError_t e = pl.p.dk == 64 ? launch_one<64>(pl, a) : launch_one<128>(pl, a);
   if (e == cudaSuccess) ++*launches;
   return e;

@@ -104,7 +104,7 @@ static mdn_status run_intra(const Plan& pl, const void* q, const void* k, int* l
                             const GateArgs& gates = GateArgs{nullptr, nullptr, nullptr, nullptr}) {
   if (!q || !k || !aligned(q, 16) || !aligned(k, 16)) return MDN_ERR_INVALID_ARG;
   cudaError_t e = pl.p.path == MDN_PATH_TENSOR ? launch_intra_tensor(pl, q, k, gates, launches)
-                                               : launch_intra_simt(pl, q, k, gates, nullptr, launches);
+                                               : launch_intra_simt(pl, q, k, gates, IntraBwd{}, launches);
   if (e != cudaSuccess) t_last_cuda_error = (int)e;
   return e == cudaSuccess ? MDN_OK : MDN_ERR_CUDA;
 }

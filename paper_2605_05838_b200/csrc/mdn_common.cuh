@@ -173,7 +173,9 @@ cudaError_t launch_gate_param(const Plan& pl, const float* x_beta, const float* 
 cudaError_t launch_qk_prep(const Plan& pl, const QkNorm& qk, const void* q, const void* k, void* q_out, void* k_out,
                            int* launches);
 cudaError_t launch_out_norm_gate(const Plan& pl, const OutPost& post, void* o, int* launches);
-cudaError_t launch_intra_simt(const Plan& pl, const void* q, const void* k, const GateArgs& gates, float* TT, int* launches);
+// What the exact backward wants besides (all NULL: nothing): T^T, and W^T dO ([slot][H][64][dv]) in the place of W.
+struct IntraBwd { const void* d_o; float* TT; float* vp; };
+cudaError_t launch_intra_simt(const Plan& pl, const void* q, const void* k, const GateArgs& gates, const IntraBwd& bwd, int* launches);
 cudaError_t launch_chain_simt(const Plan& pl, const void* q, const void* k, const void* v,
                               const float* S0, const float* M0, void* o, float* Sf, float* Mf,
                               int* launches);
@@ -205,7 +207,7 @@ cudaError_t launch_seg_combine(const Plan& pl, int G, float* E, const float* Psi
 
 // Exact backward (bwd_exact.cu).  Scratch offsets are relative to the scratch base the API layer places after the
 // forward's workspace regions.
-struct BwdScratch { uint64_t tt, states, adj, vt, total; };
+struct BwdScratch { uint64_t tt, states, adj, vt, vp, total; };
 struct BwdIo {
   const void* q; const void* k; const void* v;
   const float* beta; const float* log_alpha; const float* log_mu; const float* eta;
