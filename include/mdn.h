@@ -375,19 +375,32 @@ mdn_status mdn_chunk_bwd_saved(const mdn_params* p,
                                float* d_initial_S, float* d_initial_M,
                                void* workspace, size_t workspace_bytes, void* cuda_stream);
 
+/* mdn_chunk_bwd_saved with dq, dk, dv in the i/o dtype (bf16: each value rounded once from its fp32 sum), which is what an
+ * autograd function hands on: saves the fp32 gradients' round trip through memory. */
+mdn_status mdn_chunk_bwd_saved_io(const mdn_params* p,
+                                  const void* q, const void* k, const void* v,
+                                  const float* beta, const float* log_alpha, const float* log_mu, const float* eta,
+                                  const int32_t* cu_seqlens,
+                                  void* fwd_workspace, size_t fwd_workspace_bytes, const void* chunk_states,
+                                  const void* d_o, const float* d_final_S, const float* d_final_M,
+                                  void* dq, void* dk, void* dv,
+                                  float* dbeta, float* dlog_alpha, float* dlog_mu, float* deta,
+                                  float* d_initial_S, float* d_initial_M,
+                                  void* workspace, size_t workspace_bytes, void* cuda_stream);
+
 /*
  * Backward of mdn_chunk_fwd (Section 3.1: the training pass differentiates the same recurrence; like the paper's
- * kernels this keeps no per-token states and rebuilds them from per-chunk checkpoints):
+ * kernels this keeps no per-token states and rebuilds what it needs chunk by chunk from the chunk-start states):
  * given d_o = dL/do ([B,T,H,dv], o_dtype) and optionally dL/d(final_S), dL/d(final_M) ([N,H,dk,dv] float32, NULL =
  * zero), writes the float32 gradients
  *     dq, dk [B,T,H,dk];  dv [B,T,H,dv];  dbeta, dlog_alpha, dlog_mu, deta [B,T,H] (deta may be NULL);
  *     d_initial_S, d_initial_M [N,H,dk,dv] (either may be NULL).
  * q, k, v, the gates, the initial states, cu_seqlens, p: exactly the forward call's.  The pass recomputes the
- * forward itself, token by token in float32 (any dk, dv in {64, 128}; p->path and p->segments are ignored), so it
+ * forward's states itself, in float32 throughout (any dk, dv in {64, 128}; p->path and p->segments are ignored), so it
  * does not need the forward's outputs.  Workspace: mdn_chunk_bwd_workspace_bytes(p) bytes, 256-byte aligned,
- * scratch.  Same ownership, stream and error rules as mdn_chunk_fwd.  dv and the initial states' gradients are
- * bit-reproducible; dq, dk and the gate gradients sum over value columns through shared-memory floating-point
- * atomics, so their last bits can differ from run to run.
+ * scratch.  Same ownership, stream and error rules as mdn_chunk_fwd.  dq, dk, dv and the initial states' gradients are
+ * bit-reproducible; the gate gradients sum over key rows through shared-memory floating-point atomics, so their last
+ * bits can differ from run to run.
  */
 size_t mdn_chunk_bwd_workspace_bytes(const mdn_params* p);
 

@@ -116,6 +116,8 @@ def lib() -> ctypes.CDLL:
         L.mdn_chunk_bwd_saved_workspace_bytes.argtypes = [P]
         L.mdn_chunk_bwd_saved.restype = ctypes.c_int
         L.mdn_chunk_bwd_saved.argtypes = [P] + [vp] * 9 + [ctypes.c_size_t] + [vp] * 13 + [vp, ctypes.c_size_t, vp]
+        L.mdn_chunk_bwd_saved_io.restype = ctypes.c_int
+        L.mdn_chunk_bwd_saved_io.argtypes = L.mdn_chunk_bwd_saved.argtypes
         L.mdn_chunk_bwd.restype = ctypes.c_int
         L.mdn_chunk_bwd.argtypes = [P] + [vp] * 22 + [vp, ctypes.c_size_t, vp]
         L.mdn_chunk_bwd_workspace_bytes.restype = ctypes.c_size_t
@@ -507,6 +509,7 @@ class _ChunkAttention(torch.autograd.Function):
         o, Sf, Mf, states, ws = chunk_fwd(q, k, v, beta, log_alpha, log_mu, eta, initial_S=initial_S,
                                           initial_M=initial_M, cu_seqlens=cu_seqlens, scale=scale, path="tensor",
                                           keep_chunk_states=True)
+        ctx.set_materialize_grads(False)   # (an unused output's gradient is then None, not a tensor of zeros to read)
         ctx.save_for_backward(q, k, v, beta, log_alpha, log_mu, eta, initial_S, initial_M, cu_seqlens, states, ws)
         ctx.scale = scale
         return o, Sf, Mf
@@ -514,14 +517,18 @@ class _ChunkAttention(torch.autograd.Function):
     @staticmethod
     def backward(ctx, d_o, d_Sf, d_Mf):
         q, k, v, beta, log_alpha, log_mu, eta, initial_S, initial_M, cu_seqlens, states, ws = ctx.saved_tensors
-        g = chunk_bwd(q, k, v, beta, log_alpha, log_mu, eta, d_o.contiguous().to(q.dtype), initial_S=initial_S,
-                      initial_M=initial_M, cu_seqlens=cu_seqlens,
-                      d_final_S=None if d_Sf is None else d_Sf.contiguous().float(),
-                      d_final_M=None if d_Mf is None else d_Mf.contiguous().float(), scale=ctx.scale,
-                      method="chunked", saved=(ws, states))
-        return (g["dq"].to(q.dtype), g["dk"].to(k.dtype), g["dv"].to(v.dtype), g["dbeta"], g["dlog_alpha"], g["dlog_mu"],
-                g["deta"], None if initial_S is None else g["d_initial_S"], None if initial_M is None else g["d_initial_M"],
-                None, None)
+        d_o = torch.zeros_like(v) if d_o is None else d_o.contiguous().to(q.dtype)
+        d_Sf = None if d_Sf is None else d_Sf.contiguous().float()
+        d_Mf = None if d_Mf is None else d_Mf.contiguous().float()
+        r = (_nat or _load_native()).chunk_bwd(q, k, v, beta, log_alpha, log_mu, eta, d_o, initial_S, initial_M, cu_seqlens,
+                                               d_Sf, d_Mf, ctx.scale, None, 3, ws, states)   # dq, dk, dv in q's dtype
+        if isinstance(r, int):
+            raise MdnError(r, "mdn_chunk_bwd_saved_io")
+        if r is None:   # (an argument the native module leaves to the Python code)
+            g = chunk_bwd(q, k, v, beta, log_alpha, log_mu, eta, d_o, initial_S=initial_S, initial_M=initial_M,
+                          cu_seqlens=cu_seqlens, d_final_S=d_Sf, d_final_M=d_Mf, scale=ctx.scale, method="chunked", saved=(ws, states))
+            r = (g["dq"].to(q.dtype), g["dk"].to(k.dtype), g["dv"].to(v.dtype)) + tuple(g[n] for n in _GRADS[3:])
+        return r[:7] + (None if initial_S is None else r[7], None if initial_M is None else r[8], None, None)
 
 
 def chunk_attention(q, k, v, beta, log_alpha, log_mu, eta, *, initial_S=None, initial_M=None, cu_seqlens=None,

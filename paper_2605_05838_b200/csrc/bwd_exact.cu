@@ -471,7 +471,8 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
   else if (n > 16) body(std::integral_constant<int, 4>{});
   else body(std::integral_constant<int, 2>{});
   __syncthreads();   // DW, DW^T, DA have been read: the gate gradients' work matrices take their places
-  gate_gradients(vec, GateMats{Gam, Mm, dGe, dGm, DW, DWT}, DAS, n, tok_h, H, a.gates);
+  gate_gradients(vec, GateMats{Gam, Mm, DW, DWT}, [&](int r, int i) { return dGe[r * kLT + i]; },
+                 [&](int r, int i) { return dGm[r * kLT + i]; }, DAS, n, tok_h, H, a.gates);
 }
 
 template <int DK, int NV> cudaError_t launch_adj(const Plan& pl, const AdjArgs& a) {

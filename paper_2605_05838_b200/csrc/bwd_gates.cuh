@@ -13,18 +13,19 @@ constexpr int LG = C + 4;     // floats per row of a 64 x 64 fp32 matrix
 enum Vec : int { vAbar = 0, vB, vP, vGS, vGM, vMubar, vAlpha, vBeta, vMu, vEta, vBprev,
                  vdAbar, vdB, vdP, vdGS, vdGM, vdMubar, vdAlpha, vdBeta, vdMu, vdEta, vRed };
 
-// All [64][LG] fp32 in shared memory: gamma and m (zero above the diagonal), d Geta and d G^- (the adjoints of the masks
-// Gamma eta and G^-, zero above the diagonal), two work matrices for the adjoints of gamma and m.
-struct GateMats { const float* gam; const float* mm; const float* dge; const float* dgm; float* dg; float* dm; };
+// All [64][LG] fp32 in shared memory: gamma and m (zero above the diagonal), two work matrices for their adjoints.
+struct GateMats { const float* gam; const float* mm; float* dg; float* dm; };
 struct GateOut { float* dbeta; float* dlog_alpha; float* dlog_mu; float* deta; };
 
-// vec: the vectors above; part: 3 x 64 floats of scratch.  Called by all 256 threads after a barrier; tok0_h: index of
-// the chunk's first token in the [token][H] gate arrays.
-__device__ __forceinline__ void gate_gradients(float* vec, const GateMats& mt, float* sPart, int n, size_t tok0_h, int H,
+// vec: the vectors above; dge(r, i), dgm(r, i): the adjoints of the masks Gamma eta and G^- (asked for any r, i; zero above
+// the diagonal); sPart: 3 x 64 floats of scratch.  Called by all 256 threads after a barrier; tok0_h: index of the chunk's
+// first token in the [token][H] gate arrays.
+template <class FE, class FM>
+__device__ __forceinline__ void gate_gradients(float* vec, const GateMats& mt, FE dge_at, FM dgm_at, float* sPart, int n, size_t tok0_h, int H,
                                                const GateOut& a) {
   auto V = [&](int which) { return vec + which * C; };
   auto tok = [&](int r) { return tok0_h + (size_t)r * H; };
-  const float *sGam = mt.gam, *sMm = mt.mm, *sdGe = mt.dge, *sdGm = mt.dgm;
+  const float *sGam = mt.gam, *sMm = mt.mm;
   float *sDg = mt.dg, *sDm = mt.dm;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // In two passes.  Serial (thread i = column i, from the last row up): only the two carried adjoints
@@ -40,7 +41,7 @@ __device__ __forceinline__ void gate_gradients(float* vec, const GateMats& mt, f
     for (int rb = C - 4; rb >= 0; rb -= 4) {   // four rows' loads first: the walk itself is a chain of three FMAs per row
       float dge[4], dgm[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) { dge[u] = sdGe[(rb + u) * LG + i]; dgm[u] = sdGm[(rb + u) * LG + i]; }   // zero above the diagonal
+      for (int u = 0; u < 4; ++u) { dge[u] = dge_at(rb + u, i); dgm[u] = dgm_at(rb + u, i); }
       const float4 al4 = *reinterpret_cast<const float4*>(V(vAlpha) + rb), be4 = *reinterpret_cast<const float4*>(V(vBeta) + rb);
       const float4 mu4 = *reinterpret_cast<const float4*>(V(vMu) + rb);
       const float al[4] = {al4.x, al4.y, al4.z, al4.w}, be[4] = {be4.x, be4.y, be4.z, be4.w}, mu[4] = {mu4.x, mu4.y, mu4.z, mu4.w};
@@ -61,8 +62,8 @@ __device__ __forceinline__ void gate_gradients(float* vec, const GateMats& mt, f
     float s = 0.f;
 #pragma unroll 4
     for (int r = max(r0, i); r < r1; ++r) {
-      s = fmaf(sdGe[r * LG + i], sGam[r * LG + i], s);
-      if (r > i) s = fmaf(sdGm[r * LG + i] * V(vAlpha)[r], sGam[(r - 1) * LG + i], s);
+      s = fmaf(dge_at(r, i), sGam[r * LG + i], s);
+      if (r > i) s = fmaf(dgm_at(r, i) * V(vAlpha)[r], sGam[(r - 1) * LG + i], s);
     }
     if (part == 2) s += V(vdGS)[i] * sGam[(C - 1) * LG + i] + V(vdGM)[i] * sMm[(C - 1) * LG + i];
     sPart[part * C + i] = s;
@@ -78,7 +79,7 @@ __device__ __forceinline__ void gate_gradients(float* vec, const GateMats& mt, f
         const float dgam = sDg[r * LG + i], dmm = sDm[r * LG + i];
         sbe = fmaf(dgam, sMm[r * LG + i], sbe);
         if (i < r) {
-          sa = fmaf(sGam[(r - 1) * LG + i], fmaf(sdGm[r * LG + i], V(vEta)[i], dgam), sa);
+          sa = fmaf(sGam[(r - 1) * LG + i], fmaf(dgm_at(r, i), V(vEta)[i], dgam), sa);
           sm = fmaf(dmm, sMm[(r - 1) * LG + i], sm);
         }
       }

@@ -120,6 +120,8 @@ struct ChainArgs {
   int end_scalars_in_rk;      // (abar_C, b_C, mubar_C) of a chunk are entries 0..2 of coefficient vector 6, not the
                               // last entries of vectors 0, 1, 5 (the adjoint chain decouples them)
   float* vt_dump;             // NULL, or [chunk slot][64][H][dv] fp32: V~ of every chunk as EPI-2 reads it
+  __nv_bfloat16* dr_bf16;     // mirrored runs: NULL, or the run's "V~" (= dR) as bf16 in the mirrored problem's own [token][H][dv]
+  float* dr_f32;              // ... and (or NULL) as fp32: dL/dv
   int mirror;                 // with inject: q, k, G and T are the ORIGINAL tensors of a problem whose chunks this run
   ChunkGeom mirror_g;         // walks in reverse order (geometry mirror_g): chunk c of this run reads the rows of
                               // original chunk nchunks - 1 - c (rows past a short chunk's end meet zero coefficients)
@@ -941,6 +943,27 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
                 if (j < live) *dst = __uint_as_float(vt[j]);
             }
           }
+          if (a.dr_bf16 != nullptr) {
+            const SeqInfo os = seq_info(a.mirror_g, seq);
+            const int c0 = (nch - 1 - c) * C + r0;
+            const int live = min(kTok, os.len - c0);   // this thread's tokens inside the chunk
+            const size_t at = ((size_t)(os.tok0 + c0) * H + h) * kD + d, stride = (size_t)H * kD;
+            if (live >= kTok) {
+#pragma unroll
+              for (int j = 0; j < kTok; ++j) a.dr_bf16[at + j * stride] = __float2bfloat16_rn(__uint_as_float(vt[j]));
+              if (a.dr_f32 != nullptr) {
+#pragma unroll
+                for (int j = 0; j < kTok; ++j) a.dr_f32[at + j * stride] = __uint_as_float(vt[j]);
+              }
+            } else {
+#pragma unroll
+              for (int j = 0; j < kTok; ++j)
+                if (j < live) {
+                  a.dr_bf16[at + j * stride] = __float2bfloat16_rn(__uint_as_float(vt[j]));
+                  if (a.dr_f32 != nullptr) a.dr_f32[at + j * stride] = __uint_as_float(vt[j]);
+                }
+            }
+          }
         }
       }
     }
@@ -1012,6 +1035,7 @@ cudaError_t launch_chain_tensor(const Plan& pl, const void* q, const void* k, co
 #endif
   a.dump = pl.chain_dump; a.state_only = pl.chain_state_only; a.end_scalars_in_rk = pl.chain_end_scalars_in_rk;
   a.vt_dump = pl.chain_vt_dump; a.inject = pl.chain_inject;
+  a.dr_bf16 = pl.chain_dr_bf16; a.dr_f32 = pl.chain_dr_f32;
   a.mirror = pl.chain_mirror_geom != nullptr;
   if (a.mirror) a.mirror_g = *pl.chain_mirror_geom; else a.mirror_g = pl.geom;
   a.seg_G = 0; a.seg_phase = 0;

@@ -267,11 +267,11 @@ size_t mdn_bwd_adjoint_states_bytes(const mdn_params* p) {
   return adj_layout(p, &a) == MDN_OK ? (size_t)a.states_bytes() : 0;
 }
 
-mdn_status mdn_bwd_state_chain(const mdn_params* p, const void* q, const void* k, const void* d_o,
-                               const float* d_final_S, const float* d_final_M, const int32_t* cu_seqlens,
-                               void* fwd_workspace, size_t fwd_workspace_bytes, void* adjoint_states, float* d_initial_S,
-                               float* d_initial_M, void* workspace, size_t workspace_bytes, void* cuda_stream) {
-  t_last_launches = 0;
+// dr_bf16, dr_f32: where dR goes ([token][H][dv]; dr_f32 may be NULL); dr_bf16 NULL: into the adjoint buffer's second part.
+static mdn_status state_chain(const mdn_params* p, const void* q, const void* k, const void* d_o, const float* d_final_S,
+                              const float* d_final_M, const int32_t* cu_seqlens, void* fwd_workspace, size_t fwd_workspace_bytes,
+                              void* adjoint_states, __nv_bfloat16* dr_bf16, float* dr_f32, float* d_initial_S, float* d_initial_M,
+                              void* workspace, size_t workspace_bytes, void* cuda_stream) {
   AdjLayout al;
   mdn_status st = adj_layout(p, &al);
   if (st != MDN_OK) return st;
@@ -301,7 +301,9 @@ mdn_status mdn_bwd_state_chain(const mdn_params* p, const void* q, const void* k
   if (e != cudaSuccess) { t_last_cuda_error = (int)e; return MDN_ERR_CUDA; }
   // the forward's chain kernel on the mirrored problem, roles exchanged: its "S" is dM, its "M" is dS
   ext.chain_dump = static_cast<uint8_t*>(adjoint_states);
-  ext.chain_vt_dump = reinterpret_cast<float*>(ext.chain_dump + al.image_bytes());
+  if (dr_bf16 == nullptr) ext.chain_vt_dump = reinterpret_cast<float*>(ext.chain_dump + al.image_bytes());
+  ext.chain_dr_bf16 = dr_bf16;
+  ext.chain_dr_f32 = dr_f32;
   ext.chain_inject = 1;   // the two Q terms: q and dO (passed in the place of o) give a second update per chunk
   ext.chain_mirror_geom = &fwd.geom;   // q, k, dO and T are read in place, chunk index mirrored
   ext.chain_mirror_T = fwd.ws + fwd.lay.off_T;
@@ -311,6 +313,15 @@ mdn_status mdn_bwd_state_chain(const mdn_params* p, const void* q, const void* k
                           d_initial_S, &t_last_launches);
   if (e != cudaSuccess) { t_last_cuda_error = (int)e; return MDN_ERR_CUDA; }
   return MDN_OK;
+}
+
+mdn_status mdn_bwd_state_chain(const mdn_params* p, const void* q, const void* k, const void* d_o,
+                               const float* d_final_S, const float* d_final_M, const int32_t* cu_seqlens,
+                               void* fwd_workspace, size_t fwd_workspace_bytes, void* adjoint_states, float* d_initial_S,
+                               float* d_initial_M, void* workspace, size_t workspace_bytes, void* cuda_stream) {
+  t_last_launches = 0;
+  return state_chain(p, q, k, d_o, d_final_S, d_final_M, cu_seqlens, fwd_workspace, fwd_workspace_bytes, adjoint_states, nullptr,
+                     nullptr, d_initial_S, d_initial_M, workspace, workspace_bytes, cuda_stream);
 }
 
 // ---- the chunk-parallel backward: state-only forward keeping the chunk states, adjoint chain, per-chunk stage
@@ -343,31 +354,57 @@ size_t mdn_chunk_bwd_saved_workspace_bytes(const mdn_params* p) {
   return chunked_bwd_layout(p, &c) == MDN_OK ? (size_t)(c.total - c.adj_states) : 0;
 }
 
-// Steps 2 and 3 on states and a workspace that a mdn_chunk_fwd_keep_states call left behind.
+// Steps 2 and 3 on states and a workspace that a mdn_chunk_fwd_keep_states call left behind.  io_grads: dq, dk, dv are bf16
+// (each rounded once from fp32), else fp32; t_last_launches goes on counting.
 static mdn_status bwd_from_states(const mdn_params* p, const ChunkedBwdLayout& c, const void* q, const void* k,
-                                  const void* v, const float* beta, const float* log_alpha, const float* log_mu,
+                                  const float* beta, const float* log_alpha, const float* log_mu,
                                   const float* eta, const int32_t* cu_seqlens, const void* d_o, const float* d_final_S,
                                   const float* d_final_M, void* fwd_ws, const void* fwd_states, char* adj_states,
-                                  char* stage, float* dq, float* dk, float* dv, float* dbeta, float* dlog_alpha,
+                                  char* stage, bool io_grads, void* dq, void* dk, void* dv, float* dbeta, float* dlog_alpha,
                                   float* dlog_mu, float* deta, float* d_initial_S, float* d_initial_M,
-                                  void* cuda_stream, int launches_before) {
-  mdn_status st = mdn_bwd_state_chain(p, q, k, d_o, d_final_S, d_final_M, cu_seqlens, fwd_ws, c.lf.total_bytes, adj_states,
-                                      d_initial_S, d_initial_M, stage, c.al.total, cuda_stream);
+                                  void* cuda_stream) {
+  // dR = dv: for fp32 gradients the per-chunk stage's bf16 copy goes behind the adjoint images
+  __nv_bfloat16* dr = static_cast<__nv_bfloat16*>(io_grads ? dv : adj_states + c.al.image_bytes());
+  mdn_status st = state_chain(p, q, k, d_o, d_final_S, d_final_M, cu_seqlens, fwd_ws, c.lf.total_bytes, adj_states, dr,
+                              io_grads ? nullptr : static_cast<float*>(dv), d_initial_S, d_initial_M, stage, c.al.total, cuda_stream);
   if (st != MDN_OK) return st;
-  t_last_launches += launches_before;
   mdn_params pf = *p;
   pf.segments = 1;
   Plan fwd;
   st = make_plan(&pf, cu_seqlens, fwd_ws, c.lf.total_bytes, cuda_stream, &fwd);
   if (st != MDN_OK) return st;
   const char* fs = static_cast<const char*>(fwd_states);
-  cudaError_t e = launch_bwd_chunk_par(
+  cudaError_t e = launch_bwd_chunk_tc(
       fwd, q, k, d_o, beta, log_alpha, log_mu, eta, fs,
-      reinterpret_cast<const float*>(fs + (uint64_t)c.lf.num_slots * p->H * kStateImageBytes), adj_states,
-      reinterpret_cast<const float*>(adj_states + c.al.image_bytes()), dq, dk, dv, dbeta, dlog_alpha, dlog_mu, deta,
-      &t_last_launches);
+      reinterpret_cast<const float*>(fs + (uint64_t)c.lf.num_slots * p->H * kStateImageBytes), adj_states, dr, dq, dk, io_grads,
+      dbeta, dlog_alpha, dlog_mu, deta, &t_last_launches);
   if (e != cudaSuccess) { t_last_cuda_error = (int)e; return MDN_ERR_CUDA; }
   return MDN_OK;
+}
+
+static mdn_status bwd_saved(const mdn_params* p, const void* q, const void* k, const void* v, const float* beta,
+                            const float* log_alpha, const float* log_mu, const float* eta,
+                            const int32_t* cu_seqlens, void* fwd_workspace, size_t fwd_workspace_bytes,
+                            const void* chunk_states, const void* d_o, const float* d_final_S,
+                            const float* d_final_M, bool io_grads, void* dq, void* dk, void* dv, float* dbeta,
+                            float* dlog_alpha, float* dlog_mu, float* deta, float* d_initial_S,
+                            float* d_initial_M, void* workspace, size_t workspace_bytes, void* cuda_stream) {
+  t_last_launches = 0;
+  if (p && (p->num_seqs > 0) != (cu_seqlens != nullptr)) return MDN_ERR_INVALID_ARG;
+  ChunkedBwdLayout c;
+  mdn_status st = chunked_bwd_layout(p, &c);
+  if (st != MDN_OK) return st;
+  if (p->o_dtype != MDN_BF16) return MDN_ERR_UNSUPPORTED;
+  if (!q || !k || !v || !d_o || !beta || !log_alpha || !log_mu || !dq || !dk || !dv || !dbeta || !dlog_alpha || !dlog_mu)
+    return MDN_ERR_INVALID_ARG;
+  if (!aligned(dq, 16) || !aligned(dk, 16) || !aligned(dv, 16)) return MDN_ERR_INVALID_ARG;
+  if (!fwd_workspace || fwd_workspace_bytes < c.lf.total_bytes || !aligned(fwd_workspace, 256)) return MDN_ERR_WORKSPACE;
+  if (!chunk_states || !aligned(chunk_states, 1024)) return MDN_ERR_INVALID_ARG;
+  if (!workspace || workspace_bytes < c.total - c.adj_states || !aligned(workspace, 1024)) return MDN_ERR_WORKSPACE;
+  char* w = static_cast<char*>(workspace);   // [adjoint states | stage scratch], as in the full layout from adj_states on
+  return bwd_from_states(p, c, q, k, beta, log_alpha, log_mu, eta, cu_seqlens, d_o, d_final_S, d_final_M,
+                         fwd_workspace, chunk_states, w, w + (c.stage - c.adj_states), io_grads, dq, dk, dv, dbeta, dlog_alpha,
+                         dlog_mu, deta, d_initial_S, d_initial_M, cuda_stream);
 }
 
 mdn_status mdn_chunk_bwd_saved(const mdn_params* p, const void* q, const void* k, const void* v, const float* beta,
@@ -377,21 +414,21 @@ mdn_status mdn_chunk_bwd_saved(const mdn_params* p, const void* q, const void* k
                                const float* d_final_M, float* dq, float* dk, float* dv, float* dbeta,
                                float* dlog_alpha, float* dlog_mu, float* deta, float* d_initial_S,
                                float* d_initial_M, void* workspace, size_t workspace_bytes, void* cuda_stream) {
-  t_last_launches = 0;
-  if (p && (p->num_seqs > 0) != (cu_seqlens != nullptr)) return MDN_ERR_INVALID_ARG;
-  ChunkedBwdLayout c;
-  mdn_status st = chunked_bwd_layout(p, &c);
-  if (st != MDN_OK) return st;
-  if (p->o_dtype != MDN_BF16) return MDN_ERR_UNSUPPORTED;
-  if (!q || !k || !v || !d_o || !beta || !log_alpha || !log_mu || !dq || !dk || !dv || !dbeta || !dlog_alpha || !dlog_mu)
-    return MDN_ERR_INVALID_ARG;
-  if (!fwd_workspace || fwd_workspace_bytes < c.lf.total_bytes || !aligned(fwd_workspace, 256)) return MDN_ERR_WORKSPACE;
-  if (!chunk_states || !aligned(chunk_states, 1024)) return MDN_ERR_INVALID_ARG;
-  if (!workspace || workspace_bytes < c.total - c.adj_states || !aligned(workspace, 1024)) return MDN_ERR_WORKSPACE;
-  char* w = static_cast<char*>(workspace);   // [adjoint states | stage scratch], as in the full layout from adj_states on
-  return bwd_from_states(p, c, q, k, v, beta, log_alpha, log_mu, eta, cu_seqlens, d_o, d_final_S, d_final_M,
-                         fwd_workspace, chunk_states, w, w + (c.stage - c.adj_states), dq, dk, dv, dbeta, dlog_alpha,
-                         dlog_mu, deta, d_initial_S, d_initial_M, cuda_stream, 0);
+  return bwd_saved(p, q, k, v, beta, log_alpha, log_mu, eta, cu_seqlens, fwd_workspace, fwd_workspace_bytes, chunk_states, d_o,
+                   d_final_S, d_final_M, false, dq, dk, dv, dbeta, dlog_alpha, dlog_mu, deta, d_initial_S, d_initial_M, workspace,
+                   workspace_bytes, cuda_stream);
+}
+
+mdn_status mdn_chunk_bwd_saved_io(const mdn_params* p, const void* q, const void* k, const void* v, const float* beta,
+                                  const float* log_alpha, const float* log_mu, const float* eta,
+                                  const int32_t* cu_seqlens, void* fwd_workspace, size_t fwd_workspace_bytes,
+                                  const void* chunk_states, const void* d_o, const float* d_final_S,
+                                  const float* d_final_M, void* dq, void* dk, void* dv, float* dbeta,
+                                  float* dlog_alpha, float* dlog_mu, float* deta, float* d_initial_S,
+                                  float* d_initial_M, void* workspace, size_t workspace_bytes, void* cuda_stream) {
+  return bwd_saved(p, q, k, v, beta, log_alpha, log_mu, eta, cu_seqlens, fwd_workspace, fwd_workspace_bytes, chunk_states, d_o,
+                   d_final_S, d_final_M, true, dq, dk, dv, dbeta, dlog_alpha, dlog_mu, deta, d_initial_S, d_initial_M, workspace,
+                   workspace_bytes, cuda_stream);
 }
 
 mdn_status mdn_chunk_bwd_chunked(const mdn_params* p, const void* q, const void* k, const void* v, const float* beta,
@@ -424,9 +461,9 @@ mdn_status mdn_chunk_bwd_chunked(const mdn_params* p, const void* q, const void*
                    nullptr, nullptr);
   if (st != MDN_OK) return st;
   // 2. the adjoint state chain;  3. per (chunk, head): dq, dk, dv and the gate gradients
-  return bwd_from_states(p, c, q, k, v, beta, log_alpha, log_mu, eta, cu_seqlens, d_o, d_final_S, d_final_M, w + c.ws_fwd,
-                         w + c.fwd_states, w + c.adj_states, w + c.stage, dq, dk, dv, dbeta, dlog_alpha, dlog_mu, deta,
-                         d_initial_S, d_initial_M, cuda_stream, t_last_launches);
+  return bwd_from_states(p, c, q, k, beta, log_alpha, log_mu, eta, cu_seqlens, d_o, d_final_S, d_final_M, w + c.ws_fwd,
+                         w + c.fwd_states, w + c.adj_states, w + c.stage, false, dq, dk, dv, dbeta, dlog_alpha, dlog_mu, deta,
+                         d_initial_S, d_initial_M, cuda_stream);
 }
 
 // ---- the forward with layer operations

@@ -144,6 +144,8 @@ struct Plan {
   int chain_end_scalars_in_rk = 0;
   float* chain_vt_dump = nullptr;        // V~ per chunk slot, fp32 [slot][64][H][dv]
   int chain_inject = 0;                  // second update per chunk from q and the tensor passed as o (adjoint chain)
+  __nv_bfloat16* chain_dr_bf16 = nullptr;   // mirrored run: dR as bf16 (and fp32) in the original problem's [token][H][dv]
+  float* chain_dr_f32 = nullptr;
   const ChunkGeom* chain_mirror_geom = nullptr;   // q, k, o belong to this geometry, walked in reverse chunk order
   const char* chain_mirror_T = nullptr;           // ... and T ([slot][H][64][64] bf16 of that problem), used transposed
   int cu_total_may_be_short = 0;   // packed: cu[N] <= T instead of == T (the adjoint chain's padded problem)
@@ -154,13 +156,13 @@ struct Plan {
 // Launchers (one per .cu file).  Each returns the CUDA error of its launches and adds
 // the number of kernels it enqueued to *launches.
 cudaError_t launch_chunk_map(const Plan& pl, int* launches);
-// bwd_chunk_par.cu: gradients of q, k, v and the gates per (chunk, head) from the kept states and the adjoint states
-// (state images per chunk slot; fwd_vt = V~, adj_dr = dR per chunk slot as fp32 [slot][64][H][dv]; adj_* in the adjoint
-// chain's mirrored order: chunk c of a sequence with n chunks at the sequence's slot n - 1 - c)
-cudaError_t launch_bwd_chunk_par(const Plan& fwd, const void* q, const void* k, const void* d_o, const float* beta,
-                                 const float* log_alpha, const float* log_mu, const float* eta, const void* fwd_states,
-                                 const float* fwd_vt, const void* adj_states, const float* adj_dr, float* dq, float* dk,
-                                 float* dv, float* dbeta, float* dlog_alpha, float* dlog_mu, float* deta, int* launches);
+// bwd_chunk_tc.cu: gradients of q, k and the gates per (chunk, head) from the kept states and the adjoint states (state
+// images per chunk slot; fwd_vt = V~ per chunk slot as fp32 [slot][64][H][dv]; adj_states in the adjoint chain's mirrored
+// order: chunk c of a sequence with n chunks at the sequence's slot n - 1 - c; dr_bf16 = dR [token][H][dv]).  dq, dk: fp32, or bf16.
+cudaError_t launch_bwd_chunk_tc(const Plan& fwd, const void* q, const void* k, const void* d_o, const float* beta,
+                                const float* log_alpha, const float* log_mu, const float* eta, const void* fwd_states,
+                                const float* fwd_vt, const void* adj_states, const void* dr_bf16, void* dq, void* dk, bool grads_bf16,
+                                float* dbeta, float* dlog_alpha, float* dlog_mu, float* deta, int* launches);
 // bwd_chunk.cu: W^T dO and the coefficient vectors of the adjoint state chain's mirrored problem, from the forward's workspace
 cudaError_t launch_bwd_ext_cu(const Plan& fwd, int32_t* cu_ext, int* launches);
 cudaError_t launch_bwd_prep(const Plan& fwd, const void* d_o, void* v_ext, float* coef_ext, int* launches);

@@ -252,7 +252,7 @@ PyObject* chunk_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
 
 // chunk_bwd(q, k, v, beta, log_alpha, log_mu, eta, d_o, initial_S, initial_M, cu_seqlens, d_final_S, d_final_M, scale,
 //           workspace, method, fwd_workspace, chunk_states) -> (dq, dk, dv, dbeta, dlog_alpha, dlog_mu, deta, dS0, dM0)
-// method: 0 stepwise, 1 chunked, 2 chunked on saved states
+// method: 0 stepwise, 1 chunked, 2 chunked on saved states, 3 the same with dq, dk, dv in the i/o dtype
 PyObject* chunk_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   NATIVE_TRY
   Inputs in;
@@ -280,27 +280,32 @@ PyObject* chunk_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     ws = *t;
   }
   const Tensor *fws = nullptr, *states = nullptr;
-  if (method == 2 && (!(fws = cuda_tensor(a[16], at::kByte, in.dev)) || !(states = cuda_tensor(a[17], at::kByte, in.dev))))
+  if (method >= 2 && (!(fws = cuda_tensor(a[16], at::kByte, in.dev)) || !(states = cuda_tensor(a[17], at::kByte, in.dev))))
     return Py_NewRef(Py_None);
   Tensor g[9];
   mdn_status st;
   {
     NoGil gil;
     if (!ws.defined()) ws = empty({(int64_t)need}, at::kByte, in.dev);
-    g[0] = empty({in.B, in.T, in.H, in.dk}, at::kFloat, in.dev);
-    g[1] = empty({in.B, in.T, in.H, in.dk}, at::kFloat, in.dev);
-    g[2] = empty({in.B, in.T, in.H, in.dv}, at::kFloat, in.dev);
+    const at::ScalarType gdt = method == 3 ? in.dtype : at::kFloat;
+    g[0] = empty({in.B, in.T, in.H, in.dk}, gdt, in.dev);
+    g[1] = empty({in.B, in.T, in.H, in.dk}, gdt, in.dev);
+    g[2] = empty({in.B, in.T, in.H, in.dv}, gdt, in.dev);
     for (int i = 3; i < (in.eta ? 7 : 6); ++i) g[i] = empty({in.B, in.T, in.H}, at::kFloat, in.dev);
     g[7] = empty({nst, in.H, in.dk, in.dv}, at::kFloat, in.dev);
     g[8] = empty({nst, in.H, in.dk, in.dv}, at::kFloat, in.dev);
     float* gp[9];
-    for (int i = 0; i < 9; ++i) gp[i] = g[i].defined() ? static_cast<float*>(g[i].data_ptr()) : nullptr;
+    for (int i = 0; i < 9; ++i) gp[i] = g[i].defined() ? static_cast<float*>(g[i].data_ptr()) : nullptr;   // (0..2: the i/o dtype for method 3)
     const void *q = in.q->const_data_ptr(), *k = in.k->const_data_ptr(), *v = in.v->const_data_ptr();
     void* stream = stream_of(in.dev);
     if (method == 2)
       st = mdn_chunk_bwd_saved(&p, q, k, v, in.beta, in.log_alpha, in.log_mu, in.eta, cu, fws->data_ptr(), (size_t)fws->numel(),
                                states->const_data_ptr(), d_o->const_data_ptr(), dSf, dMf, gp[0], gp[1], gp[2], gp[3], gp[4],
                                gp[5], gp[6], gp[7], gp[8], ws.data_ptr(), (size_t)ws.numel(), stream);
+    else if (method == 3)
+      st = mdn_chunk_bwd_saved_io(&p, q, k, v, in.beta, in.log_alpha, in.log_mu, in.eta, cu, fws->data_ptr(), (size_t)fws->numel(),
+                                  states->const_data_ptr(), d_o->const_data_ptr(), dSf, dMf, gp[0], gp[1], gp[2], gp[3], gp[4],
+                                  gp[5], gp[6], gp[7], gp[8], ws.data_ptr(), (size_t)ws.numel(), stream);
     else
       st = (method == 1 ? mdn_chunk_bwd_chunked : mdn_chunk_bwd)(
           &p, q, k, v, in.beta, in.log_alpha, in.log_mu, in.eta, S0, M0, cu, d_o->const_data_ptr(), dSf, dMf, gp[0], gp[1],
