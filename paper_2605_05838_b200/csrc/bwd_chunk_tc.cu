@@ -41,12 +41,10 @@ typedef __nv_bfloat16 bf16;
 constexpr int kD = 128, kThreads = kGateThreads;
 constexpr uint32_t kVecBytes = 24 * C * 4;
 constexpr uint32_t kOffVec = 0, kOffDiag = kVecBytes, kOffA2 = 7168, kOffA1 = kOffA2 + 32768, kOffX = kOffA1 + 32768;
-constexpr uint32_t kMatF = C * LG * 4;                        // one of the gate stage's fp32 matrices (over A1, X)
-constexpr uint32_t kSmem = (kOffX + 32768 > kOffA1 + 4 * kMatF ? kOffX + 32768 : kOffA1 + 4 * kMatF) + 1024;
-static_assert(kOffDiag + C * 4 <= kOffA2 && kSmem <= 113 * 1024, "two CTAs per SM");
+constexpr uint32_t kSmem = kOffX + 32768 + 1024;
+static_assert(kOffDiag + C * 4 <= kOffA2 && kSmem <= 110 * 1024, "two CTAs per SM");
 constexpr uint32_t kColAcc = 0, kColB = 128, kColP = 128, kColQK = 192, kCols = 256;
-constexpr int kPartSlot = vRed;   // vector slots 21..23: scratch of the gate stage
-static_assert(vRed + 3 <= 24, "vector slots");
+static_assert(kGateScratch * 4 <= 32768, "the gate stage's scratch lies in A1");
 
 struct TcArgs {
   ChunkGeom g;
@@ -163,23 +161,33 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
   tc_fence_after_sync();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);
   const uint32_t tl = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + hf * 64;   // the thread's lane, its 64 columns of a 128-wide result
-  if (tid < C) {
+  if (tid < C) {   // (all loads before the first store: they must not wait for one another)
     const float* cf = a.coef + ((size_t)slot * H + h) * MDN_NUM_COEF * C;
     const int t = tid;
     const bool in = t < n;
-    V(vAbar)[t] = cf[kAbar * C + t]; V(vB)[t] = cf[kB * C + t]; V(vP)[t] = cf[kAlphaBPrev * C + t];
-    V(vGS)[t] = in ? cf[kGS * C + t] : 0.f; V(vGM)[t] = in ? cf[kGM * C + t] : 0.f; V(vMubar)[t] = cf[kMubar * C + t];
-    const size_t gi = tok(t);
-    V(vAlpha)[t] = in ? expf(a.log_alpha[gi]) : 1.f; V(vMu)[t] = in ? expf(a.log_mu[gi]) : 1.f;
-    V(vBeta)[t] = in ? a.beta[gi] : 0.f; V(vEta)[t] = in ? (a.eta ? a.eta[gi] : 1.f) : 0.f;
-    V(vBprev)[t] = t > 0 ? cf[kB * C + t - 1] : 0.f;
+    const size_t gi = tok(in ? t : 0);
+    const float x0 = __ldg(cf + kAbar * C + t), x1 = __ldg(cf + kB * C + t), x2 = __ldg(cf + kAlphaBPrev * C + t);
+    const float x3 = __ldg(cf + kGS * C + t), x4 = __ldg(cf + kGM * C + t), x5 = __ldg(cf + kMubar * C + t);
+    const float x6 = __ldg(cf + kB * C + max(t - 1, 0));
+    const float ga = __ldg(a.log_alpha + gi), gm = __ldg(a.log_mu + gi), gb = __ldg(a.beta + gi), ge = a.eta ? __ldg(a.eta + gi) : 1.f;
+    V(vAbar)[t] = x0; V(vB)[t] = x1; V(vP)[t] = x2;
+    V(vGS)[t] = in ? x3 : 0.f; V(vGM)[t] = in ? x4 : 0.f; V(vMubar)[t] = x5;
+    V(vAlpha)[t] = in ? expf(ga) : 1.f; V(vMu)[t] = in ? expf(gm) : 1.f;
+    V(vBeta)[t] = in ? gb : 0.f; V(vEta)[t] = in ? ge : 0.f;
+    V(vBprev)[t] = t > 0 ? x6 : 0.f;
   }
 
   uint32_t ph_l = 0, ph_m = 0;
   bool good = true;
-  // all threads wait for the next load / product phase and learn whether everybody's wait succeeded (also a barrier)
+  // All threads wait for the next load / product phase and learn whether everybody's wait succeeded (also a barrier).  The
+  // lanes of a warp can leave the polling loop at different times, and a block barrier does not bring them together again: the
+  // warp-collective tensor-memory loads that follow need the __syncwarp (without it they ran on parts of a warp, which
+  // ended in an illegal memory access).
   auto wait_all = [&](uint32_t bar, uint32_t& ph) {
-    good = __syncthreads_and(mbar_wait(bar, ph, &abort_flag)) != 0;
+    const bool mine = mbar_wait(bar, ph, &abort_flag);
+    __syncwarp();
+    good = __syncthreads_and(mine) != 0;
+    __syncwarp();
     ph ^= 1;
     tc_fence_after_sync();
     return good;
@@ -193,14 +201,14 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
     s = __ffma2_rn(unpack2(x.x), unpack2(y.x), s); s = __ffma2_rn(unpack2(x.y), unpack2(y.y), s);
     s = __ffma2_rn(unpack2(x.z), unpack2(y.z), s); s = __ffma2_rn(unpack2(x.w), unpack2(y.w), s);
   };
-  auto dots = [&](const uint8_t* g0, const uint8_t* g1, float2& s0, float2& s1) {   // with the state in X; g1 may be NULL
-#pragma unroll 4
-    for (int i = 0; i < 8; ++i) {
-      const uint32_t off = (tid + kThreads * i) * 16;
-      const uint4 x = *reinterpret_cast<const uint4*>(smem + kOffX + off);
-      dot8(__ldg(reinterpret_cast<const uint4*>(g0 + off)), x, s0);
-      if (g1 != nullptr) dot8(__ldg(reinterpret_cast<const uint4*>(g1 + off)), x, s1);
-    }
+  // the thread's 32-column pieces of an adjoint image, fetched long before the state they meet has arrived in X
+  auto fetch8 = [&](const uint8_t* g, uint4 (&x)[8]) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = __ldg(reinterpret_cast<const uint4*>(g + (tid + kThreads * i) * 16));
+  };
+  auto dots = [&](const uint4 (&x)[8], float2& s) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) dot8(x[i], *reinterpret_cast<const uint4*>(smem + kOffX + (tid + kThreads * i) * 16), s);
   };
   auto add_dot = [&](float2 s, float* dst, float sign) {
     float x = s.x + s.y;
@@ -220,6 +228,7 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
   // to dvec.  out: the finished row leaves for global memory instead of returning to tensor memory.
   auto epilogue = [&](uint32_t col, bool first, float w, float* dvec, float sign, TG* out) {
     float2 s = make_float2(0.f, 0.f);
+    __syncwarp();
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       uint32_t z[32];
@@ -256,6 +265,8 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
 
   do {
     // ---- Z_S
+    uint4 adj[8];
+    fetch8(imgdS, adj);
     if (!wait_all(bar_l, ph_l)) break;
     if (tid == 0) {
       const uint64_t dB = smem_desc_sw128(sb + kOffX, 16384, 1024);
@@ -264,13 +275,16 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
       umma_commit(bar_m);
     }
     float2 s0 = make_float2(0.f, 0.f), s1 = s0, s2 = s0;
-    dots(imgdS, nullptr, s1, s2);                                  // <dS', S>
+    dots(adj, s1);                                                 // <dS', S>
     if (!wait_all(bar_m, ph_m)) break;   // (also: every thread is done with S)
     if (tid == 0) { fence_proxy_async_smem(); load_image(kOffX, imgS + 32768); }
     add_dot(s1, V(vdAbar) + n - 1, 1.f);
     epilogue(kColAcc, true, k_row ? -V(vAbar)[r] : scale * V(vAbar)[r], V(vdAbar), k_row ? -1.f : scale, nullptr);
 
     // ---- Z_M
+    uint4 adj2[8];
+    fetch8(imgdS, adj);
+    fetch8(imgdM, adj2);
     if (!wait_all(bar_l, ph_l)) break;
     if (tid == 0) {
       const uint64_t dB = smem_desc_sw128(sb + kOffX, 16384, 1024);
@@ -278,7 +292,8 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
       for (int k = 0; k < 8; ++k) umma_ss(tmem + kColB, half(kOffA1, k), dB + 128 * k, id_nn, k > 0);
       umma_commit(bar_m);
     }
-    dots(imgdM, imgdS, s0, s2);                                    // <dM', M>, <dS', M>
+    dots(adj2, s0);                                                // <dM', M>
+    dots(adj, s2);                                                 // <dS', M>
     if (!wait_all(bar_m, ph_m)) break;
     if (tid == 0) {
       fence_proxy_async_smem();
@@ -366,6 +381,7 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
     {
       const uint32_t tp = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + 32 * hf;
       uint32_t hi[16], lo[16];
+      __syncwarp();
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         uint32_t p[16], x[16];
@@ -386,6 +402,7 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
           split_pack_bf16(make_float2(d[0], d[1]), hi[8 * c + i / 2], lo[8 * c + i / 2]);
         }
       }
+      __syncwarp();
       tmem_st16(tp + kColP, hi);
       tmem_st16(tp + kColP + 16, lo);
       uint8_t* zero = smem + kOffA1;
@@ -473,6 +490,7 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 1) {
+    __syncwarp();
     tc_fence_after_sync();
     tmem_dealloc(tmem, kCols);
   }
@@ -480,35 +498,8 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
     if (tid == 0) atomicCAS(a.status, kDevOk, kDevTimeout);
     return;
   }
-  // ---- gate gradients.  gamma, m by their column recurrences (thread = column) over A1 and X
-  float* Gam = reinterpret_cast<float*>(smem + kOffA1);
-  float* Mm = Gam + C * LG;
-  if (tid < C || (tid >= 128 && tid < 128 + C)) {
-    const int i = tid & 63;
-    const bool gamma = tid < C;
-    float m = 1.f, gam = 0.f;
-#pragma unroll 1
-    for (int rb = 0; rb < C; rb += 4) {
-      const float4 al = *reinterpret_cast<const float4*>(V(vAlpha) + rb), be = *reinterpret_cast<const float4*>(V(vBeta) + rb);
-      const float4 mu = *reinterpret_cast<const float4*>(V(vMu) + rb);
-      const float a4[4] = {al.x, al.y, al.z, al.w}, b4[4] = {be.x, be.y, be.z, be.w}, m4[4] = {mu.x, mu.y, mu.z, mu.w};
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int rr = rb + u;
-        if (rr > i) m *= m4[u];
-        if (gamma) {
-          if (rr >= i) gam = fmaf(a4[u], gam, b4[u] * m);
-          Gam[rr * LG + i] = rr >= i ? gam : 0.f;
-        } else {
-          Mm[rr * LG + i] = rr >= i ? m : 0.f;
-        }
-      }
-    }
-  }
-  __syncthreads();
-  gate_gradients(vec, GateMats{Gam, Mm, Mm + C * LG, Mm + 2 * C * LG},
-                 [&](int rr, int i) { return rr > i ? ge_tri[tri(rr, i)] : rr == i ? ge_diag[i] : 0.f; },
-                 [&](int rr, int i) { return rr > i ? gm_tri[tri(rr, i)] : 0.f; }, V(kPartSlot), n, tok(0), H, a.gates);
+  gate_gradients(vec, [&](int rr, int i) { return rr > i ? ge_tri[tri(rr, i)] : ge_diag[i]; },
+                 [&](int rr, int i) { return gm_tri[tri(rr, i)]; }, reinterpret_cast<float*>(smem + kOffA1), n, tok(0), H, a.gates);
 }
 
 }  // namespace

@@ -181,10 +181,10 @@ struct ParArgs {
 
 template <int DK, int DV> struct ParSmem {   // float offsets
   static constexpr int LDK = DK + 4, LDV = DV + 4, kMat = C * kLT;
-  static constexpr int kStages = 3, kStage = DK * 32, kStageArea = kStages * kStage > 2 * kMat ? kStages * kStage : 2 * kMat;
+  static constexpr int kStages = 3, kStage = DK * 32, kStageArea = kStages * kStage;
   static constexpr int K = 0, Q = K + C * LDK, vec = Q + C * LDK, st = vec + 24 * C, tiles = st + kStageArea,
                        kTiles = 3 * C * LDV > 5 * kMat ? 3 * C * LDV : 5 * kMat, kFloats = tiles + kTiles;
-  static_assert(kFloats * 4 <= 232448, "shared memory");
+  static_assert(kFloats * 4 <= 232448 && kStageArea >= kMat && kMat >= kGateScratch, "shared memory");
 };
 
 // One 256-thread CTA per (chunk, head); its two halves of 128 threads work on different products of the same step, each
@@ -207,7 +207,6 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
   float* Vt = Dr + C * LDV;
   // after the streams / the products: 64 x 64 matrices
   float* Gam = sm + L::st;
-  float* Mm = Gam + L::kMat;
   float* DW = sm + L::tiles;
   float* DWT = DW + L::kMat;
   float* DAS = DWT + L::kMat;   // DA + DA^T
@@ -263,12 +262,14 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
   const float* cf = a.coef + slot_h * MDN_NUM_COEF * C;
   for (int i = tid; i < 24 * C; i += kSimtThreads) vec[i] = 0.f;
   __syncthreads();
-  if (tid < C) {
+  if (tid < C) {   // (all loads before the first store: they must not wait for one another)
     const int r = tid;
-    V(vAbar)[r] = cf[kAbar * C + r]; V(vB)[r] = cf[kB * C + r]; V(vP)[r] = cf[kAlphaBPrev * C + r];
-    V(vGS)[r] = cf[kGS * C + r]; V(vGM)[r] = cf[kGM * C + r]; V(vMubar)[r] = cf[kMubar * C + r];
-    V(vAlpha)[r] = cf[kAlpha * C + r]; V(vMu)[r] = cf[kMu * C + r]; V(vBeta)[r] = cf[kBeta * C + r]; V(vEta)[r] = cf[kEta * C + r];
-    V(vBprev)[r] = r > 0 ? cf[kB * C + r - 1] : 0.f;
+    auto ld = [&](int which, int at) { return __ldg(cf + which * C + at); };
+    const float x0 = ld(kAbar, r), x1 = ld(kB, r), x2 = ld(kAlphaBPrev, r), x3 = ld(kGS, r), x4 = ld(kGM, r), x5 = ld(kMubar, r);
+    const float x6 = ld(kAlpha, r), x7 = ld(kMu, r), x8 = ld(kBeta, r), x9 = ld(kEta, r), x10 = ld(kB, max(r - 1, 0));
+    V(vAbar)[r] = x0; V(vB)[r] = x1; V(vP)[r] = x2; V(vGS)[r] = x3; V(vGM)[r] = x4; V(vMubar)[r] = x5;
+    V(vAlpha)[r] = x6; V(vMu)[r] = x7; V(vBeta)[r] = x8; V(vEta)[r] = x9;
+    V(vBprev)[r] = r > 0 ? x10 : 0.f;
   }
   {   // the end-of-chunk adjoints d mubar_C = <dM', M>, d abar_C = <dS', S>, d b_C = -<dS', M>
     float s0 = 0.f, s1 = 0.f, s2 = 0.f;
@@ -359,7 +360,7 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
     product(A, NP, std::integral_constant<int, 32>{}, [&](int i, int e, int r, float2 g) { add(i, e, wB * vb[r], g); }, X,
             V(half1 ? vdP : vdB), wB);
     cp_wait<0>();
-    __syncthreads();   // the ring has been read: gamma, m take its place
+    __syncthreads();   // the ring has been read: gamma takes its place
 
     if (tid < C) {          // gamma by the column recurrence of Eq. 10 (thread = column), zero above the diagonal
       const int i = tid;
@@ -369,14 +370,6 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
         if (r > i) m *= V(vMu)[r];
         if (r >= i) gam = fmaf(V(vAlpha)[r], gam, V(vBeta)[r] * m);
         Gam[r * kLT + i] = r >= i ? gam : 0.f;
-      }
-    } else if (tid >= 128 && tid < 128 + C) {   // m_{r,i} = mu_{i+1} .. mu_r
-      const int i = tid - 128;
-      float m = 1.f;
-#pragma unroll 4
-      for (int r = 0; r < C; ++r) {
-        if (r > i) m *= V(vMu)[r];
-        Mm[r * kLT + i] = r >= i ? m : 0.f;
       }
     }
     // ---- the four 64 x 64 products, lower triangle: rows rl + 8 i, columns dg + 16 e, e <= i / 2
@@ -403,7 +396,7 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
     float P[R][4], XK[R][4];
     square(P, A, LDV, Vt, LDV, DV);      // dO V~^T | dR V~^T
     square(XK, X, LDK, Ks, LDK, DK);     // Q K^T   | K K^T
-    __syncthreads();   // dO, dR, V~ have been read; gamma, m complete
+    __syncthreads();   // dO, dR, V~ have been read; gamma complete
     // (rows past the tiles' reach: the matrices' rows and columns there are cleared for the gate gradients below)
 #pragma unroll
     for (int i = 0; i < 8; ++i)
@@ -470,9 +463,9 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
   if (n > 32) body(std::integral_constant<int, 8>{});
   else if (n > 16) body(std::integral_constant<int, 4>{});
   else body(std::integral_constant<int, 2>{});
-  __syncthreads();   // DW, DW^T, DA have been read: the gate gradients' work matrices take their places
-  gate_gradients(vec, GateMats{Gam, Mm, DW, DWT}, [&](int r, int i) { return dGe[r * kLT + i]; },
-                 [&](int r, int i) { return dGm[r * kLT + i]; }, DAS, n, tok_h, H, a.gates);
+  __syncthreads();   // DW has been read: the gate gradients' scratch takes its place
+  gate_gradients(vec, [&](int r, int i) { return dGe[r * kLT + i]; }, [&](int r, int i) { return dGm[r * kLT + i]; }, DW, n, tok_h, H,
+                 a.gates);
 }
 
 template <int DK, int NV> cudaError_t launch_adj(const Plan& pl, const AdjArgs& a) {

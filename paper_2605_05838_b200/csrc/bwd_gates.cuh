@@ -13,82 +13,130 @@ constexpr int LG = C + 4;     // floats per row of a 64 x 64 fp32 matrix
 enum Vec : int { vAbar = 0, vB, vP, vGS, vGM, vMubar, vAlpha, vBeta, vMu, vEta, vBprev,
                  vdAbar, vdB, vdP, vdGS, vdGM, vdMubar, vdAlpha, vdBeta, vdMu, vdEta, vRed };
 
-// All [64][LG] fp32 in shared memory: gamma and m (zero above the diagonal), two work matrices for their adjoints.
-struct GateMats { const float* gam; const float* mm; float* dg; float* dm; };
 struct GateOut { float* dbeta; float* dlog_alpha; float* dlog_mu; float* deta; };
 
-// vec: the vectors above; dge(r, i), dgm(r, i): the adjoints of the masks Gamma eta and G^- (asked for any r, i; zero above
-// the diagonal); sPart: 3 x 64 floats of scratch.  Called by all 256 threads after a barrier; tok0_h: index of the chunk's
-// first token in the [token][H] gate arrays.
+// vec: the vectors above; dge(r, i), dgm(r, i): the adjoints of the masks Gamma eta (asked for i <= r) and G^- (i < r);
+// scratch: kGateScratch floats.  Called by all 256 threads after a barrier; tok0_h: index of the chunk's first token in
+// the [token][H] gate arrays.
+//
+// With D = d gamma_{r,i}, E = d m_{r,i} of column i, from the last row up (g_S, g_M enter in the last row):
+//     D = dg + dGeta_{r,i} eta_i,   dg <- alpha_r (D + dG^-_{r,i} eta_i),      E = dm + beta_r D,   dm <- mu_r E
+//     d alpha_r += gamma_{r-1,i} (D + dG^- eta_i),  d beta_r += D m_{r,i},  d mu_r += E m_{r-1,i},
+//     d eta_i += dGeta gamma_{r,i} + dG^- alpha_r gamma_{r-1,i}
+// A thread takes one column and ONE BLOCK OF SIXTEEN ROWS.  Down a block (gamma, m) is a linear map with three scalars
+// [[A, Cm], [0, M]] that no column changes, and (dg, dm) goes back through its transpose plus the block's own terms: so
+// every block is walked on its own (in registers), the blocks are joined by at most three such maps, and the rows' sums over columns
+// are one shuffle reduction of 48 values.  (The 64-row walks this replaces, with gamma, m, D, E as matrices in shared
+// memory, took 24 k of the 66 k cycles of a chunk and head in the tensor-core kernel: almost all of it waiting.)
+constexpr int kGateScratch = 2 * C + 4 * 4 + 4 * C * 2;
+
 template <class FE, class FM>
-__device__ __forceinline__ void gate_gradients(float* vec, const GateMats& mt, FE dge_at, FM dgm_at, float* sPart, int n, size_t tok0_h, int H,
+__device__ __forceinline__ void gate_gradients(float* vec, FE dge_at, FM dgm_at, float* scratch, int n, size_t tok0_h, int H,
                                                const GateOut& a) {
   auto V = [&](int which) { return vec + which * C; };
   auto tok = [&](int r) { return tok0_h + (size_t)r * H; };
-  const float *sGam = mt.gam, *sMm = mt.mm;
-  float *sDg = mt.dg, *sDm = mt.dm;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // In two passes.  Serial (thread i = column i, from the last row up): only the two carried adjoints
-  //     d gamma_{r,i} = dg + dGeta_{r,i} eta_i,      dg <- alpha_r (d gamma_{r,i} + dG^-_{r,i} eta_i)
-  //     d m_{r,i}     = dm + d gamma_{r,i} beta_r,   dm <- mu_r d m_{r,i}
-  // (g_S, g_M enter in the last row), written to the two work matrices.  Everything that is a sum over a
-  // row (d alpha_r, d beta_r, d mu_r) or over a column (d eta_i) of products with these follows on all threads:
-  // shared-memory atomics from the serial walk would serialise 64-way, and the walk itself is one instruction stream.
-  if (tid < C) {
-    const int i = tid;
-    const float eta_i = V(vEta)[i];
-    float dg = V(vdGS)[i] * eta_i, dm = V(vdGM)[i] * eta_i;   // what g_S, g_M give to the last row
-    for (int rb = C - 4; rb >= 0; rb -= 4) {   // four rows' loads first: the walk itself is a chain of three FMAs per row
-      float dge[4], dgm[4];
+  float2* ends = reinterpret_cast<float2*>(scratch);               // [64]: a column's (gamma, m) at the end of its own block
+  float4* maps = reinterpret_cast<float4*>(scratch + 2 * C);       // [4]: A, Cm, M of a block
+  float2* terms = reinterpret_cast<float2*>(scratch + 2 * C + 16); // [4][64]: a block's own terms of (dg, dm)
+  constexpr int RB = 16;
+  const int i = tid & 63, b = tid >> 6, bi = i >> 4, r0 = RB * b;
+  const float *al = V(vAlpha) + r0, *be = V(vBeta) + r0, *mu = V(vMu) + r0;
+  const float eta = V(vEta)[i];
+  {
+    float A = 1.f, Cm = 0.f, M = 1.f, g = 0.f, m = 0.f;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) { dge[u] = dge_at(rb + u, i); dgm[u] = dgm_at(rb + u, i); }
-      const float4 al4 = *reinterpret_cast<const float4*>(V(vAlpha) + rb), be4 = *reinterpret_cast<const float4*>(V(vBeta) + rb);
-      const float4 mu4 = *reinterpret_cast<const float4*>(V(vMu) + rb);
-      const float al[4] = {al4.x, al4.y, al4.z, al4.w}, be[4] = {be4.x, be4.y, be4.z, be4.w}, mu[4] = {mu4.x, mu4.y, mu4.z, mu4.w};
-#pragma unroll
-      for (int u = 3; u >= 0; --u) {
-        const float dgam = fmaf(dge[u], eta_i, dg);
-        const float dmm = fmaf(dgam, be[u], dm);
-        sDg[(rb + u) * LG + i] = dgam;
-        sDm[(rb + u) * LG + i] = dmm;
-        dg = al[u] * fmaf(dgm[u], eta_i, dgam);
-        dm = dmm * mu[u];
-      }
+    for (int u = 0; u < RB; ++u) {
+      const float av = al[u], bv = be[u], mv = mu[u];
+      M *= mv;
+      Cm = fmaf(av, Cm, bv * M);
+      A *= av;
+      m = r0 + u == i ? 1.f : m * mv;
+      g = fmaf(av, g, bv * m);          // (stays 0 until the column begins)
     }
-  } else {
-    // meanwhile on the other six warps, column sums that do not need the walk: d eta_i = sum_r dGeta gamma_{r,i} +
-    // dG^- alpha_r gamma_{r-1,i}, and the last row's g_S, g_M terms (three threads per column, a third of the rows each)
-    const int i = (tid - C) & 63, part = (tid - C) >> 6, r0 = 22 * part, r1 = min(C, r0 + 22);
-    float s = 0.f;
-#pragma unroll 4
-    for (int r = max(r0, i); r < r1; ++r) {
-      s = fmaf(dge_at(r, i), sGam[r * LG + i], s);
-      if (r > i) s = fmaf(dgm_at(r, i) * V(vAlpha)[r], sGam[(r - 1) * LG + i], s);
-    }
-    if (part == 2) s += V(vdGS)[i] * sGam[(C - 1) * LG + i] + V(vdGM)[i] * sMm[(C - 1) * LG + i];
-    sPart[part * C + i] = s;
+    if (bi == b) ends[i] = make_float2(g, m);
+    if (i == 0) maps[b] = make_float4(A, Cm, M, 0.f);
   }
   __syncthreads();
-  {   // row sums, four threads per row: d alpha_r += sum_i gamma_{r-1,i} (d gamma + dG^- eta_i), d beta_r += sum_i
-      // d gamma m_{r,i}, d mu_r += sum_i d m m_{r-1,i}   (columns i <= r; the terms with gamma_{r-1,i}, m_{r-1,i}: i < r)
-    const int r = tid >> 2, part = tid & 3;
-    float sa = 0.f, sbe = 0.f, sm = 0.f;
-#pragma unroll 4
-    for (int i = part; i < C; i += 4) {   // columns interleaved over the row's four threads: conflict-free
-      if (i <= r) {
-        const float dgam = sDg[r * LG + i], dmm = sDm[r * LG + i];
-        sbe = fmaf(dgam, sMm[r * LG + i], sbe);
-        if (i < r) {
-          sa = fmaf(sGam[(r - 1) * LG + i], fmaf(dgm_at(r, i), V(vEta)[i], dgam), sa);
-          sm = fmaf(dmm, sMm[(r - 1) * LG + i], sm);
+  float gam[RB + 1], mm[RB + 1];   // [0]: the row before the block
+  gam[0] = mm[0] = 0.f;
+  if (b > bi) {
+    const float2 e = ends[i];
+    float g = e.x, m = e.y;
+    for (int q = bi + 1; q < b; ++q) {
+      const float4 f = maps[q];
+      g = fmaf(f.x, g, f.y * m);
+      m *= f.z;
+    }
+    gam[0] = g; mm[0] = m;
+  }
+#pragma unroll
+  for (int u = 0; u < RB; ++u) {
+    mm[u + 1] = r0 + u == i ? 1.f : mm[u] * mu[u];
+    gam[u + 1] = fmaf(al[u], gam[u], be[u] * mm[u + 1]);
+  }
+  {   // the block's own terms of (dg, dm)
+    float dg = 0.f, dm = 0.f;
+    if (b >= bi) {
+#pragma unroll
+      for (int u = RB - 1; u >= 0; --u) {
+        const int r = r0 + u;
+        const float ge = r >= i ? dge_at(r, i) * eta : 0.f, gm = r > i ? dgm_at(r, i) * eta : 0.f;
+        const float D = dg + ge, E = fmaf(be[u], D, dm);
+        dg = al[u] * (D + gm);
+        dm = mu[u] * E;
+      }
+    }
+    terms[b * C + i] = make_float2(dg, dm);
+  }
+  __syncthreads();
+  float dg = V(vdGS)[i] * eta, dm = V(vdGM)[i] * eta;   // what g_S, g_M give to the last row
+  for (int q = 3; q > b; --q) {
+    const float4 f = maps[q];
+    const float2 t = terms[q * C + i];
+    dm = fmaf(f.z, dm, fmaf(f.y, dg, t.y));
+    dg = fmaf(f.x, dg, t.x);
+  }
+  float v[3 * RB];   // the rows' terms of d alpha, d beta, d mu
+  float de = 0.f;
+#pragma unroll
+  for (int u = RB - 1; u >= 0; --u) {
+    const int r = r0 + u;
+    const float ge = r >= i ? dge_at(r, i) : 0.f, gm = r > i ? dgm_at(r, i) : 0.f;
+    const float D = fmaf(ge, eta, dg), E = fmaf(be[u], D, dm), Dm = fmaf(gm, eta, D);
+    v[3 * u] = gam[u] * Dm;        // (gamma and m are zero before the column begins)
+    v[3 * u + 1] = D * mm[u + 1];
+    v[3 * u + 2] = E * mm[u];
+    de = fmaf(ge, gam[u + 1], fmaf(gm * al[u], gam[u], de));
+    dg = al[u] * Dm;
+    dm = mu[u] * E;
+  }
+  if (b == 3) de += V(vdGS)[i] * gam[RB] + V(vdGM)[i] * mm[RB];
+  // sums over the warp's 32 columns: halving exchange, 48 -> 3 values per lane pair
+  {
+    int cur = 3 * RB;
+#pragma unroll
+    for (int off = 16; off > 1; off >>= 1) {
+      const bool up = (lane & off) != 0;
+      cur >>= 1;
+#pragma unroll
+      for (int x = 0; x < 3 * RB / 2; ++x) {
+        if (x < cur) {
+          const float give = up ? v[x] : v[x + cur], keep = up ? v[x + cur] : v[x];
+          v[x] = keep + __shfl_xor_sync(0xffffffffu, give, off);
         }
       }
     }
-    sa += __shfl_xor_sync(0xffffffffu, sa, 1); sa += __shfl_xor_sync(0xffffffffu, sa, 2);
-    sbe += __shfl_xor_sync(0xffffffffu, sbe, 1); sbe += __shfl_xor_sync(0xffffffffu, sbe, 2);
-    sm += __shfl_xor_sync(0xffffffffu, sm, 1); sm += __shfl_xor_sync(0xffffffffu, sm, 2);
-    if (part == 0) { V(vdAlpha)[r] += sa; V(vdBeta)[r] += sbe; V(vdMu)[r] += sm; }
+#pragma unroll
+    for (int x = 0; x < 3; ++x) v[x] += __shfl_xor_sync(0xffffffffu, v[x], 1);
   }
+  if ((lane & 1) == 0) {
+    const int r = r0 + (lane >> 1);
+    atomicAdd(V(vdAlpha) + r, v[0]);
+    atomicAdd(V(vdBeta) + r, v[1]);
+    atomicAdd(V(vdMu) + r, v[2]);
+  }
+  atomicAdd(V(vdEta) + i, de);
   __syncthreads();
   // The three vector recurrences (p_r = alpha_r b_{r-1};  b_r = alpha_r b_{r-1} + beta_r mubar_r;  the cumulative
   // products) in reverse, on one warp with two rows per lane and everything in registers.  Each reverse chain
@@ -129,7 +177,7 @@ __device__ __forceinline__ void gate_gradients(float* vec, const GateMats& mt, F
     rev_scan(dMb.x, dMb.y, mu.y, mu2);
     dAl.x = fmaf(dAb.x, ab_prev0, dAl.x); dAl.y = fmaf(dAb.y, ab0, dAl.y);
     dMu.x = fmaf(dMb.x, mb_prev0, dMu.x); dMu.y = fmaf(dMb.y, mb.x, dMu.y);
-    const float de0 = sPart[e0] + sPart[C + e0] + sPart[2 * C + e0], de1 = sPart[e1] + sPart[C + e1] + sPart[2 * C + e1];
+    const float de0 = V(vdEta)[e0], de1 = V(vdEta)[e1];
     if (e0 < n) {
       const size_t gi = tok(e0);
       a.dbeta[gi] = dBe.x; a.dlog_alpha[gi] = al.x * dAl.x; a.dlog_mu[gi] = mu.x * dMu.x;
