@@ -156,6 +156,9 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
     tmem_alloc(smem_u32(&tmem_slot), kCols);
     tc_fence_before_sync();
   }
+  uint4 adj[8];   // the thread's 16-byte pieces of dS' (see dots below): under way with the tiles
+#pragma unroll
+  for (int i = 0; i < 8; ++i) adj[i] = __ldg(reinterpret_cast<const uint4*>(imgdS + (tid + kThreads * i) * 16));
   for (int i = tid; i < 24 * C; i += kThreads) vec[i] = 0.f;
   __syncthreads();
   tc_fence_after_sync();
@@ -194,7 +197,11 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
   };
   const uint32_t id_nn = idesc_bf16(128, 128, false, true, false), id_64 = idesc_bf16(128, 64, false, false, false);
   const uint32_t id_tn = idesc_bf16(128, 128, true, true, false);
-  auto half = [&](uint32_t off, int k) { return smem_desc_sw128(sb + off + (k >> 2) * 16384, 16, 1024) + 2 * (k & 3); };   // K-major, 64-column halves
+  // Products are issued by one elected lane of warp 0 while the whole warp walks the same code: addresses made warp-uniform
+  // here stay in uniform registers (a single thread's descriptor arithmetic took longer than its products)
+  const uint32_t usb = __shfl_sync(0xffffffffu, sb, 0), utm = __shfl_sync(0xffffffffu, tmem, 0);
+  const bool issuer = warp == 0;
+  auto half = [&](uint32_t off, int k) { return smem_desc_sw128(usb + off + (k >> 2) * 16384, 16, 1024) + 2 * (k & 3); };   // K-major, 64-column halves
 
   // sum over the thread's share of <global image, shared image>
   auto dot8 = [&](const uint4& x, const uint4& y, float2& s) {
@@ -265,13 +272,11 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
 
   do {
     // ---- Z_S
-    uint4 adj[8];
-    fetch8(imgdS, adj);
     if (!wait_all(bar_l, ph_l)) break;
-    if (tid == 0) {
-      const uint64_t dB = smem_desc_sw128(sb + kOffX, 16384, 1024);
+    if (issuer && elect_one()) {
+      const uint64_t dB = smem_desc_sw128(usb + kOffX, 16384, 1024);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) umma_ss(tmem + kColAcc, half(kOffA1, k), dB + 128 * k, id_nn, k > 0);
+      for (int k = 0; k < 8; ++k) umma_ss(utm + kColAcc, half(kOffA1, k), dB + 128 * k, id_nn, k > 0);
       umma_commit(bar_m);
     }
     float2 s0 = make_float2(0.f, 0.f), s1 = s0, s2 = s0;
@@ -286,10 +291,10 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
     fetch8(imgdS, adj);
     fetch8(imgdM, adj2);
     if (!wait_all(bar_l, ph_l)) break;
-    if (tid == 0) {
-      const uint64_t dB = smem_desc_sw128(sb + kOffX, 16384, 1024);
+    if (issuer && elect_one()) {
+      const uint64_t dB = smem_desc_sw128(usb + kOffX, 16384, 1024);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) umma_ss(tmem + kColB, half(kOffA1, k), dB + 128 * k, id_nn, k > 0);
+      for (int k = 0; k < 8; ++k) umma_ss(utm + kColB, half(kOffA1, k), dB + 128 * k, id_nn, k > 0);
       umma_commit(bar_m);
     }
     dots(adj2, s0);                                                // <dM', M>
@@ -365,14 +370,14 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
     tc_fence_before_sync();   // (the epilogue's tensor-memory reads of kColB)
     __syncthreads();
     // ---- P = [dO; dR] V~^T, [Q K^T; K K^T]
-    if (tid == 0) {
+    if (issuer && elect_one()) {
       tc_fence_after_sync();
 #pragma unroll
-      for (int k = 0; k < 8; ++k) umma_ss(tmem + kColP, half(kOffA1, k), half(kOffX + 8192, k), id_64, k > 0);
+      for (int k = 0; k < 8; ++k) umma_ss(utm + kColP, half(kOffA1, k), half(kOffX + 8192, k), id_64, k > 0);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) umma_ss(tmem + kColP, half(kOffA1, k), half(kOffX, k), id_64, true);
+      for (int k = 0; k < 8; ++k) umma_ss(utm + kColP, half(kOffA1, k), half(kOffX, k), id_64, true);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) umma_ss(tmem + kColQK, half(kOffA2, k), half(kOffA2 + 8192, k), id_64, k > 0);
+      for (int k = 0; k < 8; ++k) umma_ss(utm + kColQK, half(kOffA2, k), half(kOffA2 + 8192, k), id_64, k > 0);
       umma_commit(bar_m);
     }
     if (!wait_all(bar_m, ph_m)) break;
@@ -420,19 +425,19 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
     tc_fence_before_sync();
     __syncthreads();
     // ---- acc += [DW; DA] K + [0; DW^T] Q + [0; DA^T] K
-    if (tid == 0) {
+    if (issuer && elect_one()) {
       tc_fence_after_sync();
-      const uint64_t dK = smem_desc_sw128(sb + kOffA2 + 8192, 16384, 1024), dQ = smem_desc_sw128(sb + kOffA2, 16384, 1024);
+      const uint64_t dK = smem_desc_sw128(usb + kOffA2 + 8192, 16384, 1024), dQ = smem_desc_sw128(usb + kOffA2, 16384, 1024);
 #pragma unroll
       for (int part = 0; part < 2; ++part)
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          umma_ts(tmem + kColAcc, tmem + kColP + 32 * (k >> 1) + 16 * part + 8 * (k & 1), dK + 128 * k, id_nn, true);
+          umma_ts(utm + kColAcc, utm + kColP + 32 * (k >> 1) + 16 * part + 8 * (k & 1), dK + 128 * k, id_nn, true);
 #pragma unroll
       for (int m = 1; m < 4; ++m) {   // the zero block is rows 0..63 of A, m blocks further on lie rows 64..127
-        const uint64_t dA = smem_desc_sw128(sb + kOffA1, m * 8192, 1024);
+        const uint64_t dA = smem_desc_sw128(usb + kOffA1, m * 8192, 1024);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) umma_ss(tmem + kColAcc, dA + 128 * k, (m == 3 ? dK : dQ) + 128 * k, id_tn, true);
+        for (int k = 0; k < 4; ++k) umma_ss(utm + kColAcc, dA + 128 * k, (m == 3 ? dK : dQ) + 128 * k, id_tn, true);
       }
       umma_commit(bar_m);
     }
@@ -470,12 +475,12 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
 #pragma unroll 1
     for (int which = 0; which < 2; ++which) {
       if (!wait_all(bar_l, ph_l)) { broke = true; break; }
-      if (tid == 0) {
-        const uint64_t dB = smem_desc_sw128(sb + kOffA1, 16384, 1024);
+      if (issuer && elect_one()) {
+        const uint64_t dB = smem_desc_sw128(usb + kOffA1, 16384, 1024);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) umma_ss(tmem + kColB, half(kOffX, k), dB + 128 * k, id_nn, k > 0);
+        for (int k = 0; k < 8; ++k) umma_ss(utm + kColB, half(kOffX, k), dB + 128 * k, id_nn, k > 0);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) umma_ss(tmem + kColB, half(kOffX - 8192, k), dB + 128 * k, id_nn, true);
+        for (int k = 0; k < 8; ++k) umma_ss(utm + kColB, half(kOffX - 8192, k), dB + 128 * k, id_nn, true);
         umma_commit(bar_m);
       }
       if (!wait_all(bar_m, ph_m)) { broke = true; break; }
@@ -498,8 +503,8 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
     if (tid == 0) atomicCAS(a.status, kDevOk, kDevTimeout);
     return;
   }
-  gate_gradients(vec, [&](int rr, int i) { return rr > i ? ge_tri[tri(rr, i)] : ge_diag[i]; },
-                 [&](int rr, int i) { return gm_tri[tri(rr, i)]; }, reinterpret_cast<float*>(smem + kOffA1), n, tok(0), H, a.gates);
+  gate_gradients(vec, [&](int rr, int i) { return ge_tri[rr > i ? tri(rr, i) : 0]; }, [&](int i) { return ge_diag[i]; },
+                 [&](int rr, int i) { return gm_tri[rr > i ? tri(rr, i) : 0]; }, reinterpret_cast<float*>(smem + kOffA1), n, tok(0), H, a.gates);
 }
 
 }  // namespace

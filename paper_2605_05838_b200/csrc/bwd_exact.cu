@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
   else if (n > 16) body(std::integral_constant<int, 4>{});
   else body(std::integral_constant<int, 2>{});
   __syncthreads();   // DW has been read: the gate gradients' scratch takes its place
-  gate_gradients(vec, [&](int r, int i) { return dGe[r * kLT + i]; }, [&](int r, int i) { return dGm[r * kLT + i]; }, DW, n, tok_h, H,
+  gate_gradients(vec, [&](int r, int i) { return dGe[r * kLT + i]; }, [&](int i) { return dGe[i * kLT + i]; }, [&](int r, int i) { return dGm[r * kLT + i]; }, DW, n, tok_h, H,
                  a.gates);
 }
 

@@ -15,9 +15,9 @@ enum Vec : int { vAbar = 0, vB, vP, vGS, vGM, vMubar, vAlpha, vBeta, vMu, vEta, 
 
 struct GateOut { float* dbeta; float* dlog_alpha; float* dlog_mu; float* deta; };
 
-// vec: the vectors above; dge(r, i), dgm(r, i): the adjoints of the masks Gamma eta (asked for i <= r) and G^- (i < r);
-// scratch: kGateScratch floats.  Called by all 256 threads after a barrier; tok0_h: index of the chunk's first token in
-// the [token][H] gate arrays.
+// vec: the vectors above; dge(r, i), dgm(r, i): the adjoints of the masks Gamma eta and G^- strictly below the diagonal (asked
+// for any r, i: what they return elsewhere is not used), dge_diag(i): Gamma eta's on it; scratch: kGateScratch floats.
+// Called by all 256 threads after a barrier; tok0_h: index of the chunk's first token in the [token][H] gate arrays.
 //
 // With D = d gamma_{r,i}, E = d m_{r,i} of column i, from the last row up (g_S, g_M enter in the last row):
 //     D = dg + dGeta_{r,i} eta_i,   dg <- alpha_r (D + dG^-_{r,i} eta_i),      E = dm + beta_r D,   dm <- mu_r E
@@ -30,8 +30,8 @@ struct GateOut { float* dbeta; float* dlog_alpha; float* dlog_mu; float* deta; }
 // memory, took 24 k of the 66 k cycles of a chunk and head in the tensor-core kernel: almost all of it waiting.)
 constexpr int kGateScratch = 2 * C + 4 * 4 + 4 * C * 2;
 
-template <class FE, class FM>
-__device__ __forceinline__ void gate_gradients(float* vec, FE dge_at, FM dgm_at, float* scratch, int n, size_t tok0_h, int H,
+template <class FE, class FD, class FM>
+__device__ __forceinline__ void gate_gradients(float* vec, FE dge_at, FD dge_diag, FM dgm_at, float* scratch, int n, size_t tok0_h, int H,
                                                const GateOut& a) {
   auto V = [&](int which) { return vec + which * C; };
   auto tok = [&](int r) { return tok0_h + (size_t)r * H; };
@@ -41,18 +41,26 @@ __device__ __forceinline__ void gate_gradients(float* vec, FE dge_at, FM dgm_at,
   float2* terms = reinterpret_cast<float2*>(scratch + 2 * C + 16); // [4][64]: a block's own terms of (dg, dm)
   constexpr int RB = 16;
   const int i = tid & 63, b = tid >> 6, bi = i >> 4, r0 = RB * b;
-  const float *al = V(vAlpha) + r0, *be = V(vBeta) + r0, *mu = V(vMu) + r0;
-  const float eta = V(vEta)[i];
+  const float eta = V(vEta)[i], gd = dge_diag(i);
+  // four rows' values of a vector, one 16-byte load (the same address on every lane)
+  auto four = [&](int which, int u, float (&x)[4]) {
+    const float4 t = *reinterpret_cast<const float4*>(V(which) + r0 + u);
+    x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w;
+  };
   {
     float A = 1.f, Cm = 0.f, M = 1.f, g = 0.f, m = 0.f;
 #pragma unroll
-    for (int u = 0; u < RB; ++u) {
-      const float av = al[u], bv = be[u], mv = mu[u];
-      M *= mv;
-      Cm = fmaf(av, Cm, bv * M);
-      A *= av;
-      m = r0 + u == i ? 1.f : m * mv;
-      g = fmaf(av, g, bv * m);          // (stays 0 until the column begins)
+    for (int u4 = 0; u4 < RB; u4 += 4) {
+      float av[4], bv[4], mv[4];
+      four(vAlpha, u4, av); four(vBeta, u4, bv); four(vMu, u4, mv);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        M *= mv[e];
+        Cm = fmaf(av[e], Cm, bv[e] * M);
+        A *= av[e];
+        m = r0 + u4 + e == i ? 1.f : m * mv[e];
+        g = fmaf(av[e], g, bv[e] * m);          // (stays 0 until the column begins)
+      }
     }
     if (bi == b) ends[i] = make_float2(g, m);
     if (i == 0) maps[b] = make_float4(A, Cm, M, 0.f);
@@ -71,20 +79,34 @@ __device__ __forceinline__ void gate_gradients(float* vec, FE dge_at, FM dgm_at,
     gam[0] = g; mm[0] = m;
   }
 #pragma unroll
+  for (int u4 = 0; u4 < RB; u4 += 4) {
+    float av[4], bv[4], mv[4];
+    four(vAlpha, u4, av); four(vBeta, u4, bv); four(vMu, u4, mv);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int u = u4 + e;
+      mm[u + 1] = r0 + u == i ? 1.f : mm[u] * mv[e];
+      gam[u + 1] = fmaf(av[e], gam[u], bv[e] * mm[u + 1]);
+    }
+  }
+  float ge[RB], gm[RB];   // the column's mask adjoints (zero outside the mask; loads without branches)
+#pragma unroll
   for (int u = 0; u < RB; ++u) {
-    mm[u + 1] = r0 + u == i ? 1.f : mm[u] * mu[u];
-    gam[u + 1] = fmaf(al[u], gam[u], be[u] * mm[u + 1]);
+    const float x = dge_at(r0 + u, i), y = dgm_at(r0 + u, i);
+    ge[u] = r0 + u > i ? x : r0 + u == i ? gd : 0.f;
+    gm[u] = r0 + u > i ? y : 0.f;
   }
   {   // the block's own terms of (dg, dm)
     float dg = 0.f, dm = 0.f;
-    if (b >= bi) {
 #pragma unroll
-      for (int u = RB - 1; u >= 0; --u) {
-        const int r = r0 + u;
-        const float ge = r >= i ? dge_at(r, i) * eta : 0.f, gm = r > i ? dgm_at(r, i) * eta : 0.f;
-        const float D = dg + ge, E = fmaf(be[u], D, dm);
-        dg = al[u] * (D + gm);
-        dm = mu[u] * E;
+    for (int u4 = RB - 4; u4 >= 0; u4 -= 4) {
+      float av[4], bv[4], mv[4];
+      four(vAlpha, u4, av); four(vBeta, u4, bv); four(vMu, u4, mv);
+#pragma unroll
+      for (int e = 3; e >= 0; --e) {
+        const float D = fmaf(ge[u4 + e], eta, dg), E = fmaf(bv[e], D, dm);
+        dg = av[e] * fmaf(gm[u4 + e], eta, D);
+        dm = mv[e] * E;
       }
     }
     terms[b * C + i] = make_float2(dg, dm);
@@ -100,16 +122,20 @@ __device__ __forceinline__ void gate_gradients(float* vec, FE dge_at, FM dgm_at,
   float v[3 * RB];   // the rows' terms of d alpha, d beta, d mu
   float de = 0.f;
 #pragma unroll
-  for (int u = RB - 1; u >= 0; --u) {
-    const int r = r0 + u;
-    const float ge = r >= i ? dge_at(r, i) : 0.f, gm = r > i ? dgm_at(r, i) : 0.f;
-    const float D = fmaf(ge, eta, dg), E = fmaf(be[u], D, dm), Dm = fmaf(gm, eta, D);
-    v[3 * u] = gam[u] * Dm;        // (gamma and m are zero before the column begins)
-    v[3 * u + 1] = D * mm[u + 1];
-    v[3 * u + 2] = E * mm[u];
-    de = fmaf(ge, gam[u + 1], fmaf(gm * al[u], gam[u], de));
-    dg = al[u] * Dm;
-    dm = mu[u] * E;
+  for (int u4 = RB - 4; u4 >= 0; u4 -= 4) {
+    float av[4], bv[4], mv[4];
+    four(vAlpha, u4, av); four(vBeta, u4, bv); four(vMu, u4, mv);
+#pragma unroll
+    for (int e = 3; e >= 0; --e) {
+      const int u = u4 + e;
+      const float D = fmaf(ge[u], eta, dg), E = fmaf(bv[e], D, dm), Dm = fmaf(gm[u], eta, D);
+      v[3 * u] = gam[u] * Dm;        // (gamma and m are zero before the column begins)
+      v[3 * u + 1] = D * mm[u + 1];
+      v[3 * u + 2] = E * mm[u];
+      de = fmaf(ge[u], gam[u + 1], fmaf(gm[u] * av[e], gam[u], de));
+      dg = av[e] * Dm;
+      dm = mv[e] * E;
+    }
   }
   if (b == 3) de += V(vdGS)[i] * gam[RB] + V(vdGM)[i] * mm[RB];
   // sums over the warp's 32 columns: halving exchange, 48 -> 3 values per lane pair

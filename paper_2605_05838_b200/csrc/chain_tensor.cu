@@ -192,7 +192,9 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
     }
   }
   const int seq = chain / H, h = chain % H;
-  grid_dependency_wait();   // chunk map, coefficients, T and W (and segment states) come from the previous kernels
+  // what the previous kernel wrote (coefficients, T, W, V of the adjoint run) is read by the producer warp alone: see chain_tf32.cu
+  const bool early = a.seg_G == 0;
+  if (!early) grid_dependency_wait();
   SeqInfo sq = seq_info(a.g, seq);
   if (a.seg_G > 0) {        // restrict the view to this segment's chunks
     const int per = (sq.nchunks + a.seg_G - 1) / a.seg_G;
@@ -300,6 +302,7 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
     // Stage s = c & 1 serves chunk c, then (as the staged output tile) is written out and refilled for chunk c + 2.
     if (lane == 0) {
       int issued = 0;
+      if (early) grid_dependency_wait();
       for (int c = 0; c < nch + 2; ++c) {
         const int s = c & 1;
         const uint32_t st = s_base + kOffStage + s * kStageBytes;

@@ -185,7 +185,11 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
     }
   }
   const int seq = chain / H, h = chain % H;
-  grid_dependency_wait();   // chunk map, coefficients, T and W (and segment states) come from the previous kernels
+  // Coefficients, T and W come from the previous kernel, which lets this one in before it has finished (intra_mma.cu): only
+  // the producer warp waits, in front of its first load of those.  Everything else read here (the call's inputs, the chunk
+  // map) was complete before that kernel could let anybody in.  Segment states come from the kernel just before this one.
+  const bool early = a.seg_G == 0;
+  if (!early) grid_dependency_wait();
   SeqInfo sq = seq_info(a.g, seq);
   if (a.seg_G > 0) {        // restrict the view to this segment's chunks
     const int per = (sq.nchunks + a.seg_G - 1) / a.seg_G;
@@ -345,6 +349,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
         }
         if (c < nch) {
           const uint32_t fb = s ? b_full1 : b_full0;
+          if (early && c == 0) grid_dependency_wait();
           if (lane == 0) {
             const int tok0 = sq.tok0 + c * C;
             const int mat = (sq.slot0 + c) * H + h;
@@ -397,6 +402,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
           if (lazy) { g11 = n11; g12 = n12; g22 = n22; } else { g11 = 1.f; g12 = 0.f; g22 = 1.f; }
           mbar_arrive(s ? b_adj1 : b_adj0);
         } else if (c == nch) {
+          if (early && nch == 0) grid_dependency_wait();   // (every CTA ends after the previous kernel has)
           if (lane == 0) { g_final[0] = g11; g_final[1] = g12; g_final[2] = g22; }
           mbar_arrive(b_fin);
         }

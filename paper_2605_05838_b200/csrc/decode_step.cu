@@ -53,6 +53,10 @@ __global__ void __launch_bounds__(kCols * kGroups) decode_step_kernel(int H, con
   __shared__ float red[kGroups][kCols];
   __shared__ float rbuf[32];
   const int chain = blockIdx.x;       // sequence * H + head
+  // consecutive steps (and the output step behind this kernel) overlap their launches with each other's tails; everything
+  // is read after the wait
+  grid_dependency_wait();
+  grid_launch_dependents();
   const int jj = threadIdx.x % kCols;
   const int j = blockIdx.y * kCols + jj;
   const int dg = threadIdx.x / kCols;
@@ -121,21 +125,12 @@ cudaError_t dispatch(const mdn_params& p, const void* q, const void* k, const vo
                      const float* log_alpha, const float* log_mu, const float* eta, float* S, float* M, void* o,
                      const GateParam& gp, const QkNorm& qk, cudaStream_t st) {
   const bool layer = gp.raw || qk.on;
-#define MDN_DECODE_CASE(DKV, DVV)                                                                              \
-  if (p.dk == DKV && p.dv == DVV) {                                                                            \
-    if (!layer) {                                                                                              \
-      const dim3 grid((unsigned)p.B * p.H, (unsigned)p.dv / 32);                                               \
-      decode_step_kernel<TIn, TO, DKV, DVV, 32, false><<<grid, 32 * kGroups, 0, st>>>(                         \
-          p.H, static_cast<const TIn*>(q), static_cast<const TIn*>(k), static_cast<const TIn*>(v), beta, log_alpha, \
-          log_mu, eta, p.scale, S, M, static_cast<TO*>(o), gp, qk);                                            \
-    } else {                                                                                                   \
-      const dim3 grid((unsigned)p.B * p.H, (unsigned)p.dv / 32);                                               \
-      decode_step_kernel<TIn, TO, DKV, DVV, 32, true><<<grid, 32 * kGroups, 0, st>>>(                          \
-          p.H, static_cast<const TIn*>(q), static_cast<const TIn*>(k), static_cast<const TIn*>(v), beta, log_alpha, \
-          log_mu, eta, p.scale, S, M, static_cast<TO*>(o), gp, qk);                                            \
-    }                                                                                                          \
-    return cudaGetLastError();                                                                                 \
-  }
+#define MDN_DECODE_CASE(DKV, DVV)                                                                                        \
+  if (p.dk == DKV && p.dv == DVV)                                                                                      \
+    return launch_pdl(layer ? decode_step_kernel<TIn, TO, DKV, DVV, 32, true> : decode_step_kernel<TIn, TO, DKV, DVV, 32, false>, \
+                      dim3((unsigned)p.B * p.H, (unsigned)p.dv / 32), dim3(32 * kGroups), 0, st, p.H, static_cast<const TIn*>(q), \
+                      static_cast<const TIn*>(k), static_cast<const TIn*>(v), beta, log_alpha, log_mu, eta, p.scale, S, M,   \
+                      static_cast<TO*>(o), gp, qk);
   MDN_DECODE_CASE(64, 64)
   MDN_DECODE_CASE(64, 128)
   MDN_DECODE_CASE(128, 64)

@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) intra_mma_kernel(ChunkGe
                                                             QkNorm qkn, float scale,
                                                             __nv_bfloat16* __restrict__ Tout,
                                                             __nv_bfloat16* __restrict__ Wout, size_t w_lo_offset,
-                                                            int32_t* __restrict__ status) {
+                                                            int32_t* __restrict__ status, bool clear_status) {
   static_assert(!kQk || kWf32, "the q/k-norm variant uses the fp32 W staging slots");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -150,6 +150,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) intra_mma_kernel(ChunkGe
   __shared__ int abort_flag;
   const int slot = blockIdx.x / g.H, h = blockIdx.x % g.H;
   grid_dependency_wait();   // chunk map and coefficients come from the previous kernels
+  // the call's first kernel: the status word starts clean (only a wait that runs out, seconds later, can set it)
+  if (clear_status && blockIdx.x == 0 && threadIdx.x < 4) status[threadIdx.x] = 0;
   const SlotInfo si = slot_info(g, slot);
   if (si.seq < 0) return;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -476,6 +478,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) intra_mma_kernel(ChunkGe
     }
   }
   __syncthreads();   // staging read out: T takes its place
+  // The tensor memory is free: the chain kernel may come in.  It sets itself up and loads its start state and first tiles
+  // while the rest of this kernel inverts A (see the head of this file for why not earlier).
+  grid_launch_dependents();
 
   // step 1: D_b = (I + A_bb)^{-1} for the four 16x16 diagonal blocks; thread = (block, column), fp32
   if (tid < C) {
@@ -559,7 +564,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) intra_mma_kernel(ChunkGe
     *reinterpret_cast<uint4*>(Tout + mat + rr * C + c0) = packed;
   }
   if (!ok && tid == 0) atomicCAS(status, kDevOk, kDevTimeout);
-  grid_launch_dependents();   // after the tensor memory has been released (see the head of this file)
 }
 
 }  // namespace
@@ -574,7 +578,7 @@ static cudaError_t launch_intra_variant(const Plan& pl, const CUtensorMap& mq, c
                     reinterpret_cast<float*>(pl.ws + pl.lay.off_coef), gates, pl.gp, pl.qk, pl.p.scale,
                     reinterpret_cast<__nv_bfloat16*>(pl.ws + pl.lay.off_T),
                     reinterpret_cast<__nv_bfloat16*>(pl.ws + pl.lay.off_W), n_mats * C * C,
-                    reinterpret_cast<int32_t*>(pl.ws + pl.lay.off_status));
+                    reinterpret_cast<int32_t*>(pl.ws + pl.lay.off_status), pl.clear_status);
 }
 
 cudaError_t launch_intra_mma(const Plan& pl, const void* q, const void* k, const GateArgs& gates, int* launches) {

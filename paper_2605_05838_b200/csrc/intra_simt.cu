@@ -35,6 +35,7 @@ struct IntraArgs {
   IntraBwd bwd;           // set for the exact backward: T, T^T and W^T dO leave instead of T and W
   int dv;
   bool do_bf16;
+  int32_t* clear_status;  // or NULL: the status word, when this is the call's first kernel
 };
 
 template <int DK> struct IntraSmem {   // float offsets
@@ -52,6 +53,7 @@ __global__ void __launch_bounds__(kSimtThreads, 2) intra_simt_kernel(const Intra
   const int H = a.g.H, slot = blockIdx.x / H, h = blockIdx.x % H;
   grid_launch_dependents();
   grid_dependency_wait();
+  if (a.clear_status != nullptr && blockIdx.x == 0 && threadIdx.x < 4) a.clear_status[threadIdx.x] = 0;
   const SlotInfo si = slot_info(a.g, slot);
   if (si.seq < 0) return;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -309,6 +311,7 @@ cudaError_t launch_intra_simt(const Plan& pl, const void* q, const void* k, cons
   a.bwd = bwd;
   a.dv = pl.p.dv;
   a.do_bf16 = pl.p.o_dtype == MDN_BF16;
+  a.clear_status = pl.clear_status ? reinterpret_cast<int32_t*>(pl.ws + pl.lay.off_status) : nullptr;
   const cudaError_t e = pl.p.dk == 64 ? launch_one<64>(pl, a) : launch_one<128>(pl, a);
   if (e == cudaSuccess) ++*launches;
   return e;

@@ -101,16 +101,24 @@ __global__ void __launch_bounds__(256) out_norm_gate_kernel(size_t rows, OutPost
   for (int e = 0; e < E; ++e) wv[e] = post.w ? __ldg(post.w + l * E + e) : 1.f;
   const size_t warps = (size_t)gridDim.x * (blockDim.x >> 5);
   const size_t warp_id = (size_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  for (size_t row0 = warp_id * (RPW * R); row0 < rows; row0 += warps * (RPW * R)) {
+  bool first = true;   // o comes from the previous kernel, which may still be running (g and w are the call's inputs)
+  for (size_t row0 = warp_id * (RPW * R); row0 < rows || first; row0 += warps * (RPW * R)) {
     Pack<TO, E> op[R];
     Pack<TG, E> gp[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const size_t row = row0 + (size_t)r * RPW + sub;
-      if (row < rows) {
-        op[r] = *reinterpret_cast<const Pack<TO, E>*>(o + row * D + l * E);
-        gp[r] = *reinterpret_cast<const Pack<TG, E>*>(g + row * D + l * E);
-      }
+      if (row < rows) gp[r] = *reinterpret_cast<const Pack<TG, E>*>(g + row * D + l * E);
+    }
+    if (first) {
+      grid_dependency_wait();
+      grid_launch_dependents();
+      first = false;
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const size_t row = row0 + (size_t)r * RPW + sub;
+      if (row < rows) op[r] = *reinterpret_cast<const Pack<TO, E>*>(o + row * D + l * E);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -177,7 +185,8 @@ cudaError_t launch_out_norm_gate(const Plan& pl, const OutPost& post, void* o, i
   const size_t rows = (size_t)pl.p.B * pl.p.T * pl.p.H;
   const unsigned grid = blocks_for(rows, 16 * kRowsPerIter);
   const bool obf = pl.p.o_dtype == MDN_BF16, gbf = pl.p.io_dtype == MDN_BF16;
-#define MDN_OUT_CASE(TO, TG, D) out_norm_gate_kernel<TO, TG, D><<<grid, 256, 0, pl.stream>>>(rows, post, static_cast<TO*>(o))
+  cudaError_t e;
+#define MDN_OUT_CASE(TO, TG, D) e = launch_pdl(out_norm_gate_kernel<TO, TG, D>, dim3(grid), dim3(256), 0, pl.stream, rows, post, static_cast<TO*>(o))
 #define MDN_OUT_D(D)                                                   \
   if (obf && gbf) MDN_OUT_CASE(__nv_bfloat16, __nv_bfloat16, D);       \
   else if (obf) MDN_OUT_CASE(__nv_bfloat16, float, D);                 \
@@ -187,7 +196,7 @@ cudaError_t launch_out_norm_gate(const Plan& pl, const OutPost& post, void* o, i
 #undef MDN_OUT_D
 #undef MDN_OUT_CASE
   ++*launches;
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace mdn

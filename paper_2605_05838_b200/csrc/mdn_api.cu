@@ -89,15 +89,29 @@ static mdn_status make_plan(const mdn_params* p, const int32_t* cu, void* ws, si
   return MDN_OK;
 }
 
-// with_scan = false: only the status word and the chunk map (the forward runs the scan inside its intra-chunk kernel).
-static mdn_status run_prep_and_scan(const Plan& pl, const float* beta, const float* log_alpha, const float* log_mu,
-                                    const float* eta, int* launches, bool with_scan = true) {
+static mdn_status check_gates(const float* beta, const float* log_alpha, const float* log_mu, const float* eta) {
   if (!beta || !log_alpha || !log_mu) return MDN_ERR_INVALID_ARG;
   if (!aligned(beta, 4) || !aligned(log_alpha, 4) || !aligned(log_mu, 4) || (eta && !aligned(eta, 4)))
     return MDN_ERR_INVALID_ARG;
-  if (launch_chunk_map(pl, launches) != cudaSuccess) return MDN_ERR_CUDA;   // (also clears the status word)
-  if (with_scan && launch_coeff_scan(pl, beta, log_alpha, log_mu, eta, launches) != cudaSuccess) return MDN_ERR_CUDA;
   return MDN_OK;
+}
+
+static mdn_status run_prep_and_scan(const Plan& pl, const float* beta, const float* log_alpha, const float* log_mu,
+                                    const float* eta, int* launches) {
+  const mdn_status st = check_gates(beta, log_alpha, log_mu, eta);
+  if (st != MDN_OK) return st;
+  if (launch_chunk_map(pl, launches) != cudaSuccess) return MDN_ERR_CUDA;   // (also clears the status word)
+  if (launch_coeff_scan(pl, beta, log_alpha, log_mu, eta, launches) != cudaSuccess) return MDN_ERR_CUDA;
+  return MDN_OK;
+}
+
+// What precedes the intra-chunk kernel of a forward or backward (that kernel runs the coefficient scan itself).  Packed
+// input: the chunk map, which also clears the status word.  Fixed length: nothing, the intra-chunk kernel clears it (a
+// kernel of its own cost 1.5 us of a short call); only the long segmented runs keep the separate one.
+static mdn_status run_prep(Plan& pl, int* launches) {
+  pl.clear_status = pl.geom.cu == nullptr && pl.lay.segments <= 1;
+  if (pl.clear_status) return MDN_OK;
+  return launch_chunk_map(pl, launches) == cudaSuccess ? MDN_OK : MDN_ERR_CUDA;
 }
 
 static mdn_status run_intra(const Plan& pl, const void* q, const void* k, int* launches,
@@ -163,9 +177,8 @@ static mdn_status run_forward(const Plan& plan, const void* q, const void* k, co
       (final_S && !aligned(final_S, 16)) || (final_M && !aligned(final_M, 16)))
     return MDN_ERR_INVALID_ARG;
   if (!mark_stage(0, pl.stream)) return MDN_ERR_CUDA;
-  // the intra-chunk kernels run the coefficient scan themselves (one kernel and one round trip of the coefficient
-  // vectors less); the stand-alone scan kernel is the stage entry point's
-  mdn_status st = run_prep_and_scan(pl, beta, log_alpha, log_mu, eta, &t_last_launches, false);
+  mdn_status st = check_gates(beta, log_alpha, log_mu, eta);
+  if (st == MDN_OK) st = run_prep(pl, &t_last_launches);
   if (st != MDN_OK) return st;
   if (!mark_stage(1, pl.stream)) return MDN_ERR_CUDA;
   st = run_intra(pl, q, k, &t_last_launches, GateArgs{beta, log_alpha, log_mu, eta});
@@ -600,7 +613,8 @@ mdn_status mdn_chunk_bwd(const mdn_params* p, const void* q, const void* k, cons
   Plan pl;
   st = make_plan(&pe, cu_seqlens, workspace, workspace_bytes, cuda_stream, &pl);
   if (st != MDN_OK) return st;
-  if (launch_chunk_map(pl, &t_last_launches) != cudaSuccess) return MDN_ERR_CUDA;
+  st = run_prep(pl, &t_last_launches);
+  if (st != MDN_OK) return st;
   BwdScratch bs;
   bwd_scratch_layout(*p, pl.lay.num_slots, &bs);
   const BwdIo io{q, k, v, beta, log_alpha, log_mu, eta, initial_S, initial_M, d_o, d_final_S, d_final_M,

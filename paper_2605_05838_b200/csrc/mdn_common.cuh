@@ -149,6 +149,7 @@ struct Plan {
   const ChunkGeom* chain_mirror_geom = nullptr;   // q, k, o belong to this geometry, walked in reverse chunk order
   const char* chain_mirror_T = nullptr;           // ... and T ([slot][H][64][64] bf16 of that problem), used transposed
   int cu_total_may_be_short = 0;   // packed: cu[N] <= T instead of == T (the adjoint chain's padded problem)
+  bool clear_status = false;       // the intra-chunk kernel is the call's first one: it clears the status word
   bool w_f32 = false;              // tensor path: the intra-chunk kernel writes W as fp32 (chain_tf32.cu reads it so)
                                    // instead of the bf16 hi + lo pair of chain_tensor.cu
 };

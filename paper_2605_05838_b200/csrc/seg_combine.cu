@@ -2,104 +2,106 @@
 //     [S; M]_g = Phi_g [S; M]_{g-1} + Psi_g          (state at the END of segment g = start of segment g + 1)
 // with Phi_g = [Phi_SS Phi_SM; Phi_MS Phi_MM] assembled from the two basis runs of the segment (from (I, 0): the
 // column blocks Phi_SS, Phi_MS; from (0, I): Phi_SM, Phi_MM) and Psi_g the run from a zero state.  fp32 FMAs: this is
-// (G - 2) products of a 256 x 256 by a 256 x dv matrix per chain, a few percent of the segment runs themselves.
+// (G - 2) products of a 256 x 256 by a 256 x dv matrix per chain.
 //
-// grid = (chains, dv / 16); block = 256 threads: thread i owns row i of the stacked state (i < 128: S, else M) for
-// 16 value columns.  The previous state's 256 x 16 slice sits in shared memory (read as broadcasts); Phi streams
-// through shared memory in 256 x 16 tiles loaded with coalesced float4 reads (next tile prefetched into registers).
-#include "mdn_common.cuh"
+// grid = (chains, dv / 16); block = 256 threads: 8 x 8 tiles of the 256 x 16 result, every sum over the 256 state rows split
+// over four lanes (simt_tile.cuh).  Phi streams through a three-stage ring of 256 x 32 pieces, the previous state's slice
+// stays in shared memory (transposed).  Why this tile: with one row of 16 columns per thread a step spent 17 cycles of the
+// shared-memory port per 4 of the FMA pipes (18 us a step, 144 us of a 65536-token call with 16 heads).
+#include "simt_tile.cuh"
 
 namespace mdn {
 namespace {
 
-constexpr int kD = 128, kCols = 16, kThreads = 2 * kD, kMT = 16, kPad = kMT + 1;
+constexpr int kD = 128, kCols = 16, kPiece = 32, kLd = kPiece + 4, kLp = 2 * kD + 4, kStages = 3, kPieces = 2 * kD / kPiece;
+constexpr int kStage = 2 * kD * kLd;
+constexpr size_t kSmem = (size_t)(kStages * kStage + kCols * kLp) * sizeof(float);
 
-__global__ void __launch_bounds__(kThreads) seg_combine_kernel(int G, float* __restrict__ E,
-                                                              const float* __restrict__ Psi,
-                                                              const float* __restrict__ PhiS,
-                                                              const float* __restrict__ PhiM) {
-  __shared__ __align__(16) float prev[2 * kD][kCols];
-  __shared__ float phi_t[2 * kD][kPad];
+__global__ void __launch_bounds__(kSimtThreads, 1) seg_combine_kernel(int G, float* __restrict__ E,
+                                                                     const float* __restrict__ Psi,
+                                                                     const float* __restrict__ PhiS,
+                                                                     const float* __restrict__ PhiM) {
+  extern __shared__ __align__(16) float sm[];
+  float* prev = sm + kStages * kStage;   // [column][stacked row of the previous state]
   constexpr size_t kMat = (size_t)kD * kD;
-  const int chain = blockIdx.x, j0 = blockIdx.y * kCols;
-  const int i = threadIdx.x, half = i >> 7, row = i & (kD - 1);   // half 0: S rows, 1: M rows
+  const int chain = blockIdx.x, j0 = blockIdx.y * kCols, tid = threadIdx.x;
+  const int s = tid & 3, t = tid >> 2;
+  const int rt = ((t & 1) << 2) | ((t >> 1) & 3) | (t & 24), ct = t >> 5;   // rows rt + 32 i, columns 8 ct + j; a load phase's rows are four apart
   float* e_chain = E + (size_t)chain * (G - 1) * 2 * kMat;
-  {  // state at the end of segment 0 (written by its real run)
-    const float4* src = reinterpret_cast<const float4*>(e_chain + (size_t)half * kMat + (size_t)row * kD + j0);
-#pragma unroll
-    for (int c4 = 0; c4 < kCols / 4; ++c4) *reinterpret_cast<float4*>(&prev[i][c4 * 4]) = src[c4];
+  grid_dependency_wait();
+  for (int i = tid; i < 2 * kD * kCols; i += kSimtThreads) {   // state at the end of segment 0 (written by its real run)
+    const int c = i % kCols, r = i / kCols;
+    prev[c * kLp + r] = e_chain[(size_t)r * kD + j0 + c];      // (S, then M: stacked row r lies at r * 128)
   }
-  // tile loader: element f = i + 256 x covers stacked row f / 4, floats (f % 4) * 4 .. + 3 of the 16-wide tile
-  auto tile_src = [&](size_t seg_off, int mt, int x) {
-    const int f = i + kThreads * x, r = f >> 2, q4 = f & 3;
-    const int m = mt * kMT;                                 // stacked column of the previous state
-    const float* base = (m < kD ? PhiS : PhiM) + seg_off;
-    return reinterpret_cast<const float4*>(base + (size_t)(r >> 7) * kMat + (size_t)(r & (kD - 1)) * kD + (m & (kD - 1)) +
-                                           q4 * 4);
+  const int total = (G - 2) * kPieces;
+  auto fetch = [&](int p) {   // piece p: segment 1 + p / 8, stacked columns 32 (p % 8) ..
+    if (p < total) {
+      const int m = (p % kPieces) * kPiece;
+      const float* src = (m < kD ? PhiS : PhiM) + ((size_t)chain * (G - 2) + p / kPieces) * 2 * kMat + (m & (kD - 1));
+      float* dst = sm + (p % kStages) * kStage;
+#pragma unroll
+      for (int x = 0; x < 2 * kD * kPiece / 4 / kSimtThreads; ++x) {
+        const int f = tid + kSimtThreads * x, r = f >> 3, c4 = (f & 7) * 4;
+        cp16(dst + r * kLd + c4, src + (size_t)r * kD + c4, true);
+      }
+    }
+    cp_commit();
   };
-  __syncthreads();
+  fetch(0);
+  fetch(1);
+  int p = 0;
   for (int g = 1; g <= G - 2; ++g) {
-    const size_t seg_off = ((size_t)chain * (G - 2) + (g - 1)) * 2 * kMat;
-    float acc[kCols];
-    {
-      const float4* psi = reinterpret_cast<const float4*>(Psi + seg_off + (size_t)half * kMat + (size_t)row * kD + j0);
+    const float* psi = Psi + ((size_t)chain * (G - 2) + (g - 1)) * 2 * kMat + j0 + 8 * ct;
+    float4 add[2][2];   // the lane's share of Psi: rows rt + 32 (2 s + e), eight columns
 #pragma unroll
-      for (int c4 = 0; c4 < kCols / 4; ++c4) {
-        const float4 t = psi[c4];
-        acc[c4 * 4] = t.x; acc[c4 * 4 + 1] = t.y; acc[c4 * 4 + 2] = t.z; acc[c4 * 4 + 3] = t.w;
-      }
-    }
-    float4 nxt[4];
+    for (int e = 0; e < 2; ++e)
 #pragma unroll
-    for (int x = 0; x < 4; ++x) nxt[x] = *tile_src(seg_off, 0, x);
-    constexpr int kTiles = 2 * kD / kMT;
+      for (int x = 0; x < 2; ++x)
+        add[e][x] = __ldg(reinterpret_cast<const float4*>(psi + (size_t)(rt + 32 * (2 * s + e)) * kD) + x);
+    float2 acc[8][8];
+    zero2(acc);
 #pragma unroll 1
-    for (int mt = 0; mt < kTiles; ++mt) {
-      __syncthreads();   // previous tile consumed
-#pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        const int f = i + kThreads * x, r = f >> 2, q4 = f & 3;
-        phi_t[r][q4 * 4 + 0] = nxt[x].x; phi_t[r][q4 * 4 + 1] = nxt[x].y;
-        phi_t[r][q4 * 4 + 2] = nxt[x].z; phi_t[r][q4 * 4 + 3] = nxt[x].w;
-      }
-      __syncthreads();
-      if (mt + 1 < kTiles) {
-#pragma unroll
-        for (int x = 0; x < 4; ++x) nxt[x] = *tile_src(seg_off, mt + 1, x);
-      }
-#pragma unroll
-      for (int mm = 0; mm < kMT; ++mm) {
-        const float f = phi_t[i][mm];
-        const float4* pr = reinterpret_cast<const float4*>(prev[mt * kMT + mm]);
-#pragma unroll
-        for (int c4 = 0; c4 < kCols / 4; ++c4) {
-          const float4 pv = pr[c4];
-          acc[c4 * 4 + 0] = fmaf(f, pv.x, acc[c4 * 4 + 0]);
-          acc[c4 * 4 + 1] = fmaf(f, pv.y, acc[c4 * 4 + 1]);
-          acc[c4 * 4 + 2] = fmaf(f, pv.z, acc[c4 * 4 + 2]);
-          acc[c4 * 4 + 3] = fmaf(f, pv.w, acc[c4 * 4 + 3]);
-        }
-      }
+    for (int q = 0; q < kPieces; ++q, ++p) {
+      cp_wait<1>();
+      __syncthreads();   // piece p is in (and the previous state complete); piece p - 1 has been read
+      fetch(p + 2);
+      const float* a = sm + (p % kStages) * kStage + rt * kLd;
+      const float* b = prev + 8 * ct * kLp + q * kPiece;
+      dot_slices<8, 8>(acc, [&](int i) { return a + 32 * i * kLd; }, [&](int j) { return b + j * kLp; }, s, kPiece / 4, 4);
     }
-    float4* out = reinterpret_cast<float4*>(e_chain + ((size_t)g * 2 + half) * kMat + (size_t)row * kD + j0);
+    float v[64];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[8 * i + j] = hsum(acc[i][j]);
+    reduce_scatter<64, 4>(v, s);
     __syncthreads();   // everyone is done reading the previous state
+    float* out = e_chain + (size_t)g * 2 * kMat + j0 + 8 * ct;
 #pragma unroll
-    for (int c4 = 0; c4 < kCols / 4; ++c4) {
-      const float4 t = make_float4(acc[c4 * 4], acc[c4 * 4 + 1], acc[c4 * 4 + 2], acc[c4 * 4 + 3]);
-      out[c4] = t;
-      *reinterpret_cast<float4*>(&prev[i][c4 * 4]) = t;
+    for (int e = 0; e < 2; ++e) {
+      const int r = rt + 32 * (2 * s + e);
+      const float add8[8] = {add[e][0].x, add[e][0].y, add[e][0].z, add[e][0].w, add[e][1].x, add[e][1].y, add[e][1].z, add[e][1].w};
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        v[8 * e + j] += add8[j];
+        prev[(8 * ct + j) * kLp + r] = v[8 * e + j];
+      }
+      float4* o4 = reinterpret_cast<float4*>(out + (size_t)r * kD);
+      o4[0] = make_float4(v[8 * e], v[8 * e + 1], v[8 * e + 2], v[8 * e + 3]);
+      o4[1] = make_float4(v[8 * e + 4], v[8 * e + 5], v[8 * e + 6], v[8 * e + 7]);
     }
-    __syncthreads();
   }
+  cp_wait<0>();
 }
 
 }  // namespace
 
 cudaError_t launch_seg_combine(const Plan& pl, int G, float* E, const float* Psi, const float* PhiS,
                                const float* PhiM, int* launches) {
+  cudaError_t e = cudaFuncSetAttribute(seg_combine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+  if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)pl.geom.num_seqs * pl.p.H, kD / kCols);
-  seg_combine_kernel<<<grid, kThreads, 0, pl.stream>>>(G, E, Psi, PhiS, PhiM);
-  const cudaError_t e = cudaGetLastError();
+  e = launch_pdl(seg_combine_kernel, grid, dim3(kSimtThreads), kSmem, pl.stream, G, E, Psi, PhiS, PhiM);
   if (e == cudaSuccess) ++*launches;
   return e;
 }
