@@ -1093,27 +1093,41 @@ size_t seg_scratch_bytes(const mdn_params& p, int segments) {
   return chains * ((size_t)(segments - 1) * 2 + (size_t)(segments - 2) * 6) * mat;
 }
 
-// Segments per sequence for the parallel scan, from a wave-count model of the two chain launches (one CTA per
-// SM, every CTA walks ceil(nch / G) chunks; a middle segment costs three extra runs) plus about four chunk-times
-// per step of the serial combine.  The scan is used only where the model predicts at most 0.7 of the serial
-// chain's time and every segment keeps at least 8 chunks; otherwise 1 (off).
-int choose_segments(const mdn_params& p) {
-  if (!tensor_path_supported(p) || p.num_seqs > 0) return 1;
-  if (p.segments == 1) return 1;
-  if (p.segments >= 3) return p.segments;
+// How the parallel scan splits a sequence, from a wave-count model in chunk-times (one CTA per SM).  With m middle segments of
+// L chunks per chain, a last one of at most L and a first one of the rest:
+//   phase 1  the first segments' real runs (one SM each from start to end) beside the 3 m runs per chain of the middle
+//            segments on the other SMs (state-only: 0.9 of a full run);
+//   combine  m serial steps;
+//   phase 3  m + 1 real runs per chain.
+// A chunk of the first segment costs one run where one of a middle segment costs four, so the first segment is made as
+// long as phase 1 lasts anyway (equal segments: 1.35 ms of chain time for 16 chains of 1024 chunks; this split: 1.15 ms).
+// Used only where the model predicts at most 0.7 of the serial chain's time; otherwise 1 segment (off).
+SegSplit choose_segments(const mdn_params& p) {
+  const SegSplit off{1, 0, 0};
+  if (!tensor_path_supported(p) || p.num_seqs > 0 || p.segments == 1) return off;
   constexpr long kSMs = 148;
   const long nch = (p.T + C - 1) / C, chains = (long)p.B * p.H;
-  auto waves = [&](long ctas) { return (ctas + kSMs - 1) / kSMs; };
-  const long serial = waves(chains) * nch;
-  long best_cost = serial;
-  int best = 1;
-  for (int g = 3; g <= 32 && nch / g >= 8; ++g) {
-    const long per = (nch + g - 1) / g;
-    // (a state-only run takes about 0.9 of a full one: it skips the output terms, which mostly hide anyway)
-    const long cost = (waves(chains * (1 + 3 * (g - 2))) * 9 * per) / 10 + waves(chains * (g - 1)) * per + 4 * (g - 2);
-    if (cost * 10 <= serial * 7 && cost < best_cost) { best_cost = cost; best = g; }
+  if (p.segments >= 3) {   // forced: equal segments
+    const int per = (int)((nch + p.segments - 1) / p.segments);
+    return SegSplit{p.segments, per, per};
   }
-  return best;
+  auto waves = [](long ctas, long sms) { return (ctas + sms - 1) / sms; };
+  const double serial = (double)(waves(chains, kSMs) * nch);
+  if (chains >= kSMs || nch < 3 * 8) return off;   // no SM left for the middle segments; too short
+  constexpr double kState = 0.9, kRun = 1.7, kStep = 3.2, kFix = 3.;   // state-only chunk; a run's start and end; combine step; launches
+  double best = 0.7 * serial;
+  SegSplit r = off;
+  for (long m = 1; m <= 30 && (m + 1) * 8 < nch; ++m) {
+    const long w1 = waves(3 * m * chains, kSMs - chains), w3 = waves((m + 1) * chains, kSMs);
+    const long at = (long)((nch + kRun * (1 - w1)) / (kState * w1 + m + 1));   // where both kinds of phase-1 runs last equally long
+    for (long L = at > 8 ? at : 8; L <= at + 1 && (m + 1) * L < nch; ++L) {
+      const long first = nch - (m + 1) * L;
+      const double p1 = w1 * (kState * L + kRun), p0 = first + kRun;
+      const double cost = (p1 > p0 ? p1 : p0) + w3 * (L + kRun) + kStep * m * waves(chains * 8, kSMs) + kFix;
+      if (cost < best) { best = cost; r = SegSplit{(int)m + 2, (int)first, (int)L}; }
+    }
+  }
+  return r;
 }
 
 }  // namespace mdn

@@ -122,6 +122,7 @@ struct Args {
   // parallel inter-chunk scan (seg_G = 0: off, one CTA walks all chunks of its chain)
   int seg_G;
   int seg_phase;
+  int seg_first, seg_mid;   // chunks of segment 0, of every other one
   float* seg_E;
   float* seg_Psi;
   float* seg_PhiS;
@@ -174,11 +175,13 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
   // ---- work item: which chain, which segment of it, which kind of run
   int chain = blockIdx.x, seg = 0, run = 0;   // run 0: the real thing; 1: Psi; 2: Phi from (I, 0); 3: Phi from (0, I)
   if (a.seg_G > 0) {
-    if (a.seg_phase == 1) {
-      const int items = 1 + 3 * (a.seg_G - 2);
-      chain = blockIdx.x / items;
-      const int w = blockIdx.x % items;
-      if (w > 0) { seg = 1 + (w - 1) / 3; run = 1 + (w - 1) % 3; }
+    if (a.seg_phase == 1) {   // the first segments (the longest runs) lead
+      const int chains = a.g.num_seqs * H, items = 3 * (a.seg_G - 2), w = (int)blockIdx.x - chains;
+      if (w >= 0) {
+        chain = w / items;
+        seg = 1 + (w % items) / 3;
+        run = 1 + (w % items) % 3;
+      }
     } else {
       chain = blockIdx.x / (a.seg_G - 1);
       seg = 1 + blockIdx.x % (a.seg_G - 1);
@@ -192,8 +195,8 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
   if (!early) grid_dependency_wait();
   SeqInfo sq = seq_info(a.g, seq);
   if (a.seg_G > 0) {        // restrict the view to this segment's chunks
-    const int per = (sq.nchunks + a.seg_G - 1) / a.seg_G;
-    const int cb = min(sq.nchunks, seg * per), ce = min(sq.nchunks, (seg + 1) * per);
+    const int cb = seg == 0 ? 0 : min(sq.nchunks, a.seg_first + (seg - 1) * a.seg_mid);
+    const int ce = min(sq.nchunks, a.seg_first + seg * a.seg_mid);   // (G segments reach the end: choose_segments)
     sq.slot0 += cb;
     sq.tok0 += cb * C;
     sq.len = (ce > cb) ? min(sq.len - cb * C, (ce - cb) * C) : 0;
@@ -931,7 +934,7 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
   a.S0 = S0; a.M0 = M0; a.o = o; a.Sf = Sf; a.Mf = Mf;
   a.status = reinterpret_cast<int32_t*>(pl.ws + pl.lay.off_status);
   a.scale = p.scale;
-  a.seg_G = 0; a.seg_phase = 0;
+  a.seg_G = 0; a.seg_phase = 0; a.seg_first = a.seg_mid = 0;
   a.seg_E = a.seg_Psi = a.seg_PhiS = a.seg_PhiM = nullptr;
   a.qk_on = pl.qk.on; a.qk_d = pl.qk.d;
   a.post_on = pl.post.on; a.post_w = pl.post.w; a.post_g = pl.post.g; a.post_eps = pl.post.eps;
@@ -958,7 +961,9 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
   // ---- parallel inter-chunk scan: Psi / Phi of the middle segments, serial combine, then all segments for real
   constexpr size_t kMat = (size_t)kD * kD;
   float* seg = reinterpret_cast<float*>(pl.ws + pl.lay.off_seg);
+  const SegSplit split = choose_segments(p);
   a.seg_G = G;
+  a.seg_first = split.first; a.seg_mid = split.mid;
   a.seg_E = seg;
   a.seg_Psi = a.seg_E + (size_t)chains * (G - 1) * 2 * kMat;
   a.seg_PhiS = a.seg_Psi + (size_t)chains * (G - 2) * 2 * kMat;

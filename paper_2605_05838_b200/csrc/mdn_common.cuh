@@ -203,7 +203,10 @@ bool chain_uses_tf32_kernel(const Plan& pl);
 // Segment bookkeeping of the parallel inter-chunk scan: per chain (G-1) states E, (G-2) Psi and 2 (G-2) Phi
 // halves, each a pair of [dk x dv] fp32 matrices.
 size_t seg_scratch_bytes(const mdn_params& p, int segments);
-int choose_segments(const mdn_params& p);
+// The parallel inter-chunk scan's split of a sequence of nch chunks: G segments, the first `first` chunks long, the others
+// `mid` (the last one what is left).
+struct SegSplit { int G, first, mid; };
+SegSplit choose_segments(const mdn_params& p);
 cudaError_t launch_seg_combine(const Plan& pl, int G, float* E, const float* Psi, const float* PhiS,
                                const float* PhiM, int* launches);
 
