@@ -41,7 +41,7 @@ struct PrepArgs {
   float* coef_ext;                  // [slots][H][MDN_NUM_COEF][64]
 };
 
-__global__ void __launch_bounds__(kPrepThreads) bwd_prep_kernel(PrepArgs a) {
+__global__ void __launch_bounds__(kPrepThreads, 4) bwd_prep_kernel(PrepArgs a) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   // shared memory: W hi, W lo ([64][L6] each), then the dO tile ([64][LT])
   const int slot = blockIdx.x / a.g.H, h = blockIdx.x % a.g.H, H = a.g.H;
