@@ -189,10 +189,10 @@ template <int DK, int DV> struct ParSmem {   // float offsets
 
 // One 256-thread CTA per (chunk, head); its two halves of 128 threads work on different products of the same step, each
 // thread on 8 rows x dk / 16 columns (simt_tile.cuh: the tile that balances operand loads and FMAs):
-//   half 0:  V~ dS'^T (a part of dK, parked in dk),  dO S^T, dO M^T (dQ),   dO V~^T, Q K^T,  DW K
+//   half 0:  V~ dS'^T (a part of dK),  dO S^T, dO M^T (dQ),   dO V~^T, Q K^T,  DW K
 //   half 1:  V~ dM'^T, dR S^T, dR M^T (dK),                                 dR V~^T, K K^T,  DW^T Q, (DA + DA^T) K
 // The states stream through a three-stage ring (32 value columns of S or M, or 16 of dS' and dM' each); dO, dR, V~, K, Q stay in
-// shared memory, dQ and dK in registers.  Short chunks take tiles of 2 or 4 rows.  Bound by the fp32 pipes and the
+// shared memory.  Chunks of up to 32 tokens take tiles of 4 rows.  Bound by the fp32 pipes and the
 // shared-memory port alike: 9.5 M multiply-adds per chunk and head at dk = dv = 128.
 template <int DK, int DV>
 __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const ParArgs a) {
@@ -296,13 +296,14 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
 
   auto body = [&](auto rows_tag) {
     constexpr int R = decltype(rows_tag)::value;   // rows rl + 8 i, i < R, cover the chunk's n tokens
-    float2 acc[R][E2];                             // half 0: dQ, half 1: dK
-    zero2(acc);
     int step = 0;
-    // G = A B^T over the next `steps` stages of the ring (cols = 16 or 32 value columns each); f(i, e, r, column pair of G)
-    auto product = [&](const float* A, int steps, auto cols_tag, auto f, const float* X, float* dvec, float sign) {
+    // dQ (half 0) and dK (half 1) are summed in their places in global memory (L2): the accumulators of one product are all
+    // the registers can hold next to operands that are on their way
+    auto at = [&](float* g, int r, int e) { return reinterpret_cast<float2*>(g + (tok_h + (size_t)r * H) * DK + 2 * dg + 32 * e); };
+    // G = A B^T over the next `steps` stages of the ring (cols = 16 or 32 value columns each); a coefficient vector's adjoint
+    // += sign (row sums of G o X).  G's column pairs are left in G[i][e].x, G[i][e + E2].x.
+    auto product = [&](const float* A, int steps, auto cols_tag, const float* X, float* dvec, float sign, auto& G) {
       constexpr int kCols = decltype(cols_tag)::value;
-      float2 G[R][2 * E2];
       zero2(G);
       const int swz = kCols == 16 ? (dg >> 1) & 3 : dg & 7;
 #pragma unroll 1
@@ -326,7 +327,7 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
         }
       }
 #pragma unroll
-      for (int i = 0; i < R; ++i) {   // row sums of G o X are the adjoint of the product's coefficient vector
+      for (int i = 0; i < R; ++i) {
         const int r = rl + 8 * i;
         float s = 0.f;
 #pragma unroll
@@ -334,7 +335,7 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
           const float2 g = make_float2(hsum(G[i][e]), hsum(G[i][e + E2]));
           const float2 x = *reinterpret_cast<const float2*>(X + r * LDK + 2 * dg + 32 * e);
           s = fmaf(g.x, x.x, fmaf(g.y, x.y, s));
-          f(i, e, r, g);
+          G[i][e] = g;
         }
         s += __shfl_xor_sync(0xffffffffu, s, 1);
         s += __shfl_xor_sync(0xffffffffu, s, 2);
@@ -343,22 +344,38 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
         if (dg == 0) atomicAdd(dvec + r, sign * s);
       }
     };
-    auto dk_at = [&](int r, int e) { return reinterpret_cast<float2*>(a.dk + (tok_h + (size_t)r * H) * DK + 2 * dg + 32 * e); };
-    auto add = [&](int i, int e, float w, float2 g) { acc[i][e] = __ffma2_rn(make_float2(w, w), g, acc[i][e]); };
-    product(Vt, 2 * NP, std::integral_constant<int, 16>{},
-            [&](int i, int e, int r, float2 g) {
-              if (half1) add(i, e, -V(vGM)[r], g);
-              else if (r < n) *dk_at(r, e) = make_float2(V(vGS)[r] * g.x, V(vGS)[r] * g.y);
-            },
-            Ks, V(half1 ? vdGM : vdGS), half1 ? -1.f : 1.f);
+    // dst (+)= w_r G
+    auto put = [&](float* dst, float wf, const float* w, const auto& G, bool onto) {
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const int r = rl + 8 * i;
+        if (r < n) {
+          const float wr = wf * w[r];
+          float2 x[E2];
+#pragma unroll
+          for (int e = 0; e < E2; ++e) x[e] = onto ? *at(dst, r, e) : make_float2(0.f, 0.f);
+#pragma unroll
+          for (int e = 0; e < E2; ++e) *at(dst, r, e) = __ffma2_rn(make_float2(wr, wr), G[i][e], x[e]);
+        }
+      }
+    };
+    {
+      float2 G[R][2 * E2];
+      product(Vt, 2 * NP, std::integral_constant<int, 16>{}, Ks, V(half1 ? vdGM : vdGS), half1 ? -1.f : 1.f, G);
+      if (!half1) put(a.dk, 1.f, V(vGS), G, false);
+      __syncthreads();   // half 0's part of dK is there; from here on half 1 alone adds to it
+      if (half1) put(a.dk, -1.f, V(vGM), G, true);
+    }
     const float* A = half1 ? Dr : Do;
     const float* X = half1 ? Ks : Qs;
-    const float wA = half1 ? -1.f : scale, wB = half1 ? 1.f : -scale;
-    const float* vb = V(half1 ? vP : vB);
-    product(A, NP, std::integral_constant<int, 32>{}, [&](int i, int e, int r, float2 g) { add(i, e, wA * V(vAbar)[r], g); }, X,
-            V(vdAbar), wA);
-    product(A, NP, std::integral_constant<int, 32>{}, [&](int i, int e, int r, float2 g) { add(i, e, wB * vb[r], g); }, X,
-            V(half1 ? vdP : vdB), wB);
+    float* dst = half1 ? a.dk : a.dq;
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {   // against S, against M
+      float2 G[R][2 * E2];
+      const float w = (half1 ? -1.f : scale) * (pass ? -1.f : 1.f);
+      product(A, NP, std::integral_constant<int, 32>{}, X, V(pass == 0 ? vdAbar : half1 ? vdP : vdB), w, G);
+      put(dst, w, V(pass == 0 ? vAbar : half1 ? vP : vB), G, half1 || pass > 0);
+    }
     cp_wait<0>();
     __syncthreads();   // the ring has been read: gamma takes its place
 
@@ -421,6 +438,8 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
       }
     __syncthreads();
     // ---- dQ += DW K;  dK += DW^T Q + (DA + DA^T) K
+    float2 acc[R][E2];
+    zero2(acc);
     auto rows_times = [&](const float* A, const float* B) {
 #pragma unroll 1
       for (int k = 0; k < n; k += 4) {
@@ -449,20 +468,15 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
       if (r < n) {
 #pragma unroll
         for (int e = 0; e < E2; ++e) {
-          if (!half1) {
-            *reinterpret_cast<float2*>(a.dq + (tok_h + (size_t)r * H) * DK + 2 * dg + 32 * e) = acc[i][e];
-          } else {   // half 0's part has been waiting there
-            float2* at = dk_at(r, e);
-            const float2 x = *at;
-            *at = make_float2(x.x + acc[i][e].x, x.y + acc[i][e].y);
-          }
+          float2* to = at(dst, r, e);
+          const float2 x = *to;
+          *to = make_float2(x.x + acc[i][e].x, x.y + acc[i][e].y);
         }
       }
     }
   };
   if (n > 32) body(std::integral_constant<int, 8>{});
-  else if (n > 16) body(std::integral_constant<int, 4>{});
-  else body(std::integral_constant<int, 2>{});
+  else body(std::integral_constant<int, 4>{});
   __syncthreads();   // DW has been read: the gate gradients' scratch takes its place
   gate_gradients(vec, [&](int r, int i) { return dGe[r * kLT + i]; }, [&](int i) { return dGe[i * kLT + i]; }, [&](int r, int i) { return dGm[r * kLT + i]; }, DW, n, tok_h, H,
                  a.gates);
