@@ -535,6 +535,9 @@ def chunk_attention(q, k, v, beta, log_alpha, log_mu, eta, *, initial_S=None, in
                     scale: Optional[float] = None):
     """The forward as a differentiable torch function (tensor path: bf16 q, k, v, dk = dv = 128): returns
     (o, final_S, final_M); gradients come from the chunk-parallel backward on the states the forward kept."""
+    r = (_nat or _load_native()).chunk_attention(q, k, v, beta, log_alpha, log_mu, eta, initial_S, initial_M, cu_seqlens, scale)
+    if r is not None:
+        return r
     return _ChunkAttention.apply(q, k, v, beta, log_alpha, log_mu, eta, initial_S, initial_M, cu_seqlens, scale)
 
 

@@ -140,7 +140,7 @@ cudaError_t launch_bwd_prep(const Plan& fwd, const void* d_o, void* v_ext, float
   a.v_ext = static_cast<__nv_bfloat16*>(v_ext);
   a.coef_ext = coef_ext;
   const size_t smem = bwd_prep_smem_bytes();
-  cudaError_t e = cudaFuncSetAttribute(bwd_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(bwd_prep_kernel, (int)smem);
   if (e != cudaSuccess) return e;
   bwd_prep_kernel<<<dim3((unsigned)fwd.geom.num_slots * fwd.p.H), dim3(kPrepThreads), smem, fwd.stream>>>(a);
   e = cudaGetLastError();

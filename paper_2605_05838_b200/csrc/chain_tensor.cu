@@ -1046,7 +1046,7 @@ cudaError_t launch_chain_tensor(const Plan& pl, const void* q, const void* k, co
   const unsigned chains = (unsigned)pl.geom.num_seqs * p.H;
   const bool layer = a.qk_on || a.post_on;
   auto launch_as = [&](auto kern, unsigned grid) -> cudaError_t {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+    cudaError_t e = allow_smem(kern, (int)kSmemBytes);
     if (e != cudaSuccess) return e;
     const unsigned threads = layer ? Roles<token_groups(true)>::kThreads : Roles<token_groups(false)>::kThreads;
     e = launch_pdl(kern, dim3(grid), dim3(threads), kSmemBytes, pl.stream, a, mq, mk, mv, mt, mw, mo);

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "layer_ops.cuh"
 #include "mdn.h"
 
@@ -90,6 +92,31 @@ __device__ __forceinline__ SeqInfo seq_info(const ChunkGeom& g, int seq) {
 // attribute): wait for the preceding kernel's results / let the next kernel's prologue start.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// cudaFuncSetAttribute(kern, MaxDynamicSharedMemorySize, bytes), once per kernel and device: the call takes as long as a third of
+// a launch, and the smallest calls are bound by the host.  Kernels of all .cu files share the table; safe with several
+// threads (two of them may both make the call).
+inline cudaError_t allow_smem(const void* kern, int bytes) {
+  constexpr int kSlots = 128, kDevices = 16;
+  struct Slot { std::atomic<const void*> kern{nullptr}; std::atomic<int> bytes[kDevices]{}; };
+  static Slot table[kSlots];
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices)
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  for (int i = 0, at = (int)((reinterpret_cast<uintptr_t>(kern) >> 4) % kSlots); i < kSlots; ++i, at = (at + 1) % kSlots) {
+    const void* seen = nullptr;
+    Slot& s = table[at];
+    if (!s.kern.compare_exchange_strong(seen, kern) && seen != kern) continue;
+    if (s.bytes[dev].load(std::memory_order_acquire) >= bytes) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) s.bytes[dev].store(bytes, std::memory_order_release);
+    return e;
+  }
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+template <typename... A> inline cudaError_t allow_smem(void (*kern)(A...), int bytes) {
+  return allow_smem(reinterpret_cast<const void*>(kern), bytes);
+}
 
 // Launch `kern` so that its prologue may overlap the tail of the previous kernel in the stream; the kernel
 // itself calls grid_dependency_wait() before it touches anything the previous kernel wrote.

@@ -16,6 +16,7 @@
 #include <c10/cuda/CUDAFunctions.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Dtype.h>
+#include <torch/csrc/autograd/custom_function.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "mdn.h"
@@ -319,6 +320,110 @@ PyObject* chunk_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   NATIVE_CATCH
 }
 
+// ---- chunk_attention: the differentiable forward.  The same two calls as _ChunkAttention of binding.py, as a C++ autograd
+// node: a training step of a few hundred tokens takes 55 us on the GPU, and the Python node (apply, saved tensors, the
+// engine's way back into Python) made it 138 us.
+struct AttnPtrs {   // device pointers of defined tensors, NULL otherwise
+  static const float* f(const Tensor& t) { return t.defined() ? static_cast<const float*>(t.const_data_ptr()) : nullptr; }
+};
+
+class ChunkAttention : public torch::autograd::Function<ChunkAttention> {
+  static mdn_params params(const Tensor& q, const Tensor& v, const Tensor& cu, double scale) {
+    const int64_t N = cu.defined() ? cu.numel() - 1 : 0;
+    return mdn_params{(int32_t)q.size(0), (int32_t)q.size(1), (int32_t)q.size(2), (int32_t)q.size(3), (int32_t)v.size(3), 64, (int32_t)N,
+                      MDN_BF16, MDN_BF16, MDN_PATH_TENSOR, (float)scale, 1 /* the kept forward walks its chunks in order */};
+  }
+  static void check(mdn_status st, const char* where) {
+    TORCH_CHECK(st == MDN_OK, where, ": ", mdn_status_string(st), " (status ", (int)st, ")",
+                st == MDN_ERR_CUDA ? std::string(": ") + mdn_last_cuda_error_string() : std::string());
+  }
+
+ public:
+  static torch::autograd::variable_list forward(torch::autograd::AutogradContext* ctx, const Tensor& q, const Tensor& k, const Tensor& v,
+                                                const Tensor& beta, const Tensor& log_alpha, const Tensor& log_mu,
+                                                const std::optional<Tensor>& eta_, const std::optional<Tensor>& S0_,
+                                                const std::optional<Tensor>& M0_, const std::optional<Tensor>& cu_, double scale) {
+    auto get = [](const std::optional<Tensor>& t) { return t.has_value() ? *t : Tensor(); };
+    const Tensor eta = get(eta_), S0 = get(S0_), M0 = get(M0_), cu = get(cu_);
+    const mdn_params p = params(q, v, cu, scale);
+    const c10::DeviceIndex dev = q.get_device();
+    const int64_t n = p.num_seqs > 0 ? p.num_seqs : p.B;
+    const size_t need = mdn_chunk_fwd_workspace_bytes(&p), state_bytes = mdn_chunk_states_bytes(&p);
+    TORCH_CHECK(need != 0 && state_bytes != 0, "mdn_chunk_states_bytes: ", mdn_status_string(MDN_ERR_UNSUPPORTED), " (status 2)");
+    Tensor ws = empty({(int64_t)need}, at::kByte, dev), states = empty({(int64_t)state_bytes}, at::kByte, dev);
+    Tensor o = empty(v.sizes(), q.scalar_type(), dev);
+    Tensor Sf = empty({n, p.H, p.dk, p.dv}, at::kFloat, dev), Mf = empty({n, p.H, p.dk, p.dv}, at::kFloat, dev);
+    check(mdn_chunk_fwd_keep_states(&p, q.const_data_ptr(), k.const_data_ptr(), v.const_data_ptr(), AttnPtrs::f(beta),
+                                    AttnPtrs::f(log_alpha), AttnPtrs::f(log_mu), AttnPtrs::f(eta), AttnPtrs::f(S0), AttnPtrs::f(M0),
+                                    cu.defined() ? static_cast<const int32_t*>(cu.const_data_ptr()) : nullptr, o.data_ptr(),
+                                    static_cast<float*>(Sf.data_ptr()), static_cast<float*>(Mf.data_ptr()), states.data_ptr(),
+                                    ws.data_ptr(), need, stream_of(dev)),
+          "mdn_chunk_fwd_keep_states");
+    ctx->set_materialize_grads(false);
+    ctx->save_for_backward({q, k, v, beta, log_alpha, log_mu, eta, S0, M0, cu, states, ws});
+    ctx->saved_data["scale"] = scale;
+    return {o, Sf, Mf};
+  }
+
+  static torch::autograd::variable_list backward(torch::autograd::AutogradContext* ctx, torch::autograd::variable_list grads) {
+    const auto s = ctx->get_saved_variables();
+    const Tensor &q = s[0], &k = s[1], &v = s[2], &eta = s[6], &S0 = s[7], &M0 = s[8], &cu = s[9], &states = s[10], &ws = s[11];
+    const mdn_params p = params(q, v, cu, ctx->saved_data["scale"].toDouble());
+    const c10::DeviceIndex dev = q.get_device();
+    const int64_t n = p.num_seqs > 0 ? p.num_seqs : p.B;
+    const Tensor d_o = grads[0].defined() ? grads[0].to(q.scalar_type()).contiguous() : at::zeros_like(v);
+    const Tensor dSf = grads[1].defined() ? grads[1].to(at::kFloat).contiguous() : Tensor();
+    const Tensor dMf = grads[2].defined() ? grads[2].to(at::kFloat).contiguous() : Tensor();
+    const size_t need = mdn_chunk_bwd_saved_workspace_bytes(&p);
+    Tensor work = empty({(int64_t)need}, at::kByte, dev);
+    Tensor dq = empty(q.sizes(), q.scalar_type(), dev), dk = empty(q.sizes(), q.scalar_type(), dev), dv = empty(v.sizes(), q.scalar_type(), dev);
+    Tensor g[4], dS0, dM0;   // d beta, d log_alpha, d log_mu, d eta
+    float* gp[4] = {nullptr, nullptr, nullptr, nullptr};
+    for (int i = 0; i < (eta.defined() ? 4 : 3); ++i) {
+      g[i] = empty({p.B, p.T, p.H}, at::kFloat, dev);
+      gp[i] = static_cast<float*>(g[i].data_ptr());
+    }
+    if (S0.defined()) dS0 = empty({n, p.H, p.dk, p.dv}, at::kFloat, dev);
+    if (M0.defined()) dM0 = empty({n, p.H, p.dk, p.dv}, at::kFloat, dev);
+    check(mdn_chunk_bwd_saved_io(&p, q.const_data_ptr(), k.const_data_ptr(), v.const_data_ptr(), AttnPtrs::f(s[3]), AttnPtrs::f(s[4]),
+                                 AttnPtrs::f(s[5]), AttnPtrs::f(eta), cu.defined() ? static_cast<const int32_t*>(cu.const_data_ptr()) : nullptr,
+                                 ws.data_ptr(), (size_t)ws.numel(), states.const_data_ptr(), d_o.const_data_ptr(), AttnPtrs::f(dSf),
+                                 AttnPtrs::f(dMf), dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), gp[0], gp[1], gp[2], gp[3],
+                                 dS0.defined() ? static_cast<float*>(dS0.data_ptr()) : nullptr,
+                                 dM0.defined() ? static_cast<float*>(dM0.data_ptr()) : nullptr, work.data_ptr(), need, stream_of(dev)),
+          "mdn_chunk_bwd_saved_io");
+    return {dq, dk, dv, g[0], g[1], g[2], g[3], dS0, dM0, Tensor(), Tensor()};
+  }
+};
+
+// chunk_attention(q, k, v, beta, log_alpha, log_mu, eta, initial_S, initial_M, cu_seqlens, scale) -> (o, S, M)
+PyObject* chunk_attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  NATIVE_TRY
+  Inputs in;
+  float *S0, *M0, scale;
+  const int32_t* cu;
+  int64_t N;
+  if (n != 11 || !parse_inputs(a, &in) || in.dtype != at::kBFloat16 || in.dk != 128 || in.dv != 128 || !parse_cu(a[9], in.dev, &cu, &N) ||
+      (N > 0 && in.B != 1) || in.B == 0 || in.T == 0 || in.H == 0)
+    return Py_NewRef(Py_None);
+  const int64_t nst = N > 0 ? N : in.B;
+  if (!parse_state(a[7], in, nst, &S0) || !parse_state(a[8], in, nst, &M0) || !parse_scale(a[10], in.dk, &scale)) return Py_NewRef(Py_None);
+  auto maybe = [&](int i) { return a[i] == Py_None ? std::optional<Tensor>() : std::optional<Tensor>(THPVariable_Unpack(a[i])); };
+  torch::autograd::variable_list r;
+  {
+    const Tensor t[6] = {THPVariable_Unpack(a[0]), THPVariable_Unpack(a[1]), THPVariable_Unpack(a[2]),
+                         THPVariable_Unpack(a[3]), THPVariable_Unpack(a[4]), THPVariable_Unpack(a[5])};
+    const std::optional<Tensor> o[4] = {maybe(6), maybe(7), maybe(8), maybe(9)};
+    NoGil g;
+    r = ChunkAttention::apply(t[0], t[1], t[2], t[3], t[4], t[5], o[0], o[1], o[2], o[3], (double)scale);
+  }
+  PyObject* out = PyTuple_New(3);
+  if (!out) return nullptr;
+  for (int i = 0; i < 3; ++i) PyTuple_SET_ITEM(out, i, THPVariable_Wrap(r[i]));
+  return out;
+  NATIVE_CATCH
+}
+
 // ---- make_layer_ops: fills the mdn_layer_ops at an address from the binding's dicts
 bool dict_float(PyObject* d, const char* key, float* out, bool required = true) {
   PyObject* v = PyDict_GetItemString(d, key);
@@ -385,6 +490,7 @@ PyMethodDef methods[] = {
     {"decode_step", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(decode_step)), METH_FASTCALL, nullptr},
     {"chunk_fwd", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(chunk_fwd)), METH_FASTCALL, nullptr},
     {"chunk_bwd", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(chunk_bwd)), METH_FASTCALL, nullptr},
+    {"chunk_attention", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(chunk_attention)), METH_FASTCALL, nullptr},
     {"fill_layer_ops", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(fill_layer_ops)), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 

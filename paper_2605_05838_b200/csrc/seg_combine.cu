@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kSimtThreads, 1) seg_combine_kernel(int G, flo
 
 cudaError_t launch_seg_combine(const Plan& pl, int G, float* E, const float* Psi, const float* PhiS,
                                const float* PhiM, int* launches) {
-  cudaError_t e = cudaFuncSetAttribute(seg_combine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+  cudaError_t e = allow_smem(seg_combine_kernel, (int)kSmem);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)pl.geom.num_seqs * pl.p.H, kD / kCols);
   e = launch_pdl(seg_combine_kernel, grid, dim3(kSimtThreads), kSmem, pl.stream, G, E, Psi, PhiS, PhiM);
