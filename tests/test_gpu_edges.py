@@ -1,0 +1,91 @@
+"""Sizes at which the kernels' splits change: rows per tile of the exact backward (up to 32 tokens / more), value columns
+per CTA of the fp32 chains (8 while that makes at most 148 CTAs, else 16), the uneven segments of the parallel
+inter-chunk scan, and the two routes of the differentiable forward."""
+import numpy as np
+import pytest
+
+import mdn_workloads as wl
+from helpers import rel_err, run_gpu, run_oracle, to_torch
+from test_gpu_bwd import check, run_both, upstream
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mdn():
+    import paper_2605_05838_b200 as m
+    m.lib()
+    return m
+
+
+@pytest.mark.parametrize("B,H,dk,dv,T,dtype", [
+    (1, 1, 64, 64, 31, "f32"), (1, 1, 128, 64, 32, "f32"), (1, 2, 64, 128, 33, "bf16"),
+    (1, 9, 128, 128, 129, "f32"),       # 9 heads x 16 blocks of 8 columns = 144 CTAs
+    (1, 10, 128, 128, 65, "f32"),       # 160: 16 columns per CTA
+    (2, 10, 64, 64, 97, "f32")])
+def test_exact_backward_tiles(mdn, B, H, dk, dv, T, dtype):
+    """fp32 arithmetic throughout: the bound of the exact backward (1e-4 of RMS)."""
+    w = wl.Workload("edge_bwd", B=B, T=T, H=H, dk=dk, dv=dv, dtype=dtype, init_state_std=0.2, seed=T)
+    inp = wl.make_inputs(w)
+    got, ref = run_both(mdn, inp, *upstream(w, inp, T))
+    check(got, ref, "T=%d dk=%d dv=%d H=%d" % (T, dk, dv, H))
+
+
+@pytest.mark.parametrize("H,dv,T", [(9, 128, 130), (10, 128, 70), (18, 64, 64), (19, 64, 65)])
+def test_fp32_chain_columns_per_cta(mdn, H, dv, T):
+    """Both column splits meet the fp32 bound (1e-4) and give the same bits (the sums are split alike)."""
+    w = wl.Workload("edge_simt", B=2, T=T, H=H, dk=64, dv=dv, dtype="f32", init_state_std=0.2, seed=H)
+    inp = wl.make_inputs(w)
+    o, S, M = run_gpu(mdn, inp, path="simt")
+    o_ref, S_ref, M_ref = run_oracle(inp)
+    assert max(rel_err(o, o_ref), rel_err(S, S_ref), rel_err(M, M_ref)) <= 1e-4
+    t = to_torch(inp)
+    part = lambda x: x[:1, :, :1].contiguous()
+    g = [part(t[n]) for n in ("q", "k", "v", "beta", "log_alpha", "log_mu", "eta")]
+    o1, S1, M1 = mdn.chunk_fwd(*g, initial_S=t["initial_S"][:1, :1].contiguous(), initial_M=t["initial_M"][:1, :1].contiguous(),
+                               scale=inp["scale"], path="simt")
+    assert np.array_equal(o1.cpu().numpy()[0, :, 0], np.asarray(o)[0, :, 0])
+    assert np.array_equal(S1.cpu().numpy()[0, 0], np.asarray(S)[0, 0]) and np.array_equal(M1.cpu().numpy()[0, 0], np.asarray(M)[0, 0])
+
+
+@pytest.mark.parametrize("B,H,T", [(1, 1, 64 * 51 + 17), (2, 2, 64 * 61), (1, 8, 64 * 90 + 1)])
+def test_automatic_segments(mdn, B, H, T):
+    """Few long chains are split by rule into unequal segments: same recurrence within the bf16 path's bound, and the first
+    segment's tokens come from the same run as the serial chain's."""
+    import torch
+    w = wl.Workload("edge_seg", B=B, T=T, H=H, dk=128, dv=128, dtype="bf16", init_state_std=0.3, seed=T)
+    lay = mdn.workspace_layout(mdn.MdnParams(B, T, H, 128, 128, 64, 0, 1, 0, 0, 1.0, 0))
+    assert lay.segments > 1
+    inp = wl.make_inputs(w)
+    o_ref, S_ref, M_ref = run_oracle(inp)
+    o, S, M = run_gpu(mdn, inp, path="tensor", o_dtype=torch.float32)
+    assert max(rel_err(o, o_ref), rel_err(S, S_ref), rel_err(M, M_ref)) <= 2e-2
+    o1, _, _ = run_gpu(mdn, inp, path="tensor", o_dtype=torch.float32, segments=1)
+    assert np.array_equal(np.asarray(o)[:, :64], np.asarray(o1)[:, :64])
+
+
+@pytest.mark.parametrize("packed,state,eta", [(False, True, True), (True, True, False), (False, False, False)])
+def test_both_autograd_nodes_give_the_same_bits(mdn, packed, state, eta):
+    """The C++ node and the Python one run the same kernels (gate gradients: sums by atomics, last bits may differ)."""
+    import torch
+    from paper_2605_05838_b200.binding import _ChunkAttention
+    w = wl.Workload("edge_ag", B=1 if packed else 2, T=200, H=2, dk=128, dv=128, dtype="bf16", seed=7, varlen=packed, len_lo=20,
+                    len_hi=90, init_state_std=0.2 if state else 0.0)
+    t = to_torch(wl.make_inputs(w))
+    names = ["q", "k", "v", "beta", "log_alpha", "log_mu"] + (["eta"] if eta else []) + (["initial_S", "initial_M"] if state else [])
+    res = []
+    for native in (True, False):
+        x = {n: t[n].clone().requires_grad_(True) for n in names}
+        kw = dict(initial_S=x.get("initial_S"), initial_M=x.get("initial_M"), cu_seqlens=t["cu_seqlens"])
+        a = (x["q"], x["k"], x["v"], x["beta"], x["log_alpha"], x["log_mu"], x.get("eta"))
+        if native:
+            o, S, M = mdn.chunk_attention(*a, scale=0.1, **kw)
+        else:
+            o, S, M = _ChunkAttention.apply(*a, kw["initial_S"], kw["initial_M"], kw["cu_seqlens"], 0.1)
+        (o.float().square().sum() + S.square().sum()).backward()
+        res.append((o.detach(), S.detach(), M.detach()) + tuple(x[n].grad for n in names))
+    for n, x, y in zip(["o", "S", "M"] + names, *res):
+        if n in ("beta", "log_alpha", "log_mu", "eta"):
+            assert (x - y).abs().max() <= 1e-4 * y.abs().max(), n
+        else:
+            assert torch.equal(x, y), n
