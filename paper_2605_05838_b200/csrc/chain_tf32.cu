@@ -50,14 +50,17 @@ using namespace tc;
 
 constexpr int kD = 128;
 constexpr int kEpiWarps = 8, kTok = 32, kPk = 16;
-// Warp roles: warp 0 MMA issuer, warp 1 TMA producer (it also runs the scalar recurrence of G and writes each chunk's
-// coefficient vectors), warps 2..9 epilogue (lane quarter = warp % 4, as tensor memory demands), warps 10, 11 converters
+// Warp roles: warps 0..7 epilogue (lane quarter = warp % 4, as tensor memory demands), warp 8 MMA issuer, warp 9 TMA producer (it
+// also runs the scalar recurrence of G and writes each chunk's coefficient vectors), warps 10, 11 converters
 // (fp32 copies of the next chunk's K and Q tiles; they sit on the two schedulers that hold neither the MMA nor the
-// TMA warp).  Three warps per scheduler: 168 registers each.  Measured alternatives: the conversion inside the
+// TMA warp).  Three warps per scheduler: 168 registers each.  With the layer operations four more warps (12..15) run the output
+// step's second half; the register file is then split by warpgroup: 168 for the epilogue's two, 88 for the other two.  Measured alternatives: the conversion inside the
 // epilogue warps (behind the hand-over of the state-update operands) put its 1.5 k cycles of shared-memory traffic
 // on the chain's critical path; four converter warps cost the epilogue its registers.
-constexpr int kWarpMma = 0, kWarpTma = 1, kWarpEpi = 2, kWarpCvt = 10, kCvtWarps = 2;
-constexpr int kThreads = (kEpiWarps + 2 + kCvtWarps) * 32;
+constexpr int kWarpEpi = 0, kWarpMma = 8, kWarpTma = 9, kWarpCvt = 10, kCvtWarps = 2, kWarpOut = 12, kOutWarps = 4;
+constexpr int threads_of(bool layer) { return (kEpiWarps + 2 + kCvtWarps + (layer ? kOutWarps : 0)) * 32; }
+constexpr int kOutThreads = kOutWarps * 32, kRegEpi = 168, kRegRest = 88;
+static_assert(8 * 32 * kRegEpi + 8 * 32 * kRegRest <= 65536, "register file");
 constexpr int kEpiThreads = kEpiWarps * 32, kCvtThreads = kCvtWarps * 32;
 
 // shared memory (offsets from a 1024-byte aligned base)
@@ -88,7 +91,7 @@ constexpr uint32_t kColS = 0, kColM = 128, kColX = 256, kColZ = 320, kColY = 384
 
 struct Bars {
   uint64_t full[2];   // TMA loads of a stage landed                                      (1 + tx bytes)
-  uint64_t go[2];     // a stage's output tile is staged and nothing reads the stage any more (256)
+  uint64_t go[2];     // a stage's output tile is staged and nothing reads the stage any more (256; with the fused output step + 128)
   uint64_t cfull;     // bf16 K, Q of a chunk landed in their buffer                         (1 + tx bytes)
   uint64_t cfree;     // ... and read: the next chunk's may be loaded                       (64)
   uint64_t kq;        // fp32 [K; Q] of a chunk written                                   (64)
@@ -106,7 +109,7 @@ struct Bars {
   uint64_t m3;        // MMA-3 done                                                       (commit)
   uint64_t mo;        // MMA-3' done                                                      (commit)
   uint64_t zu;        // U (the chunk's output) has been read                              (256)
-  uint64_t pn;        // fused output step: the fp32 tile is staged / has been read            (256)
+  uint64_t pn[2];     // fused output step: a stage's fp32 tile is staged                     (256)
 };
 
 struct Args {
@@ -156,7 +159,7 @@ template <> __device__ __forceinline__ void stage_o<__nv_bfloat16>(uint8_t* tile
 }
 
 template <typename TO, bool kLayer>
-__global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, const __grid_constant__ CUtensorMap map_q,
+__global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const Args a, const __grid_constant__ CUtensorMap map_q,
                                                                 const __grid_constant__ CUtensorMap map_k,
                                                                 const __grid_constant__ CUtensorMap map_v,
                                                                 const __grid_constant__ CUtensorMap map_t,
@@ -238,7 +241,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
   const uint32_t b_v1b = smem_u32(&bars.v1b), b_mx = smem_u32(&bars.mx), b_m3s = smem_u32(&bars.m3s);
   const uint32_t b_m3 = smem_u32(&bars.m3), b_mo = smem_u32(&bars.mo), b_zu = smem_u32(&bars.zu);
   const uint32_t b_fin = smem_u32(&bars.fin), b_cfull = smem_u32(&bars.cfull), b_cfree = smem_u32(&bars.cfree);
-  const uint32_t b_pn = smem_u32(&bars.pn);
+  const uint32_t b_pn0 = smem_u32(&bars.pn[0]), b_pn1 = smem_u32(&bars.pn[1]);
   // kLayer = false compiles the layer operations out
   const bool qk_on = kLayer && a.qk_on;
   const float qk_dh = (qk_on && a.qk_d) ? __ldg(a.qk_d + h) : 0.f;
@@ -246,12 +249,13 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
   if (tid == 0) {
     abort_flag = 0;
     mbar_init(b_full0, 1); mbar_init(b_full1, 1);
-    mbar_init(b_go0, kEpiThreads); mbar_init(b_go1, kEpiThreads);
+    const uint32_t n_go = kEpiThreads + (kLayer && a.post_on && write_o ? kOutThreads : 0);
+    mbar_init(b_go0, n_go); mbar_init(b_go1, n_go);
     mbar_init(b_kq, kCvtThreads); mbar_init(b_adj0, 32); mbar_init(b_adj1, 32);
     mbar_init(b_fin, 32); mbar_init(b_cfull, 1); mbar_init(b_cfree, kCvtThreads);
     mbar_init(b_init, kEpiThreads); mbar_init(b_r, kEpiThreads); mbar_init(b_oi, kEpiThreads);
     mbar_init(b_v1a, kEpiThreads); mbar_init(b_v1b, kEpiThreads); mbar_init(b_zu, kEpiThreads);
-    if constexpr (kLayer) mbar_init(b_pn, kEpiThreads);
+    if constexpr (kLayer) { mbar_init(b_pn0, kEpiThreads); mbar_init(b_pn1, kEpiThreads); }
     mbar_init(b_m1, 1); mbar_init(b_m2, 1); mbar_init(b_m3, 1); mbar_init(b_mo, 1); mbar_init(b_mx, 1); mbar_init(b_m3s, 1);
     mbar_fence_init();
   }
@@ -286,9 +290,9 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
   __shared__ long long tl_sm[8][32];
 #define MDN_MARK(c, ev) \
   if (tline != nullptr && lane == 0 && (c) >= kTlFirst && (c) < kTlFirst + 8 && \
-      (warp < kWarpEpi || warp == kWarpEpi + 2 || warp >= kWarpCvt)) tl_sm[(c) - kTlFirst][(ev)] = clock64();
+      (warp >= kWarpMma || warp == kWarpEpi + 2)) tl_sm[(c) - kTlFirst][(ev)] = clock64();
 #define MDN_MARK2(c, ev) \
-  if (tline != nullptr && lane == 0 && (c) >= kTlFirst && (c) < kTlFirst + 8 && warp == 7) tl_sm[(c) - kTlFirst][(ev)] = clock64();
+  if (tline != nullptr && lane == 0 && (c) >= kTlFirst && (c) < kTlFirst + 8 && warp == 5) tl_sm[(c) - kTlFirst][(ev)] = clock64();
 #else
 #define MDN_MARK(c, ev)
 #define MDN_MARK2(c, ev)
@@ -301,6 +305,8 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
     tline[30] = clock64(); tline[31] = (long long)ns;
   }
 #endif
+  if (warp >= kWarpMma && warp < kWarpOut) {
+  if constexpr (kLayer) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegRest));   // (warpgroup 8..11)
   if (warp == kWarpTma) {
     // ================================================================== TMA producer + output stores + coefficients
     // Stage s = c & 1 serves chunk c, then (as the staged output tile) is written out and refilled for chunk c + 2.
@@ -522,7 +528,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
         MDN_MARK(c, kEvMIssued);
       }
     }
-  } else if (warp >= kWarpCvt) {
+  } else {
     // ================================================================== converter warps
     // One chunk ahead of the chain: fp32 copies of the K and Q tiles.  bf16 tile: two dk halves of [64 rows x 128 B];
     // fp32 tile: four dk quarters of [128 rows x 128 B].  A thread takes one token row (rows across the lanes:
@@ -536,41 +542,49 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
       for (int which = 0; which < (write_o ? 2 : 1); ++which) {
         const uint32_t src = s_base + kOffCvt + which * 16384 + row * 128;
         const uint32_t dst = s_base + kOffKQ32 + (which * 64 + row) * 128;
-        uint4 u[16];
+        constexpr int kBatch = kLayer ? 8 : 16;   // 16-byte pieces held at a time (88 registers with the layer operations)
+#pragma unroll 1
+        for (int p0 = 0; p0 < 16; p0 += kBatch) {
+          uint4 u[kBatch];
 #pragma unroll
-        for (int c16 = 0; c16 < 16; ++c16)
-          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                       : "=r"(u[c16].x), "=r"(u[c16].y), "=r"(u[c16].z), "=r"(u[c16].w)
-                       : "r"(src + (c16 >> 3) * 8192 + ((static_cast<uint32_t>(c16 & 7) ^ sw) << 4)));
-        if (kLayer && which == 1 && qk_dh != 0.f) {   // (kLayer = false: compiled out)
-          // fused q/k norm: the Q tile's copy is q - d k (fp32, from the two bf16 rows): the output terms then come out
-          // of the same products as for a plain q (their 1/|q - d k| rides on the coefficients)
-#pragma unroll
-          for (int c16 = 0; c16 < 16; ++c16) {
-            uint4 kk;
+          for (int i = 0; i < kBatch; ++i) {
+            const int c16 = p0 + i;
             asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(kk.x), "=r"(kk.y), "=r"(kk.z), "=r"(kk.w)
-                         : "r"(src - 16384 + (c16 >> 3) * 8192 + ((static_cast<uint32_t>(c16 & 7) ^ sw) << 4)));
-            const uint32_t qw[4] = {u[c16].x, u[c16].y, u[c16].z, u[c16].w}, kw[4] = {kk.x, kk.y, kk.z, kk.w};
-            uint32_t f[8];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              f[2 * e] = __float_as_uint(fmaf(-qk_dh, __uint_as_float(kw[e] << 16), __uint_as_float(qw[e] << 16)));
-              f[2 * e + 1] = __float_as_uint(fmaf(-qk_dh, __uint_as_float(kw[e] & 0xffff0000u), __uint_as_float(qw[e] & 0xffff0000u)));
-            }
-            const uint32_t d0 = dst + (c16 >> 2) * 16384, ch = static_cast<uint32_t>((c16 & 3) * 2);
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + ((ch ^ sw) << 4)), "r"(f[0]), "r"(f[1]), "r"(f[2]), "r"(f[3]) : "memory");
-            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + (((ch + 1) ^ sw) << 4)), "r"(f[4]), "r"(f[5]), "r"(f[6]), "r"(f[7]) : "memory");
+                         : "=r"(u[i].x), "=r"(u[i].y), "=r"(u[i].z), "=r"(u[i].w)
+                         : "r"(src + (c16 >> 3) * 8192 + ((static_cast<uint32_t>(c16 & 7) ^ sw) << 4)));
           }
-        } else {
+          if (kLayer && which == 1 && qk_dh != 0.f) {   // (kLayer = false: compiled out)
+            // fused q/k norm: the Q tile's copy is q - d k (fp32, from the two bf16 rows): the output terms then come out
+            // of the same products as for a plain q (their 1/|q - d k| rides on the coefficients)
 #pragma unroll
-        for (int c16 = 0; c16 < 16; ++c16) {
-          const uint32_t d0 = dst + (c16 >> 2) * 16384, ch = static_cast<uint32_t>((c16 & 3) * 2);
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + ((ch ^ sw) << 4)), "r"(u[c16].x << 16),
-                       "r"(u[c16].x & 0xffff0000u), "r"(u[c16].y << 16), "r"(u[c16].y & 0xffff0000u) : "memory");
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + (((ch + 1) ^ sw) << 4)), "r"(u[c16].z << 16),
-                       "r"(u[c16].z & 0xffff0000u), "r"(u[c16].w << 16), "r"(u[c16].w & 0xffff0000u) : "memory");
-        }
+            for (int i = 0; i < kBatch; ++i) {
+              const int c16 = p0 + i;
+              uint4 kk;
+              asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                           : "=r"(kk.x), "=r"(kk.y), "=r"(kk.z), "=r"(kk.w)
+                           : "r"(src - 16384 + (c16 >> 3) * 8192 + ((static_cast<uint32_t>(c16 & 7) ^ sw) << 4)));
+              const uint32_t qw[4] = {u[i].x, u[i].y, u[i].z, u[i].w}, kw[4] = {kk.x, kk.y, kk.z, kk.w};
+              uint32_t f[8];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                f[2 * e] = __float_as_uint(fmaf(-qk_dh, __uint_as_float(kw[e] << 16), __uint_as_float(qw[e] << 16)));
+                f[2 * e + 1] = __float_as_uint(fmaf(-qk_dh, __uint_as_float(kw[e] & 0xffff0000u), __uint_as_float(qw[e] & 0xffff0000u)));
+              }
+              const uint32_t d0 = dst + (c16 >> 2) * 16384, ch = static_cast<uint32_t>((c16 & 3) * 2);
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + ((ch ^ sw) << 4)), "r"(f[0]), "r"(f[1]), "r"(f[2]), "r"(f[3]) : "memory");
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + (((ch + 1) ^ sw) << 4)), "r"(f[4]), "r"(f[5]), "r"(f[6]), "r"(f[7]) : "memory");
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < kBatch; ++i) {
+              const int c16 = p0 + i;
+              const uint32_t d0 = dst + (c16 >> 2) * 16384, ch = static_cast<uint32_t>((c16 & 3) * 2);
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + ((ch ^ sw) << 4)), "r"(u[i].x << 16),
+                           "r"(u[i].x & 0xffff0000u), "r"(u[i].y << 16), "r"(u[i].y & 0xffff0000u) : "memory");
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + (((ch + 1) ^ sw) << 4)), "r"(u[i].z << 16),
+                           "r"(u[i].z & 0xffff0000u), "r"(u[i].w << 16), "r"(u[i].w & 0xffff0000u) : "memory");
+            }
+          }
         }
       }
       mbar_arrive(b_cfree);          // the bf16 tiles have been read: the next chunk's may land
@@ -578,37 +592,33 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
       mbar_arrive(b_kq);
       MDN_MARK(c, kEvCvtDone);
     }
-  } else {
-    // ================================================================== epilogue warps
-    // lane quarter q4 = warp & 3 (value columns 32 q4 .. +31 = this warp's tensor-memory lanes),
-    // token half hf = warp >> 2 (tokens 32 hf .. +31 in the per-token steps, dk columns 64 hf .. +63 of the masters)
-    const int q4 = warp & 3, hf = (warp - kWarpEpi) >> 2;
-    const int d = q4 * 32 + lane;
-    const int r0 = kTok * hf;
-    const uint32_t tl = tmem + (static_cast<uint32_t>(q4 * 32) << 16);
-    const bool post = kLayer && a.post_on && write_o;
-    uint32_t pn_phase = 0;
-    for (int c = 0; c <= nch; ++c) {
-      const float* aj = reinterpret_cast<const float*>(smem + kOffAdj + (c & 1) * kAdjBytes);
-      if constexpr (kLayer) {
-        if (post && c > 0) {
-          // Fused output step of the previous chunk, second half: y = sigmoid(g) * o / sqrt(mean_d o^2 + eps) * w_d.
-          // The staged fp32 tile is re-read row-wise: four threads per token sum its 128 squares, rescale and gate.
-          // fp32 output: written back in place (a thread rewrites only the pieces it has read); bf16 output: the final
-          // tile goes over the start of the fp32 one, once every row has been read.  Then the stage is handed back.
-          const int cp = c - 1;
-          uint8_t* stp = smem + kOffStage + (cp & 1) * kStageBytes;
-          constexpr int kTpr = 4, kPieces = 8;   // threads per token, 16-byte fp32 pieces (8-byte gate pieces) per thread
-          float* tile = reinterpret_cast<float*>(stp + kStOut);
-          const int t128 = q4 * 32 + lane, prow = r0 + t128 / kTpr, part = t128 % kTpr;
-          const bool g_live = cp * C + prow < sq.len;
+  }
+  } else if (kLayer && warp >= kWarpOut) {
+    // ================================================================== output warps
+    if constexpr (kLayer) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegRest));   // (warpgroup 12..15)
+    // Fused output step, second half: y = sigmoid(g) * o / sqrt(mean_d o^2 + eps) * w_d.  The staged fp32 tile is re-read
+    // row-wise, 32 rows at a time: four threads per token sum its 128 squares, rescale and gate.  fp32 output: written back in
+    // place (a thread rewrites only the pieces it has read); bf16 output: the final tile goes over the start of the fp32 one,
+    // 32 rows over the sixteen before them, once those have been read.  These warps work beside the whole next chunk; when
+    // the epilogue warps did this under MMA-1 (2.6 k cycles against its 2.0 k) it delayed every chunk.
+    if (a.post_on && write_o) {
+      constexpr int kTpr = 4, kPieces = 8;   // threads per token, 16-byte fp32 pieces (8-byte gate pieces) per thread
+      const int t128 = tid - kWarpOut * 32, part = t128 % kTpr;
+      for (int c = 0; c < nch; ++c) {
+        uint8_t* stp = smem + kOffStage + (c & 1) * kStageBytes;
+        float* tile = reinterpret_cast<float*>(stp + kStOut);
+        // half 0 first waits for the tile; false (on all four warps: the barrier carries the vote) if that ran out
+        auto rows32 = [&](int half) -> bool {
+          const int prow = 32 * half + t128 / kTpr;
+          const bool g_live = c * C + prow < sq.len;
           const uint2* gp = reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(a.post_g) +
-                                                           ((size_t)(sq.tok0 + cp * C + prow) * H + h) * kD) + part;
+                                                           ((size_t)(sq.tok0 + c * C + prow) * H + h) * kD) + part;
           uint2 graw[kPieces];
 #pragma unroll
           for (int i = 0; i < kPieces; ++i) graw[i] = g_live ? __ldg(gp + kTpr * i) : make_uint2(0u, 0u);
-          MDN_WAIT(b_pn, pn_phase);
-          pn_phase ^= 1;
+          uint32_t good = 1;
+          if (half == 0) good = mbar_wait((c & 1) ? b_pn1 : b_pn0, (c >> 1) & 1, abortp) ? 1u : 0u;
+          __syncwarp();
           float4 ov[kPieces];
           float ss = 0.f;
 #pragma unroll
@@ -619,10 +629,16 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
           ss += __shfl_xor_sync(0xffffffffu, ss, 1);
           ss += __shfl_xor_sync(0xffffffffu, ss, 2);
           const float rstd = rsqrtf(ss * (1.f / kD) + a.post_eps);
-          if (sizeof(TO) == 2) {   // every row read before any bf16 row lands on top of the fp32 tile
-            mbar_arrive(b_pn);
-            MDN_WAIT(b_pn, pn_phase);
-            pn_phase ^= 1;
+          if (half == 0) {   // these 32 rows have been read (what rows 32..63 turn into lies over rows 16..31)
+            asm volatile(
+                "{\n\t.reg .pred p, q;\n\t"
+                "setp.ne.u32 q, %0, 0;\n\t"
+                "barrier.cta.red.and.pred p, 1, %1, q;\n\t"
+                "selp.u32 %0, 1, 0, p;\n\t}\n"
+                : "+r"(good)
+                : "n"(kOutThreads)
+                : "memory");
+            if (good == 0) return false;
           }
 #pragma unroll
           for (int i = 0; i < kPieces; ++i) {
@@ -641,10 +657,27 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
               *reinterpret_cast<uint2*>(stp + kStOut + (prow * kD + col) * 2) = pk;
             }
           }
-          fence_proxy_async_smem();
-          mbar_arrive((cp & 1) ? b_go1 : b_go0);
-        }
+          return true;
+        };
+        ok = rows32(0);
+        if (!ok) break;
+        rows32(1);
+        fence_proxy_async_smem();
+        mbar_arrive((c & 1) ? b_go1 : b_go0);
       }
+    }
+  } else {
+    // ================================================================== epilogue warps
+    if constexpr (kLayer) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegEpi));    // (warpgroups 0..3, 4..7)
+    // lane quarter q4 = warp & 3 (value columns 32 q4 .. +31 = this warp's tensor-memory lanes),
+    // token half hf = warp >> 2 (tokens 32 hf .. +31 in the per-token steps, dk columns 64 hf .. +63 of the masters)
+    const int q4 = warp & 3, hf = (warp - kWarpEpi) >> 2;
+    const int d = q4 * 32 + lane;
+    const int r0 = kTok * hf;
+    const uint32_t tl = tmem + (static_cast<uint32_t>(q4 * 32) << 16);
+    const bool post = kLayer && a.post_on && write_o;
+    for (int c = 0; c <= nch; ++c) {
+      const float* aj = reinterpret_cast<const float*>(smem + kOffAdj + (c & 1) * kAdjBytes);
       if (c == 0) {
         // ---------------- the start state into the masters
 #pragma unroll 1
@@ -688,12 +721,6 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
       const uint32_t ph = c & 1;
       uint8_t* stg = smem + kOffStage + (c & 1) * kStageBytes;
       const __nv_bfloat16* sV = reinterpret_cast<const __nv_bfloat16*>(stg + kStV);
-      if constexpr (kLayer) if (post) {   // the chunk's output-gate rows towards L2: read at the end of the chunk
-        const int t128 = q4 * 32 + lane, prow = r0 + t128 / 4, part = t128 % 4;
-        if (part < 2 && c * C + prow < sq.len)
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const __nv_bfloat16*>(a.post_g) +
-                                                        ((size_t)(sq.tok0 + c * C + prow) * H + h) * kD + 64 * part));
-      }
       MDN_WAIT((c & 1) ? b_full1 : b_full0, (c >> 1) & 1);
       MDN_WAIT((c & 1) ? b_adj1 : b_adj0, (c >> 1) & 1);
       // ---------------- EPI-1: R^T = V^T - cX .* X + cY .* Y  -> bf16 hi, lo in X
@@ -876,11 +903,11 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
           for (int j = 0; j < kTok; ++j) stage_o<TO>(stg + kStOut, r0 + j, d, __uint_as_float(u[j]));
         } else if constexpr (kLayer) {
           // fused output step, first half: the fp32 tile (value columns across the lanes; V, T and half of the W area,
-          // all dead by now).  The rest runs at the top of the next iteration, under the next chunk's MMA-1.
+          // all dead by now).  The output warps do the rest.
           float* tile = reinterpret_cast<float*>(stg + kStOut);
 #pragma unroll
           for (int j = 0; j < kTok; ++j) tile[(r0 + j) * kD + d] = __uint_as_float(u[j]);
-          mbar_arrive(b_pn);
+          mbar_arrive((c & 1) ? b_pn1 : b_pn0);
         }
         fence_proxy_async_smem();
         MDN_MARK(c, kEvOutDone);
@@ -888,7 +915,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tf32_kernel(const Args a, c
       // the stage may be refilled once MMA-3, the last reader of its K tile, is done
       MDN_WAIT(b_m3, ph);
       MDN_MARK(c, kEvM3Seen);
-      if (!post) mbar_arrive((c & 1) ? b_go1 : b_go0);   // (fused output step: after its second half)
+      mbar_arrive((c & 1) ? b_go1 : b_go0);
     }
   }
 #undef MDN_WAIT
@@ -950,7 +977,7 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
                       : (o_bf16 ? chain_tf32_kernel<__nv_bfloat16, false> : chain_tf32_kernel<float, false>);
     cudaError_t e = allow_smem(kern, (int)kSmemBytes);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(kern, dim3(grid), dim3(kThreads), kSmemBytes, pl.stream, a, mq, mk, mv, mt, mw, mo);
+    e = launch_pdl(kern, dim3(grid), dim3(threads_of(layer)), kSmemBytes, pl.stream, a, mq, mk, mv, mt, mw, mo);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) ++*launches;
     return e;
