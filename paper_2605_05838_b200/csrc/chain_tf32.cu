@@ -53,13 +53,15 @@ constexpr int kEpiWarps = 8, kTok = 32, kPk = 16;
 // Warp roles: warps 0..7 epilogue (lane quarter = warp % 4, as tensor memory demands), warp 8 MMA issuer, warp 9 TMA producer (it
 // also runs the scalar recurrence of G and writes each chunk's coefficient vectors), warps 10, 11 converters
 // (fp32 copies of the next chunk's K and Q tiles; they sit on the two schedulers that hold neither the MMA nor the
-// TMA warp).  Three warps per scheduler: 168 registers each.  With the layer operations four more warps (12..15) run the output
-// step's second half; the register file is then split by warpgroup: 168 for the epilogue's two, 88 for the other two.  Measured alternatives: the conversion inside the
+// TMA warp).  Three warps per scheduler: 168 registers each.  Measured alternatives: the conversion inside the
 // epilogue warps (behind the hand-over of the state-update operands) put its 1.5 k cycles of shared-memory traffic
 // on the chain's critical path; four converter warps cost the epilogue its registers.
+// With the layer operations four more warps (12..15) run the output step's second half, and the register file is split
+// by warpgroup: 152 for the epilogue's two, 104 for the other two.  4 x 3001 tokens x 16 heads with q/k norm and output
+// step: 298 -> 267 us for the whole call (1 x 2048 x 16: 177 -> 151).
 constexpr int kWarpEpi = 0, kWarpMma = 8, kWarpTma = 9, kWarpCvt = 10, kCvtWarps = 2, kWarpOut = 12, kOutWarps = 4;
 constexpr int threads_of(bool layer) { return (kEpiWarps + 2 + kCvtWarps + (layer ? kOutWarps : 0)) * 32; }
-constexpr int kOutThreads = kOutWarps * 32, kRegEpi = 168, kRegRest = 88;
+constexpr int kOutThreads = kOutWarps * 32, kRegEpi = 152, kRegRest = 104;
 static_assert(8 * 32 * kRegEpi + 8 * 32 * kRegRest <= 65536, "register file");
 constexpr int kEpiThreads = kEpiWarps * 32, kCvtThreads = kCvtWarps * 32;
 
@@ -538,52 +540,72 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
       MDN_WAIT(b_cfull, c & 1);
       if (c > 0) MDN_WAIT(b_m1, (c - 1) & 1);   // the previous chunk's products have read the fp32 tiles
       MDN_MARK(c, kEvCvtStart);
-#pragma unroll 1
-      for (int which = 0; which < (write_o ? 2 : 1); ++which) {
-        const uint32_t src = s_base + kOffCvt + which * 16384 + row * 128;
-        const uint32_t dst = s_base + kOffKQ32 + (which * 64 + row) * 128;
-        constexpr int kBatch = kLayer ? 8 : 16;   // 16-byte pieces held at a time (88 registers with the layer operations)
-#pragma unroll 1
-        for (int p0 = 0; p0 < 16; p0 += kBatch) {
-          uint4 u[kBatch];
+      if constexpr (kLayer) {
+        // Fused q/k norm: the Q tile's copy is q - d k (fp32, from the two bf16 rows): the output terms then come out of the same
+        // products as for a plain q (their 1/|q - d k| rides on the coefficients).  Both rows together, four pieces of each ahead:
+        // the next chunk's MMA-1 waits for this (K then Q with K's pieces re-read one by one took 5..6 k cycles).
+        const uint32_t src = s_base + kOffCvt + row * 128, dst = s_base + kOffKQ32 + row * 128;
+        auto ld = [&](uint4& u, uint32_t at, int c16) {
+          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                       : "=r"(u.x), "=r"(u.y), "=r"(u.z), "=r"(u.w)
+                       : "r"(at + (c16 >> 3) * 8192 + ((static_cast<uint32_t>(c16 & 7) ^ sw) << 4)));
+        };
+        auto st = [&](uint32_t at, const float (&f)[8], int c16) {
+          const uint32_t d0 = at + (c16 >> 2) * 16384, ch = static_cast<uint32_t>((c16 & 3) * 2);
+          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + ((ch ^ sw) << 4)), "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]) : "memory");
+          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + (((ch + 1) ^ sw) << 4)), "f"(f[4]), "f"(f[5]), "f"(f[6]), "f"(f[7]) : "memory");
+        };
+        auto widen = [](float (&f)[8], const uint4& u) {
+          const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
-          for (int i = 0; i < kBatch; ++i) {
-            const int c16 = p0 + i;
-            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(u[i].x), "=r"(u[i].y), "=r"(u[i].z), "=r"(u[i].w)
-                         : "r"(src + (c16 >> 3) * 8192 + ((static_cast<uint32_t>(c16 & 7) ^ sw) << 4)));
+          for (int e = 0; e < 4; ++e) {
+            f[2 * e] = __uint_as_float(w[e] << 16);
+            f[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
           }
-          if (kLayer && which == 1 && qk_dh != 0.f) {   // (kLayer = false: compiled out)
-            // fused q/k norm: the Q tile's copy is q - d k (fp32, from the two bf16 rows): the output terms then come out
-            // of the same products as for a plain q (their 1/|q - d k| rides on the coefficients)
+        };
+        uint4 uk[2][4], uq[2][4];
+        auto load4 = [&](int p) {
 #pragma unroll
-            for (int i = 0; i < kBatch; ++i) {
-              const int c16 = p0 + i;
-              uint4 kk;
-              asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                           : "=r"(kk.x), "=r"(kk.y), "=r"(kk.z), "=r"(kk.w)
-                           : "r"(src - 16384 + (c16 >> 3) * 8192 + ((static_cast<uint32_t>(c16 & 7) ^ sw) << 4)));
-              const uint32_t qw[4] = {u[i].x, u[i].y, u[i].z, u[i].w}, kw[4] = {kk.x, kk.y, kk.z, kk.w};
-              uint32_t f[8];
+          for (int i = 0; i < 4; ++i) {
+            ld(uk[p & 1][i], src, 4 * p + i);
+            if (write_o) ld(uq[p & 1][i], src + 16384, 4 * p + i);
+          }
+        };
+        load4(0);
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                f[2 * e] = __float_as_uint(fmaf(-qk_dh, __uint_as_float(kw[e] << 16), __uint_as_float(qw[e] << 16)));
-                f[2 * e + 1] = __float_as_uint(fmaf(-qk_dh, __uint_as_float(kw[e] & 0xffff0000u), __uint_as_float(qw[e] & 0xffff0000u)));
-              }
-              const uint32_t d0 = dst + (c16 >> 2) * 16384, ch = static_cast<uint32_t>((c16 & 3) * 2);
-              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + ((ch ^ sw) << 4)), "r"(f[0]), "r"(f[1]), "r"(f[2]), "r"(f[3]) : "memory");
-              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + (((ch + 1) ^ sw) << 4)), "r"(f[4]), "r"(f[5]), "r"(f[6]), "r"(f[7]) : "memory");
+        for (int p = 0; p < 4; ++p) {
+          if (p < 3) load4(p + 1);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            float kf[8], qf[8];
+            widen(kf, uk[p & 1][i]);
+            st(dst, kf, 4 * p + i);
+            if (write_o) {
+              widen(qf, uq[p & 1][i]);
+#pragma unroll
+              for (int e = 0; e < 8; ++e) qf[e] = fmaf(-qk_dh, kf[e], qf[e]);
+              st(dst + 64 * 128, qf, 4 * p + i);
             }
-          } else {
+          }
+        }
+      } else {
+#pragma unroll 1
+        for (int which = 0; which < (write_o ? 2 : 1); ++which) {
+          const uint32_t src = s_base + kOffCvt + which * 16384 + row * 128;
+          const uint32_t dst = s_base + kOffKQ32 + (which * 64 + row) * 128;
+          uint4 u[16];
 #pragma unroll
-            for (int i = 0; i < kBatch; ++i) {
-              const int c16 = p0 + i;
-              const uint32_t d0 = dst + (c16 >> 2) * 16384, ch = static_cast<uint32_t>((c16 & 3) * 2);
-              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + ((ch ^ sw) << 4)), "r"(u[i].x << 16),
-                           "r"(u[i].x & 0xffff0000u), "r"(u[i].y << 16), "r"(u[i].y & 0xffff0000u) : "memory");
-              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + (((ch + 1) ^ sw) << 4)), "r"(u[i].z << 16),
-                           "r"(u[i].z & 0xffff0000u), "r"(u[i].w << 16), "r"(u[i].w & 0xffff0000u) : "memory");
-            }
+          for (int c16 = 0; c16 < 16; ++c16)
+            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(u[c16].x), "=r"(u[c16].y), "=r"(u[c16].z), "=r"(u[c16].w)
+                         : "r"(src + (c16 >> 3) * 8192 + ((static_cast<uint32_t>(c16 & 7) ^ sw) << 4)));
+#pragma unroll
+          for (int c16 = 0; c16 < 16; ++c16) {
+            const uint32_t d0 = dst + (c16 >> 2) * 16384, ch = static_cast<uint32_t>((c16 & 3) * 2);
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + ((ch ^ sw) << 4)), "r"(u[c16].x << 16),
+                         "r"(u[c16].x & 0xffff0000u), "r"(u[c16].y << 16), "r"(u[c16].y & 0xffff0000u) : "memory");
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(d0 + (((ch + 1) ^ sw) << 4)), "r"(u[c16].z << 16),
+                         "r"(u[c16].z & 0xffff0000u), "r"(u[c16].w << 16), "r"(u[c16].w & 0xffff0000u) : "memory");
           }
         }
       }
@@ -603,27 +625,33 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
     // the epilogue warps did this under MMA-1 (2.6 k cycles against its 2.0 k) it delayed every chunk.
     if (a.post_on && write_o) {
       constexpr int kTpr = 4, kPieces = 8;   // threads per token, 16-byte fp32 pieces (8-byte gate pieces) per thread
+      // piece i of a row's thread: its columns start at 4 (part + 4 (i ^ row % 4)): the four rows of a half-warp touch different
+      // banks, in the fp32 tile (512 bytes a row) and in the bf16 one (256)
       const int t128 = tid - kWarpOut * 32, part = t128 % kTpr;
+      int col4[4];   // piece 4 j + r begins at column col4[r] + 64 j
+#pragma unroll
+      for (int r = 0; r < 4; ++r) col4[r] = 4 * (part + kTpr * (r ^ ((t128 / kTpr) & 3)));
       for (int c = 0; c < nch; ++c) {
         uint8_t* stp = smem + kOffStage + (c & 1) * kStageBytes;
         float* tile = reinterpret_cast<float*>(stp + kStOut);
-        // half 0 first waits for the tile; false (on all four warps: the barrier carries the vote) if that ran out
-        auto rows32 = [&](int half) -> bool {
-          const int prow = 32 * half + t128 / kTpr;
-          const bool g_live = c * C + prow < sq.len;
-          const uint2* gp = reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(a.post_g) +
-                                                           ((size_t)(sq.tok0 + c * C + prow) * H + h) * kD) + part;
-          uint2 graw[kPieces];
+        uint2 gate[2][kPieces];   // both halves' gates before the wait
 #pragma unroll
-          for (int i = 0; i < kPieces; ++i) graw[i] = g_live ? __ldg(gp + kTpr * i) : make_uint2(0u, 0u);
-          uint32_t good = 1;
-          if (half == 0) good = mbar_wait((c & 1) ? b_pn1 : b_pn0, (c >> 1) & 1, abortp) ? 1u : 0u;
-          __syncwarp();
+        for (int half = 0; half < 2; ++half) {
+          const int prow = 32 * half + t128 / kTpr;
+          const __nv_bfloat16* gp = static_cast<const __nv_bfloat16*>(a.post_g) + ((size_t)(sq.tok0 + c * C + prow) * H + h) * kD;
+#pragma unroll
+          for (int i = 0; i < kPieces; ++i) gate[half][i] = c * C + prow < sq.len ? __ldg(reinterpret_cast<const uint2*>(gp + col4[i & 3] + 64 * (i >> 2))) : make_uint2(0u, 0u);
+        }
+        uint32_t good = mbar_wait((c & 1) ? b_pn1 : b_pn0, (c >> 1) & 1, abortp) ? 1u : 0u;
+        __syncwarp();
+        // false (on all four warps: the barrier carries the vote) if that wait ran out
+        auto rows32 = [&](int half, const uint2 (&graw)[kPieces]) -> bool {
+          const int prow = 32 * half + t128 / kTpr;
           float4 ov[kPieces];
           float ss = 0.f;
 #pragma unroll
-          for (int i = 0; i < kPieces; ++i) {   // interleaved 16-byte pieces: a row's threads cover contiguous bytes
-            ov[i] = *reinterpret_cast<const float4*>(tile + prow * kD + (part + kTpr * i) * 4);
+          for (int i = 0; i < kPieces; ++i) {
+            ov[i] = *reinterpret_cast<const float4*>(tile + prow * kD + col4[i & 3] + 64 * (i >> 2));
             ss = fmaf(ov[i].x, ov[i].x, fmaf(ov[i].y, ov[i].y, fmaf(ov[i].z, ov[i].z, fmaf(ov[i].w, ov[i].w, ss))));
           }
           ss += __shfl_xor_sync(0xffffffffu, ss, 1);
@@ -642,7 +670,7 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
           }
 #pragma unroll
           for (int i = 0; i < kPieces; ++i) {
-            const int col = (part + kTpr * i) * 4;
+            const int col = col4[i & 3] + 64 * (i >> 2);
             const float4 wv = *reinterpret_cast<const float4*>(w_sm + col);
             const uint2 gr = graw[i];
             const float g0 = __uint_as_float(gr.x << 16), g1 = __uint_as_float(gr.x & 0xffff0000u);
@@ -659,9 +687,9 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
           }
           return true;
         };
-        ok = rows32(0);
+        ok = rows32(0, gate[0]);
         if (!ok) break;
-        rows32(1);
+        rows32(1, gate[1]);
         fence_proxy_async_smem();
         mbar_arrive((c & 1) ? b_go1 : b_go0);
       }
