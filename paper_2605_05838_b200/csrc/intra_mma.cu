@@ -301,13 +301,14 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) intra_mma_kernel(ChunkGe
   float dh = 0.f;
   if constexpr (kQk) {
     // fused q/k norm, while the products run: |k|^2, |q|^2 and q . k of every token from the tiles, two threads
-    // per token (one per half of dk);  |q - d k|^2 = |q|^2 - 2 d q.k + d^2 |k|^2
+    // per token (one per half of dk; lanes 0..15 and 16..31 of a warp, so that a phase of 8 lanes reads 8 rows of one half:
+    // all banks);  |q - d k|^2 = |q|^2 - 2 d q.k + d^2 |k|^2
     dh = qkn.d ? __ldg(qkn.d + h) : 0.f;
     ok = mbar_wait(bar_t, 0, &abort_flag);
     if (ok) {
-      const int row = tid >> 1, hb = tid & 1;
-      float nq2 = 0.f, qkd = 0.f, nk2 = 0.f;
-#pragma unroll
+      const int row = warp * 16 + (lane & 15), hb = lane >> 4;
+      float2 q2 = make_float2(0.f, 0.f), qk2 = q2, k2 = q2;   // even and odd columns
+#pragma unroll 2
       for (int j = 0; j < 8; ++j) {
         const uint32_t off = q_tile_chunk(L.k1, row, hb * 8 + j);
         const uint4 uq = *reinterpret_cast<const uint4*>(smem + off);
@@ -315,16 +316,17 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) intra_mma_kernel(ChunkGe
         const uint32_t q4[4] = {uq.x, uq.y, uq.z, uq.w}, k4[4] = {uk.x, uk.y, uk.z, uk.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const float ql = __uint_as_float(q4[e] << 16), qh = __uint_as_float(q4[e] & 0xffff0000u);
-          const float kl = __uint_as_float(k4[e] << 16), kh = __uint_as_float(k4[e] & 0xffff0000u);
-          nq2 = fmaf(ql, ql, fmaf(qh, qh, nq2));
-          qkd = fmaf(ql, kl, fmaf(qh, kh, qkd));
-          nk2 = fmaf(kl, kl, fmaf(kh, kh, nk2));
+          const float2 qf = make_float2(__uint_as_float(q4[e] << 16), __uint_as_float(q4[e] & 0xffff0000u));
+          const float2 kf = make_float2(__uint_as_float(k4[e] << 16), __uint_as_float(k4[e] & 0xffff0000u));
+          q2 = __ffma2_rn(qf, qf, q2);
+          qk2 = __ffma2_rn(qf, kf, qk2);
+          k2 = __ffma2_rn(kf, kf, k2);
         }
       }
-      nq2 += __shfl_xor_sync(0xffffffffu, nq2, 1);
-      qkd += __shfl_xor_sync(0xffffffffu, qkd, 1);
-      nk2 += __shfl_xor_sync(0xffffffffu, nk2, 1);
+      float nq2 = q2.x + q2.y, qkd = qk2.x + qk2.y, nk2 = k2.x + k2.y;
+      nq2 += __shfl_xor_sync(0xffffffffu, nq2, 16);
+      qkd += __shfl_xor_sync(0xffffffffu, qkd, 16);
+      nk2 += __shfl_xor_sync(0xffffffffu, nk2, 16);
       if (hb == 0) {
         cv[6 * C + row] = 1.f / sqrtf(nk2 + qkn.eps);
         cv[7 * C + row] = 1.f / sqrtf(fmaxf(nq2 - 2.f * dh * qkd + dh * dh * nk2, 0.f) + qkn.eps);
@@ -377,8 +379,12 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) intra_mma_kernel(ChunkGe
             float4 av;
             if constexpr (kQk) {
               const float4 rki = *reinterpret_cast<const float4*>(cv + 6 * C + i);
-              av = make_float4(rn_r * f[i] * rki.x * x[j4], rn_r * f[i + 1] * rki.y * x[j4 + 1], rn_r * f[i + 2] * rki.z * x[j4 + 2],
-                               rn_r * f[i + 3] * rki.w * x[j4 + 3]);
+              const float2 rn2 = make_float2(rn_r, rn_r);
+              const float2 p0 = __fmul2_rn(__fmul2_rn(__fmul2_rn(rn2, make_float2(f[i], f[i + 1])), make_float2(rki.x, rki.y)),
+                                           make_float2(x[j4], x[j4 + 1]));
+              const float2 p1 = __fmul2_rn(__fmul2_rn(__fmul2_rn(rn2, make_float2(f[i + 2], f[i + 3])), make_float2(rki.z, rki.w)),
+                                           make_float2(x[j4 + 2], x[j4 + 3]));
+              av = make_float4(p0.x, p0.y, p1.x, p1.y);
             } else {
               const float2 p0 = __fmul2_rn(make_float2(f[i], f[i + 1]), make_float2(x[j4], x[j4 + 1]));
               const float2 p1 = __fmul2_rn(make_float2(f[i + 2], f[i + 3]), make_float2(x[j4 + 2], x[j4 + 3]));
@@ -404,32 +410,26 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) intra_mma_kernel(ChunkGe
       if (cb < reach) {
         float x[16];
         if constexpr (kQk) {   // (q_r - d k_r) . k_i / |k_i|; this row of K K^T waits in the row's staging slot
-          float y[16];
           load16(trow + cb * 16, x, ok);
-#pragma unroll
-          for (int p4 = 0; p4 < 4; ++p4) {
-            const float4 y4 = *reinterpret_cast<const float4*>(w_f32 + (((cb * 4 + p4) ^ (r & 7)) * 16));
-            y[p4 * 4] = y4.x; y[p4 * 4 + 1] = y4.y; y[p4 * 4 + 2] = y4.z; y[p4 * 4 + 3] = y4.w;
-          }
+          const float2 ndh = make_float2(-dh, -dh);
 #pragma unroll
           for (int j4 = 0; j4 < 16; j4 += 4) {
+            const float4 y = *reinterpret_cast<const float4*>(w_f32 + (((cb * 4 + j4 / 4) ^ (r & 7)) * 16));
             const float4 rki = *reinterpret_cast<const float4*>(cv + 6 * C + cb * 16 + j4);
-            x[j4] = (x[j4] - dh * y[j4]) * rki.x; x[j4 + 1] = (x[j4 + 1] - dh * y[j4 + 1]) * rki.y;
-            x[j4 + 2] = (x[j4 + 2] - dh * y[j4 + 2]) * rki.z; x[j4 + 3] = (x[j4 + 3] - dh * y[j4 + 3]) * rki.w;
+            const float2 p0 = __fmul2_rn(__ffma2_rn(ndh, make_float2(y.x, y.y), make_float2(x[j4], x[j4 + 1])), make_float2(rki.x, rki.y));
+            const float2 p1 = __fmul2_rn(__ffma2_rn(ndh, make_float2(y.z, y.w), make_float2(x[j4 + 2], x[j4 + 3])), make_float2(rki.z, rki.w));
+            x[j4] = p0.x; x[j4 + 1] = p0.y; x[j4 + 2] = p1.x; x[j4 + 3] = p1.y;
           }
         } else {
           load16(trow + cb * 16, x, ok);
         }
         float w[16];
-        if constexpr (kQk) {
 #pragma unroll
-          for (int j = 0; j < 16; ++j) w[j] = rn_r * f[cb * 16 + j] * x[j];
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; j += 2) {
-            const float2 p = __fmul2_rn(make_float2(f[cb * 16 + j], f[cb * 16 + j + 1]), make_float2(x[j], x[j + 1]));
-            w[j] = p.x; w[j + 1] = p.y;
-          }
+        for (int j = 0; j < 16; j += 2) {
+          float2 fj = make_float2(f[cb * 16 + j], f[cb * 16 + j + 1]);
+          if constexpr (kQk) fj = __fmul2_rn(make_float2(rn_r, rn_r), fj);
+          const float2 p = __fmul2_rn(fj, make_float2(x[j], x[j + 1]));
+          w[j] = p.x; w[j + 1] = p.y;
         }
         if constexpr (kWf32) {
 #pragma unroll
