@@ -666,9 +666,9 @@ def run_backward(args, w):
         "data": "synthetic", "config": {"workload": workload_desc(w), "form": (
             "chunk-parallel: state-only forward keeping the chunk states, adjoint state chain, per-chunk kernel "
             "(bf16 tensor-core products, fp32 accumulation)" if method == "chunked" else
-            "token-level adjoint recurrence, per-chunk checkpoints and recomputation (fp32)")},
+            "exact fp32: chunk-start states, adjoint chain, per-chunk kernel")},
         "gpu_launches": launches * args.steps, "workspace_bytes": need, "training_step": train,
-        "roofline": {"bound": "hbm", "kernel": "whole backward" if method == "chunked" else "bwd_stepwise", "achieved": abytes / (ms * 1e-3) / 1e9,
+        "roofline": {"bound": "hbm", "kernel": "whole backward" if method == "chunked" else "whole exact backward", "achieved": abytes / (ms * 1e-3) / 1e9,
                      "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": abytes / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
                      "traffic": None, "peak_source": peaks["source"], "algorithmic_bytes": abytes}}))
 

@@ -75,7 +75,7 @@ typedef struct {
   int32_t path;            /* mdn_path                                                       */
   float scale;             /* multiplies q; dk^-0.5 is the appendix listing's default,       */
                            /* 1.0 gives the bare o_t = S_t^T q_t                             */
-  int32_t segments;        /* tensor path, fixed-length input: split every sequence into this */
+  int32_t segments;        /* tensor path: split every sequence into this                     */
                            /* many segments whose chunk chains run in PARALLEL (see below);   */
                            /* 0 = choose automatically, 1 = off, 3..32 = forced               */
 } mdn_params;
@@ -91,7 +91,7 @@ typedef struct {
  *   2. a short serial combine over segments (fp32) giving every segment's true start state;
  *   3. in parallel: segments 1.. as usual from those start states (outputs and final state).
  * The result is the same recurrence; only rounding differs.  Chosen automatically when the call has
- * too few chains to fill the GPU and the sequences are long (e.g. B=1, H=16, T=65536).
+ * too few chains to fill the GPU and the sequences are long (e.g. B=1, H=16, T=65536; packed input: on average).
  */
 
 /* Bytes of device workspace mdn_chunk_fwd needs for these parameters (0 on invalid

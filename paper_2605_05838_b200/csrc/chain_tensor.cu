@@ -1089,7 +1089,7 @@ cudaError_t launch_chain_tensor(const Plan& pl, const void* q, const void* k, co
 
 size_t seg_scratch_bytes(const mdn_params& p, int segments) {
   if (segments <= 1) return 0;
-  const size_t chains = (size_t)p.B * p.H, mat = (size_t)p.dk * p.dv * sizeof(float);
+  const size_t chains = (size_t)(p.num_seqs > 0 ? p.num_seqs : p.B) * p.H, mat = (size_t)p.dk * p.dv * sizeof(float);
   return chains * ((size_t)(segments - 1) * 2 + (size_t)(segments - 2) * 6) * mat;
 }
 
@@ -1102,11 +1102,15 @@ size_t seg_scratch_bytes(const mdn_params& p, int segments) {
 // A chunk of the first segment costs one run where one of a middle segment costs four, so the first segment is made as
 // long as phase 1 lasts anyway (equal segments: 1.35 ms of chain time for 16 chains of 1024 chunks; this split: 1.15 ms).
 // Used only where the model predicts at most 0.7 of the serial chain's time; otherwise 1 segment (off).
+// Packed input: the lengths are known on the device only.  The model takes the mean; every sequence is then split in the same
+// proportions by its own length, so that what the longest one takes falls by the factor the model saw, and the shorter ones
+// only leave SMs free earlier.
 SegSplit choose_segments(const mdn_params& p) {
   const SegSplit off{1, 0, 0};
-  if (!tensor_path_supported(p) || p.num_seqs > 0 || p.segments == 1) return off;
+  if (!tensor_path_supported(p) || p.segments == 1) return off;
   constexpr long kSMs = 148;
-  const long nch = (p.T + C - 1) / C, chains = (long)p.B * p.H;
+  const long seqs = p.num_seqs > 0 ? p.num_seqs : p.B, tokens = p.num_seqs > 0 ? p.T / seqs : p.T;
+  const long nch = (tokens + C - 1) / C, chains = seqs * p.H;
   if (p.segments >= 3) {   // forced: equal segments
     const int per = (int)((nch + p.segments - 1) / p.segments);
     return SegSplit{p.segments, per, per};

@@ -127,7 +127,8 @@ struct Args {
   // parallel inter-chunk scan (seg_G = 0: off, one CTA walks all chunks of its chain)
   int seg_G;
   int seg_phase;
-  int seg_first, seg_mid;   // chunks of segment 0, of every other one
+  int seg_first, seg_mid;   // chunks of segment 0, of every other one; packed input: in these proportions for every sequence
+  int seg_least;            // packed input: a sequence whose middle segments would be shorter stays whole (in segment 0)
   float* seg_E;
   float* seg_Psi;
   float* seg_PhiS;
@@ -200,8 +201,14 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
   if (!early) grid_dependency_wait();
   SeqInfo sq = seq_info(a.g, seq);
   if (a.seg_G > 0) {        // restrict the view to this segment's chunks
-    const int cb = seg == 0 ? 0 : min(sq.nchunks, a.seg_first + (seg - 1) * a.seg_mid);
-    const int ce = min(sq.nchunks, a.seg_first + seg * a.seg_mid);   // (G segments reach the end: choose_segments)
+    int first = a.seg_first, mid = a.seg_mid;
+    if (a.g.cu != nullptr) {
+      mid = (int)((long long)sq.nchunks * mid / (first + (a.seg_G - 1) * mid));
+      if (mid < a.seg_least) mid = 0;
+      first = sq.nchunks - (a.seg_G - 1) * mid;
+    }
+    const int cb = seg == 0 ? 0 : min(sq.nchunks, first + (seg - 1) * mid);
+    const int ce = min(sq.nchunks, first + seg * mid);   // (G segments reach the end: choose_segments)
     sq.slot0 += cb;
     sq.tok0 += cb * C;
     sq.len = (ce > cb) ? min(sq.len - cb * C, (ce - cb) * C) : 0;
@@ -989,7 +996,7 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
   a.S0 = S0; a.M0 = M0; a.o = o; a.Sf = Sf; a.Mf = Mf;
   a.status = reinterpret_cast<int32_t*>(pl.ws + pl.lay.off_status);
   a.scale = p.scale;
-  a.seg_G = 0; a.seg_phase = 0; a.seg_first = a.seg_mid = 0;
+  a.seg_G = 0; a.seg_phase = 0; a.seg_first = a.seg_mid = a.seg_least = 0;
   a.seg_E = a.seg_Psi = a.seg_PhiS = a.seg_PhiM = nullptr;
   a.qk_on = pl.qk.on; a.qk_d = pl.qk.d;
   a.post_on = pl.post.on; a.post_w = pl.post.w; a.post_g = pl.post.g; a.post_eps = pl.post.eps;
@@ -1018,7 +1025,7 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
   float* seg = reinterpret_cast<float*>(pl.ws + pl.lay.off_seg);
   const SegSplit split = choose_segments(p);
   a.seg_G = G;
-  a.seg_first = split.first; a.seg_mid = split.mid;
+  a.seg_first = split.first; a.seg_mid = split.mid; a.seg_least = p.segments ? 1 : kSegLeast;
   a.seg_E = seg;
   a.seg_Psi = a.seg_E + (size_t)chains * (G - 1) * 2 * kMat;
   a.seg_PhiS = a.seg_Psi + (size_t)chains * (G - 2) * 2 * kMat;

@@ -57,7 +57,7 @@ static mdn_status make_layout(const mdn_params& p, mdn_ws_layout* lay) {
   lay->off_coef = off; off = align_up(off + (uint64_t)slots * p.H * MDN_NUM_COEF * C * sizeof(float), 256);
   lay->off_T = off; off = align_up(off + mats * (tensor ? 2 : 4), 256);
   lay->off_W = off; off = align_up(off + mats * 4, 256);   // fp32, or bf16 hi + bf16 lo
-  lay->segments = (tensor && !packed) ? choose_segments(p).G : 1;
+  lay->segments = tensor ? choose_segments(p).G : 1;
   lay->off_seg = off; off = align_up(off + (lay->segments > 1 ? seg_scratch_bytes(p, lay->segments) : 0), 256);
   lay->total_bytes = off;
   return MDN_OK;

@@ -64,6 +64,19 @@ def test_automatic_segments(mdn, B, H, T):
     assert np.array_equal(np.asarray(o)[:, :64], np.asarray(o1)[:, :64])
 
 
+@pytest.mark.parametrize("segments,H,lens", [(0, 1, [64 * 200 + 5, 64 * 33, 100, 64 * 140 + 63, 1]), (3, 2, [64 * 3, 64 * 2 + 1, 1, 64 * 9 + 7]),
+                                             (0, 2, [63, 64 * 150])])
+def test_segments_of_packed_sequences(mdn, segments, H, lens):
+    """Packed sequences are split in proportion to their lengths; those too short for it stay whole (empty segments behind)."""
+    import torch
+    w = wl.Workload("edge_pseg", B=1, T=sum(lens), H=H, dk=128, dv=128, dtype="bf16", varlen=True, init_state_std=0.3, seed=len(lens))
+    assert mdn.workspace_layout(mdn.MdnParams(1, w.T, H, 128, 128, 64, len(lens), 1, 0, 0, 1.0, segments)).segments > 1
+    inp = wl.make_inputs(w, lengths=np.array(lens))
+    o_ref, S_ref, M_ref = run_oracle(inp)
+    o, S, M = run_gpu(mdn, inp, path="tensor", o_dtype=torch.float32, segments=segments)
+    assert max(rel_err(o, o_ref), rel_err(S, S_ref), rel_err(M, M_ref)) <= 2e-2
+
+
 @pytest.mark.parametrize("packed,state,eta", [(False, True, True), (True, True, False), (False, False, False)])
 def test_both_autograd_nodes_give_the_same_bits(mdn, packed, state, eta):
     """The C++ node and the Python one run the same kernels (gate gradients: sums by atomics, last bits may differ)."""
