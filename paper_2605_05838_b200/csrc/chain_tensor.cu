@@ -1108,7 +1108,7 @@ size_t seg_scratch_bytes(const mdn_params& p, int segments) {
 SegSplit choose_segments(const mdn_params& p) {
   const SegSplit off{1, 0, 0};
   if (!tensor_path_supported(p) || p.segments == 1) return off;
-  constexpr long kSMs = 148;
+  constexpr long kSMs = kSegSms;
   const long seqs = p.num_seqs > 0 ? p.num_seqs : p.B, tokens = p.num_seqs > 0 ? p.T / seqs : p.T;
   const long nch = (tokens + C - 1) / C, chains = seqs * p.H;
   if (p.segments >= 3) {   // forced: equal segments
@@ -1118,7 +1118,8 @@ SegSplit choose_segments(const mdn_params& p) {
   auto waves = [](long ctas, long sms) { return (ctas + sms - 1) / sms; };
   const double serial = (double)(waves(chains, kSMs) * nch);
   if (chains >= kSMs || nch < 3 * 8) return off;   // no SM left for the middle segments; too short
-  constexpr double kState = 0.9, kRun = 1.7, kStep = 3.2, kFix = 3.;   // state-only chunk; a run's start and end; combine step; launches
+  constexpr double kState = 0.9, kRun = 1.7, kFix = 3.;   // state-only chunk; a run's start and end; launches
+  const double step = chains * 16 <= kSMs ? 2.0 : 3.2 * waves(chains * 8, kSMs);   // combine step, by its tile (seg_combine.cu)
   double best = 0.7 * serial;
   SegSplit r = off;
   for (long m = 1; m <= 30 && (m + 1) * 8 < nch; ++m) {
@@ -1127,7 +1128,7 @@ SegSplit choose_segments(const mdn_params& p) {
     for (long L = at > 8 ? at : 8; L <= at + 1 && (m + 1) * L < nch; ++L) {
       const long first = nch - (m + 1) * L;
       const double p1 = w1 * (kState * L + kRun), p0 = first + kRun;
-      const double cost = (p1 > p0 ? p1 : p0) + w3 * (L + kRun) + kStep * m * waves(chains * 8, kSMs) + kFix;
+      const double cost = (p1 > p0 ? p1 : p0) + w3 * (L + kRun) + step * m + kFix;
       if (cost < best) { best = cost; r = SegSplit{(int)m + 2, (int)first, (int)L}; }
     }
   }

@@ -233,6 +233,7 @@ size_t seg_scratch_bytes(const mdn_params& p, int segments);
 // The parallel inter-chunk scan's split of a sequence of nch chunks: G segments, the first `first` chunks long, the others
 // `mid` (the last one what is left).
 struct SegSplit { int G, first, mid; };
+constexpr int kSegSms = 148;   // SMs the split is made for
 constexpr int kSegLeast = 4;   // chunks: below that a run's start and end outweigh what running it in parallel saves
 SegSplit choose_segments(const mdn_params& p);
 cudaError_t launch_seg_combine(const Plan& pl, int G, float* E, const float* Psi, const float* PhiS,
