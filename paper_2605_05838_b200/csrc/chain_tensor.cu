@@ -1101,10 +1101,11 @@ size_t seg_scratch_bytes(const mdn_params& p, int segments) {
 //   phase 3  m + 1 real runs per chain.
 // A chunk of the first segment costs one run where one of a middle segment costs four, so the first segment is made as
 // long as phase 1 lasts anyway (equal segments: 1.35 ms of chain time for 16 chains of 1024 chunks; this split: 1.15 ms).
-// Used only where the model predicts at most 0.7 of the serial chain's time; otherwise 1 segment (off).
+// Used only where the model predicts at most 0.9 of the serial chain's time; otherwise 1 segment (off).  (Calls where it predicts
+// 0.73 .. 0.87 measured 0.77 .. 0.94, e.g. 2 x 8192 tokens x 16 heads 498 -> 395 us, 1 x 2048 x 2 118 -> 92.)
 // Packed input: the lengths are known on the device only.  The model takes the mean; every sequence is then split in the same
 // proportions by its own length, so that what the longest one takes falls by the factor the model saw, and the shorter ones
-// only leave SMs free earlier.
+// only leave SMs free earlier.  The mean says less than a length: 0.7 there.
 SegSplit choose_segments(const mdn_params& p) {
   const SegSplit off{1, 0, 0};
   if (!tensor_path_supported(p) || p.segments == 1) return off;
@@ -1120,7 +1121,7 @@ SegSplit choose_segments(const mdn_params& p) {
   if (chains >= kSMs || nch < 3 * 8) return off;   // no SM left for the middle segments; too short
   constexpr double kState = 0.9, kRun = 1.7, kFix = 3.;   // state-only chunk; a run's start and end; launches
   const double step = chains * 16 <= kSMs ? 2.0 : 3.2 * waves(chains * 8, kSMs);   // combine step, by its tile (seg_combine.cu)
-  double best = 0.7 * serial;
+  double best = (p.num_seqs > 0 ? 0.7 : 0.9) * serial;
   SegSplit r = off;
   for (long m = 1; m <= 30 && (m + 1) * 8 < nch; ++m) {
     const long w1 = waves(3 * m * chains, kSMs - chains), w3 = waves((m + 1) * chains, kSMs);

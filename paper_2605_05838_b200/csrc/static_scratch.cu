@@ -57,8 +57,8 @@ extern "C" mdn_status mdn_chunk_fwd_static_scratch(const mdn_params* p, const vo
   if (ps != MDN_OK) return ps;
   if (p->num_seqs > 0 ? cu_seqlens == nullptr : cu_seqlens != nullptr) return MDN_ERR_INVALID_ARG;
   mdn_params ps_serial = *p;
-  if (p->num_seqs > 0 && p->segments == 0 && lay.total_bytes > (uint64_t)MDN_STATIC_SCRATCH_BYTES) {
-    ps_serial.segments = 1;   // packed input: without the segment scan's scratch
+  if (p->segments == 0 && lay.total_bytes > (uint64_t)MDN_STATIC_SCRATCH_BYTES) {
+    ps_serial.segments = 1;   // without the segment scan's scratch
     if (mdn_workspace_layout(&ps_serial, &lay) != MDN_OK) return MDN_ERR_STATIC_SCRATCH;
     p = &ps_serial;
   }
