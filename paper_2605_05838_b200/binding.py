@@ -194,6 +194,13 @@ def _stream() -> ctypes.c_void_p:
     return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
 
 
+def _empty_1024(nbytes: int, device) -> torch.Tensor:
+    """A buffer that starts on a 1024-byte boundary (the allocator's blocks start on 512-byte ones)."""
+    t = torch.empty(nbytes + 1024, dtype=torch.uint8, device=device)
+    off = -t.data_ptr() % 1024
+    return t[off:off + nbytes]
+
+
 def make_params(q: torch.Tensor, v: torch.Tensor, *, num_seqs: int = 0, scale: Optional[float] = None,
                 o_dtype: Optional[torch.dtype] = None, path: str = "auto", segments: int = 0) -> MdnParams:
     B, T, H, dk = q.shape
@@ -338,7 +345,7 @@ def chunk_fwd(q, k, v, beta, log_alpha, log_mu, eta=None, *, initial_S=None, ini
         nbytes = int(lib().mdn_chunk_states_bytes(ctypes.byref(p)))
         if nbytes == 0:
             raise MdnError(2, "mdn_chunk_states_bytes")
-        states = torch.empty(nbytes, dtype=torch.uint8, device=q.device)
+        states = _empty_1024(nbytes, q.device)
         st = lib().mdn_chunk_fwd_keep_states(ctypes.byref(p), *tail[:13], _ptr(states), *tail[13:])
         if st != 0:
             raise MdnError(st, "mdn_chunk_fwd_keep_states")
@@ -403,8 +410,8 @@ def bwd_state_chain(q, k, d_o, fwd_workspace, *, v_dim: int, d_final_S=None, d_f
     need = int(lib().mdn_bwd_state_chain_workspace_bytes(ctypes.byref(p)))
     if nbytes == 0 or need == 0:
         raise MdnError(2, "mdn_bwd_state_chain_workspace_bytes")
-    adj = torch.empty(nbytes, dtype=torch.uint8, device=q.device)
-    ws = torch.empty(need, dtype=torch.uint8, device=q.device)
+    adj = _empty_1024(nbytes, q.device)
+    ws = _empty_1024(need, q.device)
     dS0 = torch.empty((nst, H, dk, v_dim), dtype=torch.float32, device=q.device) if want_initial else None
     dM0 = torch.empty((nst, H, dk, v_dim), dtype=torch.float32, device=q.device) if want_initial else None
     st = lib().mdn_bwd_state_chain(ctypes.byref(p), _ptr(q), _ptr(k), _ptr(d_o), _ptr(d_final_S), _ptr(d_final_M),
@@ -463,7 +470,7 @@ def chunk_bwd(q, k, v, beta, log_alpha, log_mu, eta, d_o, *, initial_S=None, ini
     if need == 0:
         raise MdnError(2, "mdn_chunk_bwd_workspace_bytes")
     if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=q.device)
+        workspace = _empty_1024(need, q.device)
     f32 = dict(dtype=torch.float32, device=q.device)
     g = dict(dq=torch.empty((B, T, H, dk), **f32), dk=torch.empty((B, T, H, dk), **f32),
              dv=torch.empty((B, T, H, dv), **f32), dbeta=torch.empty((B, T, H), **f32),

@@ -127,6 +127,15 @@ Tensor empty(at::IntArrayRef shape, at::ScalarType dt, c10::DeviceIndex dev) {
   return at::detail::empty_cuda(shape, dt, c10::Device(c10::kCUDA, dev), std::nullopt);
 }
 
+// A buffer that starts on a 1024-byte boundary (chunk states and the backward's workspaces): the allocator's blocks start on
+// 512-byte ones, most of them on coarser.
+Tensor empty_1024(int64_t bytes, c10::DeviceIndex dev) {
+  Tensor t = empty({bytes}, at::kByte, dev);
+  if (reinterpret_cast<uintptr_t>(t.data_ptr()) % 1024 == 0) return t;
+  t = empty({bytes + 1024}, at::kByte, dev);
+  return t.narrow(0, (int64_t)((1024 - reinterpret_cast<uintptr_t>(t.data_ptr()) % 1024) % 1024), bytes);
+}
+
 void* stream_of(c10::DeviceIndex dev) { return c10::cuda::getCurrentCUDAStream(dev).stream(); }
 
 mdn_params params_of(const Inputs& in, int64_t num_seqs, int32_t o_code, int32_t path, float scale, int32_t segments) {
@@ -229,7 +238,7 @@ PyObject* chunk_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const void *q = in.q->const_data_ptr(), *k = in.k->const_data_ptr(), *v = in.v->const_data_ptr();
     void* stream = stream_of(in.dev);
     if (keep) {
-      states = empty({(int64_t)state_bytes}, at::kByte, in.dev);
+      states = empty_1024((int64_t)state_bytes, in.dev);
       st = mdn_chunk_fwd_keep_states(&p, q, k, v, in.beta, in.log_alpha, in.log_mu, in.eta, S0, M0, cu, o.data_ptr(), sf, mf,
                                      states.data_ptr(), ws.data_ptr(), (size_t)ws.numel(), stream);
     } else {
@@ -287,7 +296,7 @@ PyObject* chunk_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   mdn_status st;
   {
     NoGil gil;
-    if (!ws.defined()) ws = empty({(int64_t)need}, at::kByte, in.dev);
+    if (!ws.defined()) ws = empty_1024((int64_t)need, in.dev);
     const at::ScalarType gdt = method == 3 ? in.dtype : at::kFloat;
     g[0] = empty({in.B, in.T, in.H, in.dk}, gdt, in.dev);
     g[1] = empty({in.B, in.T, in.H, in.dk}, gdt, in.dev);
@@ -331,7 +340,7 @@ class ChunkAttention : public torch::autograd::Function<ChunkAttention> {
   static mdn_params params(const Tensor& q, const Tensor& v, const Tensor& cu, double scale) {
     const int64_t N = cu.defined() ? cu.numel() - 1 : 0;
     return mdn_params{(int32_t)q.size(0), (int32_t)q.size(1), (int32_t)q.size(2), (int32_t)q.size(3), (int32_t)v.size(3), 64, (int32_t)N,
-                      MDN_BF16, MDN_BF16, MDN_PATH_TENSOR, (float)scale, 1 /* the kept forward walks its chunks in order */};
+                      MDN_BF16, MDN_BF16, MDN_PATH_TENSOR, (float)scale, 0};
   }
   static void check(mdn_status st, const char* where) {
     TORCH_CHECK(st == MDN_OK, where, ": ", mdn_status_string(st), " (status ", (int)st, ")",
@@ -350,7 +359,7 @@ class ChunkAttention : public torch::autograd::Function<ChunkAttention> {
     const int64_t n = p.num_seqs > 0 ? p.num_seqs : p.B;
     const size_t need = mdn_chunk_fwd_workspace_bytes(&p), state_bytes = mdn_chunk_states_bytes(&p);
     TORCH_CHECK(need != 0 && state_bytes != 0, "mdn_chunk_states_bytes: ", mdn_status_string(MDN_ERR_UNSUPPORTED), " (status 2)");
-    Tensor ws = empty({(int64_t)need}, at::kByte, dev), states = empty({(int64_t)state_bytes}, at::kByte, dev);
+    Tensor ws = empty({(int64_t)need}, at::kByte, dev), states = empty_1024((int64_t)state_bytes, dev);
     Tensor o = empty(v.sizes(), q.scalar_type(), dev);
     Tensor Sf = empty({n, p.H, p.dk, p.dv}, at::kFloat, dev), Mf = empty({n, p.H, p.dk, p.dv}, at::kFloat, dev);
     check(mdn_chunk_fwd_keep_states(&p, q.const_data_ptr(), k.const_data_ptr(), v.const_data_ptr(), AttnPtrs::f(beta),
@@ -375,7 +384,7 @@ class ChunkAttention : public torch::autograd::Function<ChunkAttention> {
     const Tensor dSf = grads[1].defined() ? grads[1].to(at::kFloat).contiguous() : Tensor();
     const Tensor dMf = grads[2].defined() ? grads[2].to(at::kFloat).contiguous() : Tensor();
     const size_t need = mdn_chunk_bwd_saved_workspace_bytes(&p);
-    Tensor work = empty({(int64_t)need}, at::kByte, dev);
+    Tensor work = empty_1024((int64_t)need, dev);
     Tensor dq = empty(q.sizes(), q.scalar_type(), dev), dk = empty(q.sizes(), q.scalar_type(), dev), dv = empty(v.sizes(), q.scalar_type(), dev);
     Tensor g[4], dS0, dM0;   // d beta, d log_alpha, d log_mu, d eta
     float* gp[4] = {nullptr, nullptr, nullptr, nullptr};
