@@ -277,8 +277,8 @@ mdn_status mdn_chunk_fwd_fused(const mdn_params* p, const mdn_layer_ops* ops /* 
  * forward's own tensor-core products read (the fp32 masters stay on chip).  Behind the images of all slots lies a
  * second part: V~ = T (V - abar.(K S) + p.(K M)) of every chunk as float32 [chunk slot][64][H][dv] (rows past the end
  * of a short chunk are not written), which the chunk-parallel backward reads instead of rebuilding it.
- * Tensor path only (bf16 input, dk = dv = 128): MDN_ERR_UNSUPPORTED otherwise.  The serial chain is used
- * (p->segments is ignored).  Workspace as for mdn_chunk_fwd.
+ * Tensor path only (bf16 input, dk = dv = 128): MDN_ERR_UNSUPPORTED otherwise.  Workspace as for
+ * mdn_chunk_fwd (one too small for p->segments but enough for the serial chain: the serial chain is used).
  */
 size_t mdn_chunk_states_bytes(const mdn_params* p);
 

@@ -101,6 +101,7 @@ struct ChainArgs {
   uint32_t w_lo_row_offset;   // rows between the hi and lo parts in the W tensor map
   // parallel inter-chunk scan (seg_G = 0: off, one CTA walks all chunks of its chain)
   int seg_G;                  // segments per sequence
+  int seg_first, seg_mid, seg_least;   // see seg_chunks
   int seg_phase;              // 1: segment 0 + the Psi / Phi runs of the middle segments; 3: segments 1.. from E
   float* seg_E;               // [chains][G-1][2][dk*dv]  state at the END of segment g (start of g+1)
   float* seg_Psi;             // [chains][G-2][2][dk*dv]  segment run from a zero state
@@ -156,7 +157,8 @@ template <> __device__ __forceinline__ void stage_o<__nv_bfloat16>(uint8_t* tile
 
 // kTrain compiles in the chunk-state dump, the state-only switch and the decoupled end-of-chunk scalars (the plain
 // forward's instantiation stays as it is: its schedule is fragile, a runtime test of these options cost it 2 %)
-template <typename TO, bool kLayer, bool kTrain = false>
+// kSeg: the parallel inter-chunk scan's runs (a template flag: as run-time tests it cost the serial chain 2 - 6 %)
+template <typename TO, bool kLayer, bool kTrain, bool kSeg>
 __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chain_tensor_kernel(const ChainArgs a,
                                                                   const __grid_constant__ CUtensorMap map_q,
                                                                   const __grid_constant__ CUtensorMap map_k,
@@ -180,12 +182,14 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
   const int H = a.g.H;
   // ---- work item: which chain, which segment of it, which kind of run
   int chain = blockIdx.x, seg = 0, run = 0;   // run 0: the real thing; 1: Psi; 2: Phi from (I, 0); 3: Phi from (0, I)
-  if (a.seg_G > 0) {
-    if (a.seg_phase == 1) {
-      const int items = 1 + 3 * (a.seg_G - 2);
-      chain = blockIdx.x / items;
-      const int w = blockIdx.x % items;
-      if (w > 0) { seg = 1 + (w - 1) / 3; run = 1 + (w - 1) % 3; }
+  if (kSeg) {
+    if (a.seg_phase == 1) {   // the first segments (the longest runs) lead
+      const int chains = a.g.num_seqs * H, items = 3 * (a.seg_G - 2), w = (int)blockIdx.x - chains;
+      if (w >= 0) {
+        chain = w / items;
+        seg = 1 + (w % items) / 3;
+        run = 1 + (w % items) % 3;
+      }
     } else {
       chain = blockIdx.x / (a.seg_G - 1);
       seg = 1 + blockIdx.x % (a.seg_G - 1);
@@ -193,12 +197,14 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
   }
   const int seq = chain / H, h = chain % H;
   // what the previous kernel wrote (coefficients, T, W, V of the adjoint run) is read by the producer warp alone: see chain_tf32.cu
-  const bool early = a.seg_G == 0;
+  const bool early = !kSeg;
   if (!early) grid_dependency_wait();
   SeqInfo sq = seq_info(a.g, seq);
-  if (a.seg_G > 0) {        // restrict the view to this segment's chunks
-    const int per = (sq.nchunks + a.seg_G - 1) / a.seg_G;
-    const int cb = min(sq.nchunks, seg * per), ce = min(sq.nchunks, (seg + 1) * per);
+  int rev0 = sq.nchunks - 1;             // mirrored runs: this run's chunk c is the original problem's chunk rev0 - c
+  if (kSeg) {        // restrict the view to this segment's chunks
+    const int2 span = seg_chunks(a.g, sq.nchunks, SegSplitArgs{a.seg_G, a.seg_first, a.seg_mid, a.seg_least}, seg);
+    const int cb = span.x, ce = span.y;
+    rev0 -= cb;
     sq.slot0 += cb;
     sq.tok0 += cb * C;
     sq.len = (ce > cb) ? min(sq.len - cb * C, (ce - cb) * C) : 0;
@@ -212,7 +218,7 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
   float* Sfp = a.Sf ? a.Sf + st_off : nullptr;
   float* Mfp = a.Mf ? a.Mf + st_off : nullptr;
   bool id_s = false, id_m = false, v_zero = false, write_o = true;
-  if (a.seg_G > 0) {
+  if (kSeg) {
     constexpr size_t kMat = (size_t)kD * kD;
     auto e_ptr = [&](int gi, int which) { return a.seg_E + (((size_t)chain * (a.seg_G - 1) + gi) * 2 + which) * kMat; };
     if (run == 0) {
@@ -233,6 +239,8 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
   if constexpr (kTrain) {
     if (a.state_only) write_o = false;
   }
+  // the runs from basis states (V = 0) have no second update; only real runs leave anything behind
+  const bool inject = kTrain && a.inject && (!kSeg || run <= 1), dump = kTrain && a.dump != nullptr && (!kSeg || run == 0);
 
   const uint32_t s_base = smem_u32(smem);
   const uint32_t b_full0 = smem_u32(&bars.full[0]), b_full1 = smem_u32(&bars.full[1]);
@@ -331,12 +339,12 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
           const int tok0 = sq.tok0 + c * C;
           const int mat = (sq.slot0 + c) * H + h;
           // state-only runs need neither Q nor W, and the V = 0 runs no V either
-          const bool inj = kTrain && a.inject;   // Q and G (into the W area) instead of Q and W
+          const bool inj = inject;               // Q and G (into the W area) instead of Q and W
           int tok0k = tok0;                      // rows of k, q, G
           int mat_t = mat;                       // which T
           if (kTrain && a.mirror) {
-            tok0k = seq_info(a.mirror_g, seq).tok0 + (nch - 1 - c) * C;
-            mat_t = (sq.slot0 + nch - 1 - c) * H + h;
+            tok0k = seq_info(a.mirror_g, seq).tok0 + (rev0 - c) * C;
+            mat_t = (seq_info(a.g, seq).slot0 + rev0 - c) * H + h;
           }
           mbar_arrive_expect_tx(fb, kTxBytes - ((write_o || inj) ? 0u : kTxQW) - (v_zero ? kTxV : 0u));
           tma_load_2d(st + kStK, &map_k, h * kD, tok0k, fb);
@@ -357,7 +365,7 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
           MDN_MARK(c, kEvTmaIssued);
           issued = c + 1;
         }
-        if (kTrain && a.dump != nullptr && c >= 1 && c <= nch) {   // the state copies of chunk c - 1 (handed over long ago)
+        if (dump && c >= 1 && c <= nch) {   // the state copies of chunk c - 1 (handed over long ago)
           MDN_WAIT(b_sb, (c - 1) & 1);
           uint8_t* dst = a.dump + ((size_t)(sq.slot0 + c - 1) * H + h) * 65536;
           for (int b = 0; b < 4; ++b) bulk_store(dst + b * 16384, s_base + kOffSb + b * 16384, 16384);
@@ -463,7 +471,7 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
           if (write_o && qk_on) MDN_MMA_1B(true);
         }
         if constexpr (kTrain) {
-          if (a.inject) {
+          if (inject) {
             // the second update (operands in Z, U and the pre-scaled masters ready since the start of the chunk, Q
             // read MN-major) needs nothing of this chunk's V~: issued here it runs while EPI-2 works, before MMA-3
             const uint64_t dQmn = smem_desc_sw128(st + kStQ, 8192, 1024);
@@ -532,7 +540,7 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
         } else {
           al = cf[kAbar * C + C - 1]; bl = cf[kB * C + C - 1]; ml = cf[kMubar * C + C - 1];
         }
-        if (kTrain && a.dump != nullptr && c > 0) MDN_WAIT(b_dump, (c - 1) & 1);
+        if (dump && c > 0) MDN_WAIT(b_dump, (c - 1) & 1);
         MDN_MARK(c, kEvFullSeen);
       }
       __syncwarp();
@@ -736,7 +744,7 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
       const float* cf = reinterpret_cast<const float*>(stg + kStCoef);
       const __nv_bfloat16* sV = reinterpret_cast<const __nv_bfloat16*>(stg + kStV);
       if constexpr (kTrain) {
-        if (a.inject) {
+        if (inject) {
           // operands of the second update: they depend on nothing the chain computes, so they are made here, while
           // MMA-1a runs.  Z, U are free in a state-only run; the previous chunk's MMA-3 (waited for in P) was their
           // last reader.
@@ -933,7 +941,7 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
         MDN_MARK(c, kEvV2Arrive);
         if constexpr (kTrain) {   // off the chain's critical path: MMA-3 is running
           const int slot_c = sq.slot0 + c;
-          if (a.vt_dump != nullptr) {
+          if (a.vt_dump != nullptr && (!kSeg || run == 0)) {
             const int live = min(C, sq.len - c * C) - r0;   // this thread's tokens inside the chunk
             float* dst = a.vt_dump + (((size_t)slot_c * C + r0) * H + h) * kD + d;
             const size_t stride = (size_t)H * kD;
@@ -946,9 +954,9 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
                 if (j < live) *dst = __uint_as_float(vt[j]);
             }
           }
-          if (a.dr_bf16 != nullptr) {
+          if (a.dr_bf16 != nullptr && (!kSeg || run == 0)) {
             const SeqInfo os = seq_info(a.mirror_g, seq);
-            const int c0 = (nch - 1 - c) * C + r0;
+            const int c0 = (rev0 - c) * C + r0;
             const int live = min(kTok, os.len - c0);   // this thread's tokens inside the chunk
             const size_t at = ((size_t)(os.tok0 + c0) * H + h) * kD + d, stride = (size_t)H * kD;
             if (live >= kTok) {
@@ -1042,30 +1050,26 @@ cudaError_t launch_chain_tensor(const Plan& pl, const void* q, const void* k, co
   a.mirror = pl.chain_mirror_geom != nullptr;
   if (a.mirror) a.mirror_g = *pl.chain_mirror_geom; else a.mirror_g = pl.geom;
   a.seg_G = 0; a.seg_phase = 0;
+  a.seg_first = a.seg_mid = a.seg_least = 0;
   a.seg_E = a.seg_Psi = a.seg_PhiS = a.seg_PhiM = nullptr;
   const unsigned chains = (unsigned)pl.geom.num_seqs * p.H;
   const bool layer = a.qk_on || a.post_on;
   auto launch_as = [&](auto kern, unsigned grid) -> cudaError_t {
     cudaError_t e = allow_smem(kern, (int)kSmemBytes);
     if (e != cudaSuccess) return e;
-    const unsigned threads = layer ? Roles<token_groups(true)>::kThreads : Roles<token_groups(false)>::kThreads;
-    e = launch_pdl(kern, dim3(grid), dim3(threads), kSmemBytes, pl.stream, a, mq, mk, mv, mt, mw, mo);
+    e = launch_pdl(kern, dim3(grid), dim3(Roles<token_groups(false)>::kThreads), kSmemBytes, pl.stream, a, mq, mk, mv, mt, mw, mo);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) ++*launches;
     return e;
   };
   auto launch = [&](unsigned grid) -> cudaError_t {
+    // (every forward without the training options runs on chain_tf32.cu)
     const bool train = a.dump != nullptr || a.state_only || a.end_scalars_in_rk || a.vt_dump != nullptr || a.inject;
-    if ((a.inject && !a.state_only) || (a.mirror && !a.inject)) return cudaErrorInvalidValue;
-    if (train) {   // plain forward with the training options (no layer operations there)
-      if (layer) return cudaErrorInvalidValue;
-      return p.o_dtype == MDN_BF16 ? launch_as(chain_tensor_kernel<__nv_bfloat16, false, true>, grid)
-                                   : launch_as(chain_tensor_kernel<float, false, true>, grid);
-    }
-    if (p.o_dtype == MDN_BF16)
-      return layer ? launch_as(chain_tensor_kernel<__nv_bfloat16, true>, grid)
-                   : launch_as(chain_tensor_kernel<__nv_bfloat16, false>, grid);
-    return layer ? launch_as(chain_tensor_kernel<float, true>, grid) : launch_as(chain_tensor_kernel<float, false>, grid);
+    if (!train || layer || (a.inject && !a.state_only) || (a.mirror && !a.inject)) return cudaErrorInvalidValue;
+    typedef __nv_bfloat16 bf16;
+    if (a.seg_G > 0)
+      return o_bf16 ? launch_as(chain_tensor_kernel<bf16, false, true, true>, grid) : launch_as(chain_tensor_kernel<float, false, true, true>, grid);
+    return o_bf16 ? launch_as(chain_tensor_kernel<bf16, false, true, false>, grid) : launch_as(chain_tensor_kernel<float, false, true, false>, grid);
   };
   const int G = pl.lay.segments;
   if (G <= 1) return launch(chains);
@@ -1073,7 +1077,9 @@ cudaError_t launch_chain_tensor(const Plan& pl, const void* q, const void* k, co
   // ---- parallel inter-chunk scan: Psi / Phi of the middle segments, serial combine, then all segments for real
   constexpr size_t kMat = (size_t)kD * kD;
   float* seg = reinterpret_cast<float*>(pl.ws + pl.lay.off_seg);
+  const SegSplit split = choose_segments(p);
   a.seg_G = G;
+  a.seg_first = split.first; a.seg_mid = split.mid; a.seg_least = p.segments ? 1 : kSegLeast;
   a.seg_E = seg;
   a.seg_Psi = a.seg_E + (size_t)chains * (G - 1) * 2 * kMat;
   a.seg_PhiS = a.seg_Psi + (size_t)chains * (G - 2) * 2 * kMat;

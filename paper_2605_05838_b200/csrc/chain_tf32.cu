@@ -127,8 +127,7 @@ struct Args {
   // parallel inter-chunk scan (seg_G = 0: off, one CTA walks all chunks of its chain)
   int seg_G;
   int seg_phase;
-  int seg_first, seg_mid;   // chunks of segment 0, of every other one; packed input: in these proportions for every sequence
-  int seg_least;            // packed input: a sequence whose middle segments would be shorter stays whole (in segment 0)
+  int seg_first, seg_mid, seg_least;   // see seg_chunks
   float* seg_E;
   float* seg_Psi;
   float* seg_PhiS;
@@ -201,14 +200,8 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
   if (!early) grid_dependency_wait();
   SeqInfo sq = seq_info(a.g, seq);
   if (a.seg_G > 0) {        // restrict the view to this segment's chunks
-    int first = a.seg_first, mid = a.seg_mid;
-    if (a.g.cu != nullptr) {
-      mid = (int)((long long)sq.nchunks * mid / (first + (a.seg_G - 1) * mid));
-      if (mid < a.seg_least) mid = 0;
-      first = sq.nchunks - (a.seg_G - 1) * mid;
-    }
-    const int cb = seg == 0 ? 0 : min(sq.nchunks, first + (seg - 1) * mid);
-    const int ce = min(sq.nchunks, first + seg * mid);   // (G segments reach the end: choose_segments)
+    const int2 span = seg_chunks(a.g, sq.nchunks, SegSplitArgs{a.seg_G, a.seg_first, a.seg_mid, a.seg_least}, seg);
+    const int cb = span.x, ce = span.y;
     sq.slot0 += cb;
     sq.tok0 += cb * C;
     sq.len = (ce > cb) ? min(sq.len - cb * C, (ce - cb) * C) : 0;

@@ -225,10 +225,13 @@ mdn_status mdn_chunk_fwd_keep_states(const mdn_params* p, const void* q, const v
   if (check_params(p) != MDN_OK) return check_params(p);
   if (resolve_path(*p) != MDN_PATH_TENSOR) return MDN_ERR_UNSUPPORTED;
   if (!chunk_states || !aligned(chunk_states, 1024)) return MDN_ERR_INVALID_ARG;
-  mdn_params ps = *p;
-  ps.segments = 1;
   Plan pl;
-  mdn_status st = make_plan(&ps, cu_seqlens, workspace, workspace_bytes, cuda_stream, &pl);
+  mdn_status st = make_plan(p, cu_seqlens, workspace, workspace_bytes, cuda_stream, &pl);
+  if (st == MDN_ERR_WORKSPACE) {   // without the segment scan's scratch
+    mdn_params ps = *p;
+    ps.segments = 1;
+    st = make_plan(&ps, cu_seqlens, workspace, workspace_bytes, cuda_stream, &pl);
+  }
   if (st != MDN_OK) return st;
   pl.chain_dump = static_cast<uint8_t*>(chunk_states);
   pl.chain_vt_dump = reinterpret_cast<float*>(pl.chain_dump + (uint64_t)pl.lay.num_slots * p->H * kStateImageBytes);
@@ -246,8 +249,7 @@ static mdn_status adj_layout(const mdn_params* p, AdjLayout* a) {
   mdn_status st = check_params(p);
   if (st != MDN_OK) return st;
   if (resolve_path(*p) != MDN_PATH_TENSOR) return MDN_ERR_UNSUPPORTED;
-  a->pe = *p;
-  a->pe.segments = 1;
+  a->pe = *p;   // (its segments too: the mirrored problem is split by the same rule)
   a->pe.path = MDN_PATH_TENSOR;
   if (p->num_seqs > 0) {   // packed: every chunk slot of the forward, padded to 64 rows (host-side bound)
     mdn_params pf = *p;
@@ -338,7 +340,7 @@ mdn_status mdn_bwd_state_chain(const mdn_params* p, const void* q, const void* k
 }
 
 // ---- the chunk-parallel backward: state-only forward keeping the chunk states, adjoint chain, per-chunk stage
-struct ChunkedBwdLayout { AdjLayout al; mdn_ws_layout lf; uint64_t ws_fwd, fwd_states, adj_states, stage, total; };
+struct ChunkedBwdLayout { AdjLayout al; mdn_ws_layout lf; uint64_t ws_fwd, ws_fwd_bytes, fwd_states, adj_states, stage, total; };
 
 static mdn_status chunked_bwd_layout(const mdn_params* p, ChunkedBwdLayout* c) {
   mdn_status st = adj_layout(p, &c->al);
@@ -349,7 +351,11 @@ static mdn_status chunked_bwd_layout(const mdn_params* p, ChunkedBwdLayout* c) {
   if (st != MDN_OK) return st;
   uint64_t off = 0;
   auto take = [&](uint64_t bytes) { uint64_t at = off; off = align_up(off + bytes, 1024); return at; };
-  c->ws_fwd = take(c->lf.total_bytes);
+  mdn_ws_layout lw;   // the forward's own workspace: with the segment scan's scratch
+  st = make_layout(*p, &lw);
+  if (st != MDN_OK) return st;
+  c->ws_fwd_bytes = lw.total_bytes;
+  c->ws_fwd = take(lw.total_bytes);
   c->fwd_states = take((uint64_t)c->lf.num_slots * p->H * (kStateImageBytes + kVtSlotBytes));
   c->adj_states = take(c->al.states_bytes());
   c->stage = take(c->al.total);
@@ -462,10 +468,8 @@ mdn_status mdn_chunk_bwd_chunked(const mdn_params* p, const void* q, const void*
   if (!workspace || workspace_bytes < c.total || !aligned(workspace, 1024)) return MDN_ERR_WORKSPACE;
   char* w = static_cast<char*>(workspace);
   // 1. the forward's states (no output terms), kept per chunk; T, W and the coefficient vectors stay in ws_fwd
-  mdn_params pf = *p;
-  pf.segments = 1;
   Plan fwd;
-  st = make_plan(&pf, cu_seqlens, w + c.ws_fwd, c.lf.total_bytes, cuda_stream, &fwd);
+  st = make_plan(p, cu_seqlens, w + c.ws_fwd, c.ws_fwd_bytes, cuda_stream, &fwd);
   if (st != MDN_OK) return st;
   fwd.chain_dump = reinterpret_cast<uint8_t*>(w + c.fwd_states);
   fwd.chain_vt_dump = reinterpret_cast<float*>(w + c.fwd_states + (uint64_t)c.lf.num_slots * p->H * kStateImageBytes);

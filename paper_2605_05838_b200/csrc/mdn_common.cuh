@@ -88,6 +88,20 @@ __device__ __forceinline__ SeqInfo seq_info(const ChunkGeom& g, int seq) {
   return s;
 }
 
+// The chunks of segment `seg` of a sequence with nchunks chunks (parallel inter-chunk scan, G segments): the first segment has
+// `first`, the others `mid`.  Packed input: in these proportions of the sequence's own length; a sequence whose middle segments
+// would be shorter than `least` stays whole, the others are empty.
+struct SegSplitArgs { int G, first, mid, least; };
+__device__ __forceinline__ int2 seg_chunks(const ChunkGeom& g, int nchunks, const SegSplitArgs& s, int seg) {
+  int first = s.first, mid = s.mid;
+  if (g.cu != nullptr) {
+    mid = (int)((long long)nchunks * mid / (first + (s.G - 1) * mid));
+    if (mid < s.least) mid = 0;
+    first = nchunks - (s.G - 1) * mid;
+  }
+  return make_int2(seg == 0 ? 0 : min(nchunks, first + (seg - 1) * mid), min(nchunks, first + seg * mid));   // (G segments reach the end)
+}
+
 // Programmatic dependent launch (no-ops unless the kernel was launched with the stream-serialization
 // attribute): wait for the preceding kernel's results / let the next kernel's prologue start.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
