@@ -1,5 +1,6 @@
 // a3 + a4 on the 5th-generation tensor cores (tcgen05, sm_100a): one CTA walks the chunks of
-// one (sequence, head) in order.  bf16 q/k/v, dk = dv = 128, chunk 64.
+// one (sequence, head) in order.  bf16 q/k/v, dk = dv = 128, chunk 64.  The first design; it runs the two chains of a
+// training step (the forward that keeps its states, the adjoint chain), every other forward runs on chain_tf32.cu.
 //
 // Everything is kept TRANSPOSED so that the value dimension (128) is the MMA M dimension and
 // fills all 128 tensor-memory lanes; the 64 tokens of a chunk are the N (or K) dimension:
@@ -22,12 +23,7 @@
 // rounding to plain bf16 would dominate the error budget); raw q/k tiles are never rescaled before
 // an MMA - every row/column scaling is applied to fp32 accumulators.
 //
-// Layer operations (template flag kLayer; Section 3.3): with the fused q/k step the accumulators X, Y are scaled by
-// 1 / |k| (folded into the coefficient vectors), EPI-1 leaves -d K S, -d K M in Z, U and MMA-1b runs after MMA-2,
-// accumulating onto them; with the fused output step the staged fp32 tile is re-read row-wise for RMSNorm, weight
-// and sigmoid gate before the TMA store.  kLayer = false is the plain forward, compiled without any of it.
-//
-// Warp roles: 8 (plain forward) or 16 (with layer operations) epilogue warps, lane quarter x token group, every one
+// Warp roles: 8 epilogue warps, lane quarter x token half, every one
 // running P, EPI-o, EPI-1, EPI-2 on its share; then the TMA producer (2-stage ring: K, Q, V, T, W_hi, W_lo, 8 coefficient vectors per chunk; it also
 // issues the output stores) and the MMA issuer (one elected lane, tensor-memory owner).  All hand-offs are
 // mbarriers with bounded waits; tensor-memory column reuse is ordered by those same barriers.
@@ -43,20 +39,11 @@ namespace {
 using namespace tc;
 
 constexpr int kD = 128;
-// Epilogue warps: 4 lane quarters (value rows 32 q .. +31 = the tensor-memory lanes a warp may touch) x TG token
-// groups of 64 / TG tokens, followed by the TMA producer warp and the MMA issuer warp.  The epilogue steps are bound
-// by fixed latencies (tensor-memory round trips, group barriers), not by instruction issue: the plain forward is
-// as fast with 8 epilogue warps (TG = 2, 168 registers per thread) as with 16; the variant with the layer
-// operations, whose output step is instruction-heavy, gains 3 % from 16 (TG = 4, 96 registers).
-template <int TG> struct Roles {
-  static_assert(TG == 2 || TG == 4, "token groups");
-  static constexpr int kTG = TG;
-  static constexpr int kTok = C / TG;          // tokens per epilogue warp in the per-token steps
-  static constexpr int kPk = kTok / 2;         // 32-bit words of packed bf16 pairs for those tokens
-  static constexpr int kEpiWarps = 4 * TG;
-  static constexpr int kThreads = (kEpiWarps + 2) * 32;
-};
-constexpr int token_groups(bool layer) { return layer ? 4 : 2; }
+// Epilogue warps: 4 lane quarters (value rows 32 q .. +31 = the tensor-memory lanes a warp may touch) x 2 token halves, followed by
+// the TMA producer warp and the MMA issuer warp.  The epilogue steps are bound by fixed latencies (tensor-memory round trips,
+// group barriers), not by instruction issue: 16 warps are no faster.
+constexpr int kTok = C / 2, kPk = kTok / 2;   // tokens per epilogue warp in the per-token steps; words of packed bf16 pairs for them
+constexpr int kEpiWarps = 8, kEpiThreads = kEpiWarps * 32, kWarpTma = kEpiWarps, kWarpMma = kEpiWarps + 1, kThreads = (kEpiWarps + 2) * 32;
 
 // shared memory (offsets from a 1024-byte aligned base)
 constexpr uint32_t kOffSb = 0, kOffMb = 32768, kOffStage = 65536;
@@ -85,7 +72,6 @@ struct Bars {
   uint64_t mo;        // MMA-3' done                                                   (commit)
   uint64_t zu;        // U (intra-chunk output) has been read                           (256)
   uint64_t dump;      // the producer has copied S_b, M_b of a chunk out (chunk-state dump only)   (1)
-  uint64_t pn[4];     // fused output step: the staged rows of a token group are in shared memory (128 each)
 };
 
 struct ChainArgs {
@@ -107,13 +93,6 @@ struct ChainArgs {
   float* seg_Psi;             // [chains][G-2][2][dk*dv]  segment run from a zero state
   float* seg_PhiS;            // [chains][G-2][2][dk*dv]  segment run with V = 0 from (S, M) = (I, 0)
   float* seg_PhiM;            // [chains][G-2][2][dk*dv]  ... from (0, I)
-  // layer operations absorbed by this kernel (Section 3.3)
-  int qk_on;                  // q <- L2Norm(q - d k), k <- L2Norm(k): coefficient vectors 6, 7 hold 1/|k|, 1/|q - d k|
-  const float* qk_d;          // [H] or NULL
-  int post_on;                // o <- sigmoid(g) * RMSNorm(o) * w in the output epilogue
-  const float* post_w;        // [dv] or NULL
-  const void* post_g;         // [B,T,H,dv] bf16
-  float post_eps;
   // training / backward support
   uint8_t* dump;              // NULL, or [slot][H][65536]: the bf16 copies S_b^T | M_b^T of the state at the START of
                               // every chunk, as they lie in shared memory (two [128 x 128 B] swizzled blocks each)
@@ -140,13 +119,6 @@ enum Ev : int { kEvMmaStart = 0, kEvM1Seen, kEvRArrive, kEvM2Seen, kEvVArrive, k
                 kEvZqArrive, kEvMoSeen, kEvZuArrive, kEvMmaIssued, kEvRSeen, kEvVSeen, kEvTmaIssued, kEvFullSeen,
                 kEvStoresDone, kEvV2Arrive, kEvPrescaled };
 
-// sigmoid(x) = (1 + tanh(x / 2)) / 2 with the one-instruction tanh approximation (relative error ~2^-11)
-__device__ __forceinline__ float sigmoid_fast(float x) {
-  float t;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(0.5f * x));
-  return fmaf(0.5f, t, 0.5f);
-}
-
 template <typename TO> __device__ __forceinline__ void stage_o(uint8_t* tile, int r, int d, float x);
 template <> __device__ __forceinline__ void stage_o<float>(uint8_t* tile, int r, int d, float x) {
   reinterpret_cast<float*>(tile)[r * kD + d] = x;
@@ -155,11 +127,9 @@ template <> __device__ __forceinline__ void stage_o<__nv_bfloat16>(uint8_t* tile
   reinterpret_cast<__nv_bfloat16*>(tile)[r * kD + d] = __float2bfloat16_rn(x);
 }
 
-// kTrain compiles in the chunk-state dump, the state-only switch and the decoupled end-of-chunk scalars (the plain
-// forward's instantiation stays as it is: its schedule is fragile, a runtime test of these options cost it 2 %)
 // kSeg: the parallel inter-chunk scan's runs (a template flag: as run-time tests it cost the serial chain 2 - 6 %)
-template <typename TO, bool kLayer, bool kTrain, bool kSeg>
-__global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chain_tensor_kernel(const ChainArgs a,
+template <typename TO, bool kSeg>
+__global__ void __launch_bounds__(kThreads, 1) chain_tensor_kernel(const ChainArgs a,
                                                                   const __grid_constant__ CUtensorMap map_q,
                                                                   const __grid_constant__ CUtensorMap map_k,
                                                                   const __grid_constant__ CUtensorMap map_v,
@@ -171,13 +141,7 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
   __shared__ __align__(8) Bars bars;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
-  __shared__ __align__(16) float w_sm[kLayer ? kD : 4];   // RMSNorm weight of the fused output step
 
-  using R = Roles<token_groups(kLayer)>;
-  constexpr int kTG = R::kTG, kTok = R::kTok, kPk = R::kPk, kEpiWarps = R::kEpiWarps;
-  constexpr int kWarpTma = kEpiWarps, kWarpMma = kEpiWarps + 1;
-  constexpr bool kWarpArrive = kLayer;   // epilogue hand-overs: one mbarrier arrival per warp, or one per thread
-  constexpr int kArrivals = kWarpArrive ? kEpiWarps : kEpiWarps * 32;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int H = a.g.H;
   // ---- work item: which chain, which segment of it, which kind of run
@@ -236,11 +200,11 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
       Sfp = base; Mfp = base + kMat;
     }
   }
-  if constexpr (kTrain) {
+  {
     if (a.state_only) write_o = false;
   }
   // the runs from basis states (V = 0) have no second update; only real runs leave anything behind
-  const bool inject = kTrain && a.inject && (!kSeg || run <= 1), dump = kTrain && a.dump != nullptr && (!kSeg || run == 0);
+  const bool inject = a.inject && (!kSeg || run <= 1), dump = a.dump != nullptr && (!kSeg || run == 0);
 
   const uint32_t s_base = smem_u32(smem);
   const uint32_t b_full0 = smem_u32(&bars.full[0]), b_full1 = smem_u32(&bars.full[1]);
@@ -249,24 +213,18 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
   const uint32_t b_r = smem_u32(&bars.r), b_m2 = smem_u32(&bars.m2);
   const uint32_t b_v1 = smem_u32(&bars.v1), b_v2 = smem_u32(&bars.v2), b_m3 = smem_u32(&bars.m3);
   const uint32_t b_mo = smem_u32(&bars.mo), b_zu = smem_u32(&bars.zu), b_dump = smem_u32(&bars.dump);
-  // kLayer = false compiles the layer operations out: the plain forward keeps its instruction count
-  const bool qk_on = kLayer && a.qk_on;
-  const bool post = kLayer && a.post_on && write_o;
-  const float dh = (qk_on && a.qk_d) ? __ldg(a.qk_d + h) : 0.f;
 
   if (tid == 0) {
     abort_flag = 0;
     mbar_init(b_full0, 1); mbar_init(b_full1, 1);
-    mbar_init(b_go0, kArrivals); mbar_init(b_go1, kArrivals);
-    mbar_init(b_sb, kArrivals); mbar_init(b_r, kArrivals); mbar_init(b_v1, kArrivals);
-    mbar_init(b_v2, kArrivals);
-    mbar_init(b_zu, kArrivals);
+    mbar_init(b_go0, kEpiThreads); mbar_init(b_go1, kEpiThreads);
+    mbar_init(b_sb, kEpiThreads); mbar_init(b_r, kEpiThreads); mbar_init(b_v1, kEpiThreads);
+    mbar_init(b_v2, kEpiThreads);
+    mbar_init(b_zu, kEpiThreads);
     mbar_init(b_dump, 1);
     mbar_init(b_m1, 1); mbar_init(b_mq, 1); mbar_init(b_m2, 1); mbar_init(b_m3, 1); mbar_init(b_mo, 1);
-    for (int i = 0; i < kTG; ++i) mbar_init(smem_u32(&bars.pn[i]), 128);
     mbar_fence_init();
   }
-  if (kLayer && tid < kD) w_sm[tid] = (a.post_on && a.post_w) ? __ldg(a.post_w + tid) : 1.f;
   if (warp == kWarpMma) tmem_alloc(smem_u32(&tmem_slot), 512);
   if (warp == kWarpTma && lane == 0) {
     prefetch_tensormap(&map_q); prefetch_tensormap(&map_k); prefetch_tensormap(&map_v);
@@ -286,18 +244,6 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
 #ifdef MDN_DEBUG
   long long* const tline = (blockIdx.x == 0) ? a.timeline : nullptr;
 #endif
-  // Hand-over arrivals of the epilogue.  With 16 epilogue warps (layer variant) one arrival per warp, after the warp
-  // has converged (every lane's stores and fences precede it): 32 x fewer shared-memory atomics in front of every
-  // hand-over, 2 % of the step.  The 8-warp plain forward measured 1 % slower that way and keeps one per thread.
-#define MDN_WARP_ARRIVE(bar)             \
-  {                                      \
-    if constexpr (kWarpArrive) {         \
-      __syncwarp();                      \
-      if (lane == 0) mbar_arrive(bar);   \
-    } else {                             \
-      mbar_arrive(bar);                  \
-    }                                    \
-  }
 #ifdef MDN_DEBUG
 #define MDN_MARK(c, ev) \
   if (tline != nullptr && lane == 0 && (warp == 0 || warp >= kEpiWarps)) tline[(c) * 32 + (ev)] = clock64();
@@ -319,8 +265,8 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
           MDN_WAIT(s ? b_go1 : b_go0, (co >> 1) & 1);
           const int n = min(C, sq.len - co * C);
           const int tok0 = sq.tok0 + co * C;
-          // the finished tile: at the start of the stage, except the bf16 tile of the fused output step (T / W area)
-          const uint32_t src = st + ((post && sizeof(TO) == 2) ? kStT : 0u);
+          // the finished tile: at the start of the stage
+          const uint32_t src = st;
           if (!write_o) {
             // Psi / Phi runs of the parallel scan produce states only
           } else if (n == C) {
@@ -342,7 +288,7 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
           const bool inj = inject;               // Q and G (into the W area) instead of Q and W
           int tok0k = tok0;                      // rows of k, q, G
           int mat_t = mat;                       // which T
-          if (kTrain && a.mirror) {
+          if (a.mirror) {
             tok0k = seq_info(a.mirror_g, seq).tok0 + (rev0 - c) * C;
             mat_t = (seq_info(a.g, seq).slot0 + rev0 - c) * H + h;
           }
@@ -415,35 +361,19 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
         for (int k = 0; k < 8; ++k)
           umma_ss(tmem + kColY, ((k >> 2) ? dMb1 : dMb0) + 2 * (k & 3), ((k >> 2) ? dK1 : dK0) + 2 * (k & 3), id64, k > 0);
         umma_commit(b_m1);
-        // ---- MMA-1b: Z = S_b Q^T, U = M_b Q^T (U of the previous chunk must have been read).  With the fused q/k
-        // step it runs after MMA-2 instead and ACCUMULATES onto -d K S, -d K M, which EPI-1 has put into Z, U.
-#define MDN_MMA_1B(onto)                                                                                                  \
-  {                                                                                                                        \
-    MDN_WAIT(b_zu, ph ^ 1);                                                                                                \
-    tc_fence_after_sync();                                                                                                 \
-    _Pragma("unroll") for (int k = 0; k < 8; ++k)                                                                          \
-        umma_ss(tmem + kColZ, ((k >> 2) ? dSb1 : dSb0) + 2 * (k & 3), ((k >> 2) ? dQ1 : dQ0) + 2 * (k & 3), id64, (onto) || k > 0); \
-    _Pragma("unroll") for (int k = 0; k < 8; ++k)                                                                          \
-        umma_ss(tmem + kColU, ((k >> 2) ? dMb1 : dMb0) + 2 * (k & 3), ((k >> 2) ? dQ1 : dQ0) + 2 * (k & 3), id64, (onto) || k > 0); \
-    umma_commit(b_mq);                                                                                                     \
-  }
         // ---- MMA-1b (output terms, off the critical path).  The tensor pipe runs its MMAs in issue order, so a group
         // issued here delays MMA-2 by whatever of it is still running when EPI-1 is done: only Z = S_b Q^T is issued
         // here (it fits under EPI-1) ...
-        if constexpr (!kLayer) {
-          if (write_o) {
+        if (write_o) {
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-              umma_ss(tmem + kColZ, ((k >> 2) ? dSb1 : dSb0) + 2 * (k & 3), ((k >> 2) ? dQ1 : dQ0) + 2 * (k & 3), id64, k > 0);
-          }
-        } else {
-          if (write_o && !qk_on) MDN_MMA_1B(false);
+          for (int k = 0; k < 8; ++k)
+            umma_ss(tmem + kColZ, ((k >> 2) ? dSb1 : dSb0) + 2 * (k & 3), ((k >> 2) ? dQ1 : dQ0) + 2 * (k & 3), id64, k > 0);
         }
         // ---- MMA-2: Y = (R_hi + R_lo)^T T^T
         MDN_WAIT(b_r, ph);
         tc_fence_after_sync();
         MDN_MARK(c, kEvRSeen);
-        if (kTrain && a.mirror) {   // T^T: the same tile read MN-major (16 rows = 2048 bytes per K step)
+        if (a.mirror) {   // T^T: the same tile read MN-major (16 rows = 2048 bytes per K step)
           const uint64_t dTmn = smem_desc_sw128(st + kStT, 8192, 1024);
           const uint32_t id64_mn = idesc_bf16(128, 64, false, true, false);
           for (int k = 0; k < 8; ++k)
@@ -458,19 +388,15 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
         }
         umma_commit(b_m2);
         // ... and U = M_b Q^T here: it fits under EPI-2 and is done before MMA-3 can start
-        if constexpr (!kLayer) {
-          if (write_o) {
-            MDN_WAIT(b_zu, ph ^ 1);
-            tc_fence_after_sync();
+        if (write_o) {
+          MDN_WAIT(b_zu, ph ^ 1);
+          tc_fence_after_sync();
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-              umma_ss(tmem + kColU, ((k >> 2) ? dMb1 : dMb0) + 2 * (k & 3), ((k >> 2) ? dQ1 : dQ0) + 2 * (k & 3), id64, k > 0);
-            umma_commit(b_mq);
-          }
-        } else {
-          if (write_o && qk_on) MDN_MMA_1B(true);
+          for (int k = 0; k < 8; ++k)
+            umma_ss(tmem + kColU, ((k >> 2) ? dMb1 : dMb0) + 2 * (k & 3), ((k >> 2) ? dQ1 : dQ0) + 2 * (k & 3), id64, k > 0);
+          umma_commit(b_mq);
         }
-        if constexpr (kTrain) {
+        {
           if (inject) {
             // the second update (operands in Z, U and the pre-scaled masters ready since the start of the chunk, Q
             // read MN-major) needs nothing of this chunk's V~: issued here it runs while EPI-2 works, before MMA-3
@@ -519,8 +445,6 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
     const int d = q4 * 32 + lane;
     const int r0 = kTok * hf;
     const uint32_t tl = tmem + (static_cast<uint32_t>(q4 * 32) << 16);
-    uint32_t pn_phase = 0;
-    const uint32_t b_pn = smem_u32(&bars.pn[hf]);
     float oi[kTok];   // scale (abar .* Q S - b .* Q M) for this thread's tokens, carried to the output step
 
 #pragma unroll
@@ -535,7 +459,7 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
       if (c < nch) {
         MDN_WAIT((c & 1) ? b_full1 : b_full0, (c >> 1) & 1);
         const float* cf = reinterpret_cast<const float*>(smem + kOffStage + (c & 1) * kStageBytes + kStCoef);
-        if (kTrain && a.end_scalars_in_rk) {
+        if (a.end_scalars_in_rk) {
           al = cf[kRk * C + 0]; bl = cf[kRk * C + 1]; ml = cf[kRk * C + 2];
         } else {
           al = cf[kAbar * C + C - 1]; bl = cf[kB * C + C - 1]; ml = cf[kMubar * C + C - 1];
@@ -545,7 +469,7 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
       }
       __syncwarp();
       tc_fence_after_sync();
-      if constexpr (kTG == 2) {   // two passes of 32 dk columns (kept textually apart: the plain forward's schedule is fragile)
+      {   // two passes of 32 dk columns
 #pragma unroll 1
         for (int i = 0; i < 2; ++i) {
           const int cs = 2 * hf + i;   // 32-column slice of dk
@@ -598,83 +522,20 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
             }
           }
         }
-      } else {
-        constexpr int kPw = (kTG == 4) ? 16 : 32;   // dk columns per pass (a warp owns 128 / kTG of them)
-#pragma unroll 1
-        for (int i = 0; i < 128 / kTG / kPw; ++i) {
-          const int col0 = hf * (128 / kTG) + i * kPw;
-          uint32_t sr[kPw], mr[kPw];
-          if (c == 0) {
-#pragma unroll
-            for (int j = 0; j < kPw; ++j) {
-              const float unit = (col0 + j == d) ? 1.f : 0.f;
-              sr[j] = __float_as_uint(S0p ? __ldg(S0p + (size_t)(col0 + j) * kD + d) : (id_s ? unit : 0.f));
-              mr[j] = __float_as_uint(M0p ? __ldg(M0p + (size_t)(col0 + j) * kD + d) : (id_m ? unit : 0.f));
-            }
-          } else {
-            tmem_ld_n<kPw>(tl + kColS + col0, sr);
-            tmem_ld_n<kPw>(tl + kColM + col0, mr);
-            tmem_wait_ld();
-          }
-          if (c < nch) {
-            uint8_t* sb = smem + kOffSb + (col0 >> 6) * 16384;
-            uint8_t* mb = smem + kOffMb + (col0 >> 6) * 16384;
-#pragma unroll
-            for (int j8 = 0; j8 < kPw / 8; ++j8) {
-              uint4 ps, pm;
-              ps.x = pack_bf16(__uint_as_float(sr[j8 * 8 + 0]), __uint_as_float(sr[j8 * 8 + 1]));
-              ps.y = pack_bf16(__uint_as_float(sr[j8 * 8 + 2]), __uint_as_float(sr[j8 * 8 + 3]));
-              ps.z = pack_bf16(__uint_as_float(sr[j8 * 8 + 4]), __uint_as_float(sr[j8 * 8 + 5]));
-              ps.w = pack_bf16(__uint_as_float(sr[j8 * 8 + 6]), __uint_as_float(sr[j8 * 8 + 7]));
-              pm.x = pack_bf16(__uint_as_float(mr[j8 * 8 + 0]), __uint_as_float(mr[j8 * 8 + 1]));
-              pm.y = pack_bf16(__uint_as_float(mr[j8 * 8 + 2]), __uint_as_float(mr[j8 * 8 + 3]));
-              pm.z = pack_bf16(__uint_as_float(mr[j8 * 8 + 4]), __uint_as_float(mr[j8 * 8 + 5]));
-              pm.w = pack_bf16(__uint_as_float(mr[j8 * 8 + 6]), __uint_as_float(mr[j8 * 8 + 7]));
-              const uint32_t off = sw128_offset(d, (col0 & 63) + j8 * 8);
-              *reinterpret_cast<uint4*>(sb + off) = ps;
-              *reinterpret_cast<uint4*>(mb + off) = pm;
-            }
-            // masters scaled by this chunk's (abar_C, b_C, mubar_C) so that MMA-3 can accumulate straight into
-            // them; the stores are asynchronous and only waited for before V~_S, V~_M are handed over
-#pragma unroll
-            for (int j = 0; j < kPw; ++j) {
-              const float sv = __uint_as_float(sr[j]), mv = __uint_as_float(mr[j]);
-              sr[j] = __float_as_uint(al * sv - bl * mv);
-              mr[j] = __float_as_uint(ml * mv);
-            }
-            tmem_st_n<kPw>(tl + kColS + col0, sr);
-            tmem_st_n<kPw>(tl + kColM + col0, mr);
-          } else {
-#pragma unroll
-            for (int j = 0; j < kPw; ++j) {
-              if (Sfp) Sfp[(size_t)(col0 + j) * kD + d] = __uint_as_float(sr[j]);
-              if (Mfp) Mfp[(size_t)(col0 + j) * kD + d] = __uint_as_float(mr[j]);
-            }
-          }
-        }
       }
       if (c < nch) {
         fence_proxy_async_smem();
-        MDN_WARP_ARRIVE(b_sb);
+        mbar_arrive(b_sb);
         MDN_MARK(c, kEvSbArrive);
       }
       // ---------------- output of the previous chunk (under MMA-1a): o^T = oi + U, staged as a [64 x 128] tile in
       // the previous chunk's stage (all its MMAs are done and nobody reads its tiles any more)
       if (c > 0 && !write_o) {
         // state-only run: MMA-3 of the previous chunk (waited for above) was the last reader of its stage
-        MDN_WARP_ARRIVE(((c - 1) & 1) ? b_go1 : b_go0);
+        mbar_arrive(((c - 1) & 1) ? b_go1 : b_go0);
       } else if (c > 0) {
         const int cp = c - 1;
         uint8_t* stp = smem + kOffStage + (cp & 1) * kStageBytes;
-        // fused output step: this thread's share of the chunk's output-gate rows is four threads per token, 8-byte
-        // pieces (each warp-load covers eight full 32-byte sectors); the rows are pulled towards L2 here and read
-        // once the tile is staged, when registers are free again
-        constexpr int kTpr = 128 / kTok, kPieces = 32 / kTpr;   // threads per row, 16-byte pieces per thread
-        const int t128 = q4 * 32 + lane, prow = r0 + t128 / kTpr, part = t128 % kTpr;
-        const bool g_live = post && cp * C + prow < sq.len;
-        const uint2* gp = reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(a.post_g) +
-                                                         ((size_t)(sq.tok0 + cp * C + prow) * H + h) * kD) + part;
-        if (g_live && part < 2) asm volatile("prefetch.global.L2 [%0];" ::"l"(gp + 15 * part));   // bytes 0 and 128 of the row (parts 0, 1)
         MDN_WAIT(b_mo, cp & 1);
         __syncwarp();
         tc_fence_after_sync();
@@ -684,57 +545,13 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
           tmem_ld_n<kTok>(tl + kColU + r0, u);
           tmem_wait_ld();
           tc_fence_before_sync();
-          MDN_WARP_ARRIVE(b_zu);
+          mbar_arrive(b_zu);
           MDN_MARK(cp, kEvZuArrive);
-          if (!post) {
 #pragma unroll
-            for (int j = 0; j < kTok; ++j) stage_o<TO>(stp, r0 + j, d, oi[j] + __uint_as_float(u[j]));
-          } else {
-            // fused output step: y = sigmoid(g) * o / sqrt(mean_d o^2 + eps) * w_d.  The fp32 tile is staged first
-            // (value columns across lanes), then re-read row-wise: four threads per token sum its 128 squares,
-            // rescale, gate and write the final tile (in place for fp32 output, into the T / W area for bf16).
-            float* tile = reinterpret_cast<float*>(stp);
-#pragma unroll
-            for (int j = 0; j < kTok; ++j) tile[(r0 + j) * kD + d] = oi[j] + __uint_as_float(u[j]);
-            uint2 graw[kPieces];
-#pragma unroll
-            for (int i = 0; i < kPieces; ++i) graw[i] = g_live ? __ldg(gp + kTpr * i) : make_uint2(0u, 0u);
-            mbar_arrive(b_pn);
-            MDN_WAIT(b_pn, pn_phase);
-            pn_phase ^= 1;
-            __syncwarp();
-            const int row = prow;
-            float4 ov[kPieces];
-            float ss = 0.f;
-#pragma unroll
-            for (int i = 0; i < kPieces; ++i) {   // interleaved 16-byte pieces: a row's threads cover contiguous bytes
-              ov[i] = *reinterpret_cast<const float4*>(tile + row * kD + (part + kTpr * i) * 4);
-              ss = fmaf(ov[i].x, ov[i].x, fmaf(ov[i].y, ov[i].y, fmaf(ov[i].z, ov[i].z, fmaf(ov[i].w, ov[i].w, ss))));
-            }
-#pragma unroll
-            for (int off = 1; off < kTpr; off <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-            const float rstd = rsqrtf(ss * (1.f / kD) + a.post_eps);
-#pragma unroll
-            for (int i = 0; i < kPieces; ++i) {
-              const int col = (part + kTpr * i) * 4;
-              const float4 wv = *reinterpret_cast<const float4*>(w_sm + col);
-              const uint2 gr = graw[i];
-              const float g0 = __uint_as_float(gr.x << 16), g1 = __uint_as_float(gr.x & 0xffff0000u);
-              const float g2 = __uint_as_float(gr.y << 16), g3 = __uint_as_float(gr.y & 0xffff0000u);
-              const float y0 = ov[i].x * rstd * wv.x * sigmoid_fast(g0), y1 = ov[i].y * rstd * wv.y * sigmoid_fast(g1);
-              const float y2 = ov[i].z * rstd * wv.z * sigmoid_fast(g2), y3 = ov[i].w * rstd * wv.w * sigmoid_fast(g3);
-              if (sizeof(TO) == 4) {
-                *reinterpret_cast<float4*>(tile + row * kD + col) = make_float4(y0, y1, y2, y3);
-              } else {
-                uint2 pk;
-                pk.x = pack_bf16(y0, y1); pk.y = pack_bf16(y2, y3);
-                *reinterpret_cast<uint2*>(stp + kStT + (row * kD + col) * 2) = pk;
-              }
-            }
-          }
+          for (int j = 0; j < kTok; ++j) stage_o<TO>(stp, r0 + j, d, oi[j] + __uint_as_float(u[j]));
         }
         fence_proxy_async_smem();
-        MDN_WARP_ARRIVE((cp & 1) ? b_go1 : b_go0);
+        mbar_arrive((cp & 1) ? b_go1 : b_go0);
       }
       if (c == nch) break;
       MDN_MARK(c, kEvPrescaled);
@@ -743,7 +560,7 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
       const uint8_t* stg = smem + kOffStage + (c & 1) * kStageBytes;
       const float* cf = reinterpret_cast<const float*>(stg + kStCoef);
       const __nv_bfloat16* sV = reinterpret_cast<const __nv_bfloat16*>(stg + kStV);
-      if constexpr (kTrain) {
+      {
         if (inject) {
           // operands of the second update: they depend on nothing the chain computes, so they are made here, while
           // MMA-1a runs.  Z, U are free in a state-only run; the previous chunk's MMA-3 (waited for in P) was their
@@ -767,7 +584,7 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
           }
           tmem_wait_st();
           tc_fence_before_sync();
-          MDN_WARP_ARRIVE(b_v2);
+          mbar_arrive(b_v2);
         }
       }
       // ---------------- EPI-1: R^T = V^T - abar .* X + (alpha b^-) .* Y  -> bf16 hi, lo in X
@@ -790,37 +607,12 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
           for (int j = 0; j < kTok; j += 4) {
             const float4 ab = *reinterpret_cast<const float4*>(cf + kAbar * C + r0 + j);
             const float4 pb = *reinterpret_cast<const float4*>(cf + kAlphaBPrev * C + r0 + j);
-            float e0, e1, e2, e3;
-            if (qk_on) {
-              // k' = k / |k|: X, Y are products with the raw k tile, so the norm scales the accumulators (vector 2
-              // already carries the factor); the output correction q - d k turns Q S into Q S - d K S (same for M):
-              // its K terms are X, Y themselves, handed to the tensor core as the start value of Z, U
-              const float4 rk = *reinterpret_cast<const float4*>(cf + kRk * C + r0 + j);
-              const float x0 = __uint_as_float(x[j + 0]), x1 = __uint_as_float(x[j + 1]);
-              const float x2 = __uint_as_float(x[j + 2]), x3 = __uint_as_float(x[j + 3]);
-              const float y0 = __uint_as_float(y[j + 0]), y1 = __uint_as_float(y[j + 1]);
-              const float y2 = __uint_as_float(y[j + 2]), y3 = __uint_as_float(y[j + 3]);
-              e0 = vv[j + 0] - (rk.x * ab.x) * x0 + pb.x * y0;
-              e1 = vv[j + 1] - (rk.y * ab.y) * x1 + pb.y * y1;
-              e2 = vv[j + 2] - (rk.z * ab.z) * x2 + pb.z * y2;
-              e3 = vv[j + 3] - (rk.w * ab.w) * x3 + pb.w * y3;
-              // -d K S, -d K M: MMA-1b will accumulate Q S, Q M onto them
-              x[j + 0] = __float_as_uint(-dh * x0); x[j + 1] = __float_as_uint(-dh * x1);
-              x[j + 2] = __float_as_uint(-dh * x2); x[j + 3] = __float_as_uint(-dh * x3);
-              y[j + 0] = __float_as_uint(-dh * y0); y[j + 1] = __float_as_uint(-dh * y1);
-              y[j + 2] = __float_as_uint(-dh * y2); y[j + 3] = __float_as_uint(-dh * y3);
-            } else {
-              e0 = vv[j + 0] - ab.x * __uint_as_float(x[j + 0]) + pb.x * __uint_as_float(y[j + 0]);
-              e1 = vv[j + 1] - ab.y * __uint_as_float(x[j + 1]) + pb.y * __uint_as_float(y[j + 1]);
-              e2 = vv[j + 2] - ab.z * __uint_as_float(x[j + 2]) + pb.z * __uint_as_float(y[j + 2]);
-              e3 = vv[j + 3] - ab.w * __uint_as_float(x[j + 3]) + pb.w * __uint_as_float(y[j + 3]);
-            }
+            const float e0 = vv[j + 0] - ab.x * __uint_as_float(x[j + 0]) + pb.x * __uint_as_float(y[j + 0]);
+            const float e1 = vv[j + 1] - ab.y * __uint_as_float(x[j + 1]) + pb.y * __uint_as_float(y[j + 1]);
+            const float e2 = vv[j + 2] - ab.z * __uint_as_float(x[j + 2]) + pb.z * __uint_as_float(y[j + 2]);
+            const float e3 = vv[j + 3] - ab.w * __uint_as_float(x[j + 3]) + pb.w * __uint_as_float(y[j + 3]);
             split_pack_bf16(e0, e1, hi[j >> 1], lo[j >> 1]);
             split_pack_bf16(e2, e3, hi[(j >> 1) + 1], lo[(j >> 1) + 1]);
-          }
-          if (qk_on && write_o) {   // own lanes only; MMA-3' of the previous chunk and this thread's read of U are done
-            tmem_st_n<kTok>(tl + kColZ + r0, x);
-            tmem_st_n<kTok>(tl + kColU + r0, y);
           }
         }
         // hi and lo both go into the columns this warp has just read (its own kTok columns of X): no other warp
@@ -830,40 +622,8 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
         tmem_wait_st();
       }
       tc_fence_before_sync();
-      MDN_WARP_ARRIVE(b_r);
+      mbar_arrive(b_r);
       MDN_MARK(c, kEvRArrive);
-      // ---------------- inter-chunk output terms: oi = scale (abar .* Q S - b .* Q M), under MMA-2; with the fused
-      // q/k step Z, U arrive later (MMA-1b follows MMA-2) and already hold Q S - d K S, Q M - d K M: then this
-      // step runs under MMA-3 instead
-#define MDN_INTER_CHUNK_TERMS()                                                                              \
-  {                                                                                                          \
-    MDN_WAIT(b_mq, ph);                                                                                      \
-    __syncwarp();                                                                                            \
-    tc_fence_after_sync();                                                                                   \
-    MDN_MARK(c, kEvMqSeen);                                                                                  \
-    uint32_t z[kTok], u[kTok];                                                                               \
-    tmem_ld_n<kTok>(tl + kColZ + r0, z);                                                                     \
-    tmem_ld_n<kTok>(tl + kColU + r0, u);                                                                     \
-    tmem_wait_ld();                                                                                          \
-    tc_fence_before_sync();                                                                                  \
-    MDN_MARK(c, kEvZqArrive);                                                                                \
-    _Pragma("unroll") for (int j = 0; j < kTok; j += 4) {                                                    \
-      const float4 ab = *reinterpret_cast<const float4*>(cf + kAbar * C + r0 + j);                           \
-      const float4 bb = *reinterpret_cast<const float4*>(cf + kB * C + r0 + j);                              \
-      float4 sc = make_float4(a.scale, a.scale, a.scale, a.scale);                                           \
-      if (qk_on) { /* q' = (q - d k) / |q - d k| */                                                          \
-        const float4 rq = *reinterpret_cast<const float4*>(cf + kRq * C + r0 + j);                           \
-        sc.x *= rq.x; sc.y *= rq.y; sc.z *= rq.z; sc.w *= rq.w;                                              \
-      }                                                                                                      \
-      oi[j + 0] = sc.x * (ab.x * __uint_as_float(z[j + 0]) - bb.x * __uint_as_float(u[j + 0]));              \
-      oi[j + 1] = sc.y * (ab.y * __uint_as_float(z[j + 1]) - bb.y * __uint_as_float(u[j + 1]));              \
-      oi[j + 2] = sc.z * (ab.z * __uint_as_float(z[j + 2]) - bb.z * __uint_as_float(u[j + 2]));              \
-      oi[j + 3] = sc.w * (ab.w * __uint_as_float(z[j + 3]) - bb.w * __uint_as_float(u[j + 3]));              \
-    }                                                                                                        \
-  }
-      if constexpr (kLayer) {
-        if (write_o && !qk_on) MDN_INTER_CHUNK_TERMS();
-      }
       // ---------------- EPI-2: V~ -> (gamma_C eta) V~, ((mubar_C/mubar) eta) V~ [part a], V~ [part b]; bf16 hi, lo
       MDN_WAIT(b_m2, ph);
       __syncwarp();
@@ -900,9 +660,10 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
         }
         tmem_wait_st();          // also covers the pre-scaled masters stored in P part 2
         tc_fence_before_sync();
-        MDN_WARP_ARRIVE(b_v1);
+        mbar_arrive(b_v1);
         MDN_MARK(c, kEvVArrive);
-        if constexpr (!kLayer) {
+        // inter-chunk output terms: oi = scale (abar .* Q S - b .* Q M), under MMA-3
+        {
           if (write_o) {
             MDN_WAIT(b_mq, ph);
             __syncwarp();
@@ -924,8 +685,6 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
               oi[j + 3] = a.scale * (ab.w * __uint_as_float(z[j + 3]) - bb.w * __uint_as_float(u[j + 3]));
             }
           }
-        } else {
-          if (write_o && qk_on) MDN_INTER_CHUNK_TERMS();
         }
         // part b (under MMA-3): V~ itself for the intra-chunk output, into Z
         if (write_o) {
@@ -936,10 +695,10 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
           tmem_st_n<kPk>(tl + kColZ + r0 + kPk, vl);
           tmem_wait_st();
           tc_fence_before_sync();
-          MDN_WARP_ARRIVE(b_v2);
+          mbar_arrive(b_v2);
         }
         MDN_MARK(c, kEvV2Arrive);
-        if constexpr (kTrain) {   // off the chain's critical path: MMA-3 is running
+        {   // off the chain's critical path: MMA-3 is running
           const int slot_c = sq.slot0 + c;
           if (a.vt_dump != nullptr && (!kSeg || run == 0)) {
             const int live = min(C, sq.len - c * C) - r0;   // this thread's tokens inside the chunk
@@ -979,9 +738,6 @@ __global__ void __launch_bounds__(Roles<token_groups(kLayer)>::kThreads, 1) chai
       }
     }
   }
-#undef MDN_INTER_CHUNK_TERMS
-#undef MDN_MMA_1B
-#undef MDN_WARP_ARRIVE
 #undef MDN_WAIT
 #undef MDN_MARK
 
@@ -1028,8 +784,6 @@ cudaError_t launch_chain_tensor(const Plan& pl, const void* q, const void* k, co
   if (!encode_tma_2d(&mo, TmaMap2D{o, row, tokens_qko, row * (o_bf16 ? 2u : 4u), 128, 64, false}, !o_bf16))
     return cudaErrorInvalidValue;
   ChainArgs a;
-  a.qk_on = pl.qk.on; a.qk_d = pl.qk.d;
-  a.post_on = pl.post.on; a.post_w = pl.post.w; a.post_g = pl.post.g; a.post_eps = pl.post.eps;
   a.g = pl.geom;
   a.coef = reinterpret_cast<const float*>(pl.ws + pl.lay.off_coef);
   a.S0 = S0; a.M0 = M0; a.o = o; a.Sf = Sf; a.Mf = Mf;
@@ -1053,11 +807,11 @@ cudaError_t launch_chain_tensor(const Plan& pl, const void* q, const void* k, co
   a.seg_first = a.seg_mid = a.seg_least = 0;
   a.seg_E = a.seg_Psi = a.seg_PhiS = a.seg_PhiM = nullptr;
   const unsigned chains = (unsigned)pl.geom.num_seqs * p.H;
-  const bool layer = a.qk_on || a.post_on;
+  const bool layer = pl.qk.on || pl.post.on;
   auto launch_as = [&](auto kern, unsigned grid) -> cudaError_t {
     cudaError_t e = allow_smem(kern, (int)kSmemBytes);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(kern, dim3(grid), dim3(Roles<token_groups(false)>::kThreads), kSmemBytes, pl.stream, a, mq, mk, mv, mt, mw, mo);
+    e = launch_pdl(kern, dim3(grid), dim3(kThreads), kSmemBytes, pl.stream, a, mq, mk, mv, mt, mw, mo);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) ++*launches;
     return e;
@@ -1068,8 +822,8 @@ cudaError_t launch_chain_tensor(const Plan& pl, const void* q, const void* k, co
     if (!train || layer || (a.inject && !a.state_only) || (a.mirror && !a.inject)) return cudaErrorInvalidValue;
     typedef __nv_bfloat16 bf16;
     if (a.seg_G > 0)
-      return o_bf16 ? launch_as(chain_tensor_kernel<bf16, false, true, true>, grid) : launch_as(chain_tensor_kernel<float, false, true, true>, grid);
-    return o_bf16 ? launch_as(chain_tensor_kernel<bf16, false, true, false>, grid) : launch_as(chain_tensor_kernel<float, false, true, false>, grid);
+      return o_bf16 ? launch_as(chain_tensor_kernel<bf16, true>, grid) : launch_as(chain_tensor_kernel<float, true>, grid);
+    return o_bf16 ? launch_as(chain_tensor_kernel<bf16, false>, grid) : launch_as(chain_tensor_kernel<float, false>, grid);
   };
   const int G = pl.lay.segments;
   if (G <= 1) return launch(chains);
