@@ -744,7 +744,10 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tensor_kernel(const ChainAr
   if (!ok && lane == 0) atomicCAS(a.status, kDevOk, kDevTimeout);
   tc_fence_before_sync();
   __syncthreads();
-  if (warp == kWarpMma) tmem_dealloc(tmem, 512);
+  if (warp == kWarpMma) {
+    __syncwarp();
+    tmem_dealloc(tmem, 512);
+  }
 }
 
 }  // namespace

@@ -728,6 +728,7 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
       if (c == nch) {
         // ---------------- final states: [S; M] = G [Sh; Mh]  (the last chunk's MMA-3 was waited for below)
         MDN_WAIT(b_fin, 0);
+        __syncwarp();
         const float g11 = g_final[0], g12 = g_final[1], g22 = g_final[2];
         tc_fence_after_sync();
 #pragma unroll 1
@@ -962,7 +963,10 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
   }
   if (tline != nullptr && tid < 256) tline[(kTlFirst + (tid >> 5)) * 32 + (tid & 31)] = (tid & 31) < 30 ? tl_sm[tid >> 5][tid & 31] : 0;
 #endif
-  if (warp == kWarpMma) tmem_dealloc(tmem, 512);
+  if (warp == kWarpMma) {
+    __syncwarp();
+    tmem_dealloc(tmem, 512);
+  }
 }
 
 }  // namespace

@@ -460,6 +460,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) intra_mma_kernel(ChunkGe
   tc_fence_before_sync();
   __syncthreads();   // A and the W staging complete
   if (warp == 2) {   // every warp's tensor-memory loads completed before the barrier
+    __syncwarp();
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
   }

@@ -67,6 +67,8 @@ constexpr uint32_t kSpinLimit = 1u << 22;   // try_wait suspends internally; thi
 
 // Bounded wait.  Returns false when the limit ran out or another thread already gave up
 // (*abort_flag != 0); the caller then unwinds to the kernel's common exit.
+// The lanes of a warp can leave the loop at different times and nothing brings them together again, a block barrier
+// included: a warp-collective instruction behind it (tcgen05.ld, .st, .dealloc) needs a __syncwarp() first.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                           uint32_t limit = kSpinLimit) {
   // A phase that is already complete is seen by a plain poll in ~40 cycles; try_wait takes 200-350 cycles to say the

@@ -292,7 +292,10 @@ __global__ void __launch_bounds__(128) tf32_probe_kernel(int mode, const float* 
   if (!ok && tid == 0) atomicCAS(status, kDevOk, kDevTimeout);
   tc_fence_before_sync();
   __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, 256);
+  if (warp == 0) {
+    __syncwarp();
+    tmem_dealloc(tmem, 256);
+  }
 }
 
 // Issue-to-completion time of a stream of tcgen05 products of one shape (operand contents irrelevant): how the
@@ -359,7 +362,10 @@ __global__ void __launch_bounds__(128) mma_timing_kernel(int tf32, int a_tmem, i
   if (!ok && tid == 0) atomicCAS(status, kDevOk, kDevTimeout);
   tc_fence_before_sync();
   __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, 512);
+  if (warp == 0) {
+    __syncwarp();
+    tmem_dealloc(tmem, 512);
+  }
 }
 
 // One CTA waits, at most `spin_limit` polls, on an mbarrier in its own shared memory that nothing ever arrives at

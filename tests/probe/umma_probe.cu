@@ -225,7 +225,10 @@ __global__ void __launch_bounds__(128) umma_probe_kernel(int mode, const __nv_bf
   if (!ok && tid == 0) atomicCAS(status, kDevOk, kDevTimeout);
   tc_fence_before_sync();
   __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, 256);
+  if (warp == 0) {
+    __syncwarp();
+    tmem_dealloc(tmem, 256);
+  }
 }
 
 }  // namespace
