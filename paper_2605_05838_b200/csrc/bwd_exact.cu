@@ -67,8 +67,8 @@ __global__ void __launch_bounds__(kChainThreads<NV>, 1) adj_chain_kernel(const A
   const int H = a.g.H, DV = a.dv, NVB = DV / NV;
   const int vb = blockIdx.x % NVB, h = (blockIdx.x / NVB) % H, seq = blockIdx.x / (NVB * H);
   const int j0 = vb * NV;
-  grid_launch_dependents();
   grid_dependency_wait();
+  grid_launch_dependents();
   const SeqInfo sq = seq_info(a.g, seq);
   const size_t st_off = ((size_t)seq * H + h) * DK * DV;
   const size_t es = a.in_bf16 ? 2 : 4;
@@ -215,8 +215,8 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
   auto V = [&](int which) { return vec + which * C; };
 
   const int H = a.g.H, slot = blockIdx.x / H, h = blockIdx.x % H;
-  grid_launch_dependents();
   grid_dependency_wait();
+  grid_launch_dependents();
   const SlotInfo si = slot_info(a.g, slot);
   if (si.seq < 0) return;
   const int n = si.n;

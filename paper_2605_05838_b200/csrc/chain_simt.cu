@@ -69,8 +69,8 @@ __global__ void __launch_bounds__(kChainThreads<NV>, 1) chain_simt_kernel(const 
   const int H = a.g.H, DV = a.dv, NVB = DV / NV;
   const int vb = blockIdx.x % NVB, h = (blockIdx.x / NVB) % H, seq = blockIdx.x / (NVB * H);
   const int j0 = vb * NV;
-  grid_launch_dependents();
   grid_dependency_wait();
+  grid_launch_dependents();
   const SeqInfo sq = seq_info(a.g, seq);
   const size_t st_off = ((size_t)seq * H + h) * DK * DV;
   const size_t es = a.in_bf16 ? 2 : 4;

@@ -51,8 +51,8 @@ __global__ void __launch_bounds__(kSimtThreads, 2) intra_simt_kernel(const Intra
   using L = IntraSmem<DK>;
   constexpr int LDK = L::LDK, LP = 36;
   const int H = a.g.H, slot = blockIdx.x / H, h = blockIdx.x % H;
-  grid_launch_dependents();
   grid_dependency_wait();
+  grid_launch_dependents();
   if (a.clear_status != nullptr && blockIdx.x == 0 && threadIdx.x < 4) a.clear_status[threadIdx.x] = 0;
   const SlotInfo si = slot_info(a.g, slot);
   if (si.seq < 0) return;

@@ -101,7 +101,9 @@ __global__ void __launch_bounds__(256) out_norm_gate_kernel(size_t rows, OutPost
   for (int e = 0; e < E; ++e) wv[e] = post.w ? __ldg(post.w + l * E + e) : 1.f;
   const size_t warps = (size_t)gridDim.x * (blockDim.x >> 5);
   const size_t warp_id = (size_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  bool first = true;   // o comes from the previous kernel, which may still be running (g and w are the call's inputs)
+  // o comes from the previous kernel, which may still be running; g and w are the call's inputs, complete before that kernel
+  // let this one in (launch_pdl)
+  bool first = true;
   for (size_t row0 = warp_id * (RPW * R); row0 < rows || first; row0 += warps * (RPW * R)) {
     Pack<TO, E> op[R];
     Pack<TG, E> gp[R];

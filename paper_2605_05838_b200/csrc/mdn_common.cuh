@@ -133,7 +133,9 @@ template <typename... A> inline cudaError_t allow_smem(void (*kern)(A...), int b
 }
 
 // Launch `kern` so that its prologue may overlap the tail of the previous kernel in the stream; the kernel
-// itself calls grid_dependency_wait() before it touches anything the previous kernel wrote.
+// itself calls grid_dependency_wait() before it touches anything the previous kernel wrote.  No kernel lets its dependents in
+// before its own wait is over: so whatever was complete when the PREVIOUS kernel began its work (a call's inputs, whoever
+// made them and however early that kernel let its dependents in) is complete here before the wait, and may be read there.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                               Args&&... args) {

@@ -123,3 +123,27 @@ def test_both_autograd_nodes_give_the_same_bits(mdn, packed, state, eta):
             assert (x - y).abs().max() <= 1e-4 * y.abs().max(), n
         else:
             assert torch.equal(x, y), n
+
+
+@pytest.mark.parametrize("T,H,dtype", [(64, 1, "float32"), (1, 4, "float32"), (3000, 8, "float32"), (1, 64, "bfloat16")])
+def test_output_gate_made_by_the_call_before(mdn, T, H, dtype):
+    """The output step's gate is what the call just before wrote on the same stream (its last kernel lets the next ones in before it
+    stores): the same bits as with a synchronisation between the two.  T = 1: also through decode_step."""
+    import torch
+    dt = getattr(torch, dtype)
+    g = torch.Generator(device="cuda").manual_seed(T)
+    r = lambda *s: torch.randn(s, device="cuda", generator=g)
+    q, k, v = (x.to(dt) for x in (0.1 * r(2, T, H, 64), 0.1 * r(2, T, H, 64), r(2, T, H, 64)))
+    gates = (0.1 * r(2, T, H).abs(), -r(2, T, H).abs(), -0.1 * r(2, T, H).abs(), 1 + 0.1 * r(2, T, H))
+    step = lambda gate: mdn.make_layer_ops(q, v, out_norm_gate=dict(g=gate, eps=1e-5))
+    S = r(2, H, 64, 64)
+    calls = [lambda gate: mdn.chunk_fwd(q, k, v, *gates, layer_ops=step(gate))[0]]
+    if T == 1:
+        calls.append(lambda gate: mdn.decode_step(q, k, v, *gates, S.clone(), S.clone(), layer_ops=step(gate)))
+    for call in calls:
+        first = call(v)
+        torch.cuda.synchronize()
+        want = call(first)
+        torch.cuda.synchronize()
+        for _ in range(50):
+            assert torch.equal(call(call(v)), want)

@@ -36,3 +36,27 @@ def unsynced_tensor_memory_access(lines):
 @pytest.mark.parametrize("path", [p for p in SOURCES + PROBES if "tmem_dealloc(" in open(p).read()], ids=os.path.basename)
 def test_warps_reconverge_before_tensor_memory_instructions(path):
     assert unsynced_tensor_memory_access(code_lines(path)) == []
+
+
+def kernels(lines):
+    """The lines of every __global__ function: (name, lines)."""
+    out = []
+    for no, text in lines:
+        if "__global__" in text:
+            out.append([None, []])
+        if out:
+            out[-1][1].append((no, text))
+            m = re.search(r"\b(\w+_kernel)\(", text)
+            if out[-1][0] is None and m:
+                out[-1][0] = m.group(1)
+    return out
+
+
+@pytest.mark.parametrize("path", SOURCES, ids=os.path.basename)
+def test_no_kernel_lets_its_dependents_in_before_its_own_wait(path):
+    """Kernels that are let in early read the call's inputs before their wait: that needs every kernel in front of them to
+    have waited for its own predecessor first."""
+    for name, lines in kernels(code_lines(path)):
+        calls = [(m.group(0), no) for no, t in lines for m in re.finditer(r"grid_(dependency_wait|launch_dependents)(?=\(\))", t)]
+        if any(c == "grid_launch_dependents" for c, _ in calls):
+            assert calls[0][0] == "grid_dependency_wait", (name, calls)
