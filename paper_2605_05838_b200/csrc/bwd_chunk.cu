@@ -127,8 +127,6 @@ cudaError_t launch_bwd_ext_cu(const Plan& fwd, int32_t* cu_ext, int* launches) {
   return cudaGetLastError();
 }
 
-size_t bwd_prep_smem_bytes() { return (size_t)2 * C * L6 * 2 + (size_t)C * LT * 2; }
-
 cudaError_t launch_bwd_prep(const Plan& fwd, const void* d_o, void* v_ext, float* coef_ext, int* launches) {
   PrepArgs a;
   a.g = fwd.geom;
@@ -139,8 +137,8 @@ cudaError_t launch_bwd_prep(const Plan& fwd, const void* d_o, void* v_ext, float
   a.scale = fwd.p.scale;
   a.v_ext = static_cast<__nv_bfloat16*>(v_ext);
   a.coef_ext = coef_ext;
-  const size_t smem = bwd_prep_smem_bytes();
-  cudaError_t e = allow_smem(bwd_prep_kernel, (int)smem);
+  constexpr size_t smem = (size_t)2 * C * L6 * 2 + (size_t)C * LT * 2;
+  cudaError_t e = allow_smem<(int)smem>(bwd_prep_kernel);
   if (e != cudaSuccess) return e;
   bwd_prep_kernel<<<dim3((unsigned)fwd.geom.num_slots * fwd.p.H), dim3(kPrepThreads), smem, fwd.stream>>>(a);
   e = cudaGetLastError();

@@ -533,7 +533,7 @@ cudaError_t launch_bwd_chunk_tc(const Plan& fwd, const void* q, const void* k, c
   a.wide = ((reinterpret_cast<uintptr_t>(dq) | reinterpret_cast<uintptr_t>(dk)) & 31) == 0;
   a.gates = GateOut{dbeta, dlog_alpha, dlog_mu, deta};
   auto launch = [&](auto kern) -> cudaError_t {
-    cudaError_t e = allow_smem(kern, (int)kSmem);
+    cudaError_t e = allow_smem<(int)kSmem>(kern);
     if (e != cudaSuccess) return e;
     e = launch_pdl(kern, dim3((unsigned)fwd.geom.num_slots * fwd.p.H), dim3(kThreads), kSmem, fwd.stream, a, mq, mk, mdo, mdr, mvt);
     if (e == cudaSuccess) ++*launches;

@@ -484,14 +484,14 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
 
 template <int DK, int NV> cudaError_t launch_adj(const Plan& pl, const AdjArgs& a) {
   const size_t smem = AdjSmem<DK, NV>::bytes(a.in_bf16);
-  const cudaError_t e = allow_smem(adj_chain_kernel<DK, NV>, (int)smem);
+  const cudaError_t e = allow_smem<(int)AdjSmem<DK, NV>::bytes(true)>(adj_chain_kernel<DK, NV>);
   if (e != cudaSuccess) return e;
   return launch_pdl(adj_chain_kernel<DK, NV>, dim3((unsigned)pl.geom.num_seqs * pl.p.H * (a.dv / NV)), dim3(kChainThreads<NV>), smem,
                     pl.stream, a);
 }
 template <int DK, int DV> cudaError_t launch_par(const Plan& pl, const ParArgs& a) {
   constexpr size_t smem = (size_t)ParSmem<DK, DV>::kFloats * 4;
-  const cudaError_t e = allow_smem(bwd_exact_par_kernel<DK, DV>, (int)smem);
+  const cudaError_t e = allow_smem<(int)smem>(bwd_exact_par_kernel<DK, DV>);
   if (e != cudaSuccess) return e;
   return launch_pdl(bwd_exact_par_kernel<DK, DV>, dim3((unsigned)pl.geom.num_slots * pl.p.H), dim3(kSimtThreads), smem, pl.stream, a);
 }

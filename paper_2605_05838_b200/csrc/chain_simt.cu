@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(kChainThreads<NV>, 1) chain_simt_kernel(const 
 template <int DK, int NV, bool kOut> cudaError_t launch_one(const Plan& pl, const ChainArgs& a) {
   const size_t smem = ChainSmem<DK, NV>::bytes(kOut, a.in_bf16);
   auto kern = chain_simt_kernel<DK, NV, kOut>;
-  const cudaError_t e = allow_smem(kern, (int)smem);
+  const cudaError_t e = allow_smem<(int)ChainSmem<DK, NV>::bytes(kOut, true)>(kern);
   if (e != cudaSuccess) return e;
   const unsigned grid = (unsigned)pl.geom.num_seqs * pl.p.H * (a.dv / NV);
   return launch_pdl(kern, dim3(grid), dim3(kChainThreads<NV>), smem, pl.stream, a);

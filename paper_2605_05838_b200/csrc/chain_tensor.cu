@@ -812,7 +812,7 @@ cudaError_t launch_chain_tensor(const Plan& pl, const void* q, const void* k, co
   const unsigned chains = (unsigned)pl.geom.num_seqs * p.H;
   const bool layer = pl.qk.on || pl.post.on;
   auto launch_as = [&](auto kern, unsigned grid) -> cudaError_t {
-    cudaError_t e = allow_smem(kern, (int)kSmemBytes);
+    cudaError_t e = allow_smem<(int)kSmemBytes>(kern);
     if (e != cudaSuccess) return e;
     e = launch_pdl(kern, dim3(grid), dim3(kThreads), kSmemBytes, pl.stream, a, mq, mk, mv, mt, mw, mo);
     if (e == cudaSuccess) e = cudaGetLastError();

@@ -1007,7 +1007,7 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
   auto launch = [&](unsigned grid) -> cudaError_t {
     auto kern = layer ? (o_bf16 ? chain_tf32_kernel<__nv_bfloat16, true> : chain_tf32_kernel<float, true>)
                       : (o_bf16 ? chain_tf32_kernel<__nv_bfloat16, false> : chain_tf32_kernel<float, false>);
-    cudaError_t e = allow_smem(kern, (int)kSmemBytes);
+    cudaError_t e = allow_smem<(int)kSmemBytes>(kern);
     if (e != cudaSuccess) return e;
     e = launch_pdl(kern, dim3(grid), dim3(threads_of(layer)), kSmemBytes, pl.stream, a, mq, mk, mv, mt, mw, mo);
     if (e == cudaSuccess) e = cudaGetLastError();

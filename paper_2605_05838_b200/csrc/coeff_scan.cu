@@ -174,7 +174,7 @@ cudaError_t launch_coeff_scan(const Plan& pl, const float* beta, const float* lo
                               const float* eta, int* launches) {
   const size_t smem = (size_t)4 * C * pl.p.H * sizeof(float);
   if (smem > 48 * 1024) {
-    cudaError_t e = allow_smem(coeff_scan_kernel, (int)smem);
+    cudaError_t e = allow_smem<kSmemOptin>(coeff_scan_kernel);
     if (e != cudaSuccess) return e;
   }
   coeff_scan_kernel<<<pl.geom.num_slots, kScanWarps * 32, smem, pl.stream>>>(

@@ -573,7 +573,7 @@ template <bool kQk, bool kWf32>
 static cudaError_t launch_intra_variant(const Plan& pl, const CUtensorMap& mq, const CUtensorMap& mk, const GateArgs& gates,
                                         size_t n_mats) {
   constexpr uint32_t smem_bytes = lay_of(kQk).smem;
-  cudaError_t e = allow_smem(intra_mma_kernel<kQk, kWf32>, (int)smem_bytes);
+  cudaError_t e = allow_smem<(int)smem_bytes>(intra_mma_kernel<kQk, kWf32>);
   if (e != cudaSuccess) return e;
   return launch_pdl(intra_mma_kernel<kQk, kWf32>, dim3((unsigned)n_mats), dim3(kThreads), smem_bytes, pl.stream, pl.geom, mq, mk,
                     reinterpret_cast<float*>(pl.ws + pl.lay.off_coef), gates, pl.gp, pl.qk, pl.p.scale,

@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kSimtThreads, 2) intra_simt_kernel(const Intra
 
 template <int DK> cudaError_t launch_one(const Plan& pl, const IntraArgs& a) {
   const size_t smem = IntraSmem<DK>::bytes(a.in_bf16, a.bwd.TT ? a.dv : 0);
-  const cudaError_t e = allow_smem(intra_simt_kernel<DK>, (int)smem);
+  const cudaError_t e = allow_smem<(int)IntraSmem<DK>::bytes(true, 128)>(intra_simt_kernel<DK>);
   if (e != cudaSuccess) return e;
   return launch_pdl(intra_simt_kernel<DK>, dim3((unsigned)pl.geom.num_slots * pl.p.H), dim3(kSimtThreads), smem, pl.stream, a);
 }

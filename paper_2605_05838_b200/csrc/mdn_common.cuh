@@ -5,8 +5,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <atomic>
-
 #include "layer_ops.cuh"
 #include "mdn.h"
 
@@ -107,29 +105,13 @@ __device__ __forceinline__ int2 seg_chunks(const ChunkGeom& g, int nchunks, cons
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// cudaFuncSetAttribute(kern, MaxDynamicSharedMemorySize, bytes), once per kernel and device: the call takes as long as a third of
-// a launch, and the smallest calls are bound by the host.  Kernels of all .cu files share the table; safe with several
-// threads (two of them may both make the call).
-inline cudaError_t allow_smem(const void* kern, int bytes) {
-  constexpr int kSlots = 128, kDevices = 16;
-  struct Slot { std::atomic<const void*> kern{nullptr}; std::atomic<int> bytes[kDevices]{}; };
-  static Slot table[kSlots];
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices)
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  for (int i = 0, at = (int)((reinterpret_cast<uintptr_t>(kern) >> 4) % kSlots); i < kSlots; ++i, at = (at + 1) % kSlots) {
-    const void* seen = nullptr;
-    Slot& s = table[at];
-    if (!s.kern.compare_exchange_strong(seen, kern) && seen != kern) continue;
-    if (s.bytes[dev].load(std::memory_order_acquire) >= bytes) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) s.bytes[dev].store(bytes, std::memory_order_release);
-    return e;
-  }
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-}
-template <typename... A> inline cudaError_t allow_smem(void (*kern)(A...), int bytes) {
-  return allow_smem(reinterpret_cast<const void*>(kern), bytes);
+// Lets `kern` be launched with up to kBytes of dynamic shared memory.  Made before every launch (60 ns): the limit belongs to
+// the kernel in the current context, which a device reset takes away.  kBytes is a constant, the most that any launch of that
+// kernel asks for: threads that launch it with different sizes at the same time set the same limit.
+constexpr int kSmemOptin = 232448;   // the most a block can have
+template <int kBytes, typename... A> inline cudaError_t allow_smem(void (*kern)(A...)) {
+  static_assert(kBytes <= kSmemOptin, "shared memory");
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
 }
 
 // Launch `kern` so that its prologue may overlap the tail of the previous kernel in the stream; the kernel

@@ -107,7 +107,7 @@ cudaError_t launch_seg_combine(const Plan& pl, int G, float* E, const float* Psi
   const unsigned chains = (unsigned)pl.geom.num_seqs * pl.p.H;
   auto run = [&](auto cols) -> cudaError_t {
     constexpr int kCols = decltype(cols)::value;
-    cudaError_t e = allow_smem(seg_combine_kernel<kCols>, (int)kSmem<kCols>);
+    cudaError_t e = allow_smem<(int)kSmem<kCols>>(seg_combine_kernel<kCols>);
     if (e != cudaSuccess) return e;
     return launch_pdl(seg_combine_kernel<kCols>, dim3(chains, kD / kCols), dim3(kSimtThreads), kSmem<kCols>, pl.stream, G, E, Psi, PhiS,
                       PhiM);

@@ -2,6 +2,10 @@
 Python binding raises its own error, and gives the Python binding's results otherwise.  An int `scale` is one of the
 arguments it declines: the same value as int and as float takes the two routes."""
 import ctypes
+import os
+import subprocess
+import sys
+import threading
 
 import pytest
 import torch
@@ -56,3 +60,36 @@ def test_both_routes_give_the_same_bits(dtype, dk, dv, T):
     assert g1.keys() == g2.keys() and torch.equal(g1["dv"], g2["dv"]) and torch.equal(g1["d_initial_S"], g2["d_initial_S"])
     with pytest.raises(mdn.MdnError):
         mdn.chunk_fwd(*a, scale=1.0, segments=2)
+
+
+@pytest.mark.gpu
+def test_kernels_run_after_a_device_reset():
+    """The kernels' shared-memory limits are gone with the old context and set anew."""
+    child = os.path.join(os.path.dirname(os.path.abspath(__file__)), "probe", "reset_child.py")
+    r = subprocess.run([sys.executable, child], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and r.stdout.strip() == "[0, 0, 0, 0]", r.stdout + r.stderr
+
+
+@pytest.mark.gpu
+def test_threads_that_launch_one_kernel_with_different_sizes():
+    """The fp32 kernels take more shared memory for bf16 input and wider values: threads that use both at the same time."""
+    errors = []
+
+    def work(dtype, dv, stream):
+        try:
+            with torch.cuda.stream(stream):
+                a = args(1, 70, 2, 128, dv, dtype, "cuda")
+                want = mdn.chunk_fwd(*a, path="simt")[0]
+                for _ in range(200):
+                    assert torch.equal(mdn.chunk_fwd(*a, path="simt")[0], want)
+                    mdn.chunk_bwd(*a, a[2])
+                stream.synchronize()
+        except Exception as e:   # handed to the test's thread
+            errors.append(e)
+    threads = [threading.Thread(target=work, args=(dt, dv, torch.cuda.Stream()))
+               for dt in (torch.float32, torch.bfloat16) for dv in (64, 128)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
