@@ -76,6 +76,7 @@ def _load_native():
     if _nat is None:
         lib()
         from . import _native
+        _native.set_error_class(MdnError)
         _nat = _native
     return _nat
 

@@ -16,6 +16,7 @@
 #include <c10/cuda/CUDAFunctions.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Dtype.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/custom_function.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -150,13 +151,13 @@ bool parse_ops(PyObject* obj, const mdn_layer_ops** ops) {
   return !PyErr_Occurred();
 }
 
+// C++ exceptions as torch's own functions hand them on: out of memory, ValueError and so on as those types, and what Python code
+// raised underneath (saved-tensor hooks, which activation checkpointing leaves by an exception) as itself.
 #define NATIVE_TRY try {
-#define NATIVE_CATCH                                        \
-  } catch (const c10::OutOfMemoryError&) {                  \
-    return Py_NewRef(Py_None); /* the Python code raises */ \
-  } catch (const std::exception& e) {                       \
-    PyErr_SetString(PyExc_RuntimeError, e.what());          \
-    return nullptr;                                         \
+#define NATIVE_CATCH                                                 \
+  } catch (const std::exception&) {                                  \
+    torch::translate_exception_to_python(std::current_exception());  \
+    return nullptr;                                                  \
   }
 
 // decode_step(q, k, v, beta, log_alpha, log_mu, eta, S, M, scale, o_dtype, out, ops) -> o
@@ -329,6 +330,32 @@ PyObject* chunk_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   NATIVE_CATCH
 }
 
+PyObject* mdn_error = nullptr;   // binding.py's MdnError, set when it loads this module
+
+// set_error_class(MdnError)
+PyObject* set_error_class(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  if (n != 1) { PyErr_SetString(PyExc_TypeError, "set_error_class(class)"); return nullptr; }
+  Py_XDECREF(mdn_error);
+  mdn_error = Py_NewRef(a[0]);
+  return Py_NewRef(Py_None);
+}
+
+// Throws MdnError(status, where) for a failed call: it arrives as that in Python, from autograd's threads too.  The GIL need not
+// be held.
+void check(mdn_status st, const char* where) {
+  if (st == MDN_OK) return;
+  const PyGILState_STATE gil = PyGILState_Ensure();
+  PyObject* e = PyObject_CallFunction(mdn_error, "is", (int)st, where);
+  if (e) {
+    PyErr_SetObject(mdn_error, e);
+    Py_DECREF(e);
+  }
+  python_error err;
+  err.persist();
+  PyGILState_Release(gil);
+  throw err;
+}
+
 // ---- chunk_attention: the differentiable forward.  The same two calls as _ChunkAttention of binding.py, as a C++ autograd
 // node: a training step of a few hundred tokens takes 55 us on the GPU, and the Python node (apply, saved tensors, the
 // engine's way back into Python) made it 138 us.
@@ -342,10 +369,6 @@ class ChunkAttention : public torch::autograd::Function<ChunkAttention> {
     return mdn_params{(int32_t)q.size(0), (int32_t)q.size(1), (int32_t)q.size(2), (int32_t)q.size(3), (int32_t)v.size(3), 64, (int32_t)N,
                       MDN_BF16, MDN_BF16, MDN_PATH_TENSOR, (float)scale, 0};
   }
-  static void check(mdn_status st, const char* where) {
-    TORCH_CHECK(st == MDN_OK, where, ": ", mdn_status_string(st), " (status ", (int)st, ")",
-                st == MDN_ERR_CUDA ? std::string(": ") + mdn_last_cuda_error_string() : std::string());
-  }
 
  public:
   static torch::autograd::variable_list forward(torch::autograd::AutogradContext* ctx, const Tensor& q, const Tensor& k, const Tensor& v,
@@ -358,7 +381,7 @@ class ChunkAttention : public torch::autograd::Function<ChunkAttention> {
     const c10::DeviceIndex dev = q.get_device();
     const int64_t n = p.num_seqs > 0 ? p.num_seqs : p.B;
     const size_t need = mdn_chunk_fwd_workspace_bytes(&p), state_bytes = mdn_chunk_states_bytes(&p);
-    TORCH_CHECK(need != 0 && state_bytes != 0, "mdn_chunk_states_bytes: ", mdn_status_string(MDN_ERR_UNSUPPORTED), " (status 2)");
+    check(need != 0 && state_bytes != 0 ? MDN_OK : MDN_ERR_UNSUPPORTED, "mdn_chunk_fwd_workspace_bytes");
     Tensor ws = empty({(int64_t)need}, at::kByte, dev), states = empty_1024((int64_t)state_bytes, dev);
     Tensor o = empty(v.sizes(), q.scalar_type(), dev);
     Tensor Sf = empty({n, p.H, p.dk, p.dv}, at::kFloat, dev), Mf = empty({n, p.H, p.dk, p.dv}, at::kFloat, dev);
@@ -500,6 +523,7 @@ PyMethodDef methods[] = {
     {"chunk_fwd", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(chunk_fwd)), METH_FASTCALL, nullptr},
     {"chunk_bwd", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(chunk_bwd)), METH_FASTCALL, nullptr},
     {"chunk_attention", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(chunk_attention)), METH_FASTCALL, nullptr},
+    {"set_error_class", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(set_error_class)), METH_FASTCALL, nullptr},
     {"fill_layer_ops", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(fill_layer_ops)), METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 

@@ -93,3 +93,61 @@ def test_threads_that_launch_one_kernel_with_different_sizes():
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+def misaligned(t):
+    """The same values in a contiguous tensor that starts two bytes behind a 16-byte boundary."""
+    buf = torch.empty(t.numel() + 8, dtype=t.dtype, device=t.device)
+    m = buf[1:1 + t.numel()].view(t.shape)
+    return m.copy_(t)
+
+
+def attention_args(T=100):
+    return [t.requires_grad_() for t in args(1, T, 2, 128, 128, torch.bfloat16, "cuda")]
+
+
+@pytest.mark.gpu
+def test_a_refused_call_of_the_differentiable_forward_is_an_MdnError():
+    """In the forward (q) and, through the autograd engine's thread, in the backward (d_o)."""
+    a = attention_args()
+    with pytest.raises(mdn.MdnError) as e:
+        mdn.chunk_attention(misaligned(a[0].detach()), *a[1:])
+    assert e.value.status == 1
+    o, _, _ = mdn.chunk_attention(*a)
+    with pytest.raises(mdn.MdnError) as e:
+        torch.autograd.grad(o, a, misaligned(torch.ones_like(o)))
+    assert e.value.status == 1
+
+
+@pytest.mark.gpu
+def test_exceptions_of_saved_tensor_hooks_pass_through():
+    class Mine(Exception):
+        pass
+
+    def fail(_):
+        raise Mine("hook")
+    a = attention_args()
+    with pytest.raises(Mine), torch.autograd.graph.saved_tensors_hooks(fail, lambda x: x):
+        mdn.chunk_attention(*a)
+    with torch.autograd.graph.saved_tensors_hooks(lambda x: x, fail):
+        o, _, _ = mdn.chunk_attention(*a)
+    with pytest.raises(Mine):
+        o.float().sum().backward()
+
+
+def grads_of(run, a):
+    o, S, _ = run(*a)
+    return torch.autograd.grad(o.float().square().sum() + S.square().sum(), a)
+
+
+def same_gradients(x, y):   # (gate gradients: sums by atomics, last bits may differ)
+    return all(torch.equal(u, w) if u.dtype == torch.bfloat16 else (u - w).abs().max() <= 1e-4 * w.abs().max() for u, w in zip(x, y))
+
+
+@pytest.mark.gpu
+def test_activation_checkpointing():
+    """The recomputation ends with an exception out of the last saved tensor's hook, which the checkpoint catches."""
+    from torch.utils.checkpoint import checkpoint
+    a = attention_args()
+    want = grads_of(mdn.chunk_attention, a)
+    assert same_gradients(grads_of(lambda *x: checkpoint(mdn.chunk_attention, *x, use_reentrant=False), a), want)
