@@ -369,6 +369,18 @@ class ChunkAttention : public torch::autograd::Function<ChunkAttention> {
     return mdn_params{(int32_t)q.size(0), (int32_t)q.size(1), (int32_t)q.size(2), (int32_t)q.size(3), (int32_t)v.size(3), 64, (int32_t)N,
                       MDN_BF16, MDN_BF16, MDN_PATH_TENSOR, (float)scale, 0};
   }
+  // A saved tensor as it was handed to save_for_backward: hooks may have brought back something else.
+  static const Tensor& same(const Tensor& t, at::ScalarType dtype, c10::DeviceIndex dev, at::IntArrayRef shape) {
+    TORCH_CHECK_VALUE(!t.defined() || (t.is_cuda() && t.get_device() == dev && t.scalar_type() == dtype && t.is_contiguous() && t.sizes() == shape),
+                      "a tensor saved for chunk_attention's backward came back with another device, type, shape or stride");
+    return t;
+  }
+  // A byte buffer of the forward on the boundary that it needs (copied there where hooks have moved it).
+  static Tensor buffer(const Tensor& t, int64_t bytes, c10::DeviceIndex dev) {
+    same(t, at::kByte, dev, {bytes});
+    if (reinterpret_cast<uintptr_t>(t.const_data_ptr()) % 1024 == 0) return t;
+    return empty_1024(bytes, dev).copy_(t);
+  }
 
  public:
   static torch::autograd::variable_list forward(torch::autograd::AutogradContext* ctx, const Tensor& q, const Tensor& k, const Tensor& v,
@@ -394,15 +406,24 @@ class ChunkAttention : public torch::autograd::Function<ChunkAttention> {
     ctx->set_materialize_grads(false);
     ctx->save_for_backward({q, k, v, beta, log_alpha, log_mu, eta, S0, M0, cu, states, ws});
     ctx->saved_data["scale"] = scale;
+    ctx->saved_data["device"] = (int64_t)dev;
+    ctx->saved_data["qk"] = q.sizes().vec();
+    ctx->saved_data["v"] = v.sizes().vec();
+    ctx->saved_data["seqs"] = (int64_t)p.num_seqs;
     return {o, Sf, Mf};
   }
 
   static torch::autograd::variable_list backward(torch::autograd::AutogradContext* ctx, torch::autograd::variable_list grads) {
     const auto s = ctx->get_saved_variables();
-    const Tensor &q = s[0], &k = s[1], &v = s[2], &eta = s[6], &S0 = s[7], &M0 = s[8], &cu = s[9], &states = s[10], &ws = s[11];
+    const c10::DeviceIndex dev = (c10::DeviceIndex)ctx->saved_data["device"].toInt();
+    const auto qk_shape = ctx->saved_data["qk"].toIntVector(), v_shape = ctx->saved_data["v"].toIntVector();
+    const Tensor &q = same(s[0], at::kBFloat16, dev, qk_shape), &k = same(s[1], at::kBFloat16, dev, qk_shape);
+    const Tensor &v = same(s[2], at::kBFloat16, dev, v_shape), &cu = same(s[9], at::kInt, dev, {ctx->saved_data["seqs"].toInt() + 1});
+    for (int i = 3; i < 7; ++i) same(s[i], at::kFloat, dev, {qk_shape[0], qk_shape[1], qk_shape[2]});
+    const Tensor &eta = s[6], &S0 = s[7], &M0 = s[8];
     const mdn_params p = params(q, v, cu, ctx->saved_data["scale"].toDouble());
-    const c10::DeviceIndex dev = q.get_device();
     const int64_t n = p.num_seqs > 0 ? p.num_seqs : p.B;
+    const Tensor states = buffer(s[10], (int64_t)mdn_chunk_states_bytes(&p), dev), ws = buffer(s[11], (int64_t)mdn_chunk_fwd_workspace_bytes(&p), dev);
     const Tensor d_o = grads[0].defined() ? grads[0].to(q.scalar_type()).contiguous() : at::zeros_like(v);
     const Tensor dSf = grads[1].defined() ? grads[1].to(at::kFloat).contiguous() : Tensor();
     const Tensor dMf = grads[2].defined() ? grads[2].to(at::kFloat).contiguous() : Tensor();

@@ -151,3 +151,28 @@ def test_activation_checkpointing():
     a = attention_args()
     want = grads_of(mdn.chunk_attention, a)
     assert same_gradients(grads_of(lambda *x: checkpoint(mdn.chunk_attention, *x, use_reentrant=False), a), want)
+
+
+@pytest.mark.gpu
+def test_saved_tensors_that_come_back_elsewhere():
+    """Hooks that keep the saved tensors on the host (or copy them): the kept states need their 1024-byte boundary again.  What comes
+    back in other strides or another type is refused."""
+    a = attention_args()
+    want = grads_of(mdn.chunk_attention, a)
+    with torch.autograd.graph.save_on_cpu(pin_memory=True):
+        assert same_gradients(grads_of(mdn.chunk_attention, a), want)
+
+    def shifted(t):   # every byte buffer 256 bytes behind a 1024-byte boundary
+        if t.dtype != torch.uint8:
+            return t.clone()
+        buf = torch.empty(t.numel() + 2048, dtype=t.dtype, device=t.device)
+        at = -buf.data_ptr() % 1024 + 256
+        return buf[at:at + t.numel()].copy_(t)
+    with torch.autograd.graph.saved_tensors_hooks(shifted, lambda x: x):
+        assert same_gradients(grads_of(mdn.chunk_attention, a), want)
+    for bad in (lambda t: t.transpose(1, 2).contiguous().transpose(1, 2), lambda t: t.float()):
+        change = lambda t: bad(t) if t.dim() == 4 and t.dtype == torch.bfloat16 else t
+        with torch.autograd.graph.saved_tensors_hooks(change, lambda x: x):
+            o, _, _ = mdn.chunk_attention(*a)
+        with pytest.raises(ValueError):
+            o.float().sum().backward()
