@@ -340,7 +340,8 @@ mdn_status mdn_bwd_state_chain(const mdn_params* p,
  * dk = dv = 128; MDN_ERR_UNSUPPORTED otherwise.  Operands are bf16 / tf32 with fp32 accumulation, so the gradients
  * carry the forward's bf16-level error (see the tests), not mdn_chunk_bwd's fp32 exactness; d_final_S, d_final_M
  * enter the tensor-core products through a bf16 copy (one rounding, up to 2^-8 of their largest element).  deta,
- * d_initial_S, d_initial_M may be NULL.  Workspace: mdn_chunk_bwd_chunked_workspace_bytes(p), 1024-byte aligned.
+ * d_initial_S, d_initial_M may be NULL.  dq, dk: 8-byte aligned (32 is fastest), dv: 16.
+ * Workspace: mdn_chunk_bwd_chunked_workspace_bytes(p), 1024-byte aligned.
  */
 size_t mdn_chunk_bwd_chunked_workspace_bytes(const mdn_params* p);
 
@@ -376,7 +377,7 @@ mdn_status mdn_chunk_bwd_saved(const mdn_params* p,
                                void* workspace, size_t workspace_bytes, void* cuda_stream);
 
 /* mdn_chunk_bwd_saved with dq, dk, dv in the i/o dtype (bf16: each value rounded once from its fp32 sum), which is what an
- * autograd function hands on: saves the fp32 gradients' round trip through memory. */
+ * autograd function hands on: saves the fp32 gradients' round trip through memory.  dq, dk, dv: 16-byte aligned. */
 mdn_status mdn_chunk_bwd_saved_io(const mdn_params* p,
                                   const void* q, const void* k, const void* v,
                                   const float* beta, const float* log_alpha, const float* log_mu, const float* eta,

@@ -54,37 +54,40 @@ struct TcArgs {
   int32_t* status;                                        // the forward workspace's status word
   float scale;
   void* dq; void* dk;
-  bool wide;                                              // dq, dk are 32-byte aligned
+  int align;                                              // of dq, dk: 8, 16 or 32 bytes
   GateOut gates;
 };
 
 // 32 consecutive values of a row to global memory
-template <typename TG> __device__ __forceinline__ void store_row32(TG* dst, const float2 (&x)[16], bool wide);
-__device__ __forceinline__ void st_v8(void* p, const uint32_t (&w)[8], bool wide) {
-  if (wide) {
+template <typename TG> __device__ __forceinline__ void store_row32(TG* dst, const float2 (&x)[16], int align);
+__device__ __forceinline__ void st_v8(void* p, const uint32_t (&w)[8], int align) {
+  if (align == 32) {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]),
                  "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
-  } else {
+  } else if (align == 16) {
     static_cast<uint4*>(p)[0] = make_uint4(w[0], w[1], w[2], w[3]);
     static_cast<uint4*>(p)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) static_cast<uint2*>(p)[i] = make_uint2(w[2 * i], w[2 * i + 1]);
   }
 }
-template <> __device__ __forceinline__ void store_row32<bf16>(bf16* dst, const float2 (&x)[16], bool wide) {
+template <> __device__ __forceinline__ void store_row32<bf16>(bf16* dst, const float2 (&x)[16], int align) {
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     uint32_t w[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) w[e] = pack_bf16(x[8 * i + e].x, x[8 * i + e].y);
-    st_v8(dst + 16 * i, w, wide);
+    st_v8(dst + 16 * i, w, align);
   }
 }
-template <> __device__ __forceinline__ void store_row32<float>(float* dst, const float2 (&x)[16], bool wide) {
+template <> __device__ __forceinline__ void store_row32<float>(float* dst, const float2 (&x)[16], int align) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     uint32_t w[8];
 #pragma unroll
     for (int e = 0; e < 4; ++e) { w[2 * e] = __float_as_uint(x[4 * i + e].x); w[2 * e + 1] = __float_as_uint(x[4 * i + e].y); }
-    st_v8(dst + 8 * i, w, wide);
+    st_v8(dst + 8 * i, w, align);
   }
 }
 
@@ -256,7 +259,7 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
         for (int i = 0; i < 16; ++i) x[i] = __ffma2_rn(make_float2(w, w), f2(z[2 * i], z[2 * i + 1]), f2(acc[2 * i], acc[2 * i + 1]));
       }
       if (out != nullptr) {
-        if (live) store_row32<TG>(out + 32 * c, x, a.wide);
+        if (live) store_row32<TG>(out + 32 * c, x, a.align);
         __syncwarp();
       } else {
         uint32_t y[32];
@@ -466,7 +469,7 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_chunk_tc_kernel(const TcArgs 
         float2 x[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) x[i] = f2(acc[2 * i], acc[2 * i + 1]);
-        if (live) store_row32<TG>(static_cast<TG*>(a.dq) + tok(r) * kD + 64 * hf + 32 * c, x, a.wide);
+        if (live) store_row32<TG>(static_cast<TG*>(a.dq) + tok(r) * kD + 64 * hf + 32 * c, x, a.align);
         __syncwarp();
       }
     }
@@ -530,7 +533,9 @@ cudaError_t launch_bwd_chunk_tc(const Plan& fwd, const void* q, const void* k, c
   a.status = reinterpret_cast<int32_t*>(fwd.ws + fwd.lay.off_status);
   a.scale = fwd.p.scale;
   a.dq = dq; a.dk = dk;
-  a.wide = ((reinterpret_cast<uintptr_t>(dq) | reinterpret_cast<uintptr_t>(dk)) & 31) == 0;
+  const uintptr_t at = reinterpret_cast<uintptr_t>(dq) | reinterpret_cast<uintptr_t>(dk);
+  if (at & 7) return cudaErrorInvalidValue;
+  a.align = at & 15 ? 8 : at & 31 ? 16 : 32;
   a.gates = GateOut{dbeta, dlog_alpha, dlog_mu, deta};
   auto launch = [&](auto kern) -> cudaError_t {
     cudaError_t e = allow_smem<(int)kSmem>(kern);

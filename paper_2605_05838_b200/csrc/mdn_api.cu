@@ -416,7 +416,8 @@ static mdn_status bwd_saved(const mdn_params* p, const void* q, const void* k, c
   if (p->o_dtype != MDN_BF16) return MDN_ERR_UNSUPPORTED;
   if (!q || !k || !v || !d_o || !beta || !log_alpha || !log_mu || !dq || !dk || !dv || !dbeta || !dlog_alpha || !dlog_mu)
     return MDN_ERR_INVALID_ARG;
-  if (!aligned(dq, 16) || !aligned(dk, 16) || !aligned(dv, 16)) return MDN_ERR_INVALID_ARG;
+  const uintptr_t grad_align = io_grads ? 16 : 8;
+  if (!aligned(dq, grad_align) || !aligned(dk, grad_align) || !aligned(dv, 16)) return MDN_ERR_INVALID_ARG;
   if (!fwd_workspace || fwd_workspace_bytes < c.lf.total_bytes || !aligned(fwd_workspace, 256)) return MDN_ERR_WORKSPACE;
   if (!chunk_states || !aligned(chunk_states, 1024)) return MDN_ERR_INVALID_ARG;
   if (!workspace || workspace_bytes < c.total - c.adj_states || !aligned(workspace, 1024)) return MDN_ERR_WORKSPACE;
@@ -465,6 +466,7 @@ mdn_status mdn_chunk_bwd_chunked(const mdn_params* p, const void* q, const void*
   if (p->o_dtype != MDN_BF16) return MDN_ERR_UNSUPPORTED;
   if (!q || !k || !v || !d_o || !beta || !log_alpha || !log_mu || !dq || !dk || !dv || !dbeta || !dlog_alpha || !dlog_mu)
     return MDN_ERR_INVALID_ARG;
+  if (!aligned(dq, 8) || !aligned(dk, 8) || !aligned(dv, 16)) return MDN_ERR_INVALID_ARG;
   if (!workspace || workspace_bytes < c.total || !aligned(workspace, 1024)) return MDN_ERR_WORKSPACE;
   char* w = static_cast<char*>(workspace);
   // 1. the forward's states (no output terms), kept per chunk; T, W and the coefficient vectors stay in ws_fwd

@@ -159,3 +159,19 @@ def test_training_buffer_sizes_and_state_image_unpacking(mdn):
     assert torch.equal(mdn.unpack_chunk_vt(buf, H), vt)
     with pytest.raises(ValueError):
         mdn.unpack_chunk_states(buf[:-4], H)
+
+
+def test_gradient_alignment_is_checked_before_anything_runs(mdn):
+    """The chunk-parallel backward's vector stores: dq, dk on 8 bytes, dv on 16 (no workspace is given: a call that passes the
+    checks is answered with the workspace status)."""
+    p = params(mdn, dk=128, dv=128, io_dtype=1, o_dtype=1)
+    ok = [ctypes.c_void_p(1 << 20)] * 7
+    for which in range(3):
+        for off, status in ((4, 1), (8, 1 if which == 2 else 3), (16, 3)):
+            d = [ctypes.c_void_p((1 << 20) + (off if i == which else 0)) for i in range(3)]
+            st = mdn.lib().mdn_chunk_bwd_chunked(ctypes.byref(p), *ok, None, None, None, ok[0], None, None, *d, *ok[:3], None, None, None,
+                                                 None, 0, None)
+            assert st == status, (which, off, st)
+            st = mdn.lib().mdn_chunk_bwd_saved(ctypes.byref(p), *ok, None, None, 0, ok[0], ok[0], None, None, *d, *ok[:3], None, None, None,
+                                               None, 0, None)
+            assert st == status, (which, off, st)

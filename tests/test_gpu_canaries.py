@@ -108,3 +108,31 @@ def test_fused_layer_operations_stay_inside_their_buffers(mdn, o_bf16):
     assert guards_intact(ws_buf, ws_bytes), "workspace"
     assert guards_intact(o_buf, o_bytes), "o"
     assert torch.isfinite(o.float()).all()
+
+
+@pytest.mark.parametrize("offset", [0, 8, 16])
+def test_chunked_backward_into_gradients_at_narrower_alignments(mdn, offset):
+    """fp32 dq, dk that start 8 (or 16) bytes behind a 32-byte boundary: the same values as on it, nothing around them written."""
+    import torch
+    w = wl.Workload("canary_bwd", B=1, T=100, H=2, dk=128, dv=128, dtype="bf16", seed=51)
+    t = to_torch(wl.make_inputs(w))
+    d_o = torch.randn(t["v"].shape, generator=torch.Generator().manual_seed(1)).to(torch.bfloat16).cuda()
+    names = ("q", "k", "v", "beta", "log_alpha", "log_mu", "eta")
+    want = mdn.chunk_bwd(*(t[n] for n in names), d_o, scale=0.1, method="chunked")
+    p = mdn.make_params(t["q"], t["v"], scale=0.1, o_dtype=torch.bfloat16, path="tensor")
+    vp = lambda x: None if x is None else ctypes.c_void_p(x.data_ptr())
+    need = int(mdn.lib().mdn_chunk_bwd_chunked_workspace_bytes(ctypes.byref(p)))
+    ws = torch.empty(need + 1024, dtype=torch.uint8, device="cuda")
+    ws = ws[-ws.data_ptr() % 1024:]
+    nbytes = t["q"].numel() * 4
+    bufs = [torch.full((nbytes + 2 * GUARD,), PATTERN, dtype=torch.uint8, device="cuda") for _ in range(2)]
+    dq, dk = (ctypes.c_void_p(b.data_ptr() + GUARD + offset) for b in bufs)
+    rest = [torch.empty_like(want[n]) for n in ("dv", "dbeta", "dlog_alpha", "dlog_mu", "deta")]
+    st = mdn.lib().mdn_chunk_bwd_chunked(ctypes.byref(p), *(vp(t[n]) for n in names), None, None, None, vp(d_o), None, None, dq, dk,
+                                         *(vp(x) for x in rest), None, None, vp(ws), need, None)
+    torch.cuda.synchronize()
+    assert st == 0
+    for b, n in zip(bufs, ("dq", "dk")):
+        lo = GUARD + offset
+        assert torch.equal(b[lo:lo + nbytes].clone().view(torch.float32).view(want[n].shape), want[n]), n
+        assert bool((b[:lo] == PATTERN).all()) and bool((b[lo + nbytes:] == PATTERN).all()), n
