@@ -95,8 +95,11 @@ typedef struct {
  */
 
 /* Bytes of device workspace mdn_chunk_fwd needs for these parameters (0 on invalid
- * parameters).  Holds the chunk map, the per-chunk coefficient vectors and the
- * per-chunk T and W matrices; contents are scratch. */
+ * parameters).  Holds the chunk map, the per-chunk coefficient vectors, the
+ * per-chunk T and W matrices and the parallel inter-chunk scan's segment states;
+ * contents are scratch.  The scan makes the size of a shorter call the larger one at
+ * times: with segments = 0, every call with a workspace (or arena) argument also takes one
+ * that suffices for segments = 1, and runs that way. */
 size_t mdn_chunk_fwd_workspace_bytes(const mdn_params* p);
 
 /*

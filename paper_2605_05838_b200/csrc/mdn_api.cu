@@ -63,6 +63,15 @@ static mdn_status make_layout(const mdn_params& p, mdn_ws_layout* lay) {
   return MDN_OK;
 }
 
+// The same call without the parallel inter-chunk scan, whose scratch is the part of a workspace that a SHORTER call can need more of
+// (more segments, or segments at all): a workspace too small for it, but enough without, is taken that way where the caller
+// left the choice open.
+static mdn_params serial(const mdn_params& p) {
+  mdn_params s = p;
+  s.segments = 1;
+  return s;
+}
+
 static mdn_status make_plan(const mdn_params* p, const int32_t* cu, void* ws, size_t ws_bytes, void* stream,
                             Plan* pl) {
   mdn_status st = check_params(p);
@@ -71,6 +80,10 @@ static mdn_status make_plan(const mdn_params* p, const int32_t* cu, void* ws, si
   pl->p = *p;
   pl->p.path = resolve_path(*p);
   st = make_layout(*p, &pl->lay);
+  if (st == MDN_OK && p->segments == 0 && ws_bytes < pl->lay.total_bytes) {
+    pl->p.segments = 1;
+    st = make_layout(pl->p, &pl->lay);
+  }
   if (st != MDN_OK) return st;
   if (!ws || ws_bytes < pl->lay.total_bytes || !aligned(ws, 256)) return MDN_ERR_WORKSPACE;
   pl->ws = static_cast<char*>(ws);
@@ -228,8 +241,7 @@ mdn_status mdn_chunk_fwd_keep_states(const mdn_params* p, const void* q, const v
   Plan pl;
   mdn_status st = make_plan(p, cu_seqlens, workspace, workspace_bytes, cuda_stream, &pl);
   if (st == MDN_ERR_WORKSPACE) {   // without the segment scan's scratch
-    mdn_params ps = *p;
-    ps.segments = 1;
+    const mdn_params ps = serial(*p);
     st = make_plan(&ps, cu_seqlens, workspace, workspace_bytes, cuda_stream, &pl);
   }
   if (st != MDN_OK) return st;
@@ -252,10 +264,8 @@ static mdn_status adj_layout(const mdn_params* p, AdjLayout* a) {
   a->pe = *p;   // (its segments too: the mirrored problem is split by the same rule)
   a->pe.path = MDN_PATH_TENSOR;
   if (p->num_seqs > 0) {   // packed: every chunk slot of the forward, padded to 64 rows (host-side bound)
-    mdn_params pf = *p;
-    pf.segments = 1;
     mdn_ws_layout lf;
-    st = make_layout(pf, &lf);
+    st = make_layout(serial(*p), &lf);
     if (st != MDN_OK) return st;
     a->pe.B = 1;
     a->pe.T = p->chunk * (int)lf.num_slots;
@@ -293,9 +303,9 @@ static mdn_status state_chain(const mdn_params* p, const void* q, const void* k,
   if (!q || !k || !d_o || !adjoint_states || !aligned(adjoint_states, 1024)) return MDN_ERR_INVALID_ARG;
   if (!aligned(q, 16) || !aligned(k, 16) || !aligned(d_o, 16)) return MDN_ERR_INVALID_ARG;
   if (p->o_dtype != MDN_BF16) return MDN_ERR_UNSUPPORTED;   // d_o is read as bf16
+  const mdn_params pf = serial(*p);
+  if (workspace_bytes < al.total) adj_layout(&pf, &al);
   if (!workspace || workspace_bytes < al.total || !aligned(workspace, 1024)) return MDN_ERR_WORKSPACE;
-  mdn_params pf = *p;
-  pf.segments = 1;
   Plan fwd;
   st = make_plan(&pf, cu_seqlens, fwd_workspace, fwd_workspace_bytes, cuda_stream, &fwd);
   if (st != MDN_OK) return st;
@@ -345,9 +355,7 @@ struct ChunkedBwdLayout { AdjLayout al; mdn_ws_layout lf; uint64_t ws_fwd, ws_fw
 static mdn_status chunked_bwd_layout(const mdn_params* p, ChunkedBwdLayout* c) {
   mdn_status st = adj_layout(p, &c->al);
   if (st != MDN_OK) return st;
-  mdn_params pf = *p;
-  pf.segments = 1;
-  st = make_layout(pf, &c->lf);
+  st = make_layout(serial(*p), &c->lf);
   if (st != MDN_OK) return st;
   uint64_t off = 0;
   auto take = [&](uint64_t bytes) { uint64_t at = off; off = align_up(off + bytes, 1024); return at; };
@@ -387,8 +395,7 @@ static mdn_status bwd_from_states(const mdn_params* p, const ChunkedBwdLayout& c
   mdn_status st = state_chain(p, q, k, d_o, d_final_S, d_final_M, cu_seqlens, fwd_ws, c.lf.total_bytes, adj_states, dr,
                               io_grads ? nullptr : static_cast<float*>(dv), d_initial_S, d_initial_M, stage, c.al.total, cuda_stream);
   if (st != MDN_OK) return st;
-  mdn_params pf = *p;
-  pf.segments = 1;
+  const mdn_params pf = serial(*p);
   Plan fwd;
   st = make_plan(&pf, cu_seqlens, fwd_ws, c.lf.total_bytes, cuda_stream, &fwd);
   if (st != MDN_OK) return st;
@@ -420,6 +427,11 @@ static mdn_status bwd_saved(const mdn_params* p, const void* q, const void* k, c
   if (!aligned(dq, grad_align) || !aligned(dk, grad_align) || !aligned(dv, 16)) return MDN_ERR_INVALID_ARG;
   if (!fwd_workspace || fwd_workspace_bytes < c.lf.total_bytes || !aligned(fwd_workspace, 256)) return MDN_ERR_WORKSPACE;
   if (!chunk_states || !aligned(chunk_states, 1024)) return MDN_ERR_INVALID_ARG;
+  const mdn_params ps = serial(*p);
+  if (workspace_bytes < c.total - c.adj_states) {
+    p = &ps;
+    chunked_bwd_layout(p, &c);
+  }
   if (!workspace || workspace_bytes < c.total - c.adj_states || !aligned(workspace, 1024)) return MDN_ERR_WORKSPACE;
   char* w = static_cast<char*>(workspace);   // [adjoint states | stage scratch], as in the full layout from adj_states on
   return bwd_from_states(p, c, q, k, beta, log_alpha, log_mu, eta, cu_seqlens, d_o, d_final_S, d_final_M,
@@ -467,6 +479,11 @@ mdn_status mdn_chunk_bwd_chunked(const mdn_params* p, const void* q, const void*
   if (!q || !k || !v || !d_o || !beta || !log_alpha || !log_mu || !dq || !dk || !dv || !dbeta || !dlog_alpha || !dlog_mu)
     return MDN_ERR_INVALID_ARG;
   if (!aligned(dq, 8) || !aligned(dk, 8) || !aligned(dv, 16)) return MDN_ERR_INVALID_ARG;
+  const mdn_params ps = serial(*p);
+  if (workspace_bytes < c.total) {
+    p = &ps;
+    chunked_bwd_layout(p, &c);
+  }
   if (!workspace || workspace_bytes < c.total || !aligned(workspace, 1024)) return MDN_ERR_WORKSPACE;
   char* w = static_cast<char*>(workspace);
   // 1. the forward's states (no output terms), kept per chunk; T, W and the coefficient vectors stay in ws_fwd
@@ -549,6 +566,12 @@ mdn_status mdn_chunk_fwd_fused(const mdn_params* p, const mdn_layer_ops* ops, co
   if (st != MDN_OK) return st;
   SepLayout sl;
   sep_layout(*p, *ops, pl.lay, &sl);
+  if (workspace_bytes < sl.total && p->segments == 0) {
+    const mdn_params ps = serial(*p);
+    st = make_plan(&ps, cu_seqlens, workspace, workspace_bytes, cuda_stream, &pl);
+    if (st != MDN_OK) return st;
+    sep_layout(ps, *ops, pl.lay, &sl);
+  }
   if (workspace_bytes < sl.total) return MDN_ERR_WORKSPACE;
   if (!q || !k || !aligned(q, 16) || !aligned(k, 16) || !o || !aligned(o, 16)) return MDN_ERR_INVALID_ARG;
   if (ops->raw_gates) {
@@ -774,6 +797,11 @@ mdn_status mdn_chunk_fwd_host(const mdn_params* p, const void* q, const void* k,
                               float* final_S, float* final_M, void* arena, size_t arena_bytes, void* cuda_stream) {
   HostArena a;
   if (!host_arena(p, &a)) return check_params(p) != MDN_OK ? check_params(p) : MDN_ERR_UNSUPPORTED;
+  const mdn_params one_run = serial(*p);
+  if (arena_bytes < a.total && p->segments == 0) {
+    p = &one_run;
+    host_arena(p, &a);
+  }
   if (!arena || arena_bytes < a.total || !aligned(arena, 256)) return MDN_ERR_WORKSPACE;
   if (!q || !k || !v || !beta || !log_alpha || !log_mu || !o) return MDN_ERR_INVALID_ARG;
   if ((p->num_seqs > 0) != (cu_seqlens != nullptr)) return MDN_ERR_INVALID_ARG;

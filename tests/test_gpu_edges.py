@@ -147,3 +147,56 @@ def test_output_gate_made_by_the_call_before(mdn, T, H, dtype):
         torch.cuda.synchronize()
         for _ in range(50):
             assert torch.equal(call(call(v)), want)
+
+
+def test_workspace_enough_for_the_serial_chain(mdn):
+    """A workspace kept for the largest call also serves the shorter ones that the scan would split (and need more for): the result of
+    segments = 1, for every call that takes a workspace."""
+    import ctypes
+    import torch
+    byref = ctypes.byref
+    L = mdn.lib()
+    for lens, B, T, H in ((None, 1, 3000, 2), ([7000, 1900, 100], 1, 9000, 1)):
+        w = wl.Workload("edge_ws", B=B, T=T, H=H, dk=128, dv=128, dtype="bf16", varlen=lens is not None, init_state_std=0.1, seed=3)
+        inp = wl.make_inputs(w, lengths=np.array(lens)) if lens else wl.make_inputs(w)
+        t = to_torch(inp)
+        a = [t[n] for n in ("q", "k", "v", "beta", "log_alpha", "log_mu", "eta")]
+        kw = dict(initial_S=t["initial_S"], initial_M=t["initial_M"], cu_seqlens=t["cu_seqlens"], scale=0.1)
+        N = len(lens) if lens else 0
+        p, p1 = (mdn.make_params(a[0], a[2], num_seqs=N, scale=0.1, segments=s) for s in (0, 1))
+        assert mdn.workspace_layout(p).segments > 1
+        buf = lambda n: torch.empty(int(n) + 1024, dtype=torch.uint8, device="cuda")
+        cut = lambda b, n: b[-b.data_ptr() % 1024:][:int(n)]
+        space = lambda n: cut(buf(n), n)
+        same = lambda x, y: all(torch.equal(u, v) for u, v in zip(x, y))
+        # the forward, alone and with the layer operations as passes of their own
+        ops = mdn.make_layer_ops(a[0], a[2], qk_norm=dict(eps=1e-6), out_norm_gate=dict(g=a[2], eps=1e-5), placement="separate")
+        for lo in (None, ops):
+            one = mdn.chunk_fwd(*a, segments=1, layer_ops=lo, **kw)
+            n = mdn.workspace_bytes(p1) if lo is None else L.mdn_chunk_fwd_fused_workspace_bytes(byref(p1), byref(lo))
+            n0 = mdn.workspace_bytes(p) if lo is None else L.mdn_chunk_fwd_fused_workspace_bytes(byref(p), byref(lo))
+            assert n < n0
+            assert same(mdn.chunk_fwd(*a, workspace=space(n), layer_ops=lo, **kw), one)
+            with pytest.raises(mdn.MdnError):
+                mdn.chunk_fwd(*a, workspace=space(n - 256), layer_ops=lo, **kw)
+            with pytest.raises(mdn.MdnError):
+                mdn.chunk_fwd(*a, workspace=space(n), segments=4, layer_ops=lo, **kw)
+        # host buffers
+        h = {k: (v.cpu().pin_memory() if v is not None else None) for k, v in t.items()}
+        ha = [h[n] for n in ("q", "k", "v", "beta", "log_alpha", "log_mu", "eta")]
+        hkw = dict(initial_S=h["initial_S"], initial_M=h["initial_M"], cu_seqlens=h["cu_seqlens"], scale=0.1)
+        got = mdn.chunk_fwd_host(*ha, arena=space(mdn.host_arena_bytes(p1)), **hkw)
+        assert same([x.cuda() for x in got], mdn.chunk_fwd(*a, segments=1, **kw))
+        # training: the backward with and without kept states
+        d_o = torch.randn(a[2].shape, generator=torch.Generator().manual_seed(2)).to(torch.bfloat16).cuda()
+        st = mdn.chunk_fwd(*a, path="tensor", keep_chunk_states=True, workspace=space(mdn.workspace_bytes(p1)), **kw)
+        want = mdn.chunk_bwd(*a, d_o, method="stepwise", **kw)
+        pb, pb1 = (mdn.make_params(a[0], a[2], num_seqs=N, scale=0.1, path="tensor", segments=s) for s in (0, 1))
+        for saved, size in ((None, L.mdn_chunk_bwd_chunked_workspace_bytes), ((st[4], st[3]), L.mdn_chunk_bwd_saved_workspace_bytes)):
+            assert size(byref(pb1)) < size(byref(pb))
+            got = mdn.chunk_bwd(*a, d_o, method="chunked", saved=saved, workspace=space(size(byref(pb1))), **kw)
+            for n in want:   # (5e-3 in RMS: the tensor-core backward's bound)
+                x, y = got[n].double(), want[n].double()
+                assert (x - y).norm() <= 5e-3 * y.norm(), n
+            with pytest.raises(mdn.MdnError):
+                mdn.chunk_bwd(*a, d_o, method="chunked", saved=saved, workspace=space(size(byref(pb1)) - 1024), **kw)
