@@ -875,8 +875,8 @@ SegSplit choose_segments(const mdn_params& p) {
   constexpr long kSMs = kSegSms;
   const long seqs = p.num_seqs > 0 ? p.num_seqs : p.B, tokens = p.num_seqs > 0 ? p.T / seqs : p.T;
   const long nch = (tokens + C - 1) / C, chains = seqs * p.H;
-  if (p.segments >= 3) {   // forced: equal segments
-    const int per = (int)((nch + p.segments - 1) / p.segments);
+  if (p.segments >= 3) {   // forced: equal segments (at least a chunk: packed input can have fewer tokens than sequences)
+    const int per = nch > 0 ? (int)((nch + p.segments - 1) / p.segments) : 1;
     return SegSplit{p.segments, per, per};
   }
   auto waves = [](long ctas, long sms) { return (ctas + sms - 1) / sms; };

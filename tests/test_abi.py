@@ -175,3 +175,20 @@ def test_gradient_alignment_is_checked_before_anything_runs(mdn):
             st = mdn.lib().mdn_chunk_bwd_saved(ctypes.byref(p), *ok, None, None, 0, ok[0], ok[0], None, None, *d, *ok[:3], None, None, None,
                                                None, 0, None)
             assert st == status, (which, off, st)
+
+
+def test_every_split_of_the_scan_has_chunks(mdn):
+    """Packed sequences are cut in the proportions of the split: one without chunks would be a division by zero in the kernels."""
+    class Split(ctypes.Structure):   # mdn::SegSplit
+        _fields_ = [("G", ctypes.c_int), ("first", ctypes.c_int), ("mid", ctypes.c_int)]
+    choose = getattr(mdn.lib(), "_ZN3mdn15choose_segmentsERK10mdn_params")
+    choose.restype, choose.argtypes = Split, [ctypes.c_void_p]
+    for segments in (0, 3, 32):
+        for B, T, H, seqs in ((1, 1, 1, 2), (1, 5, 2, 300), (1, 64, 1, 64), (1, 100000, 2, 8), (1, 1, 1, 0), (2, 70, 1, 0), (1, 9000, 2, 0)):
+            p = params(mdn, B=B, T=T, H=H, dk=128, dv=128, io_dtype=1, num_seqs=seqs, segments=segments)
+            s = choose(ctypes.addressof(p))
+            assert s.G == mdn.workspace_layout(p).segments and (segments == 0 or s.G == segments)
+            if s.G > 1:
+                assert s.first >= 1 and s.mid >= 1
+                if seqs == 0:
+                    assert s.first + (s.G - 1) * s.mid >= (T + 63) // 64

@@ -200,3 +200,21 @@ def test_workspace_enough_for_the_serial_chain(mdn):
                 assert (x - y).norm() <= 5e-3 * y.norm(), n
             with pytest.raises(mdn.MdnError):
                 mdn.chunk_bwd(*a, d_o, method="chunked", saved=saved, workspace=space(size(byref(pb1)) - 1024), **kw)
+
+
+@pytest.mark.parametrize("lens", [[0, 0, 5, 0], [1, 0, 0, 0, 0], [0, 70, 0]])
+def test_forced_segments_with_fewer_tokens_than_sequences(mdn, lens):
+    """Such sequences stay whole: the serial chain's bits, and an empty one hands its start state on."""
+    import torch
+    N, H, T = len(lens), 2, sum(lens)
+    g = torch.Generator(device="cuda").manual_seed(N)
+    r = lambda *s: torch.randn(s, device="cuda", generator=g)
+    a = [(0.1 * r(1, T, H, 128)).bfloat16(), (0.1 * r(1, T, H, 128)).bfloat16(), r(1, T, H, 128).bfloat16(),
+         0.1 * r(1, T, H).abs(), -r(1, T, H).abs(), -0.1 * r(1, T, H).abs(), 1 + 0.1 * r(1, T, H)]
+    S0, M0 = r(N, H, 128, 128), r(N, H, 128, 128)
+    cu = torch.tensor(np.concatenate([[0], np.cumsum(lens)]), dtype=torch.int32, device="cuda")
+    one, three = (mdn.chunk_fwd(*a, initial_S=S0, initial_M=M0, cu_seqlens=cu, path="tensor", segments=s) for s in (1, 3))
+    assert torch.equal(one[0], three[0])
+    for x, y, z in zip(one[1:], three[1:], (S0, M0)):
+        for n in range(N):
+            assert torch.equal(x[n], y[n]) and (lens[n] > 0 or torch.equal(y[n], z[n])), n
