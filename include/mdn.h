@@ -295,6 +295,20 @@ mdn_status mdn_chunk_fwd_keep_states(const mdn_params* p,
                                      void* chunk_states,
                                      void* workspace, size_t workspace_bytes, void* cuda_stream);
 
+/* The same with the parallel inter-chunk scan's scratch in a buffer of its own: the last total_bytes - off_seg bytes of
+ * mdn_workspace_layout (256-byte aligned; not needed, and may be NULL, where that layout has one segment).  It is free again
+ * when the call has run; `workspace`, which the backward reads, is then off_seg bytes. */
+mdn_status mdn_chunk_fwd_keep_states_scratch(const mdn_params* p,
+                                             const void* q, const void* k, const void* v,
+                                             const float* beta, const float* log_alpha, const float* log_mu,
+                                             const float* eta,
+                                             const float* initial_S, const float* initial_M,
+                                             const int32_t* cu_seqlens,
+                                             void* o, float* final_S, float* final_M,
+                                             void* chunk_states,
+                                             void* workspace, size_t workspace_bytes,
+                                             void* scan_scratch, size_t scan_scratch_bytes, void* cuda_stream);
+
 /*
  * Chunk-parallel backward, stage 1 (Section 3.2 differentiated chunk by chunk): the adjoint of the inter-chunk
  * state recurrence.  With dS', dM' the adjoints of the carried pair at the END of a chunk,

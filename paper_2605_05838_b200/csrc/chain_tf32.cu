@@ -1019,7 +1019,7 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
 
   // ---- parallel inter-chunk scan: Psi / Phi of the middle segments, serial combine, then all segments for real
   constexpr size_t kMat = (size_t)kD * kD;
-  float* seg = reinterpret_cast<float*>(pl.ws + pl.lay.off_seg);
+  float* seg = reinterpret_cast<float*>(pl.seg);
   const SegSplit split = choose_segments(p);
   a.seg_G = G;
   a.seg_first = split.first; a.seg_mid = split.mid; a.seg_least = p.segments ? 1 : kSegLeast;

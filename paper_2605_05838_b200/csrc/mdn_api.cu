@@ -87,6 +87,7 @@ static mdn_status make_plan(const mdn_params* p, const int32_t* cu, void* ws, si
   if (st != MDN_OK) return st;
   if (!ws || ws_bytes < pl->lay.total_bytes || !aligned(ws, 256)) return MDN_ERR_WORKSPACE;
   pl->ws = static_cast<char*>(ws);
+  pl->seg = pl->ws + pl->lay.off_seg;
   pl->stream = static_cast<cudaStream_t>(stream);
   pl->gp = GateParam{};
   pl->qk = QkNorm{};
@@ -228,6 +229,14 @@ size_t mdn_chunk_states_bytes(const mdn_params* p) {
   return (size_t)lay.num_slots * p->H * (kStateImageBytes + kVtSlotBytes);
 }
 
+static mdn_status keep_states(Plan& pl, const void* q, const void* k, const void* v, const float* beta, const float* log_alpha,
+                              const float* log_mu, const float* eta, const float* initial_S, const float* initial_M, void* o,
+                              float* final_S, float* final_M, void* chunk_states) {
+  pl.chain_dump = static_cast<uint8_t*>(chunk_states);
+  pl.chain_vt_dump = reinterpret_cast<float*>(pl.chain_dump + (uint64_t)pl.lay.num_slots * pl.p.H * kStateImageBytes);
+  return run_forward(pl, q, k, v, beta, log_alpha, log_mu, eta, initial_S, initial_M, o, final_S, final_M);
+}
+
 mdn_status mdn_chunk_fwd_keep_states(const mdn_params* p, const void* q, const void* k, const void* v,
                                      const float* beta, const float* log_alpha, const float* log_mu,
                                      const float* eta, const float* initial_S, const float* initial_M,
@@ -245,9 +254,33 @@ mdn_status mdn_chunk_fwd_keep_states(const mdn_params* p, const void* q, const v
     st = make_plan(&ps, cu_seqlens, workspace, workspace_bytes, cuda_stream, &pl);
   }
   if (st != MDN_OK) return st;
-  pl.chain_dump = static_cast<uint8_t*>(chunk_states);
-  pl.chain_vt_dump = reinterpret_cast<float*>(pl.chain_dump + (uint64_t)pl.lay.num_slots * p->H * kStateImageBytes);
-  return run_forward(pl, q, k, v, beta, log_alpha, log_mu, eta, initial_S, initial_M, o, final_S, final_M);
+  return keep_states(pl, q, k, v, beta, log_alpha, log_mu, eta, initial_S, initial_M, o, final_S, final_M, chunk_states);
+}
+
+mdn_status mdn_chunk_fwd_keep_states_scratch(const mdn_params* p, const void* q, const void* k, const void* v,
+                                             const float* beta, const float* log_alpha, const float* log_mu,
+                                             const float* eta, const float* initial_S, const float* initial_M,
+                                             const int32_t* cu_seqlens, void* o, float* final_S, float* final_M,
+                                             void* chunk_states, void* workspace, size_t workspace_bytes,
+                                             void* scan_scratch, size_t scan_scratch_bytes, void* cuda_stream) {
+  t_last_launches = 0;
+  if (check_params(p) != MDN_OK) return check_params(p);
+  if (resolve_path(*p) != MDN_PATH_TENSOR) return MDN_ERR_UNSUPPORTED;
+  if (!chunk_states || !aligned(chunk_states, 1024)) return MDN_ERR_INVALID_ARG;
+  const mdn_params ps = serial(*p);
+  Plan pl;
+  mdn_status st = make_plan(&ps, cu_seqlens, workspace, workspace_bytes, cuda_stream, &pl);
+  if (st != MDN_OK) return st;
+  mdn_ws_layout lay;   // (its parts before the scan's are those of the serial layout)
+  st = make_layout(*p, &lay);
+  if (st != MDN_OK) return st;
+  if (lay.segments > 1) {
+    if (!scan_scratch || scan_scratch_bytes < lay.total_bytes - lay.off_seg || !aligned(scan_scratch, 256)) return MDN_ERR_WORKSPACE;
+    pl.p.segments = p->segments;
+    pl.lay = lay;
+    pl.seg = static_cast<char*>(scan_scratch);
+  }
+  return keep_states(pl, q, k, v, beta, log_alpha, log_mu, eta, initial_S, initial_M, o, final_S, final_M, chunk_states);
 }
 
 // ---- chunk-parallel backward, stage 1: the adjoint of the inter-chunk state recurrence

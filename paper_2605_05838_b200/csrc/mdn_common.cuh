@@ -171,6 +171,7 @@ struct Plan {
   int chain_inject = 0;                  // second update per chunk from q and the tensor passed as o (adjoint chain)
   __nv_bfloat16* chain_dr_bf16 = nullptr;   // mirrored run: dR as bf16 (and fp32) in the original problem's [token][H][dv]
   float* chain_dr_f32 = nullptr;
+  char* seg = nullptr;             // the parallel inter-chunk scan's scratch
   const ChunkGeom* chain_mirror_geom = nullptr;   // q, k, o belong to this geometry, walked in reverse chunk order
   const char* chain_mirror_T = nullptr;           // ... and T ([slot][H][64][64] bf16 of that problem), used transposed
   int cu_total_may_be_short = 0;   // packed: cu[N] <= T instead of == T (the adjoint chain's padded problem)

@@ -392,16 +392,21 @@ class ChunkAttention : public torch::autograd::Function<ChunkAttention> {
     const mdn_params p = params(q, v, cu, scale);
     const c10::DeviceIndex dev = q.get_device();
     const int64_t n = p.num_seqs > 0 ? p.num_seqs : p.B;
-    const size_t need = mdn_chunk_fwd_workspace_bytes(&p), state_bytes = mdn_chunk_states_bytes(&p);
-    check(need != 0 && state_bytes != 0 ? MDN_OK : MDN_ERR_UNSUPPORTED, "mdn_chunk_fwd_workspace_bytes");
-    Tensor ws = empty({(int64_t)need}, at::kByte, dev), states = empty_1024((int64_t)state_bytes, dev);
+    const size_t state_bytes = mdn_chunk_states_bytes(&p);
+    mdn_ws_layout lay;
+    check(state_bytes != 0 ? mdn_workspace_layout(&p, &lay) : MDN_ERR_UNSUPPORTED, "mdn_chunk_fwd_workspace_bytes");
+    // the scan's scratch is given back here: what is kept for the backward lives until then, in every layer
+    const int64_t need = (int64_t)lay.off_seg, scan = (int64_t)(lay.total_bytes - lay.off_seg);
+    Tensor ws = empty({need}, at::kByte, dev), states = empty_1024((int64_t)state_bytes, dev), scratch;
+    if (scan > 0) scratch = empty({scan}, at::kByte, dev);
     Tensor o = empty(v.sizes(), q.scalar_type(), dev);
     Tensor Sf = empty({n, p.H, p.dk, p.dv}, at::kFloat, dev), Mf = empty({n, p.H, p.dk, p.dv}, at::kFloat, dev);
-    check(mdn_chunk_fwd_keep_states(&p, q.const_data_ptr(), k.const_data_ptr(), v.const_data_ptr(), AttnPtrs::f(beta),
-                                    AttnPtrs::f(log_alpha), AttnPtrs::f(log_mu), AttnPtrs::f(eta), AttnPtrs::f(S0), AttnPtrs::f(M0),
-                                    cu.defined() ? static_cast<const int32_t*>(cu.const_data_ptr()) : nullptr, o.data_ptr(),
-                                    static_cast<float*>(Sf.data_ptr()), static_cast<float*>(Mf.data_ptr()), states.data_ptr(),
-                                    ws.data_ptr(), need, stream_of(dev)),
+    check(mdn_chunk_fwd_keep_states_scratch(
+              &p, q.const_data_ptr(), k.const_data_ptr(), v.const_data_ptr(), AttnPtrs::f(beta), AttnPtrs::f(log_alpha),
+              AttnPtrs::f(log_mu), AttnPtrs::f(eta), AttnPtrs::f(S0), AttnPtrs::f(M0),
+              cu.defined() ? static_cast<const int32_t*>(cu.const_data_ptr()) : nullptr, o.data_ptr(), static_cast<float*>(Sf.data_ptr()),
+              static_cast<float*>(Mf.data_ptr()), states.data_ptr(), ws.data_ptr(), (size_t)need, scan > 0 ? scratch.data_ptr() : nullptr,
+              (size_t)scan, stream_of(dev)),
           "mdn_chunk_fwd_keep_states");
     ctx->set_materialize_grads(false);
     ctx->save_for_backward({q, k, v, beta, log_alpha, log_mu, eta, S0, M0, cu, states, ws});
@@ -423,7 +428,9 @@ class ChunkAttention : public torch::autograd::Function<ChunkAttention> {
     const Tensor &eta = s[6], &S0 = s[7], &M0 = s[8];
     const mdn_params p = params(q, v, cu, ctx->saved_data["scale"].toDouble());
     const int64_t n = p.num_seqs > 0 ? p.num_seqs : p.B;
-    const Tensor states = buffer(s[10], (int64_t)mdn_chunk_states_bytes(&p), dev), ws = buffer(s[11], (int64_t)mdn_chunk_fwd_workspace_bytes(&p), dev);
+    mdn_ws_layout lay;
+    check(mdn_workspace_layout(&p, &lay), "mdn_workspace_layout");
+    const Tensor states = buffer(s[10], (int64_t)mdn_chunk_states_bytes(&p), dev), ws = buffer(s[11], (int64_t)lay.off_seg, dev);
     const Tensor d_o = grads[0].defined() ? grads[0].to(q.scalar_type()).contiguous() : at::zeros_like(v);
     const Tensor dSf = grads[1].defined() ? grads[1].to(at::kFloat).contiguous() : Tensor();
     const Tensor dMf = grads[2].defined() ? grads[2].to(at::kFloat).contiguous() : Tensor();

@@ -1,6 +1,8 @@
 """Sizes at which the kernels' splits change: rows per tile of the exact backward (up to 32 tokens / more), value columns
 per CTA of the fp32 chains (8 while that makes at most 148 CTAs, else 16), the uneven segments of the parallel
 inter-chunk scan, and the two routes of the differentiable forward."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -152,7 +154,6 @@ def test_output_gate_made_by_the_call_before(mdn, T, H, dtype):
 def test_workspace_enough_for_the_serial_chain(mdn):
     """A workspace kept for the largest call also serves the shorter ones that the scan would split (and need more for): the result of
     segments = 1, for every call that takes a workspace."""
-    import ctypes
     import torch
     byref = ctypes.byref
     L = mdn.lib()
@@ -218,3 +219,32 @@ def test_forced_segments_with_fewer_tokens_than_sequences(mdn, lens):
     for x, y, z in zip(one[1:], three[1:], (S0, M0)):
         for n in range(N):
             assert torch.equal(x[n], y[n]) and (lens[n] > 0 or torch.equal(y[n], z[n])), n
+
+
+def training_tensors(T, H):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(T)
+    r = lambda *s: torch.randn(s, device="cuda", generator=g)
+    n = lambda x: (x / x.norm(dim=-1, keepdim=True)).bfloat16()
+    return [n(r(1, T, H, 128)), n(r(1, T, H, 128)), r(1, T, H, 128).bfloat16(), 0.05 * r(1, T, H).abs(), -0.1 * r(1, T, H).abs(),
+            -0.1 * r(1, T, H).abs(), 1 + 0.1 * r(1, T, H)]
+
+
+def test_training_keeps_no_scan_scratch(mdn):
+    """Between forward and backward a call that the scan splits holds what the serial chain holds: outputs, states, and the workspace
+    without the segments' states."""
+    import torch
+    a = [t.requires_grad_() for t in training_tensors(3000, 2)]
+    p, p1 = (mdn.make_params(a[0], a[2], path="tensor", segments=s) for s in (0, 1))
+    scan = mdn.workspace_bytes(p) - mdn.workspace_bytes(p1)
+    assert scan > 4 << 20
+    torch.cuda.synchronize()
+    before = torch.cuda.memory_allocated()
+    o, S, M = mdn.chunk_attention(*a)
+    held = torch.cuda.memory_allocated() - before
+    kept = int(mdn.lib().mdn_chunk_states_bytes(ctypes.byref(p))) + mdn.workspace_bytes(p1) + sum(x.numel() * x.element_size() for x in (o, S, M))
+    assert kept <= held <= kept + (2 << 20)   # (the allocator's rounding)
+    o.float().sum().backward()
+    ref = mdn.chunk_bwd(*(t.detach() for t in a), torch.ones_like(o), method="stepwise")
+    for x, n in zip(a, ("dq", "dk", "dv", "dbeta", "dlog_alpha", "dlog_mu", "deta")):
+        assert (x.grad.float() - ref[n]).norm() <= 5e-3 * ref[n].norm(), n   # 5e-3 in RMS: the tensor-core backward's bound
