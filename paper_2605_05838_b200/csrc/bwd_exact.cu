@@ -8,9 +8,10 @@
 //     dK  = -abar.(dR S^T) + p.(dR M^T) + g_S.(V~ dS'^T) - g_M.(V~ dM'^T) + DW^T Q + (DA + DA^T) K,
 //                                                                         DA = G^- o dA,  dA = -tril(dR V~^T, -1),
 // the coefficient vectors' adjoints as row sums of products that dQ, dK need anyway, and the gate gradients from those
-// by the scans of Eq. 10 in reverse (bwd_gates.cuh).  Five kernels:
-//   status / chunk map;  intra_simt (scan, T, T^T, W^T dO);  chain_simt without output terms (the states at every chunk's start, V~);
+// by the scans of Eq. 10 in reverse (bwd_gates.cuh).  Four kernels (packed input: the chunk map before them):
+//   intra_simt (scan, T, T^T, W^T dO);  chain_simt without output terms (the states at every chunk's start, V~);
 //   the adjoint chain (dS', dM' at every chunk's end, dR);  the per-chunk kernel (everything else, all chunks in parallel).
+// Short sequences go token by token instead (bwd_short.cu, which holds the rule).
 //
 // Why: the serial part of a backward is two walks over the chunks.  The token-by-token form this replaces was serial
 // over tokens (3.4 us per token and chain whatever the GPU's size: 3.4 ms for T = 1023, B H = 16); here 64 tokens cost
@@ -36,6 +37,7 @@ struct AdjArgs {
   float* adj;            // [slot][H][2][dk][dv]: dS', dM' at the chunk's end
   float* dv_out;         // dR = dL/dv, [B,T,H,dv]
   float* dS0; float* dM0;
+  int short_limit;       // sequences of up to so many tokens are bwd_short.cu's
 };
 
 template <int DK, int NV> struct AdjSmem {   // float offsets
@@ -70,6 +72,7 @@ __global__ void __launch_bounds__(kChainThreads<NV>, 1) adj_chain_kernel(const A
   grid_dependency_wait();
   grid_launch_dependents();
   const SeqInfo sq = seq_info(a.g, seq);
+  if (short_sequence(sq, a.short_limit)) return;
   const size_t st_off = ((size_t)seq * H + h) * DK * DV;
   const size_t es = a.in_bf16 ? 2 : 4;
   const int nch = sq.nchunks;
@@ -177,6 +180,7 @@ struct ParArgs {
   float scale;
   float* dq; float* dk;
   GateOut gates;
+  int short_limit;
 };
 
 template <int DK, int DV> struct ParSmem {   // float offsets
@@ -218,7 +222,7 @@ __global__ void __launch_bounds__(kSimtThreads, 1) bwd_exact_par_kernel(const Pa
   grid_dependency_wait();
   grid_launch_dependents();
   const SlotInfo si = slot_info(a.g, slot);
-  if (si.seq < 0) return;
+  if (si.seq < 0 || short_sequence(si, a.short_limit)) return;
   const int n = si.n;
   const int tid = threadIdx.x, lane = tid & 31;
   const bool half1 = tid >= 128;
@@ -498,8 +502,10 @@ template <int DK, int DV> cudaError_t launch_par(const Plan& pl, const ParArgs& 
 
 }  // namespace
 
-void bwd_scratch_layout(const mdn_params& p, int num_slots, BwdScratch* s) {
-  const uint64_t mats = (uint64_t)num_slots * p.H;
+void bwd_scratch_layout(const mdn_params& p, int num_slots, bool allow_short, BwdScratch* s) {
+  s->shorts = allow_short ? bwd_short_plan(p) : BwdShort{-1, 0, 0};
+  s->chunks = p.T > s->shorts.limit;
+  const uint64_t mats = s->chunks ? (uint64_t)num_slots * p.H : 0;
   uint64_t off = 0;
   auto take = [&](uint64_t floats) { const uint64_t at = off; off = (off + floats * 4 + 255) / 256 * 256; return at; };
   s->tt = take(mats * C * C);
@@ -507,6 +513,7 @@ void bwd_scratch_layout(const mdn_params& p, int num_slots, BwdScratch* s) {
   s->adj = take(mats * 2 * p.dk * p.dv);
   s->vt = take(mats * C * p.dv);
   s->vp = take(mats * C * p.dv);
+  s->tokens = take(s->shorts.scratch_bytes / 4);
   s->total = off;
 }
 
@@ -516,9 +523,14 @@ cudaError_t launch_bwd_exact(const Plan& pl, const BwdIo& io, char* scratch, con
   float* adj = reinterpret_cast<float*>(scratch + sl.adj);
   float* vt = reinterpret_cast<float*>(scratch + sl.vt);
   float* vp = reinterpret_cast<float*>(scratch + sl.vp);
-  cudaError_t e = launch_intra_simt(pl, io.q, io.k, GateArgs{io.beta, io.log_alpha, io.log_mu, io.eta}, IntraBwd{io.d_o, tt, vp}, launches);
+  const int limit = sl.shorts.limit;
+  if (limit >= 0) {
+    const cudaError_t es = launch_bwd_short(pl, io, sl.shorts, scratch + sl.tokens, launches);
+    if (es != cudaSuccess || !sl.chunks) return es;
+  }
+  cudaError_t e = launch_intra_simt(pl, io.q, io.k, GateArgs{io.beta, io.log_alpha, io.log_mu, io.eta}, IntraBwd{io.d_o, tt, vp, limit}, launches);
   if (e != cudaSuccess) return e;
-  e = launch_chain_simt_keep(pl, io.k, io.v, io.S0, io.M0, states, vt, launches);
+  e = launch_chain_simt_keep(pl, io.k, io.v, io.S0, io.M0, states, vt, limit, launches);
   if (e != cudaSuccess) return e;
   const bool in_bf16 = pl.p.io_dtype == MDN_BF16, do_bf16 = pl.p.o_dtype == MDN_BF16;
   const float* coef = reinterpret_cast<const float*>(pl.ws + pl.lay.off_coef);
@@ -532,6 +544,7 @@ cudaError_t launch_bwd_exact(const Plan& pl, const BwdIo& io, char* scratch, con
   a.scale = pl.p.scale;
   a.adj = adj; a.dv_out = io.dv;
   a.dS0 = io.dS0; a.dM0 = io.dM0;
+  a.short_limit = limit;
   const bool narrow = simt_narrow_columns(pl);
   if (pl.p.dk == 64) e = narrow ? launch_adj<64, 8>(pl, a) : launch_adj<64, 16>(pl, a);
   else e = narrow ? launch_adj<128, 8>(pl, a) : launch_adj<128, 16>(pl, a);
@@ -545,6 +558,7 @@ cudaError_t launch_bwd_exact(const Plan& pl, const BwdIo& io, char* scratch, con
   b.scale = pl.p.scale;
   b.dq = io.dq; b.dk = io.dk;
   b.gates = GateOut{io.dbeta, io.dlog_alpha, io.dlog_mu, io.deta};
+  b.short_limit = limit;
   if (pl.p.dk == 64) e = pl.p.dv == 64 ? launch_par<64, 64>(pl, b) : launch_par<64, 128>(pl, b);
   else e = pl.p.dv == 64 ? launch_par<128, 64>(pl, b) : launch_par<128, 128>(pl, b);
   if (e == cudaSuccess) ++*launches;

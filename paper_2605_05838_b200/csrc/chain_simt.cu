@@ -35,6 +35,7 @@ struct ChainArgs {
   float* Sf; float* Mf;
   float* keep_states;   // kOut = false: [slot][H][2][dk][dv]
   float* keep_vt;       //               [slot][H][64][dv]
+  int short_limit;      // kOut = false: sequences of up to so many tokens are left out
 };
 
 template <int DK, int NV> struct ChainSmem {   // float offsets
@@ -72,6 +73,7 @@ __global__ void __launch_bounds__(kChainThreads<NV>, 1) chain_simt_kernel(const 
   grid_dependency_wait();
   grid_launch_dependents();
   const SeqInfo sq = seq_info(a.g, seq);
+  if (!kOut && short_sequence(sq, a.short_limit)) return;
   const size_t st_off = ((size_t)seq * H + h) * DK * DV;
   const size_t es = a.in_bf16 ? 2 : 4;
 
@@ -211,7 +213,7 @@ ChainArgs chain_args(const Plan& pl, const void* q, const void* k, const void* v
 
 // Eight value columns per CTA as long as that makes no more CTAs than SMs (a chunk's latency is what counts then);
 // sixteen beyond (twice the arithmetic per operand load).
-bool simt_narrow_columns(const Plan& pl) { return (int64_t)pl.geom.num_seqs * pl.p.H * (pl.p.dv / 8) <= 148; }
+bool simt_narrow_columns(const Plan& pl) { return (int64_t)pl.geom.num_seqs * pl.p.H * (pl.p.dv / 8) <= kSms; }
 
 cudaError_t launch_chain_simt(const Plan& pl, const void* q, const void* k, const void* v, const float* S0,
                               const float* M0, void* o, float* Sf, float* Mf, int* launches) {
@@ -223,9 +225,10 @@ cudaError_t launch_chain_simt(const Plan& pl, const void* q, const void* k, cons
 }
 
 cudaError_t launch_chain_simt_keep(const Plan& pl, const void* k, const void* v, const float* S0, const float* M0,
-                                   float* states, float* vt, int* launches) {
+                                   float* states, float* vt, int short_limit, int* launches) {
   ChainArgs a = chain_args(pl, nullptr, k, v, S0, M0);
   a.keep_states = states; a.keep_vt = vt;
+  a.short_limit = short_limit;
   const cudaError_t e = launch_dims<false>(pl, a);
   if (e == cudaSuccess) ++*launches;
   return e;

@@ -872,7 +872,6 @@ size_t seg_scratch_bytes(const mdn_params& p, int segments) {
 SegSplit choose_segments(const mdn_params& p) {
   const SegSplit off{1, 0, 0};
   if (!tensor_path_supported(p) || p.segments == 1) return off;
-  constexpr long kSMs = kSegSms;
   const long seqs = p.num_seqs > 0 ? p.num_seqs : p.B, tokens = p.num_seqs > 0 ? p.T / seqs : p.T;
   const long nch = (tokens + C - 1) / C, chains = seqs * p.H;
   if (p.segments >= 3) {   // forced: equal segments (at least a chunk: packed input can have fewer tokens than sequences)
@@ -880,14 +879,14 @@ SegSplit choose_segments(const mdn_params& p) {
     return SegSplit{p.segments, per, per};
   }
   auto waves = [](long ctas, long sms) { return (ctas + sms - 1) / sms; };
-  const double serial = (double)(waves(chains, kSMs) * nch);
-  if (chains >= kSMs || nch < 3 * 8) return off;   // no SM left for the middle segments; too short
+  const double serial = (double)(waves(chains, kSms) * nch);
+  if (chains >= kSms || nch < 3 * 8) return off;   // no SM left for the middle segments; too short
   constexpr double kState = 0.9, kRun = 1.7, kFix = 3.;   // state-only chunk; a run's start and end; launches
-  const double step = chains * 16 <= kSMs ? 2.0 : 3.2 * waves(chains * 8, kSMs);   // combine step, by its tile (seg_combine.cu)
+  const double step = chains * 16 <= kSms ? 2.0 : 3.2 * waves(chains * 8, kSms);   // combine step, by its tile (seg_combine.cu)
   double best = (p.num_seqs > 0 ? 0.7 : 0.9) * serial;
   SegSplit r = off;
   for (long m = 1; m <= 30 && (m + 1) * 8 < nch; ++m) {
-    const long w1 = waves(3 * m * chains, kSMs - chains), w3 = waves((m + 1) * chains, kSMs);
+    const long w1 = waves(3 * m * chains, kSms - chains), w3 = waves((m + 1) * chains, kSms);
     const long at = (long)((nch + kRun * (1 - w1)) / (kState * w1 + m + 1));   // where both kinds of phase-1 runs last equally long
     for (long L = at > 8 ? at : 8; L <= at + 1 && (m + 1) * L < nch; ++L) {
       const long first = nch - (m + 1) * L;

@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(kSimtThreads, 2) intra_simt_kernel(const Intra
   grid_launch_dependents();
   if (a.clear_status != nullptr && blockIdx.x == 0 && threadIdx.x < 4) a.clear_status[threadIdx.x] = 0;
   const SlotInfo si = slot_info(a.g, slot);
-  if (si.seq < 0) return;
+  if (si.seq < 0 || (a.bwd.TT != nullptr && short_sequence(si, a.bwd.short_limit))) return;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   float* Ks = sm + L::K;
   float* Qs = sm + L::Q;

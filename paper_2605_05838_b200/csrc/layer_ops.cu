@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(256) out_norm_gate_kernel(size_t rows, OutPost
 
 inline unsigned blocks_for(size_t items, int per_block) {
   const size_t b = (items + per_block - 1) / per_block;
-  return (unsigned)(b < 148 * 32 ? (b ? b : 1) : 148 * 32);
+  return (unsigned)(b < kSms * 32 ? (b ? b : 1) : kSms * 32);
 }
 
 }  // namespace

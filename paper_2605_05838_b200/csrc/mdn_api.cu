@@ -646,12 +646,16 @@ static mdn_params bwd_params(const mdn_params& p) {
   return pe;
 }
 
-size_t mdn_chunk_bwd_workspace_bytes(const mdn_params* p) {
+static size_t exact_bwd_layout(const mdn_params* p, bool allow_short, BwdScratch* bs) {
   mdn_ws_layout lay;
   if (check_params(p) != MDN_OK || make_layout(bwd_params(*p), &lay) != MDN_OK) return 0;
+  bwd_scratch_layout(*p, lay.num_slots, allow_short, bs);
+  return (size_t)(lay.total_bytes + bs->total);
+}
+
+size_t mdn_chunk_bwd_workspace_bytes(const mdn_params* p) {
   BwdScratch bs;
-  bwd_scratch_layout(*p, lay.num_slots, &bs);
-  return (size_t)(lay.total_bytes + bs.total);
+  return exact_bwd_layout(p, true, &bs);
 }
 
 mdn_status mdn_chunk_bwd(const mdn_params* p, const void* q, const void* k, const void* v, const float* beta,
@@ -664,7 +668,9 @@ mdn_status mdn_chunk_bwd(const mdn_params* p, const void* q, const void* k, cons
   mdn_status st = check_params(p);
   if (st != MDN_OK) return st;
   if ((p->num_seqs > 0) != (cu_seqlens != nullptr)) return MDN_ERR_INVALID_ARG;
-  const size_t need = mdn_chunk_bwd_workspace_bytes(p);
+  BwdScratch bs;
+  size_t need = exact_bwd_layout(p, true, &bs);
+  if (workspace_bytes < need) need = exact_bwd_layout(p, false, &bs);   // (a workspace kept for longer sequences: all of them by chunks)
   if (!workspace || workspace_bytes < need || !aligned(workspace, 256)) return MDN_ERR_WORKSPACE;
   if (!q || !k || !v || !beta || !log_alpha || !log_mu || !d_o || !dq || !dk || !dv || !dbeta || !dlog_alpha || !dlog_mu)
     return MDN_ERR_INVALID_ARG;
@@ -677,8 +683,6 @@ mdn_status mdn_chunk_bwd(const mdn_params* p, const void* q, const void* k, cons
   if (st != MDN_OK) return st;
   st = run_prep(pl, &t_last_launches);
   if (st != MDN_OK) return st;
-  BwdScratch bs;
-  bwd_scratch_layout(*p, pl.lay.num_slots, &bs);
   const BwdIo io{q, k, v, beta, log_alpha, log_mu, eta, initial_S, initial_M, d_o, d_final_S, d_final_M,
                  dq, dk, dv, dbeta, dlog_alpha, dlog_mu, deta, d_initial_S, d_initial_M};
   const cudaError_t e = launch_bwd_exact(pl, io, pl.ws + pl.lay.total_bytes, bs, &t_last_launches);

@@ -86,6 +86,11 @@ __device__ __forceinline__ SeqInfo seq_info(const ChunkGeom& g, int seq) {
   return s;
 }
 
+// Whether a sequence is one that the exact backward takes token by token (bwd_short.cu): up to `limit` tokens (-1: none).  For
+// the kernels that work by slots: chunk 0 with so few tokens is a whole sequence.
+__device__ __forceinline__ bool short_sequence(const SeqInfo& s, int limit) { return limit >= 0 && s.nchunks <= 1 && s.len <= limit; }
+__device__ __forceinline__ bool short_sequence(const SlotInfo& s, int limit) { return s.local == 0 && s.n <= limit; }
+
 // The chunks of segment `seg` of a sequence with nchunks chunks (parallel inter-chunk scan, G segments): the first segment has
 // `first`, the others `mid`.  Packed input: in these proportions of the sequence's own length; a sequence whose middle segments
 // would be shorter than `least` stays whole, the others are empty.
@@ -108,6 +113,7 @@ __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddep
 // Lets `kern` be launched with up to kBytes of dynamic shared memory.  Made before every launch (60 ns): the limit belongs to
 // the kernel in the current context, which a device reset takes away.  kBytes is a constant, the most that any launch of that
 // kernel asks for: threads that launch it with different sizes at the same time set the same limit.
+constexpr int kSms = 148;            // streaming multiprocessors
 constexpr int kSmemOptin = 232448;   // the most a block can have
 template <int kBytes, typename... A> inline cudaError_t allow_smem(void (*kern)(A...)) {
   static_assert(kBytes <= kSmemOptin, "shared memory");
@@ -203,14 +209,15 @@ cudaError_t launch_qk_prep(const Plan& pl, const QkNorm& qk, const void* q, cons
                            int* launches);
 cudaError_t launch_out_norm_gate(const Plan& pl, const OutPost& post, void* o, int* launches);
 // What the exact backward wants besides (all NULL: nothing): T^T, and W^T dO ([slot][H][64][dv]) in the place of W.
-struct IntraBwd { const void* d_o; float* TT; float* vp; };
+// Sequences of up to short_limit tokens are left out.
+struct IntraBwd { const void* d_o; float* TT; float* vp; int short_limit; };
 cudaError_t launch_intra_simt(const Plan& pl, const void* q, const void* k, const GateArgs& gates, const IntraBwd& bwd, int* launches);
 cudaError_t launch_chain_simt(const Plan& pl, const void* q, const void* k, const void* v,
                               const float* S0, const float* M0, void* o, float* Sf, float* Mf,
                               int* launches);
 // ... without the output terms, keeping every chunk's start state [slot][H][2][dk][dv] and V~ [slot][H][64][dv]
 cudaError_t launch_chain_simt_keep(const Plan& pl, const void* k, const void* v, const float* S0, const float* M0,
-                                   float* states, float* vt, int* launches);
+                                   float* states, float* vt, int short_limit, int* launches);
 bool simt_narrow_columns(const Plan& pl);   // value columns per CTA of the fp32 chains: 8 or 16
 
 // Tensor-core (tcgen05) path: bf16 q/k/v, dk = dv = 128.
@@ -232,7 +239,6 @@ size_t seg_scratch_bytes(const mdn_params& p, int segments);
 // The parallel inter-chunk scan's split of a sequence of nch chunks: G segments, the first `first` chunks long, the others
 // `mid` (the last one what is left).
 struct SegSplit { int G, first, mid; };
-constexpr int kSegSms = 148;   // SMs the split is made for
 constexpr int kSegLeast = 4;   // chunks: below that a run's start and end outweigh what running it in parallel saves
 SegSplit choose_segments(const mdn_params& p);
 cudaError_t launch_seg_combine(const Plan& pl, int G, float* E, const float* Psi, const float* PhiS,
@@ -241,7 +247,9 @@ cudaError_t launch_seg_combine(const Plan& pl, int G, float* E, const float* Psi
 
 // Exact backward (bwd_exact.cu).  Scratch offsets are relative to the scratch base the API layer places after the
 // forward's workspace regions.
-struct BwdScratch { uint64_t tt, states, adj, vt, vp, total; };
+// bwd_short.cu: sequences of up to `limit` tokens (-1: none) token by token, on `ctas` CTAs.
+struct BwdShort { int limit, ctas; uint64_t scratch_bytes; };
+struct BwdScratch { uint64_t tt, states, adj, vt, vp, tokens, total; BwdShort shorts; bool chunks; };   // chunks: some sequences go by chunks
 struct BwdIo {
   const void* q; const void* k; const void* v;
   const float* beta; const float* log_alpha; const float* log_mu; const float* eta;
@@ -250,7 +258,9 @@ struct BwdIo {
   float* dq; float* dk; float* dv; float* dbeta; float* dlog_alpha; float* dlog_mu; float* deta;
   float* dS0; float* dM0;
 };
-void bwd_scratch_layout(const mdn_params& p, int num_slots, BwdScratch* s);
+void bwd_scratch_layout(const mdn_params& p, int num_slots, bool allow_short, BwdScratch* s);
+BwdShort bwd_short_plan(const mdn_params& p);
+cudaError_t launch_bwd_short(const Plan& pl, const BwdIo& io, const BwdShort& plan, void* scratch, int* launches);
 cudaError_t launch_bwd_exact(const Plan& pl, const BwdIo& io, char* scratch, const BwdScratch& sl, int* launches);
 
 // Recurrent decode step (one token per sequence, state updated in place).

@@ -112,7 +112,7 @@ cudaError_t launch_seg_combine(const Plan& pl, int G, float* E, const float* Psi
     return launch_pdl(seg_combine_kernel<kCols>, dim3(chains, kD / kCols), dim3(kSimtThreads), kSmem<kCols>, pl.stream, G, E, Psi, PhiS,
                       PhiM);
   };
-  cudaError_t e = chains * (kD / 8) <= kSegSms ? run(std::integral_constant<int, 8>{}) : run(std::integral_constant<int, 16>{});
+  cudaError_t e = chains * (kD / 8) <= kSms ? run(std::integral_constant<int, 8>{}) : run(std::integral_constant<int, 16>{});
   if (e == cudaSuccess) ++*launches;
   return e;
 }

@@ -248,3 +248,54 @@ def test_training_keeps_no_scan_scratch(mdn):
     ref = mdn.chunk_bwd(*(t.detach() for t in a), torch.ones_like(o), method="stepwise")
     for x, n in zip(a, ("dq", "dk", "dv", "dbeta", "dlog_alpha", "dlog_mu", "deta")):
         assert (x.grad.float() - ref[n]).norm() <= 5e-3 * ref[n].norm(), n   # 5e-3 in RMS: the tensor-core backward's bound
+
+
+@pytest.mark.parametrize("dk,dv,dtype", [(64, 64, "f32"), (128, 128, "bf16"), (128, 64, "f32"), (64, 128, "bf16")])
+@pytest.mark.parametrize("B,T,H", [(1, 1, 1), (2, 8, 3), (1, 9, 2), (3, 18, 5), (1, 19, 2), (1, 25, 1), (5, 36, 15), (2, 41, 35), (2, 56, 50),
+                                   (1, 57, 100), (200, 5, 1)])
+def test_exact_backward_of_short_sequences(mdn, B, T, H, dk, dv, dtype):
+    """The lengths around which the exact backward goes token by token (sums of 4, blocks of 8 tokens, up to 18 .. 56 tokens by the number
+    of CTAs and dk, more chains than CTAs): the fp32 bound, 1e-4 of RMS; all but the gates' gradients bit-reproducible."""
+    import torch
+    w = wl.Workload("edge_short", B=B, T=T, H=H, dk=dk, dv=dv, dtype=dtype, init_state_std=0.2, seed=T)
+    inp = wl.make_inputs(w)
+    got, ref = run_both(mdn, inp, *upstream(w, inp, T))
+    check(got, ref, "short B=%d T=%d H=%d" % (B, T, H))
+    t = to_torch(inp)
+    a = [t[n] for n in ("q", "k", "v", "beta", "log_alpha", "log_mu", "eta")]
+    x, y = (mdn.chunk_bwd(*a, t["v"], scale=0.1) for _ in range(2))
+    assert all(torch.equal(x[n], y[n]) for n in ("dq", "dk", "dv", "d_initial_S", "d_initial_M"))
+
+
+@pytest.mark.parametrize("lens", [[3, 9, 1], [2, 0, 5, 1], [100, 28, 29, 56, 57, 64, 0, 1] + [7] * 92, [2] * 300, [150, 70, 20]])
+@pytest.mark.parametrize("dv", [64, 128])
+def test_exact_backward_of_packed_short_sequences(mdn, lens, dv):
+    """Packed input: every sequence by its own length, some by chunks and some token by token; the same as one by one, and in a workspace
+    without room for the second kind (all by chunks) the same to rounding."""
+    import torch
+    N, H, T, dk = len(lens), 2, sum(lens), 128
+    g = torch.Generator(device="cuda").manual_seed(N)
+    r = lambda *s: torch.randn(s, device="cuda", generator=g)
+    n = lambda x: x / x.norm(dim=-1, keepdim=True)
+    a = [n(r(1, T, H, dk)), n(r(1, T, H, dk)), r(1, T, H, dv), 0.05 * r(1, T, H).abs(), -0.1 * r(1, T, H).abs(), -0.1 * r(1, T, H).abs(),
+         1 + 0.1 * r(1, T, H)]
+    d_o = r(1, T, H, dv)
+    st = {k: 0.2 * r(N, H, dk, dv) for k in ("initial_S", "initial_M", "d_final_S", "d_final_M")}
+    cu = torch.tensor(np.concatenate([[0], np.cumsum(lens)]), dtype=torch.int32, device="cuda")
+    got = mdn.chunk_bwd(*a, d_o, cu_seqlens=cu, **st)
+
+    def close(x, y, what):   # fp32 sums in another order
+        assert float((x - y).norm()) <= 2e-5 * float(y.norm()), what
+    for i in sorted(set(range(0, N, max(1, N // 8))) | set(range(min(N, 8)))):
+        if lens[i] == 0:
+            assert torch.equal(got["d_initial_S"][i], st["d_final_S"][i])
+            continue
+        t0, t1 = int(cu[i]), int(cu[i + 1])
+        one = mdn.chunk_bwd(*[x[:, t0:t1].contiguous() for x in a], d_o[:, t0:t1].contiguous(), **{k: x[i:i + 1].contiguous() for k, x in st.items()})
+        for k, x in one.items():
+            close(got[k][i:i + 1] if k.startswith("d_init") else got[k][:, t0:t1], x, (k, i, lens[i]))
+    if N == 100:   # both kinds (all short: the chunk form needs more)
+        need = int(mdn.lib().mdn_chunk_bwd_workspace_bytes(ctypes.byref(mdn.make_params(a[0], a[2], num_seqs=N))))
+        fewer = mdn.chunk_bwd(*a, d_o, cu_seqlens=cu, workspace=torch.empty(need - 256, dtype=torch.uint8, device="cuda"), **st)
+        for k in got:
+            close(fewer[k], got[k], k)
