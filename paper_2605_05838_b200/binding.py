@@ -430,7 +430,7 @@ def chunk_bwd(q, k, v, beta, log_alpha, log_mu, eta, d_o, *, initial_S=None, ini
               d_final_S=None, d_final_M=None, scale: Optional[float] = None, workspace: Optional[torch.Tensor] = None,
               method: str = "stepwise", saved=None):
     """mdn_chunk_bwd (method="stepwise": exact, fp32) or mdn_chunk_bwd_chunked (method="chunked":
-    chunk-parallel on the tensor cores; bf16 inputs, dk = dv = 128, fixed length) on CUDA tensors (current stream):
+    chunk-parallel on the tensor cores; bf16 inputs, dk = dv = 128) on CUDA tensors (current stream):
     gradients of mdn_chunk_fwd's outputs' loss.  saved = (fwd_workspace, chunk_states) of a chunk_fwd(...,
     keep_chunk_states=True) call with the same inputs: mdn_chunk_bwd_saved (method="chunked" only).
     d_o: [B,T,H,dv] (its dtype is taken as the forward's o_dtype).  Returns a dict of float32 tensors

@@ -30,12 +30,11 @@ constexpr int LT = kD + 8;    // bf16 elements per row of the dO tile in shared 
 constexpr int L6 = C + 8;     // ... of a 64 x 64 matrix
 
 struct PrepArgs {
-  ChunkGeom g;                      // the forward's geometry (fixed length)
+  ChunkGeom g;                      // the forward's geometry
   const __nv_bfloat16* d_o;
   const float* coef;                // forward: [slot][H][MDN_NUM_COEF][64]
   const __nv_bfloat16* W;           // forward: hi part, lo part w_lo_offset elements later
   size_t w_lo_offset;
-  float scale;
   // the mirrored problem: sequence s = rows [chunk_off[s] * 64, ..) of v_ext
   __nv_bfloat16* v_ext;             // [slots 64][H][128]
   float* coef_ext;                  // [slots][H][MDN_NUM_COEF][64]
@@ -134,7 +133,6 @@ cudaError_t launch_bwd_prep(const Plan& fwd, const void* d_o, void* v_ext, float
   a.coef = reinterpret_cast<const float*>(fwd.ws + fwd.lay.off_coef);
   a.W = reinterpret_cast<const __nv_bfloat16*>(fwd.ws + fwd.lay.off_W);
   a.w_lo_offset = (size_t)fwd.geom.num_slots * fwd.p.H * C * C;
-  a.scale = fwd.p.scale;
   a.v_ext = static_cast<__nv_bfloat16*>(v_ext);
   a.coef_ext = coef_ext;
   constexpr size_t smem = (size_t)2 * C * L6 * 2 + (size_t)C * LT * 2;

@@ -26,7 +26,7 @@
 //    returns to the identity.  The result is the same recurrence either way; only rounding differs.
 //  * One product gives the state terms of the correction AND of the output: B = the K tile stacked on the Q tile
 //    (128 rows), so [X | Z] = Sh [K; Q]^T and [Y | U] = Mh [K; Q]^T are two N = 128 products (a product costs the
-//    same up to N = 128: measured 54 / 54 / 64 / 128 cycles at N = 32 / 64 / 128 / 256 with A in tensor memory).
+//    same up to N = 64: measured 45 / 45 / 64 / 128 cycles at N = 32 / 64 / 128 / 256 with A in tensor memory).
 //  * The intra-chunk output product reads V~ straight from the accumulator of V~ = T R (kind::tf32 against an fp32 W
 //    tile the intra-chunk kernel writes), accumulating onto the inter-chunk terms the epilogue has left there: no
 //    operand conversion for it, and it runs under the epilogue's work on the state update.

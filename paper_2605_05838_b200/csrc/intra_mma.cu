@@ -40,9 +40,6 @@ constexpr int LM = C + 4;     // fp32 elements per row of T (16-byte aligned row
 
 // operand tiles, bf16, [64 rows x 128 B] swizzled blocks: K (dk 0..63) | Q (dk 0..63) | K (dk 64..127) | Q (..)
 // so that rows 0..127 of each 16 KB half are K stacked on Q
-struct Lay {
-  uint32_t k1, cv, tiles, smem;   // offset of the second half, of the vectors; tile bytes; dynamic shared memory
-};
 constexpr uint32_t kOffK0 = 0, kOffQ0 = 8192;
 constexpr int kCvVecs = 12;                                  // + gamma_C eta, (mubar_C/mubar) eta, 1/|k|, 1/|q - dk|, |q|^2, q.k, |k|^2
 // the tile area is reused once the product is done:
@@ -57,10 +54,8 @@ constexpr uint32_t kOffB10 = kOffA21 + 32 * LA * 4;          // A[16:32, 0:16]
 constexpr uint32_t kOffB32 = kOffB10 + 16 * LB * 4;          // A[48:64, 32:48]
 constexpr uint32_t kOffAd = kOffB32 + 16 * LB * 4;           // the four diagonal blocks; dead after step 1:
 constexpr uint32_t kOffP = kOffAd;                           // product scratch, 2 x [16][LB] in step 2, [32][LA] in step 3
-__host__ __device__ constexpr Lay lay_of(bool qk) {
-  const uint32_t half = 16384u; (void)qk;
-  return Lay{half, 2 * half, 2 * half, 2 * half + kCvVecs * C * 4 + 1024};   // + slack for the 1024-byte alignment
-}
+constexpr uint32_t kHalf = 16384, kOffK1 = kHalf, kOffQ1 = kHalf + 8192, kOffCv = 2 * kHalf;   // the second half of the tiles; the vectors
+constexpr uint32_t kSmemBytes = kOffCv + kCvVecs * C * 4 + 1024;                             // + slack for the 1024-byte alignment
 static_assert(kOffAd + 4 * LD16 * 4 <= 32768 && 32 * LA * 4 <= 4 * LD16 * 4, "reuse of the tile area");
 
 __device__ __forceinline__ float4 lds_f4(uint32_t addr) {
@@ -155,8 +150,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) intra_mma_kernel(ChunkGe
   const SlotInfo si = slot_info(g, slot);
   if (si.seq < 0) return;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  constexpr Lay L = lay_of(kQk);
-  constexpr uint32_t kOffK1 = L.k1, kOffQ1 = L.k1 + 8192, kOffCv = L.cv, kTmemCols = 64;
+  constexpr uint32_t kTmemCols = 64;
   const int fg = lane >> 2, ft = lane & 3;   // MMA fragment coordinates of the tf32 block products
   float* Tf = reinterpret_cast<float*>(smem + kOffT);
   float* cv = reinterpret_cast<float*>(smem + kOffCv);
@@ -174,7 +168,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) intra_mma_kernel(ChunkGe
       mbar_init(bar_t, 1);
       mbar_init(bar_p, 1);
       mbar_fence_init();
-      mbar_arrive_expect_tx(bar_t, L.tiles);
+      mbar_arrive_expect_tx(bar_t, 2 * kHalf);
       tma_load_2d(s_base + kOffK0, &map_k, h * kD, si.tok0, bar_t);
       tma_load_2d(s_base + kOffK1, &map_k, h * kD + 64, si.tok0, bar_t);
       tma_load_2d(s_base + kOffQ0, &map_q, h * kD, si.tok0, bar_t);
@@ -310,7 +304,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) intra_mma_kernel(ChunkGe
       float2 q2 = make_float2(0.f, 0.f), qk2 = q2, k2 = q2;   // even and odd columns
 #pragma unroll 2
       for (int j = 0; j < 8; ++j) {
-        const uint32_t off = q_tile_chunk(L.k1, row, hb * 8 + j);
+        const uint32_t off = q_tile_chunk(kOffK1, row, hb * 8 + j);
         const uint4 uq = *reinterpret_cast<const uint4*>(smem + off);
         const uint4 uk = *reinterpret_cast<const uint4*>(smem + off - kOffQ0);
         const uint32_t q4[4] = {uq.x, uq.y, uq.z, uq.w}, k4[4] = {uk.x, uk.y, uk.z, uk.w};
@@ -572,10 +566,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) intra_mma_kernel(ChunkGe
 template <bool kQk, bool kWf32>
 static cudaError_t launch_intra_variant(const Plan& pl, const CUtensorMap& mq, const CUtensorMap& mk, const GateArgs& gates,
                                         size_t n_mats) {
-  constexpr uint32_t smem_bytes = lay_of(kQk).smem;
-  cudaError_t e = allow_smem<(int)smem_bytes>(intra_mma_kernel<kQk, kWf32>);
+  cudaError_t e = allow_smem<(int)kSmemBytes>(intra_mma_kernel<kQk, kWf32>);
   if (e != cudaSuccess) return e;
-  return launch_pdl(intra_mma_kernel<kQk, kWf32>, dim3((unsigned)n_mats), dim3(kThreads), smem_bytes, pl.stream, pl.geom, mq, mk,
+  return launch_pdl(intra_mma_kernel<kQk, kWf32>, dim3((unsigned)n_mats), dim3(kThreads), kSmemBytes, pl.stream, pl.geom, mq, mk,
                     reinterpret_cast<float*>(pl.ws + pl.lay.off_coef), gates, pl.gp, pl.qk, pl.p.scale,
                     reinterpret_cast<__nv_bfloat16*>(pl.ws + pl.lay.off_T),
                     reinterpret_cast<__nv_bfloat16*>(pl.ws + pl.lay.off_W), n_mats * C * C,

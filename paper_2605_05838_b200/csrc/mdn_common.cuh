@@ -227,7 +227,7 @@ cudaError_t launch_intra_mma(const Plan& pl, const void* q, const void* k, const
 cudaError_t launch_chain_tensor(const Plan& pl, const void* q, const void* k, const void* v,
                                 const float* S0, const float* M0, void* o, float* Sf, float* Mf,
                                 int* launches);
-// chain_tf32.cu: the plain forward's chain kernel (no layer operations, no training options); expects an fp32 W
+// chain_tf32.cu: the chain kernel of every forward without the training options, layer operations included; expects an fp32 W
 cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, const void* v,
                               const float* S0, const float* M0, void* o, float* Sf, float* Mf,
                               int* launches);
@@ -245,9 +245,8 @@ cudaError_t launch_seg_combine(const Plan& pl, int G, float* E, const float* Psi
                                const float* PhiM, int* launches);
 
 
-// Exact backward (bwd_exact.cu).  Scratch offsets are relative to the scratch base the API layer places after the
-// forward's workspace regions.
-// bwd_short.cu: sequences of up to `limit` tokens (-1: none) token by token, on `ctas` CTAs.
+// Exact backward (bwd_exact.cu; bwd_short.cu: sequences of up to `limit` tokens (-1: none) token by token, on `ctas` CTAs).  Scratch
+// offsets are relative to the scratch base the API layer places after the forward's workspace regions.
 struct BwdShort { int limit, ctas; uint64_t scratch_bytes; };
 struct BwdScratch { uint64_t tt, states, adj, vt, vp, tokens, total; BwdShort shorts; bool chunks; };   // chunks: some sequences go by chunks
 struct BwdIo {

@@ -83,7 +83,8 @@ def test_segments_of_packed_sequences(mdn, segments, H, lens):
 @pytest.mark.parametrize("B,H,T,lens", [(1, 1, 64 * 45 + 17, None), (2, 2, 64 * 40, None), (1, 1, 0, [64 * 110 + 3, 64 * 40, 70])])
 def test_training_with_segments(mdn, B, H, T, lens):
     """Few long chains: both chains of a training step are split as the forward is.  Against the exact fp32 backward (1e-4 of the
-    oracle): the tensor-core backward's bounds, 2e-2 of RMS per element and 5e-3 in RMS."""
+    oracle): the tensor-core backward's bounds, 2e-2 of RMS per element (dv 3e-2: largest of 1e5 .. 1e6 values rounded to bf16 on the
+    way, the serial chain's own is 2.1e-2 here and up to 2.8e-2 elsewhere) and 5e-3 in RMS."""
     import torch
     w = wl.Workload("edge_tseg", B=B, T=T or sum(lens), H=H, dk=128, dv=128, dtype="bf16", varlen=lens is not None, init_state_std=0.1, seed=B + 7)
     assert mdn.workspace_layout(mdn.MdnParams(B, w.T, H, 128, 128, 64, len(lens) if lens else 0, 1, 1, 0, 1.0, 0)).segments > 1
@@ -97,7 +98,7 @@ def test_training_with_segments(mdn, B, H, T, lens):
         got = mdn.chunk_bwd(*args, d_o, method="chunked", saved=saved, **kw)
         for name, y in ref.items():
             x, y = got[name].double().cpu().numpy(), y.double().cpu().numpy()
-            assert rel_err(x, y) <= (3e-2 if name == "dv" else 2e-2), name   # (dv: the serial chain reaches 2.1e-2 on these inputs)
+            assert rel_err(x, y) <= (3e-2 if name == "dv" else 2e-2), name
             assert np.sqrt(np.mean((x - y) ** 2)) <= 5e-3 * np.sqrt(np.mean(y ** 2)), name
 
 
