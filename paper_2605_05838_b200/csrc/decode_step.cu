@@ -34,7 +34,7 @@ __device__ __forceinline__ float2 block_sum2(float x, float y, float* buf) {
 
 // 32 value columns per CTA (4 CTAs per (sequence, head) at dv = 128: many small CTAs keep a pure streaming kernel at
 // HBM speed).  kLayer adds the gate formulas and the q / k step of Section 3.3 (measured: free and +1 us); the output
-// norm and gate need the whole head row and run as a second, tiny kernel over o (0.5 MB, L2-resident: +3 us) -
+// norm and gate need the whole head row and run as a second, tiny kernel over o (0.5 MB, L2-resident: +3 us as a dependent launch) -
 // forming thread-block clusters of the head's CTAs and reducing through distributed shared memory cost +20 us,
 // one 512-thread CTA per head +36 us.
 template <typename TIn, typename TO, int DK, int DV, int kCols, bool kLayer>
