@@ -408,7 +408,8 @@ mdn_status mdn_chunk_bwd_saved_io(const mdn_params* p,
 
 /*
  * Backward of mdn_chunk_fwd (Section 3.1: the training pass differentiates the same recurrence; like the paper's
- * kernels this keeps no per-token states and rebuilds what it needs chunk by chunk from the chunk-start states):
+ * kernels this keeps no per-token states and rebuilds what it needs chunk by chunk from the chunk-start states; short
+ * sequences token by token):
  * given d_o = dL/do ([B,T,H,dv], o_dtype) and optionally dL/d(final_S), dL/d(final_M) ([N,H,dk,dv] float32, NULL =
  * zero), writes the float32 gradients
  *     dq, dk [B,T,H,dk];  dv [B,T,H,dv];  dbeta, dlog_alpha, dlog_mu, deta [B,T,H] (deta may be NULL);
@@ -416,8 +417,8 @@ mdn_status mdn_chunk_bwd_saved_io(const mdn_params* p,
  * q, k, v, the gates, the initial states, cu_seqlens, p: exactly the forward call's.  The pass recomputes the
  * forward's states itself, in float32 throughout (any dk, dv in {64, 128}; p->path and p->segments are ignored), so it
  * does not need the forward's outputs.  Workspace: mdn_chunk_bwd_workspace_bytes(p) bytes, 256-byte aligned,
- * scratch.  Same ownership, stream and error rules as mdn_chunk_fwd.  dq, dk, dv and the initial states' gradients are
- * bit-reproducible; the gate gradients sum over key rows through shared-memory floating-point atomics, so their last
+ * scratch (one that suffices for the chunk form alone is taken too).  Same ownership, stream and error rules as
+ * mdn_chunk_fwd.  dq, dk, dv and the initial states' gradients are bit-reproducible; the gate gradients sum over key rows through shared-memory floating-point atomics, so their last
  * bits can differ from run to run.
  */
 size_t mdn_chunk_bwd_workspace_bytes(const mdn_params* p);
