@@ -1,0 +1,838 @@
+// a3 + a4 of the plain forward for calls that leave SMs idle: TWO CTAs walk the chunks of one (sequence, head), each with half of
+// the value columns.  The same recurrence, products and roundings as chain_tf32.cu (lazily scaled fp32 masters in tensor memory,
+// read as tf32; see there); bf16 q/k/v, dk = dv = 128, chunk 64.
+//
+// What the split buys.  A product costs the same for 64 accumulator lanes as for 128, so half the value columns alone would save
+// nothing.  Here the 128 lanes hold BOTH states of the CTA's 64 value columns: of the 32 lanes of a quarter the lower sixteen are
+// rows of S^T, the upper sixteen the same rows of M^T.  One product then gives K S and K M (the masters times the K tile), one
+// Q S and Q M, and one updates both states: per chunk 16 + 16 products for the state terms and 8 for the updates where chain_tf32.cu
+// has 32 (twice as wide) and 16.  What combines S and M terms (R, the output, the rescaling) needs both in one thread: the
+// epilogue accesses tensor memory sixteen lanes at a time (16x256b / 16x128b), where a thread gets the same (column, token) of
+// both halves, without a shuffle; R^T and V~ stand in both halves of the lanes, so that V~ = T R comes out where either state's
+// update operand is made.  The thread layout is that of the warp-level matrix instructions: V comes in and o leaves by
+// ldmatrix / stmatrix (transposed).
+//
+// Per chunk:  MMA-1x X = P K^T (P: both masters)  ->  EPI-1 R^T (bf16 hi + lo) into X  ->  MMA-2 Y = R^T T^T  ->  EPI-2 wS V~ | -wM V~
+//             (bf16 hi + lo) into X  ->  MMA-3 P += X K  ->  next chunk's MMA-1x.
+// Off that path: MMA-1z Z = P Q^T (under EPI-1), o_inter into Z (under MMA-2), MMA-3' Z += V~^T W^T (under EPI-2), output tile.
+//
+// What bounds a chunk: the serial chain of the three product groups (0.72 + 0.36 + 0.51 k cycles), their commit-to-wake latencies
+// and the two epilogue steps; the tensor pipe is busy about 60 % of it, the shared-memory port about as much (the fp32 K
+// and Q copies).  Registers and tensor memory (320 of 512 columns) are not the limit here.
+//
+// With the layer operations the RMSNorm of the output step sums over all 128 value columns: the two CTAs of a chain are a
+// thread-block cluster and exchange each token's sum of squares through distributed shared memory.
+#include "chain_tf32.cuh"
+#include "mdn_common.cuh"
+#include "tc_utils.cuh"
+
+namespace mdn {
+namespace {
+
+using namespace tc;
+
+constexpr int kD = 128, kN = 64;   // key columns; value columns of a CTA
+// Warps 0..7 epilogue (lane quarter = warp % 4, token half = warp / 4), 8 MMA issuer, 9 loads of K and Q, 10 coefficients, 11 output
+// stores and the loads behind them, 12..15 converters, with the layer operations 16..19 output step.  (With one producer
+// warp for all of it the coefficients came 0.45 k cycles before the epilogue needed them and the next K tile's copy 0.4 k late.)
+constexpr int kEpiWarps = 8, kWarpMma = 8, kWarpKq = 9, kWarpCoef = 10, kWarpTma = 11, kWarpCvt = 12, kCvtWarps = 4, kWarpOut = 16, kOutWarps = 4;
+constexpr int threads_of(bool layer) { return (kWarpOut + (layer ? kOutWarps : 0)) * 32; }
+constexpr int kEpiThreads = kEpiWarps * 32, kCvtThreads = kCvtWarps * 32, kOutThreads = kOutWarps * 32;
+constexpr int kTok = 32, kPk = 16;   // tokens of an epilogue warp; their packed bf16 pairs
+
+// Shared memory (offsets from a 1024-byte aligned base).  The fp32 K copy is double-buffered: it is made as soon as the K tile
+// has landed, whatever the chain is at.  The fp32 Q copy is single (its readers are done early in a chunk).
+constexpr uint32_t kOffK32 = 0, kK32Bytes = 32768;   // [64 tokens x 128 dk] fp32: four dk quarters x [64 rows x 128 B], swizzled
+constexpr uint32_t kOffQ32 = 65536;
+constexpr uint32_t kOffQb = 98304;                   // bf16 Q tile waiting for its copy: two dk halves x [64 rows x 128 B]
+constexpr uint32_t kOffStage = 114688;
+constexpr uint32_t kStK = 0, kStV = 16384, kStT = 24576, kStW = 32768, kStCoef = 49152;
+constexpr uint32_t kCoefBytes = kChainCoefs * C * sizeof(float);
+constexpr uint32_t kStageBytes = 51200;
+constexpr uint32_t kTxK = 16384, kTxV = 8192, kTxT = 8192, kTxW = 16384;
+constexpr uint32_t kStOut = kStV;                    // the finished output tile: V area (bf16), V + T (fp32); both dead by then
+constexpr uint32_t kOffAdj = kOffStage + 2 * kStageBytes;
+constexpr uint32_t kSmemBytes = kOffAdj + 2 * kAdjBytes + 1024;
+static_assert(kStCoef + kCoefBytes <= kStageBytes && kSmemBytes <= kSmemOptin - 4096, "shared-memory layout");
+
+// tensor memory columns: masters P (lanes: S^T | M^T), X, Z, Y
+constexpr uint32_t kColP = 0, kColX = 128, kColZ = 192, kColY = 256;
+constexpr uint32_t kUpper = 16u << 16;               // the upper sixteen lanes of a warp's quarter: M
+
+// A barrier that a waiter could fall a whole phase behind comes in pairs, by the chunk's parity.
+struct Bars {
+  uint64_t kfull[2];  // bf16 K tile of a stage landed                                    (1 + tx bytes)
+  uint64_t full[2];   // V, T, W of a stage landed                                        (1 + tx bytes)
+  uint64_t cfull[2];  // coefficient vectors of a stage landed                            (1 + tx bytes)
+  uint64_t qfull;     // bf16 Q tile landed                                               (1 + tx bytes)
+  uint64_t qfree;     // ... and read                                                     (4 warps)
+  uint64_t k32[2];    // fp32 K copy written                                              (4 warps)
+  uint64_t q32;       // fp32 Q copy written                                              (4 warps)
+  uint64_t adj[2];    // a chunk's coefficient block written                              (1)
+  uint64_t fin;       // G after the last chunk written                                   (1)
+  uint64_t init;      // masters of chunk 0 stored                                        (8 warps)
+  uint64_t mx[2];     // X done: the fp32 K copy is free too                              (commit)
+  uint64_t mz;        // Z done: the fp32 Q copy is free too                              (commit)
+  uint64_t r;         // EPI-1 done: R^T in X                                             (8 warps)
+  uint64_t m2;        // V~ in Y                                                          (commit)
+  uint64_t oi;        // inter-chunk output terms in Z                                    (8 warps)
+  uint64_t v;         // EPI-2 done: update operand in X (eager chunks: masters rescaled)  (8 warps)
+  uint64_t m3[2];     // masters updated: the stage's K tile is free too                  (commit)
+  uint64_t mo;        // MMA-3' done                                                      (commit)
+  uint64_t zu;        // Z (the chunk's output) has been read                             (8 warps)
+  uint64_t go[2];     // the output tile is staged                                        (8 warps; fused output step 4)
+  uint64_t pn[2];     // fused output step: the fp32 tile is staged                       (8 warps)
+  uint64_t peer[2];   // ... and the other CTA's sums of squares have arrived             (64)
+};
+
+enum Ev : int { kEvTop = 0, kEvXIssued, kEvZIssued, kEvRSeen, kEvM2Issued, kEvMoIssued, kEvVSeen, kEvM3Issued,
+                kEvMxSeen, kEvRArrive, kEvOiArrive, kEvM2Seen, kEvVArrive, kEvMoSeen, kEvOutDone, kEvCvtK, kEvCvtKDone, kEvCvtQ,
+                kEvCvtQDone, kEvTma, kEvAdj, kEvTmaKq, kEvStored, kEvPn, kEvSsSent, kEvPeer, kEvGo };
+
+template <typename TO, bool kLayer>
+__global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const ChainTf32Args a, const __grid_constant__ CUtensorMap map_q,
+                                                                const __grid_constant__ CUtensorMap map_k,
+                                                                const __grid_constant__ CUtensorMap map_v,
+                                                                const __grid_constant__ CUtensorMap map_t,
+                                                                const __grid_constant__ CUtensorMap map_w,
+                                                                const __grid_constant__ CUtensorMap map_o) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ __align__(8) Bars bars;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_flag;
+  __shared__ float g_final[4];   // G after the last chunk: what the final states are read through
+  __shared__ __align__(16) float w_sm[kLayer ? kN : 4];        // RMSNorm weight of the fused output step
+  __shared__ float peer_ss[2][kLayer ? C : 1];                 // the other CTA's sums of squares, by chunk parity
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int H = a.g.H;
+  // Coefficients, T and W come from the previous kernel, which lets this one in before it has finished (intra_mma.cu): only
+  // the two warps that load those wait.  Everything else read here (the call's inputs, the chunk
+  // map) was complete before that kernel could let anybody in.  Segment states come from the kernel just before this one.
+  const bool early = a.seg_G == 0;
+  if (!early) grid_dependency_wait();
+  const ChainRun rn = chain_run(a, (int)blockIdx.x >> 1);
+  const int v0 = ((int)blockIdx.x & 1) * kN;   // first value column
+  const SeqInfo sq = rn.sq;
+  const int h = rn.h, nch = sq.nchunks;
+  const bool v_zero = rn.v_zero, write_o = rn.write_o;
+
+  const uint32_t s_base = smem_u32(smem);
+  auto bar = [](uint64_t& b) { return smem_u32(&b); };
+  // One arrival per warp, for what its lanes have done before (tensor memory: behind the wait for it and the fence).  An arrival
+  // per thread is 256 shared-memory operations per hand-over: 3.9 -> 3.65 k cycles per chunk.
+  auto warp_arrive = [&](uint64_t& b) {
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&b));
+  };
+  const bool qk_on = kLayer && a.qk_on;
+  const float qk_dh = (qk_on && a.qk_d) ? __ldg(a.qk_d + h) : 0.f;
+  const bool post = kLayer && a.post_on && write_o;
+  const uint32_t peer_rank = kLayer ? cluster_rank() ^ 1u : 0u;
+
+  if (tid == 0) {
+    abort_flag = 0;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(bar(bars.kfull[i]), 1); mbar_init(bar(bars.full[i]), 1); mbar_init(bar(bars.cfull[i]), 1);
+      mbar_init(bar(bars.k32[i]), kCvtWarps); mbar_init(bar(bars.adj[i]), 1);
+      mbar_init(bar(bars.mx[i]), 1); mbar_init(bar(bars.m3[i]), 1);
+      mbar_init(bar(bars.go[i]), post ? kOutWarps : kEpiWarps);
+      mbar_init(bar(bars.pn[i]), kEpiWarps); mbar_init(bar(bars.peer[i]), C);
+    }
+    mbar_init(bar(bars.qfull), 1); mbar_init(bar(bars.qfree), kCvtWarps); mbar_init(bar(bars.q32), kCvtWarps);
+    mbar_init(bar(bars.fin), 1); mbar_init(bar(bars.init), kEpiWarps);
+    mbar_init(bar(bars.mz), 1); mbar_init(bar(bars.m2), 1); mbar_init(bar(bars.mo), 1);
+    mbar_init(bar(bars.r), kEpiWarps); mbar_init(bar(bars.oi), kEpiWarps); mbar_init(bar(bars.v), kEpiWarps);
+    mbar_init(bar(bars.zu), kEpiWarps);
+    mbar_fence_init();
+  }
+  if (kLayer && tid < kN) w_sm[tid] = (a.post_on && a.post_w) ? __ldg(a.post_w + v0 + tid) : 1.f;
+  if (warp == kWarpMma) tmem_alloc(smem_u32(&tmem_slot), 512);
+  if (warp == kWarpTma && lane == 0) {
+    prefetch_tensormap(&map_q); prefetch_tensormap(&map_k); prefetch_tensormap(&map_v);
+    prefetch_tensormap(&map_t); prefetch_tensormap(&map_w); prefetch_tensormap(&map_o);
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  if constexpr (kLayer) cluster_sync_all();   // the other CTA's barriers are set up before anything arrives at them
+  tc_fence_after_sync();
+  const uint32_t tmem = tmem_slot;
+  bool ok = true;
+  volatile int* abortp = &abort_flag;
+#define MDN_WAIT(b, par)                                    \
+  if (!mbar_wait(smem_u32(&bars.b), (par), abortp)) {       \
+    ok = false;                                             \
+    break;                                                  \
+  }
+  // waits on the chain's critical path poll without suspending
+#define MDN_SPIN(b, par)                                    \
+  if (!mbar_wait_spin(smem_u32(&bars.b), (par), abortp)) {  \
+    ok = false;                                             \
+    break;                                                  \
+  }
+#ifdef MDN_DEBUG
+  // Stamps go to shared memory for the chunks kTlFirst .. kTlFirst + 7 and are copied out when the kernel ends.
+  long long* const tline = a.timeline != nullptr ? a.timeline + 1024 * (size_t)blockIdx.x : nullptr;   // (1024 words per CTA)
+  constexpr int kTlFirst = 16;
+  __shared__ long long tl_sm[8][32];
+#define MDN_MARK(c, ev) \
+  if (tline != nullptr && lane == 0 && (c) >= kTlFirst && (c) < kTlFirst + 8 && \
+      ((warp >= kWarpMma && warp <= kWarpCvt) || warp == 2 || warp == kWarpOut)) tl_sm[(c) - kTlFirst][(ev)] = clock64();
+  auto now = [&](int i) {   // ... and the nanosecond stamps of the run as a whole in the words before them
+    unsigned long long ns;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns));
+    if (tline != nullptr && lane == 0) tline[i] = (long long)ns;
+  };
+#define MDN_NOW(i) now(i)
+#else
+#define MDN_MARK(c, ev)
+#define MDN_NOW(i) (void)0
+#endif
+
+  if (warp == 0) { MDN_NOW(0); }
+#ifdef MDN_DEBUG
+  if (tline != nullptr && tid == 0) {
+    uint32_t smid;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
+    tline[7] = smid;
+  }
+#endif
+  if (warp == kWarpKq) {
+    // ================================================================== K and Q tiles, for the converters and MMA-3
+    // A stage's K tile is refilled (for chunk c + 2) as soon as MMA-3 has read it, the Q buffer as soon as it is converted.
+    int issued = 0;
+    for (int c = 0; c < nch; ++c) {
+      const int s = c & 1, tok0 = sq.tok0 + c * C;
+      const uint32_t st = s_base + kOffStage + s * kStageBytes;
+      if (c >= 2) MDN_WAIT(m3[s], ((c - 2) >> 1) & 1);
+      if (lane == 0) {
+        mbar_arrive_expect_tx(bar(bars.kfull[s]), kTxK);
+        tma_load_2d(st + kStK, &map_k, h * kD, tok0, bar(bars.kfull[s]));
+        tma_load_2d(st + kStK + 8192, &map_k, h * kD + 64, tok0, bar(bars.kfull[s]));
+      }
+      issued = c + 1;
+      if (write_o) {
+        if (c > 0) MDN_WAIT(qfree, (c - 1) & 1);
+        if (lane == 0) {
+          mbar_arrive_expect_tx(bar(bars.qfull), kTxK);
+          tma_load_2d(s_base + kOffQb, &map_q, h * kD, tok0, bar(bars.qfull));
+          tma_load_2d(s_base + kOffQb + 8192, &map_q, h * kD + 64, tok0, bar(bars.qfull));
+        }
+      }
+      MDN_MARK(c, kEvTmaKq);
+    }
+    if (!ok && lane == 0) {   // giving up: let the copies already in flight land before the CTA exits
+      for (int c = max(0, issued - 2); c < issued; ++c)
+        for (uint32_t it = 0; it < (1u << 16) && !mbar_try_wait(bar(bars.kfull[c & 1]), (c >> 1) & 1); ++it) {}
+      for (int c = max(0, issued - 2); c < issued && write_o; ++c)   // (the last or the last but one is in flight)
+        for (uint32_t it = 0; it < (1u << 16) && !mbar_try_wait(bar(bars.qfull), c & 1); ++it) {}
+    }
+  } else if (warp == kWarpCoef) {
+    // ================================================================== coefficients: a chunk ahead of their use
+    int issued = 0;
+    float g11 = 1.f, g12 = 0.f, g22 = 1.f;
+    auto load = [&](int c) {   // (the stage's vectors have been read when its chunk's block is published)
+      if (c >= nch) return;
+      if (lane == 0) {
+        const uint32_t fb = bar(bars.cfull[c & 1]);
+        mbar_arrive_expect_tx(fb, kCoefBytes);
+        bulk_load(s_base + kOffStage + (c & 1) * kStageBytes + kStCoef, a.coef + (size_t)((sq.slot0 + c) * H + h) * MDN_NUM_COEF * C,
+                  kCoefBytes, fb);
+      }
+      issued = c + 1;
+    };
+    if (early) grid_dependency_wait();
+    MDN_NOW(1);
+    load(0);
+    load(1);
+    for (int c = 0; c < nch; ++c) {
+      const int s = c & 1;
+      MDN_WAIT(cfull[s], (c >> 1) & 1);
+      if (c >= 2) MDN_WAIT(m3[s], ((c - 2) >> 1) & 1);   // chunk c - 2's block has been read
+      publish_coefs<kLayer>(reinterpret_cast<const float*>(smem + kOffStage + s * kStageBytes + kStCoef),
+                            reinterpret_cast<float*>(smem + kOffAdj + s * kAdjBytes), a.scale, lane, g11, g12, g22);
+      warp_arrive(bars.adj[s]);
+      MDN_MARK(c, kEvAdj);
+      __syncwarp();
+      load(c + 2);
+    }
+    if (ok) {
+      if (lane == 0) {
+        g_final[0] = g11; g_final[1] = g12; g_final[2] = g22;
+        mbar_arrive(bar(bars.fin));
+      }
+    } else if (lane == 0) {
+      for (int c = max(0, issued - 2); c < issued; ++c)
+        for (uint32_t it = 0; it < (1u << 16) && !mbar_try_wait(bar(bars.cfull[c & 1]), (c >> 1) & 1); ++it) {}
+    }
+  } else if (warp == kWarpTma) {
+    // ================================================================== output stores, V, T, W tiles
+    // Stage s = c & 1 serves chunk c; its V, T, W are refilled for chunk c + 2 once the output tile staged over V and T has left.
+    int issued = 0;
+    if (early) grid_dependency_wait();
+    for (int c = 0; c < nch + 2; ++c) {
+      const int s = c & 1;
+      const uint32_t st = s_base + kOffStage + s * kStageBytes;
+      if (c >= 2) {
+        const int co = c - 2;
+        MDN_WAIT(go[s], (co >> 1) & 1);
+        if (lane == 0) {
+          const int n = min(C, sq.len - co * C);
+          const int tok = sq.tok0 + co * C;
+          const uint32_t src = st + kStOut;
+          if (!write_o) {
+            // Psi / Phi runs of the parallel scan produce states only
+          } else if (n == C) {
+            tma_store_2d(&map_o, h * kD + v0, tok, src);
+          } else {   // short chunk: rows >= n belong to another sequence; one bulk copy per valid row (an unswizzled tile)
+            for (int r = 0; r < n; ++r)
+              bulk_store(static_cast<uint8_t*>(a.o) + (((size_t)(tok + r) * H + h) * kD + v0) * sizeof(TO),
+                         src + r * kN * (uint32_t)sizeof(TO), kN * (uint32_t)sizeof(TO));
+          }
+          tma_store_commit();
+          tma_store_wait_read();
+        }
+        __syncwarp();
+        MDN_MARK(co, kEvStored);
+      }
+      if (c < nch) {
+        if (lane == 0) {
+          const uint32_t fb = bar(bars.full[s]);
+          const int mat = (sq.slot0 + c) * H + h;
+          mbar_arrive_expect_tx(fb, kTxT + (write_o ? kTxW : 0u) + (v_zero ? 0u : kTxV));
+          if (!v_zero) tma_load_2d(st + kStV, &map_v, h * kD + v0, sq.tok0 + c * C, fb);
+          tma_load_2d(st + kStT, &map_t, 0, mat * C, fb);
+          if (write_o) {
+            tma_load_2d(st + kStW, &map_w, 0, mat * C, fb);
+            tma_load_2d(st + kStW + 8192, &map_w, 32, mat * C, fb);
+          }
+        }
+        __syncwarp();
+        MDN_MARK(c, kEvTma);
+        issued = c + 1;
+      }
+    }
+    if (lane == 0) {
+      for (int c = max(0, issued - 2); c < issued && !ok; ++c)
+        for (uint32_t it = 0; it < (1u << 16) && !mbar_try_wait(bar(bars.full[c & 1]), (c >> 1) & 1); ++it) {}
+      tma_store_wait_all();
+    }
+  } else if (warp == kWarpMma) {
+    // ================================================================== MMA issuer
+    // The whole warp walks the loop and waits (warp-uniform control flow and operands); one elected lane issues the products and
+    // the commits.  A product that reads what the one just before it accumulates waits for that one's commit: MMA-1x issued
+    // right behind MMA-3 read masters that lacked part of the update (o off by 3e-4 of its RMS), and was no faster.
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t sb = __shfl_sync(0xffffffffu, s_base, 0);
+    const bool lead = elect_one();
+    // Column of the bf16 A operands the epilogue leaves in X: K-step k covers tokens 16k .. 16k + 15; the warp that owns those tokens
+    // keeps hi (part 0) and lo (part 1) inside its own kTok columns
+    auto a_col = [](int part, int k) {
+      return static_cast<uint32_t>(kTok * ((16 * k) / kTok) + kPk * part + ((16 * k) % kTok) / 2);
+    };
+    const uint32_t id64 = idesc_bf16(128, 64, false, false, false);
+    const uint32_t id128_mn = idesc_bf16(128, 128, false, true, false);
+    const uint32_t id64_tf32 = idesc_tf32(128, 64, false, false, false);
+    const uint64_t dK_0 = smem_desc_sw128(sb + kOffK32, 16, 1024), dK_1 = dK_0 + (kK32Bytes >> 4);   // + (j >> 2) * 8192 + (j & 3) * 32 bytes per K step
+    const uint64_t dQ = smem_desc_sw128(sb + kOffQ32, 16, 1024);
+    const uint64_t dT_0 = smem_desc_sw128(sb + kOffStage + kStT, 16, 1024), dT_1 = dT_0 + (kStageBytes >> 4);
+    const uint64_t dW_0 = smem_desc_sw128(sb + kOffStage + kStW, 16, 1024), dW_1 = dW_0 + (kStageBytes >> 4);
+    const uint64_t dKmn_0 = smem_desc_sw128(sb + kOffStage + kStK, 8192, 1024), dKmn_1 = dKmn_0 + (kStageBytes >> 4);
+    // ---- MMA-1x: X = P K^T (K S and K M)
+    auto mma1x = [&](int c) {
+      const uint64_t dK = (c & 1) ? dK_1 : dK_0;
+      if (lead) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          umma_ts_tf32(tm + kColX, tm + kColP + 8 * j, dK + (uint64_t)((j >> 2) * 512 + (j & 3) * 2), id64_tf32, j > 0);
+        umma_commit(bar(bars.mx[c & 1]));
+      }
+      MDN_MARK(c, kEvXIssued);
+    };
+    for (int c = 0; c < nch; ++c) {
+      const int s = c & 1;
+      const uint32_t ph = c & 1;
+      if (c == 0) {
+        MDN_WAIT(k32[0], 0);
+        MDN_WAIT(init, 0);
+        __syncwarp();
+        tc_fence_after_sync();
+        MDN_NOW(2);
+        mma1x(0);
+      }
+      const uint64_t dT = s ? dT_1 : dT_0, dW = s ? dW_1 : dW_0, dKmn = s ? dKmn_1 : dKmn_0;
+      MDN_MARK(c, kEvTop);
+      // ---- MMA-1z: Z = P Q^T (Q S and Q M), once the previous chunk's output has been read out of Z
+      if (write_o) {
+        MDN_SPIN(q32, ph);
+        MDN_SPIN(zu, ph ^ 1);
+        tc_fence_after_sync();
+        if (lead) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            umma_ts_tf32(tm + kColZ, tm + kColP + 8 * j, dQ + (uint64_t)((j >> 2) * 512 + (j & 3) * 2), id64_tf32, j > 0);
+          umma_commit(bar(bars.mz));
+        }
+        MDN_MARK(c, kEvZIssued);
+      }
+      // (T, W and the K tile of the stage have landed: the epilogue waited for V, which came with T and W, the converters for K)
+      // ---- MMA-2: Y = (R_hi + R_lo)^T T^T
+      MDN_SPIN(r, ph);
+      tc_fence_after_sync();
+      MDN_MARK(c, kEvRSeen);
+      if (lead) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) umma_ts(tm + kColY, tm + kColX + a_col(k >> 2, k & 3), dT + 2 * (k & 3), id64, k > 0);
+        umma_commit(bar(bars.m2));
+      }
+      MDN_MARK(c, kEvM2Issued);
+      // ---- MMA-3': Z += V~^T W^T, V~ read as tf32 from the accumulator MMA-2 has just filled
+      if (write_o) {
+        MDN_SPIN(m2, ph);
+        MDN_SPIN(oi, ph);
+        tc_fence_after_sync();
+        if (lead) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            umma_ts_tf32(tm + kColZ, tm + kColY + 8 * j, dW + (uint64_t)((j >> 2) * 512 + (j & 3) * 2), id64_tf32, true);
+          umma_commit(bar(bars.mo));
+        }
+        MDN_MARK(c, kEvMoIssued);
+      }
+      // ---- MMA-3: P += [wS V~ | -wM V~]^T K   (K tile read MN-major: N = dk, K = tokens)
+      MDN_SPIN(v, ph);
+      tc_fence_after_sync();
+      MDN_MARK(c, kEvVSeen);
+      if (lead) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          umma_ts(tm + kColP, tm + kColX + a_col(k >> 2, k & 3), dKmn + 128 * (k & 3), id128_mn, true);
+        umma_commit(bar(bars.m3[s]));
+      }
+      MDN_MARK(c, kEvM3Issued);
+      if (c == 0) { MDN_NOW(3); }
+      if (c == nch - 1) { MDN_NOW(4); }
+      if (c + 1 < nch) {
+        MDN_SPIN(k32[s ^ 1], ((c + 1) >> 1) & 1);
+        MDN_SPIN(m3[s], (c >> 1) & 1);
+        tc_fence_after_sync();
+        mma1x(c + 1);
+      }
+    }
+  } else if (warp >= kWarpCvt && warp < kWarpOut) {
+    // ================================================================== converter warps
+    // fp32 copies of the K tile (from the stage, into the buffer that the chunk before the previous one has left) and of the Q tile.
+    // A thread takes half a token row (rows across the lanes: minimal wavefronts in both swizzled layouts): the loads first.
+    const uint32_t t128 = static_cast<uint32_t>(tid - kWarpCvt * 32), row = t128 & 63, half = t128 >> 6, sw = row & 7;
+    auto load8 = [&](uint4 (&u)[8], uint32_t tile) {   // dk half `half`: [64 rows x 128 B]
+#pragma unroll
+      for (uint32_t i = 0; i < 8; ++i)
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(u[i].x), "=r"(u[i].y), "=r"(u[i].z), "=r"(u[i].w)
+                     : "r"(tile + half * 8192 + row * 128 + ((i ^ sw) << 4)));
+    };
+    // piece i (8 of the half's 64 columns) of the fp32 copy: quarter 2 half + i / 4, 16-byte chunks 2 (i % 4), + 1 of its row
+    auto store4 = [&](uint32_t copy, uint32_t i, int e, uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3) {
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                   ::"r"(copy + (2 * half + (i >> 2)) * 8192 + row * 128 + ((((i & 3) * 2 + e) ^ sw) << 4)), "r"(x0), "r"(x1), "r"(x2), "r"(x3)
+                   : "memory");
+    };
+    auto store8 = [&](uint32_t copy, const uint4 (&u)[8]) {
+#pragma unroll
+      for (uint32_t i = 0; i < 8; ++i) {
+        store4(copy, i, 0, u[i].x << 16, u[i].x & 0xffff0000u, u[i].y << 16, u[i].y & 0xffff0000u);
+        store4(copy, i, 1, u[i].z << 16, u[i].z & 0xffff0000u, u[i].w << 16, u[i].w & 0xffff0000u);
+      }
+    };
+    for (int c = 0; c < nch; ++c) {
+      const int s = c & 1;
+      const uint32_t k_tile = s_base + kOffStage + s * kStageBytes + kStK;
+      MDN_WAIT(kfull[s], (c >> 1) & 1);
+      if (c >= 2) MDN_WAIT(mx[s], ((c - 2) >> 1) & 1);   // chunk c - 2's product has read this copy
+      MDN_MARK(c, kEvCvtK);
+      uint4 uk[8];
+      load8(uk, k_tile);
+      store8(s_base + kOffK32 + s * kK32Bytes, uk);
+      fence_proxy_async_smem();
+      warp_arrive(bars.k32[s]);
+      MDN_MARK(c, kEvCvtKDone);
+      if (write_o) {
+        MDN_WAIT(qfull, c & 1);
+        uint4 uq[8];
+        load8(uq, s_base + kOffQb);
+        warp_arrive(bars.qfree);
+        if (c > 0) MDN_WAIT(mz, (c - 1) & 1);             // the previous chunk's product has read the copy
+        MDN_MARK(c, kEvCvtQ);
+        if constexpr (kLayer) {
+          // fused q/k norm: the copy is q - d k (its 1/|q - d k| rides on the output terms' coefficients)
+#pragma unroll
+          for (uint32_t i = 0; i < 8; ++i) {
+            const uint32_t wk[4] = {uk[i].x, uk[i].y, uk[i].z, uk[i].w}, wq[4] = {uq[i].x, uq[i].y, uq[i].z, uq[i].w};
+            uint32_t f[8];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              f[2 * e] = __float_as_uint(fmaf(-qk_dh, __uint_as_float(wk[e] << 16), __uint_as_float(wq[e] << 16)));
+              f[2 * e + 1] = __float_as_uint(fmaf(-qk_dh, __uint_as_float(wk[e] & 0xffff0000u), __uint_as_float(wq[e] & 0xffff0000u)));
+            }
+            store4(s_base + kOffQ32, i, 0, f[0], f[1], f[2], f[3]);
+            store4(s_base + kOffQ32, i, 1, f[4], f[5], f[6], f[7]);
+          }
+        } else {
+          store8(s_base + kOffQ32, uq);
+        }
+        fence_proxy_async_smem();
+        warp_arrive(bars.q32);
+        MDN_MARK(c, kEvCvtQDone);
+      }
+    }
+  } else if (kLayer && warp >= kWarpOut) {
+    // ================================================================== output warps
+    // Fused output step, second half: y = sigmoid(g) * o / sqrt(mean_d o^2 + eps) * w_d, the mean over both CTAs' columns.  Two
+    // threads per token, 32 of its 64 values each, in eight 16-byte pieces whose places rotate with the token (no bank is
+    // touched twice by eight neighbouring lanes).  The whole fp32 tile is in registers before anything is written over it.
+    if (post) {
+      const int t128 = tid - kWarpOut * 32, row = t128 >> 1, part = t128 & 1;
+      const uint32_t peer_bar[2] = {map_to_cta(bar(bars.peer[0]), peer_rank), map_to_cta(bar(bars.peer[1]), peer_rank)};
+      const uint32_t peer_at = map_to_cta(smem_u32(&peer_ss[0][row]), peer_rank);
+      const int swz = ((row >> 1) & 3) * 2;   // (the epilogue's store rotates a row's 16-byte pieces by this)
+      int place[8], col[8];                   // a piece's place in the row, its first column
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        place[i] = 2 * ((i + row) & 7) + part;
+        col[i] = 4 * (place[i] ^ swz);
+      }
+      for (int c = 0; c < nch; ++c) {
+        const int s = c & 1;
+        const uint32_t ph2 = (c >> 1) & 1;
+        uint8_t* const out = smem + kOffStage + s * kStageBytes + kStOut;
+        const int n = min(C, sq.len - c * C);
+        const __nv_bfloat16* gp = static_cast<const __nv_bfloat16*>(a.post_g) + ((size_t)(sq.tok0 + c * C + row) * H + h) * kD + v0;
+        uint2 gate[8];   // before the wait
+#pragma unroll
+        for (int i = 0; i < 8; ++i) gate[i] = row < n ? __ldg(reinterpret_cast<const uint2*>(gp + col[i])) : make_uint2(0u, 0u);
+        uint32_t good = mbar_wait(bar(bars.pn[s]), ph2, abortp) ? 1u : 0u;
+        __syncwarp();
+        MDN_MARK(c, kEvPn);
+        float4 ov[8];
+        float ss = 0.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          ov[i] = *reinterpret_cast<const float4*>(out + row * kN * 4 + place[i] * 16);
+          ss = fmaf(ov[i].x, ov[i].x, fmaf(ov[i].y, ov[i].y, fmaf(ov[i].z, ov[i].z, fmaf(ov[i].w, ov[i].w, ss))));
+        }
+        ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+        if (part == 0) {
+          st_cluster_f32(peer_at + s * (uint32_t)sizeof(peer_ss[0]), ss);
+          mbar_arrive_cluster(peer_bar[s]);
+        }
+        MDN_MARK(c, kEvSsSent);
+        if (!mbar_wait_cluster(bar(bars.peer[s]), ph2, abortp)) good = 0;
+        __syncwarp();
+        MDN_MARK(c, kEvPeer);
+        ss += *const_cast<volatile float*>(&peer_ss[s][row]);
+        const float rstd = rsqrtf(ss * (1.f / kD) + a.post_eps);
+        // the tile has been read by all four warps (the barrier carries the vote whether every wait has ended)
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\t"
+            "setp.ne.u32 q, %0, 0;\n\t"
+            "barrier.cta.red.and.pred p, 1, %1, q;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}\n"
+            : "+r"(good)
+            : "n"(kOutThreads)
+            : "memory");
+        if (good == 0) { ok = false; break; }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float4 wv = *reinterpret_cast<const float4*>(w_sm + col[i]);
+          const float g0 = __uint_as_float(gate[i].x << 16), g1 = __uint_as_float(gate[i].x & 0xffff0000u);
+          const float g2 = __uint_as_float(gate[i].y << 16), g3 = __uint_as_float(gate[i].y & 0xffff0000u);
+          const float y0 = ov[i].x * rstd * wv.x * sigmoid_fast(g0), y1 = ov[i].y * rstd * wv.y * sigmoid_fast(g1);
+          const float y2 = ov[i].z * rstd * wv.z * sigmoid_fast(g2), y3 = ov[i].w * rstd * wv.w * sigmoid_fast(g3);
+          if (sizeof(TO) == 4) {
+            *reinterpret_cast<float4*>(out + (row * kN + col[i]) * 4) = make_float4(y0, y1, y2, y3);
+          } else {   // 128-byte rows, swizzled as the store's tensor map has it (short chunks: plain rows)
+            uint2 pk;
+            pk.x = pack_bf16(y0, y1); pk.y = pack_bf16(y2, y3);
+            const int ch = (col[i] >> 3) ^ (n == C ? row & 7 : 0);
+            *reinterpret_cast<uint2*>(out + row * 128 + ch * 16 + (col[i] & 4) * 2) = pk;
+          }
+        }
+        fence_proxy_async_smem();
+        warp_arrive(bars.go[s]);
+        MDN_MARK(c, kEvGo);
+      }
+    }
+  } else if (warp < kEpiWarps) {
+    // ================================================================== epilogue warps
+    const int q4 = warp & 3, hf = warp >> 2;
+    const int r0 = kTok * hf;                      // first token of the per-token steps
+    const int row = lane >> 2, cp = 2 * (lane & 3);   // this thread's value columns 16 q4 + row, + 8; tokens r0 + 8 j + cp, + 1
+    const uint32_t tl = tmem + (static_cast<uint32_t>(q4 * 32) << 16);
+    // ldmatrix / stmatrix: lane's 16-byte row: token (lane & 7) + 8 (lane >> 4) of a pair of token groups, value columns 8 ((lane >> 3) & 1)
+    const uint32_t m_tok = r0 + (lane & 7) + 8 * (lane >> 4), m_ch = 2 * q4 + ((lane >> 3) & 1);
+    // whole states between global memory and the masters: one lane per row (lower sixteen: S, upper: M)
+    const int dg = v0 + 16 * q4 + (lane & 15);
+    const bool is_m = lane >= 16;
+    for (int c = 0; c <= nch; ++c) {
+      const int s = c & 1;
+      const uint32_t ph = c & 1, ph2 = (c >> 1) & 1;
+      const float* aj = reinterpret_cast<const float*>(smem + kOffAdj + s * kAdjBytes);
+      if (c == 0) {
+        // ---------------- the start state into the masters
+        const float* src = is_m ? rn.M0 : rn.S0;
+        const bool id = is_m ? rn.id_m : rn.id_s;
+#pragma unroll 1
+        for (int i = 0; i < 2; ++i) {
+          const int col0 = hf * 64 + i * 32;
+          uint32_t x[32];
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            x[j] = __float_as_uint(src ? __ldg(src + (size_t)(col0 + j) * kD + dg) : (id && col0 + j == dg ? 1.f : 0.f));
+          __syncwarp();
+          tmem_st32(tl + kColP + col0, x);
+        }
+        tmem_wait_st();
+        tc_fence_before_sync();
+        warp_arrive(bars.init);
+      }
+      if (c == nch) {
+        // ---------------- final states: [S; M] = G [Sh; Mh]  (the last chunk's MMA-3 was waited for below)
+        MDN_WAIT(fin, 0);
+        __syncwarp();
+        const float g11 = g_final[0], g12 = g_final[1], g22 = g_final[2];
+        tc_fence_after_sync();
+        float* dst = is_m ? rn.Mf : rn.Sf;
+#pragma unroll 1
+        for (int i = 0; i < 2; ++i) {
+          const int col0 = hf * 64 + i * 32;
+          uint32_t x[32];
+          tmem_ld32(tl + kColP + col0, x);
+          tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const float mine = __uint_as_float(x[j]), other = __shfl_xor_sync(0xffffffffu, mine, 16);
+            const float y = is_m ? g22 * mine : unscale_s(g11, mine, g12, other);
+            if (dst) dst[(size_t)(col0 + j) * kD + dg] = y;
+          }
+        }
+        break;
+      }
+      uint8_t* stg = smem + kOffStage + s * kStageBytes;
+      MDN_WAIT(full[s], ph2);
+      MDN_WAIT(adj[s], ph2);
+      __syncwarp();
+      // a vector's values for this thread's four token pairs
+      auto coef4 = [&](float2 (&f)[4], int vec) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) f[j] = *reinterpret_cast<const float2*>(aj + vec + r0 + 8 * j + cp);
+      };
+      auto pair = [](const uint32_t (&x)[16], int j, int e) { return make_float2(__uint_as_float(x[4 * j + 2 * e]), __uint_as_float(x[4 * j + 2 * e + 1])); };
+      // ---------------- EPI-1: R^T = V^T - cX .* (K S) + cY .* (K M)  -> bf16 hi, lo into X, in both halves of the lanes
+      {
+        // V and the coefficients are fetched before the wait
+        uint32_t vr[8];   // [pair of token groups][m]: token group 2 g + m / 2, value column half m % 2
+        if (!v_zero) {
+#pragma unroll
+          for (int g = 0; g < 2; ++g)
+            ldmatrix_x4_trans(s_base + kOffStage + s * kStageBytes + kStV + (m_tok + 16 * g) * 128 + ((m_ch ^ (m_tok & 7)) << 4), vr + 4 * g);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) vr[i] = 0u;
+        }
+        float2 cx[4], cy[4];
+        coef4(cx, kCx);   // (-cX)
+        coef4(cy, kCy);
+        MDN_WAIT(mx[s], ph2);
+        __syncwarp();
+        tc_fence_after_sync();
+        MDN_MARK(c, kEvMxSeen);
+        uint32_t xs[16], xm[16];
+        tmem_ld_16x256_x4(tl + kColX + r0, xs);
+        tmem_ld_16x256_x4(tl + kUpper + kColX + r0, xm);
+        tmem_wait_ld();
+        uint32_t hi[8], lo[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const uint32_t vw = vr[4 * (j >> 1) + 2 * (j & 1) + e];
+            float2 x = make_float2(__uint_as_float(vw << 16), __uint_as_float(vw & 0xffff0000u));
+            x = __ffma2_rn(cx[j], pair(xs, j, e), x);
+            x = __ffma2_rn(cy[j], pair(xm, j, e), x);
+            split_pack_bf16(x, hi[2 * j + e], lo[2 * j + e]);
+          }
+        // (the columns this warp has just read)
+        tmem_st_16x128_x4(tl + kColX + r0, hi);
+        tmem_st_16x128_x4(tl + kUpper + kColX + r0, hi);
+        tmem_st_16x128_x4(tl + kColX + r0 + kPk, lo);
+        tmem_st_16x128_x4(tl + kUpper + kColX + r0 + kPk, lo);
+        tmem_wait_st();
+      }
+      tc_fence_before_sync();
+      warp_arrive(bars.r);
+      MDN_MARK(c, kEvRArrive);
+      // ---------------- inter-chunk output terms cZ .* (Q S) + cU .* (Q M) into the lower lanes of Z, for MMA-3' to accumulate onto
+      // (the upper lanes accumulate onto Q M: nobody reads them)
+      if (write_o) {
+        float2 cz[4], cu[4];
+        coef4(cz, kCz);
+        coef4(cu, kCu);
+        MDN_WAIT(mz, ph);
+        __syncwarp();
+        tc_fence_after_sync();
+        uint32_t zs[16], zm[16];
+        tmem_ld_16x256_x4(tl + kColZ + r0, zs);
+        tmem_ld_16x256_x4(tl + kUpper + kColZ + r0, zm);
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const float2 o2 = __ffma2_rn(cz[j], pair(zs, j, e), __fmul2_rn(cu[j], pair(zm, j, e)));
+            zs[4 * j + 2 * e] = __float_as_uint(o2.x);
+            zs[4 * j + 2 * e + 1] = __float_as_uint(o2.y);
+          }
+        tmem_st_16x256_x4(tl + kColZ + r0, zs);
+        tmem_wait_st();
+        tc_fence_before_sync();
+        warp_arrive(bars.oi);
+        MDN_MARK(c, kEvOiArrive);
+      }
+      // ---------------- EPI-2: wS .* V~ | -wM .* V~ -> X as bf16 hi, lo.  Eager chunks: the masters take G' = D_c G first (under MMA-2;
+      // MMA-1 of this chunk, their last reader, is done) and the update is added in true coordinates.
+      const bool eager = aj[kLazy] == 0.f;
+      const float n11 = aj[kN11], n12 = aj[kN12], n22 = aj[kN22];
+              if (eager) {   // Sh <- n11 Sh + n12 Mh, Mh <- n22 Mh
+      #pragma unroll 1
+                for (int i = 0; i < 2; ++i) {
+                  const uint32_t col0 = kColP + hf * 64 + i * 32;
+                  uint32_t ps[16], pm[16];
+                  tmem_ld_16x256_x4(tl + col0, ps);
+                  tmem_ld_16x256_x4(tl + kUpper + col0, pm);
+                  tmem_wait_ld();
+      #pragma unroll
+                  for (int j = 0; j < 16; ++j) {
+                    ps[j] = __float_as_uint(unscale_s(n11, __uint_as_float(ps[j]), n12, __uint_as_float(pm[j])));
+                    pm[j] = __float_as_uint(n22 * __uint_as_float(pm[j]));
+                  }
+                  tmem_st_16x256_x4(tl + col0, ps);
+                  tmem_st_16x256_x4(tl + kUpper + col0, pm);
+                }
+              }
+      {
+        float2 ws[4], wm[4];
+        coef4(ws, kWs);
+        coef4(wm, kWm);
+        MDN_WAIT(m2, ph);
+        __syncwarp();
+        tc_fence_after_sync();
+        MDN_MARK(c, kEvM2Seen);
+        uint32_t vt[16];
+        tmem_ld_16x256_x4(tl + kColY + r0, vt);
+        tmem_wait_ld();
+        uint32_t hi[8], lo[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) split_pack_bf16(__fmul2_rn(ws[j], pair(vt, j, e)), hi[2 * j + e], lo[2 * j + e]);
+        tmem_st_16x128_x4(tl + kColX + r0, hi);          // X is free: MMA-2 has consumed R
+        tmem_st_16x128_x4(tl + kColX + r0 + kPk, lo);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int e = 0; e < 2; ++e)
+            split_pack_bf16(__fmul2_rn(make_float2(-wm[j].x, -wm[j].y), pair(vt, j, e)), hi[2 * j + e], lo[2 * j + e]);
+        tmem_st_16x128_x4(tl + kUpper + kColX + r0, hi);
+        tmem_st_16x128_x4(tl + kUpper + kColX + r0 + kPk, lo);
+        tmem_wait_st();
+        tc_fence_before_sync();
+        warp_arrive(bars.v);
+        MDN_MARK(c, kEvVArrive);
+      }
+      // ---------------- the chunk's output tile (under MMA-3): Z -> [64 tokens x 64 value columns] over the stage's V (and T)
+      if (write_o) {
+        MDN_WAIT(mo, ph);
+        __syncwarp();
+        tc_fence_after_sync();
+        MDN_MARK(c, kEvMoSeen);
+        uint32_t u[16];
+        tmem_ld_16x256_x4(tl + kColZ + r0, u);
+        tmem_wait_ld();
+        tc_fence_before_sync();
+        warp_arrive(bars.zu);
+        if (post || sizeof(TO) == 4) {
+          // an fp32 tile; for the output warps a row's 16-byte pieces are rotated by its token pair (no bank is touched twice)
+          float* tile = reinterpret_cast<float*>(stg + kStOut);
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int t = r0 + 8 * j + cp + (e & 1), d = 16 * q4 + row + 8 * (e >> 1);
+              tile[t * kN + (post ? d ^ (((t >> 1) & 3) << 3) : d)] = __uint_as_float(u[4 * j + e]);
+            }
+        } else {
+          uint32_t pk[8];
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) pk[2 * j + e] = pack_bf16(__uint_as_float(u[4 * j + 2 * e]), __uint_as_float(u[4 * j + 2 * e + 1]));
+          const uint32_t swz = sq.len - c * C >= C ? m_tok & 7 : 0;   // (a short chunk leaves row by row)
+#pragma unroll
+          for (int g = 0; g < 2; ++g)
+            stmatrix_x4_trans(s_base + kOffStage + s * kStageBytes + kStOut + (m_tok + 16 * g) * 128 + ((m_ch ^ swz) << 4), pk + 4 * g);
+        }
+        fence_proxy_async_smem();
+        if (post) warp_arrive(bars.pn[s]);
+        MDN_MARK(c, kEvOutDone);
+      }
+      if (!post) warp_arrive(bars.go[s]);
+      if (c == nch - 1) MDN_WAIT(m3[s], ph2);   // the final states follow
+    }
+  }
+#undef MDN_WAIT
+#undef MDN_SPIN
+#undef MDN_MARK
+  if (warp == 0) { MDN_NOW(6); }
+
+  if (!ok && lane == 0) atomicCAS(a.status, kDevOk, kDevTimeout);
+  tc_fence_before_sync();
+  __syncthreads();
+  if constexpr (kLayer) cluster_sync_all();   // neither CTA's shared memory goes while the other may still write to it
+#ifdef MDN_DEBUG
+  if (warp == 0) { MDN_NOW(5); }
+  if (tline != nullptr && tid < 256) tline[(kTlFirst + (tid >> 5)) * 32 + (tid & 31)] = tl_sm[tid >> 5][tid & 31];
+#endif
+  if (warp == kWarpMma) {
+    __syncwarp();
+    tmem_dealloc(tmem, 512);
+  }
+}
+
+}  // namespace
+
+cudaError_t launch_chain_half(const Plan& pl, const ChainTf32Args& a, const ChainTensors& in, unsigned items, int* launches) {
+  const mdn_params& p = pl.p;
+  const uint64_t tokens = (uint64_t)p.B * p.T, mats = (uint64_t)pl.geom.num_slots * p.H, row = (uint64_t)p.H * kD;
+  CUtensorMap mq, mk, mv, mt, mw, mo;
+  const bool o_bf16 = p.o_dtype == MDN_BF16;
+  if (!encode_tma_2d_bf16(&mq, TmaMap2D{in.q, row, tokens, row * 2, 64, 64, true}) ||
+      !encode_tma_2d_bf16(&mk, TmaMap2D{in.k, row, tokens, row * 2, 64, 64, true}) ||
+      !encode_tma_2d_bf16(&mv, TmaMap2D{in.v, row, tokens, row * 2, kN, 64, true}) ||
+      !encode_tma_2d_bf16(&mt, TmaMap2D{pl.ws + pl.lay.off_T, 64, mats * C, 128, 64, 64, true}) ||
+      !encode_tma_2d(&mw, TmaMap2D{pl.ws + pl.lay.off_W, 64, mats * C, 256, 32, 64, true}, true) ||
+      !encode_tma_2d(&mo, TmaMap2D{a.o, row, tokens, row * (o_bf16 ? 2u : 4u), kN, 64, o_bf16}, !o_bf16))
+    return cudaErrorInvalidValue;
+  const bool layer = a.qk_on || a.post_on;
+  auto kern = layer ? (o_bf16 ? chain_half_kernel<__nv_bfloat16, true> : chain_half_kernel<float, true>)
+                    : (o_bf16 ? chain_half_kernel<__nv_bfloat16, false> : chain_half_kernel<float, false>);
+  cudaError_t e = allow_smem<(int)kSmemBytes>(kern);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl_cluster(layer ? 2 : 1, kern, dim3(2 * items), dim3(threads_of(layer)), kSmemBytes, pl.stream, a, mq, mk, mv, mt, mw, mo);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e == cudaSuccess) ++*launches;
+  return e;
+}
+
+}  // namespace mdn

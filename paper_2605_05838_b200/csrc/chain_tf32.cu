@@ -40,6 +40,7 @@
 #include <cstdlib>
 #include <cstring>
 
+#include "chain_tf32.cuh"
 #include "mdn_common.cuh"
 #include "tc_utils.cuh"
 
@@ -79,14 +80,8 @@ constexpr uint32_t kTxBytes = 2 * 16384 + 8192 + 16384 + kCoefBytes;
 constexpr uint32_t kTxW = 16384, kTxV = 16384;   // bytes of the W tile, of the V tile
 constexpr uint32_t kStOut = kStV;       // the finished output tile: V area (bf16), V + T + half of W (fp32); all dead by then
 constexpr uint32_t kOffAdj = kOffStage + 2 * kStageBytes;
-constexpr uint32_t kAdjBytes = 2048;
 constexpr uint32_t kSmemBytes = kOffAdj + 2 * kAdjBytes + 1024;
 static_assert(kStCoef + kCoefBytes <= kStageBytes && kSmemBytes <= 232448, "shared-memory layout");
-
-// per-chunk block the producer warp publishes (float indices)
-enum Adj : int { kCx = 0, kCy = 64, kCz = 128, kCu = 192, kWs = 256, kWm = 320, kN11 = 384, kN12, kN22, kLazy };
-constexpr float kLazyMin = 5.421010862427522e-20f;   // 2^-64: smallest g11', g22' a lazy chunk may leave
-constexpr float kLazyMix = 1.f;                      // largest |g12'| / g22' (beyond it the two hat terms of S cancel too much)
 
 // tensor memory columns (512 x 128 lanes x 32 bit)
 constexpr uint32_t kColS = 0, kColM = 128, kColX = 256, kColZ = 320, kColY = 384, kColU = 448;
@@ -114,40 +109,6 @@ struct Bars {
   uint64_t pn[2];     // fused output step: a stage's fp32 tile is staged                     (256)
 };
 
-struct Args {
-  ChunkGeom g;
-  const float* coef;
-  const float* S0;
-  const float* M0;
-  void* o;
-  float* Sf;
-  float* Mf;
-  int32_t* status;
-  float scale;
-  // parallel inter-chunk scan (seg_G = 0: off, one CTA walks all chunks of its chain)
-  int seg_G;
-  int seg_phase;
-  int seg_first, seg_mid, seg_least;   // see seg_chunks
-  float* seg_E;
-  float* seg_Psi;
-  float* seg_PhiS;
-  float* seg_PhiM;
-  long long* timeline;   // debug builds: CTA 0 writes clock64() at [chunk * 32 + event]
-  // layer operations (Section 3.3), kLayer instantiation only
-  int qk_on;             // q <- L2Norm(q - d k), k <- L2Norm(k): 1/|k|, 1/|q - d k| arrive as coefficient vectors 6, 7
-  const float* qk_d;     // [H] or NULL
-  int post_on;           // o <- sigmoid(g) * RMSNorm(o) * w in the output step
-  const float* post_w;   // [dv] or NULL
-  const void* post_g;    // [B,T,H,dv] bf16
-  float post_eps;
-};
-
-__device__ __forceinline__ float sigmoid_fast(float x) {
-  float t;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(0.5f * x));
-  return fmaf(0.5f, t, 0.5f);
-}
-
 enum Ev : int { kEvMma1 = 0, kEvM1Seen, kEvRArrive, kEvOiArrive, kEvM2Seen, kEvV1Arrive, kEvOutDone, kEvM3Seen, kEvRSeen,
                 kEvV1Seen, kEvCvtStart, kEvCvtDone, kEvTmaIssued, kEvStoresDone, kEvM2Own, kEvEager,
                 kEvXzIssued, kEvYuIssued, kEvM2Issued, kEvSIssued, kEvMIssued, kEvV1bSeen, kEvV1bArrive, kEvZuArrive, kEvMoIssued, kEvM3sOwn, kEvKqSeen, kEvLoopTop, kEvRArrive2, kEvV1Arrive2 };
@@ -161,7 +122,7 @@ template <> __device__ __forceinline__ void stage_o<__nv_bfloat16>(uint8_t* tile
 }
 
 template <typename TO, bool kLayer>
-__global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const Args a, const __grid_constant__ CUtensorMap map_q,
+__global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const ChainTf32Args a, const __grid_constant__ CUtensorMap map_q,
                                                                 const __grid_constant__ CUtensorMap map_k,
                                                                 const __grid_constant__ CUtensorMap map_v,
                                                                 const __grid_constant__ CUtensorMap map_t,
@@ -177,62 +138,19 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int H = a.g.H;
-  // ---- work item: which chain, which segment of it, which kind of run
-  int chain = blockIdx.x, seg = 0, run = 0;   // run 0: the real thing; 1: Psi; 2: Phi from (I, 0); 3: Phi from (0, I)
-  if (a.seg_G > 0) {
-    if (a.seg_phase == 1) {   // the first segments (the longest runs) lead
-      const int chains = a.g.num_seqs * H, items = 3 * (a.seg_G - 2), w = (int)blockIdx.x - chains;
-      if (w >= 0) {
-        chain = w / items;
-        seg = 1 + (w % items) / 3;
-        run = 1 + (w % items) % 3;
-      }
-    } else {
-      chain = blockIdx.x / (a.seg_G - 1);
-      seg = 1 + blockIdx.x % (a.seg_G - 1);
-    }
-  }
-  const int seq = chain / H, h = chain % H;
   // Coefficients, T and W come from the previous kernel, which lets this one in before it has finished (intra_mma.cu): only
   // the producer warp waits, in front of its first load of those.  Everything else read here (the call's inputs, the chunk
   // map) was complete before that kernel could let anybody in.  Segment states come from the kernel just before this one.
   const bool early = a.seg_G == 0;
   if (!early) grid_dependency_wait();
-  SeqInfo sq = seq_info(a.g, seq);
-  if (a.seg_G > 0) {        // restrict the view to this segment's chunks
-    const int2 span = seg_chunks(a.g, sq.nchunks, SegSplitArgs{a.seg_G, a.seg_first, a.seg_mid, a.seg_least}, seg);
-    const int cb = span.x, ce = span.y;
-    sq.slot0 += cb;
-    sq.tok0 += cb * C;
-    sq.len = (ce > cb) ? min(sq.len - cb * C, (ce - cb) * C) : 0;
-    sq.nchunks = ce - cb;
-  }
-  const int nch = sq.nchunks;
-  const size_t st_off = (size_t)chain * kD * kD;
-  // ---- where the start state comes from, where the end state goes, whether V counts, whether o is written
-  const float* S0p = a.S0 ? a.S0 + st_off : nullptr;
-  const float* M0p = a.M0 ? a.M0 + st_off : nullptr;
-  float* Sfp = a.Sf ? a.Sf + st_off : nullptr;
-  float* Mfp = a.Mf ? a.Mf + st_off : nullptr;
-  bool id_s = false, id_m = false, v_zero = false, write_o = true;
-  if (a.seg_G > 0) {
-    constexpr size_t kMat = (size_t)kD * kD;
-    auto e_ptr = [&](int gi, int which) { return a.seg_E + (((size_t)chain * (a.seg_G - 1) + gi) * 2 + which) * kMat; };
-    if (run == 0) {
-      if (seg > 0) { S0p = e_ptr(seg - 1, 0); M0p = e_ptr(seg - 1, 1); }
-      if (seg < a.seg_G - 1) {
-        Sfp = (seg == 0) ? e_ptr(0, 0) : nullptr;
-        Mfp = (seg == 0) ? e_ptr(0, 1) : nullptr;
-      }
-    } else {
-      write_o = false;
-      S0p = M0p = nullptr;
-      id_s = run == 2; id_m = run == 3; v_zero = run >= 2;
-      float* base = (run == 1 ? a.seg_Psi : run == 2 ? a.seg_PhiS : a.seg_PhiM) +
-                    (((size_t)chain * (a.seg_G - 2) + (seg - 1)) * 2) * kMat;
-      Sfp = base; Mfp = base + kMat;
-    }
-  }
+  const ChainRun rn = chain_run(a, (int)blockIdx.x);
+  const SeqInfo sq = rn.sq;
+  const int h = rn.h, nch = sq.nchunks;
+  const float* const S0p = rn.S0;
+  const float* const M0p = rn.M0;
+  float* const Sfp = rn.Sf;
+  float* const Mfp = rn.Mf;
+  const bool id_s = rn.id_s, id_m = rn.id_m, v_zero = rn.v_zero, write_o = rn.write_o;
 
   const uint32_t s_base = smem_u32(smem);
   const uint32_t b_full0 = smem_u32(&bars.full[0]), b_full1 = smem_u32(&bars.full[1]);
@@ -383,34 +301,7 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
           MDN_WAIT(fb, (c >> 1) & 1);
           float* aj = reinterpret_cast<float*>(smem + kOffAdj + s * kAdjBytes);
           const float* cf = reinterpret_cast<const float*>(smem + kOffStage + s * kStageBytes + kStCoef);
-          const float aC = cf[kAbar * C + C - 1], bC = cf[kB * C + C - 1], mC = cf[kMubar * C + C - 1];
-          const float n11 = __fmul_rn(aC, g11), n12 = __fsub_rn(__fmul_rn(aC, g12), __fmul_rn(bC, g22)), n22 = __fmul_rn(mC, g22);
-          const bool lazy = n11 >= kLazyMin && n22 >= kLazyMin && fabsf(n12) <= kLazyMix * n22;
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int t = 2 * lane + e;
-            const float ab = cf[kAbar * C + t], bb = cf[kB * C + t], pp = cf[kAlphaBPrev * C + t];
-            const float gs = cf[kGS * C + t], gm = cf[kGM * C + t];
-            // fused q/k norm: k^ = k / |k| scales the rows of K S, K M (vectors 2, 3, 4 carry that factor already),
-            // q^ = (q - d k) / |q - d k| those of the output terms (the converter warps subtract d k from the Q tile)
-            float cx, cy, cz, cu;
-            if constexpr (kLayer) {
-              const float rk = cf[kRk * C + t], sq_ = a.scale * cf[kRq * C + t];
-              cx = ab * rk * g11; cy = pp * g22 - ab * rk * g12;
-              cz = sq_ * (ab * g11); cu = sq_ * (ab * g12 - bb * g22);
-            } else {
-              cx = ab * g11; cy = pp * g22 - ab * g12;
-              cz = a.scale * cx; cu = a.scale * (ab * g12 - bb * g22);
-            }
-            aj[kCx + t] = -cx;     // stored negated: the epilogue's first step is one packed FMA per token pair
-            aj[kCy + t] = cy;
-            aj[kCz + t] = cz;
-            aj[kCu + t] = cu;
-            aj[kWs + t] = lazy ? (gs + (n12 / n22) * gm) / n11 : gs;
-            aj[kWm + t] = lazy ? gm / n22 : gm;
-          }
-          if (lane == 0) { aj[kN11] = n11; aj[kN12] = n12; aj[kN22] = n22; aj[kLazy] = lazy ? 1.f : 0.f; }
-          if (lazy) { g11 = n11; g12 = n12; g22 = n22; } else { g11 = 1.f; g12 = 0.f; g22 = 1.f; }
+          publish_coefs<kLayer>(cf, aj, a.scale, lane, g11, g12, g22);
           mbar_arrive(s ? b_adj1 : b_adj0);
         } else if (c == nch) {
           if (early && nch == 0) grid_dependency_wait();   // (every CTA ends after the previous kernel has)
@@ -741,7 +632,7 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             const float sv = __uint_as_float(sr[j]), mv = __uint_as_float(mr[j]);
-            if (Sfp) Sfp[(size_t)(col0 + j) * kD + d] = g11 * sv + g12 * mv;
+            if (Sfp) Sfp[(size_t)(col0 + j) * kD + d] = unscale_s(g11, sv, g12, mv);
             if (Mfp) Mfp[(size_t)(col0 + j) * kD + d] = g22 * mv;
           }
         }
@@ -879,7 +770,7 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
             tmem_ld32(tl + kColM + col0, mr);
             tmem_wait_ld();
 #pragma unroll
-            for (int j = 0; j < 32; ++j) sr[j] = __float_as_uint(n11 * __uint_as_float(sr[j]) + n12 * __uint_as_float(mr[j]));
+            for (int j = 0; j < 32; ++j) sr[j] = __float_as_uint(unscale_s(n11, __uint_as_float(sr[j]), n12, __uint_as_float(mr[j])));
             tmem_st32(tl + kColS + col0, sr);
           }
         }
@@ -987,7 +878,7 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
   const bool o_bf16 = p.o_dtype == MDN_BF16;
   if (!encode_tma_2d(&mo, TmaMap2D{o, row, tokens, row * (o_bf16 ? 2u : 4u), 128, 64, false}, !o_bf16))
     return cudaErrorInvalidValue;
-  Args a;
+  ChainTf32Args a;
   a.g = pl.geom;
   a.coef = reinterpret_cast<const float*>(pl.ws + pl.lay.off_coef);
   a.S0 = S0; a.M0 = M0; a.o = o; a.Sf = Sf; a.Mf = Mf;
@@ -1005,6 +896,7 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
 #endif
   const unsigned chains = (unsigned)pl.geom.num_seqs * p.H;
   auto launch = [&](unsigned grid) -> cudaError_t {
+    if (!layer && 2 * grid <= (unsigned)kSms) return launch_chain_half(pl, a, ChainTensors{q, k, v}, grid, launches);
     auto kern = layer ? (o_bf16 ? chain_tf32_kernel<__nv_bfloat16, true> : chain_tf32_kernel<float, true>)
                       : (o_bf16 ? chain_tf32_kernel<__nv_bfloat16, false> : chain_tf32_kernel<float, false>);
     cudaError_t e = allow_smem<(int)kSmemBytes>(kern);

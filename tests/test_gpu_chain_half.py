@@ -1,0 +1,54 @@
+"""The forward's chain on two CTAs per chain (up to 74 runs at once) against the oracle and against the kernel with one CTA per
+chain, which a batch of 38 copies of the same rows (76 chains) takes."""
+import numpy as np
+import pytest
+
+import mdn_workloads as wl
+from helpers import rel_err, run_gpu, run_oracle, to_torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mdn():
+    import paper_2605_05838_b200 as m
+    m.lib()
+    return m
+
+
+# (tokens, preset): chunk edges, two and more chunks; preset F forgets fast: the masters are rescaled in every chunk
+CASES = [(T, "S") for T in (1, 63, 64, 65, 128, 200, 449)] + [(65, "F"), (333, "F")]
+
+
+@pytest.mark.parametrize("T,preset", CASES)
+def test_two_ctas_per_chain(mdn, T, preset):
+    """Both kernels make the same products in the same order; a last bit that differs can change what a tf32 operand truncates to
+    (2^-10 of one of 128 terms): 2e-3 of RMS between them, 2e-2 to the oracle as everywhere on this path.  A bf16 o may besides
+    differ by one place between them (2^-7 of the largest value) and carries its own rounding against the oracle."""
+    import torch
+    w = wl.Workload("half", B=1, T=T, H=2, dk=128, dv=128, dtype="bf16", init_state_std=0.2, seed=T, preset=preset)
+    inp = wl.make_inputs(w)
+    ref = run_oracle(inp)
+    t = to_torch(inp)
+    names = ("q", "k", "v", "beta", "log_alpha", "log_mu", "eta")
+    for o_dtype in (torch.float32, torch.bfloat16):
+        got = run_gpu(mdn, inp, o_dtype=o_dtype)
+        place = 0.0 if o_dtype == torch.float32 else 2.0 ** -7 * np.abs(ref[0]).max() / np.sqrt(np.mean(ref[0] ** 2))
+        assert rel_err(got[0], ref[0]) <= 2e-2 + place / 2 and max(rel_err(x, y) for x, y in zip(got[1:], ref[1:])) <= 2e-2
+        many = mdn.chunk_fwd(*(t[n].expand(38, *t[n].shape[1:]).contiguous() for n in names), scale=inp["scale"], o_dtype=o_dtype,
+                             initial_S=t["initial_S"].expand(38, -1, -1, -1).contiguous(),
+                             initial_M=t["initial_M"].expand(38, -1, -1, -1).contiguous())
+        for i, (x, y) in enumerate(zip(got, many)):
+            y = y.double().cpu().numpy()
+            assert rel_err(np.asarray(x), y[:1]) <= 2e-3 + (place if i == 0 else 0.0)
+            assert np.array_equal(y[:1], y[37:])
+
+
+def test_two_ctas_per_chain_packed(mdn):
+    """Short, empty-tailed and chunk-aligned sequences in one row, each with its own start state."""
+    lens = np.array([1, 64, 130, 63, 200])
+    w = wl.Workload("half_packed", B=1, T=int(lens.sum()), H=3, dk=128, dv=128, dtype="bf16", varlen=True, init_state_std=0.2, seed=5)
+    inp = wl.make_inputs(w, lengths=lens)
+    import torch
+    got, ref = run_gpu(mdn, inp, o_dtype=torch.float32), run_oracle(inp)
+    assert max(rel_err(x, y) for x, y in zip(got, ref)) <= 2e-2
