@@ -14,11 +14,15 @@
 //
 // Per chunk:  MMA-1x X = P K^T (P: both masters)  ->  EPI-1 R^T (bf16 hi + lo) into X  ->  MMA-2 Y = R^T T^T  ->  EPI-2 wS V~ | -wM V~
 //             (bf16 hi + lo) into X  ->  MMA-3 P += X K  ->  next chunk's MMA-1x.
-// Off that path: MMA-1z Z = P Q^T (under EPI-1), o_inter into Z (under MMA-2), MMA-3' Z += V~^T W^T (under EPI-2), output tile.
+// The rest is cut to fit the two gaps in which the tensor pipe would wait for the epilogue: MMA-1z Z = P Q^T in two halves, the first
+// under EPI-1, the second under EPI-2 (whole under EPI-1 it delayed MMA-2 by 0.4 k cycles); o_inter into Z behind EPI-2; MMA-3'
+// Z += V~^T W^T behind the NEXT chunk's MMA-1x; output tile under that chunk's MMA-2.  Z is double-buffered for that.
 //
 // What bounds a chunk: the serial chain of the three product groups (0.72 + 0.36 + 0.51 k cycles), their commit-to-wake latencies
-// and the two epilogue steps; the tensor pipe is busy about 60 % of it, the shared-memory port about as much (the fp32 K
-// and Q copies).  Registers and tensor memory (320 of 512 columns) are not the limit here.
+// and the two epilogue steps.  Registers, shared memory and tensor memory (448 of 512 columns) are not the limit here.
+// Two warps issue products: one those of the serial chain alone (three waits per chunk), one those of the output.  A wait in the
+// issuing warp costs 0.2 .. 0.4 k cycles even if its phase is long complete (one warp for all, with eight waits: 4.3 k cycles per
+// chunk).
 //
 // With the layer operations the RMSNorm of the output step sums over all 128 value columns: the two CTAs of a chain are a
 // thread-block cluster and exchange each token's sum of squares through distributed shared memory.
@@ -32,62 +36,59 @@ namespace {
 using namespace tc;
 
 constexpr int kD = 128, kN = 64;   // key columns; value columns of a CTA
-// Warps 0..7 epilogue (lane quarter = warp % 4, token half = warp / 4), 8 MMA issuer, 9 loads of K and Q, 10 coefficients, 11 output
-// stores and the loads behind them, 12..15 converters, with the layer operations 16..19 output step.  (With one producer
-// warp for all of it the coefficients came 0.45 k cycles before the epilogue needed them and the next K tile's copy 0.4 k late.)
-constexpr int kEpiWarps = 8, kWarpMma = 8, kWarpKq = 9, kWarpCoef = 10, kWarpTma = 11, kWarpCvt = 12, kCvtWarps = 4, kWarpOut = 16, kOutWarps = 4;
+// Warps 0..7 epilogue (lane quarter = warp % 4, token half = warp / 4), 8 the products of the state's serial chain, 9 loads and
+// coefficients, 10 the products of the output, 11 output stores, 12..15 converters, with the layer operations 16..19 output step.
+constexpr int kEpiWarps = 8, kWarpMma = 8, kWarpLoad = 9, kWarpMmaOut = 10, kWarpStore = 11, kWarpCvt = 12, kCvtWarps = 4, kWarpOut = 16, kOutWarps = 4;
 constexpr int threads_of(bool layer) { return (kWarpOut + (layer ? kOutWarps : 0)) * 32; }
-constexpr int kEpiThreads = kEpiWarps * 32, kCvtThreads = kCvtWarps * 32, kOutThreads = kOutWarps * 32;
+constexpr int kOutThreads = kOutWarps * 32;
 constexpr int kTok = 32, kPk = 16;   // tokens of an epilogue warp; their packed bf16 pairs
 
-// Shared memory (offsets from a 1024-byte aligned base).  The fp32 K copy is double-buffered: it is made as soon as the K tile
-// has landed, whatever the chain is at.  The fp32 Q copy is single (its readers are done early in a chunk).
-constexpr uint32_t kOffK32 = 0, kK32Bytes = 32768;   // [64 tokens x 128 dk] fp32: four dk quarters x [64 rows x 128 B], swizzled
-constexpr uint32_t kOffQ32 = 65536;
-constexpr uint32_t kOffQb = 98304;                   // bf16 Q tile waiting for its copy: two dk halves x [64 rows x 128 B]
-constexpr uint32_t kOffStage = 114688;
+// Shared memory (offsets from a 1024-byte aligned base)
+constexpr uint32_t kOffK32 = 0, kOffQ32 = 32768;     // fp32 K and Q [64 tokens x 128 dk]: four dk quarters x [64 rows x 128 B], swizzled
+constexpr uint32_t kOffQb = 65536;                   // bf16 Q tile waiting for its copy: two dk halves x [64 rows x 128 B]
+constexpr uint32_t kOffOut = 81920, kOutBytes = 16384;   // two output tiles (bf16 or fp32), by the chunk's parity
+constexpr uint32_t kOffStage = 114688;               // two stages, by the chunk's parity
 constexpr uint32_t kStK = 0, kStV = 16384, kStT = 24576, kStW = 32768, kStCoef = 49152;
 constexpr uint32_t kCoefBytes = kChainCoefs * C * sizeof(float);
 constexpr uint32_t kStageBytes = 51200;
 constexpr uint32_t kTxK = 16384, kTxV = 8192, kTxT = 8192, kTxW = 16384;
-constexpr uint32_t kStOut = kStV;                    // the finished output tile: V area (bf16), V + T (fp32); both dead by then
 constexpr uint32_t kOffAdj = kOffStage + 2 * kStageBytes;
 constexpr uint32_t kSmemBytes = kOffAdj + 2 * kAdjBytes + 1024;
 static_assert(kStCoef + kCoefBytes <= kStageBytes && kSmemBytes <= kSmemOptin - 4096, "shared-memory layout");
 
-// tensor memory columns: masters P (lanes: S^T | M^T), X, Z, Y
-constexpr uint32_t kColP = 0, kColX = 128, kColZ = 192, kColY = 256;
+// tensor memory columns: masters P (lanes: S^T | M^T), X, two Y, two Z (by the chunk's parity)
+constexpr uint32_t kColP = 0, kColX = 128, kColY = 192, kColZ = 320;
 constexpr uint32_t kUpper = 16u << 16;               // the upper sixteen lanes of a warp's quarter: M
 
 // A barrier that a waiter could fall a whole phase behind comes in pairs, by the chunk's parity.
 struct Bars {
-  uint64_t kfull[2];  // bf16 K tile of a stage landed                                    (1 + tx bytes)
-  uint64_t full[2];   // V, T, W of a stage landed                                        (1 + tx bytes)
-  uint64_t cfull[2];  // coefficient vectors of a stage landed                            (1 + tx bytes)
+  uint64_t kfull[2];  // bf16 K and V tiles of a stage landed                             (1 + tx bytes)
+  uint64_t full[2];   // T, W, coefficient vectors                                        (1 + tx bytes)
   uint64_t qfull;     // bf16 Q tile landed                                               (1 + tx bytes)
   uint64_t qfree;     // ... and read                                                     (4 warps)
-  uint64_t k32[2];    // fp32 K copy written                                              (4 warps)
+  uint64_t xr;        // MMA-1x may start: fp32 K copy written, masters updated           (4 warps + commit)
   uint64_t q32;       // fp32 Q copy written                                              (4 warps)
-  uint64_t adj[2];    // a chunk's coefficient block written                              (1)
+  uint64_t adj[2];    // a chunk's coefficient block written, its T and W landed          (1)
   uint64_t fin;       // G after the last chunk written                                   (1)
   uint64_t init;      // masters of chunk 0 stored                                        (8 warps)
-  uint64_t mx[2];     // X done: the fp32 K copy is free too                              (commit)
+  uint64_t mx;        // X done: the fp32 K copy is free too                              (commit)
   uint64_t mz;        // Z done: the fp32 Q copy is free too                              (commit)
   uint64_t r;         // EPI-1 done: R^T in X                                             (8 warps)
   uint64_t m2;        // V~ in Y                                                          (commit)
   uint64_t oi;        // inter-chunk output terms in Z                                    (8 warps)
-  uint64_t v;         // EPI-2 done: update operand in X (eager chunks: masters rescaled)  (8 warps)
-  uint64_t m3[2];     // masters updated: the stage's K tile is free too                  (commit)
+  uint64_t v;         // MMA-3 may start: update operand in X (eager chunks: masters rescaled), MMA-1z done  (8 warps + 1)
+  uint64_t m3[2];     // masters updated: the stage's K, V, T are free too                (commit)
   uint64_t mo;        // MMA-3' done                                                      (commit)
-  uint64_t zu;        // Z (the chunk's output) has been read                             (8 warps)
+  uint64_t zu[2];     // Z (the chunk's output) has been read: W and the coefficient block are free too  (8 warps)
   uint64_t go[2];     // the output tile is staged                                        (8 warps; fused output step 4)
+  uint64_t ofree[2];  // ... and read by its store                                        (1)
   uint64_t pn[2];     // fused output step: the fp32 tile is staged                       (8 warps)
-  uint64_t peer[2];   // ... and the other CTA's sums of squares have arrived             (64)
+  uint64_t peer[2];   // ... and the other CTA's sums of squares have arrived             (1 + 256 bytes)
 };
 
 enum Ev : int { kEvTop = 0, kEvXIssued, kEvZIssued, kEvRSeen, kEvM2Issued, kEvMoIssued, kEvVSeen, kEvM3Issued,
                 kEvMxSeen, kEvRArrive, kEvOiArrive, kEvM2Seen, kEvVArrive, kEvMoSeen, kEvOutDone, kEvCvtK, kEvCvtKDone, kEvCvtQ,
-                kEvCvtQDone, kEvTma, kEvAdj, kEvTmaKq, kEvStored, kEvPn, kEvSsSent, kEvPeer, kEvGo };
+                kEvCvtQDone, kEvTma, kEvAdj, kEvStored, kEvPn, kEvSsSent, kEvPeer, kEvGo };
 
 template <typename TO, bool kLayer>
 __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const ChainTf32Args a, const __grid_constant__ CUtensorMap map_q,
@@ -108,7 +109,7 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int H = a.g.H;
   // Coefficients, T and W come from the previous kernel, which lets this one in before it has finished (intra_mma.cu): only
-  // the two warps that load those wait.  Everything else read here (the call's inputs, the chunk
+  // the warp that loads those waits.  Everything else read here (the call's inputs, the chunk
   // map) was complete before that kernel could let anybody in.  Segment states come from the kernel just before this one.
   const bool early = a.seg_G == 0;
   if (!early) grid_dependency_wait();
@@ -135,22 +136,20 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
     abort_flag = 0;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      mbar_init(bar(bars.kfull[i]), 1); mbar_init(bar(bars.full[i]), 1); mbar_init(bar(bars.cfull[i]), 1);
-      mbar_init(bar(bars.k32[i]), kCvtWarps); mbar_init(bar(bars.adj[i]), 1);
-      mbar_init(bar(bars.mx[i]), 1); mbar_init(bar(bars.m3[i]), 1);
-      mbar_init(bar(bars.go[i]), post ? kOutWarps : kEpiWarps);
-      mbar_init(bar(bars.pn[i]), kEpiWarps); mbar_init(bar(bars.peer[i]), C);
+      mbar_init(bar(bars.kfull[i]), 1); mbar_init(bar(bars.full[i]), 1);
+      mbar_init(bar(bars.adj[i]), 1); mbar_init(bar(bars.m3[i]), 1); mbar_init(bar(bars.zu[i]), kEpiWarps);
+      mbar_init(bar(bars.go[i]), post ? kOutWarps : kEpiWarps); mbar_init(bar(bars.ofree[i]), 1);
+      mbar_init(bar(bars.pn[i]), kEpiWarps); mbar_init(bar(bars.peer[i]), 1);
     }
-    mbar_init(bar(bars.qfull), 1); mbar_init(bar(bars.qfree), kCvtWarps); mbar_init(bar(bars.q32), kCvtWarps);
+    mbar_init(bar(bars.qfull), 1); mbar_init(bar(bars.qfree), kCvtWarps); mbar_init(bar(bars.q32), kCvtWarps); mbar_init(bar(bars.xr), kCvtWarps + 1);
     mbar_init(bar(bars.fin), 1); mbar_init(bar(bars.init), kEpiWarps);
-    mbar_init(bar(bars.mz), 1); mbar_init(bar(bars.m2), 1); mbar_init(bar(bars.mo), 1);
-    mbar_init(bar(bars.r), kEpiWarps); mbar_init(bar(bars.oi), kEpiWarps); mbar_init(bar(bars.v), kEpiWarps);
-    mbar_init(bar(bars.zu), kEpiWarps);
+    mbar_init(bar(bars.mx), 1); mbar_init(bar(bars.mz), 1); mbar_init(bar(bars.m2), 1); mbar_init(bar(bars.mo), 1);
+    mbar_init(bar(bars.r), kEpiWarps); mbar_init(bar(bars.oi), kEpiWarps); mbar_init(bar(bars.v), kEpiWarps + (write_o ? 1 : 0));
     mbar_fence_init();
   }
   if (kLayer && tid < kN) w_sm[tid] = (a.post_on && a.post_w) ? __ldg(a.post_w + v0 + tid) : 1.f;
   if (warp == kWarpMma) tmem_alloc(smem_u32(&tmem_slot), 512);
-  if (warp == kWarpTma && lane == 0) {
+  if (warp == kWarpLoad && lane == 0) {
     prefetch_tensormap(&map_q); prefetch_tensormap(&map_k); prefetch_tensormap(&map_v);
     prefetch_tensormap(&map_t); prefetch_tensormap(&map_w); prefetch_tensormap(&map_o);
   }
@@ -161,16 +160,16 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
   const uint32_t tmem = tmem_slot;
   bool ok = true;
   volatile int* abortp = &abort_flag;
-#define MDN_WAIT(b, par)                                    \
-  if (!mbar_wait(smem_u32(&bars.b), (par), abortp)) {       \
+#define MDN_WAIT(b, par)                                                            \
+  if (!warp_wait(smem_u32(&bars.b), (par), abortp)) { \
     ok = false;                                             \
     break;                                                  \
   }
-  // waits on the chain's critical path poll without suspending
-#define MDN_SPIN(b, par)                                    \
-  if (!mbar_wait_spin(smem_u32(&bars.b), (par), abortp)) {  \
-    ok = false;                                             \
-    break;                                                  \
+  // waits on the chain's critical path poll, in place (a call there costs 0.2 .. 0.4 k cycles)
+#define MDN_POLL(b, par)                                            \
+  if (!warp_poll(smem_u32(&bars.b), (par), abortp)) {               \
+    ok = false;                                                     \
+    break;                                                          \
   }
 #ifdef MDN_DEBUG
   // Stamps go to shared memory for the chunks kTlFirst .. kTlFirst + 7 and are copied out when the kernel ends.
@@ -199,20 +198,26 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
     tline[7] = smid;
   }
 #endif
-  if (warp == kWarpKq) {
-    // ================================================================== K and Q tiles, for the converters and MMA-3
-    // A stage's K tile is refilled (for chunk c + 2) as soon as MMA-3 has read it, the Q buffer as soon as it is converted.
+  if (warp == kWarpLoad) {
+    // ================================================================== loads, coefficients
+    // A stage's K, V and T tiles are refilled (for chunk c + 2) as soon as MMA-3 has read K, the Q buffer as soon as it is converted, W
+    // when the output it belongs to has been read.  A chunk's coefficient block is published when its T and W have landed too and the
+    // output that its Z held has been read: who waits for the block need not wait for those.
     int issued = 0;
+    float g11 = 1.f, g12 = 0.f, g22 = 1.f;
+#pragma unroll 1
     for (int c = 0; c < nch; ++c) {
-      const int s = c & 1, tok0 = sq.tok0 + c * C;
+      const int s = c & 1, tok0 = sq.tok0 + c * C, mat = (sq.slot0 + c) * H + h;
+      const uint32_t ph2 = (c >> 1) & 1;
       const uint32_t st = s_base + kOffStage + s * kStageBytes;
-      if (c >= 2) MDN_WAIT(m3[s], ((c - 2) >> 1) & 1);
+      if (c >= 2) MDN_WAIT(m3[s], ph2 ^ 1);
       if (lane == 0) {
-        mbar_arrive_expect_tx(bar(bars.kfull[s]), kTxK);
-        tma_load_2d(st + kStK, &map_k, h * kD, tok0, bar(bars.kfull[s]));
-        tma_load_2d(st + kStK + 8192, &map_k, h * kD + 64, tok0, bar(bars.kfull[s]));
+        const uint32_t fb = bar(bars.kfull[s]);
+        mbar_arrive_expect_tx(fb, kTxK + (v_zero ? 0u : kTxV));
+        tma_load_2d(st + kStK, &map_k, h * kD, tok0, fb);
+        tma_load_2d(st + kStK + 8192, &map_k, h * kD + 64, tok0, fb);
+        if (!v_zero) tma_load_2d(st + kStV, &map_v, h * kD + v0, tok0, fb);
       }
-      issued = c + 1;
       if (write_o) {
         if (c > 0) MDN_WAIT(qfree, (c - 1) & 1);
         if (lane == 0) {
@@ -220,110 +225,73 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
           tma_load_2d(s_base + kOffQb, &map_q, h * kD, tok0, bar(bars.qfull));
           tma_load_2d(s_base + kOffQb + 8192, &map_q, h * kD + 64, tok0, bar(bars.qfull));
         }
+        if (c >= 2) MDN_WAIT(zu[s], ph2 ^ 1);
       }
-      MDN_MARK(c, kEvTmaKq);
-    }
-    if (!ok && lane == 0) {   // giving up: let the copies already in flight land before the CTA exits
-      for (int c = max(0, issued - 2); c < issued; ++c)
-        for (uint32_t it = 0; it < (1u << 16) && !mbar_try_wait(bar(bars.kfull[c & 1]), (c >> 1) & 1); ++it) {}
-      for (int c = max(0, issued - 2); c < issued && write_o; ++c)   // (the last or the last but one is in flight)
-        for (uint32_t it = 0; it < (1u << 16) && !mbar_try_wait(bar(bars.qfull), c & 1); ++it) {}
-    }
-  } else if (warp == kWarpCoef) {
-    // ================================================================== coefficients: a chunk ahead of their use
-    int issued = 0;
-    float g11 = 1.f, g12 = 0.f, g22 = 1.f;
-    auto load = [&](int c) {   // (the stage's vectors have been read when its chunk's block is published)
-      if (c >= nch) return;
+      if (early && c == 0) { grid_dependency_wait(); MDN_NOW(1); }
       if (lane == 0) {
-        const uint32_t fb = bar(bars.cfull[c & 1]);
-        mbar_arrive_expect_tx(fb, kCoefBytes);
-        bulk_load(s_base + kOffStage + (c & 1) * kStageBytes + kStCoef, a.coef + (size_t)((sq.slot0 + c) * H + h) * MDN_NUM_COEF * C,
-                  kCoefBytes, fb);
+        const uint32_t fb = bar(bars.full[s]);
+        mbar_arrive_expect_tx(fb, kCoefBytes + kTxT + (write_o ? kTxW : 0u));
+        bulk_load(st + kStCoef, a.coef + (size_t)mat * MDN_NUM_COEF * C, kCoefBytes, fb);
+        tma_load_2d(st + kStT, &map_t, 0, mat * C, fb);
+        if (write_o) {
+          tma_load_2d(st + kStW, &map_w, 0, mat * C, fb);
+          tma_load_2d(st + kStW + 8192, &map_w, 32, mat * C, fb);
+        }
       }
       issued = c + 1;
-    };
-    if (early) grid_dependency_wait();
-    MDN_NOW(1);
-    load(0);
-    load(1);
-    for (int c = 0; c < nch; ++c) {
-      const int s = c & 1;
-      MDN_WAIT(cfull[s], (c >> 1) & 1);
-      if (c >= 2) MDN_WAIT(m3[s], ((c - 2) >> 1) & 1);   // chunk c - 2's block has been read
+      MDN_MARK(c, kEvTma);
+      MDN_WAIT(full[s], ph2);
       publish_coefs<kLayer>(reinterpret_cast<const float*>(smem + kOffStage + s * kStageBytes + kStCoef),
                             reinterpret_cast<float*>(smem + kOffAdj + s * kAdjBytes), a.scale, lane, g11, g12, g22);
       warp_arrive(bars.adj[s]);
       MDN_MARK(c, kEvAdj);
-      __syncwarp();
-      load(c + 2);
     }
+    if (early && nch == 0) grid_dependency_wait();   // (every CTA ends after the previous kernel has)
     if (ok) {
       if (lane == 0) {
         g_final[0] = g11; g_final[1] = g12; g_final[2] = g22;
         mbar_arrive(bar(bars.fin));
       }
-    } else if (lane == 0) {
-      for (int c = max(0, issued - 2); c < issued; ++c)
-        for (uint32_t it = 0; it < (1u << 16) && !mbar_try_wait(bar(bars.cfull[c & 1]), (c >> 1) & 1); ++it) {}
+    } else if (lane == 0) {   // giving up: let the copies already in flight land before the CTA exits
+#pragma unroll 1
+      for (int c = max(0, issued - 2); c <= issued; ++c) {   // (of chunk `issued` the first copies may have been issued)
+        uint32_t it = 0;
+#pragma unroll 1
+        while (it < (1u << 18) && !(mbar_try_wait(bar(bars.kfull[c & 1]), (c >> 1) & 1) &&
+                                    mbar_try_wait(bar(bars.full[c & 1]), (c >> 1) & 1) && (!write_o || mbar_try_wait(bar(bars.qfull), c & 1)))) ++it;
+      }
     }
-  } else if (warp == kWarpTma) {
-    // ================================================================== output stores, V, T, W tiles
-    // Stage s = c & 1 serves chunk c; its V, T, W are refilled for chunk c + 2 once the output tile staged over V and T has left.
-    int issued = 0;
-    if (early) grid_dependency_wait();
-    for (int c = 0; c < nch + 2; ++c) {
+  } else if (warp == kWarpStore) {
+    // ================================================================== output stores
+#pragma unroll 1
+    for (int c = 0; c < (write_o ? nch : 0); ++c) {
       const int s = c & 1;
-      const uint32_t st = s_base + kOffStage + s * kStageBytes;
-      if (c >= 2) {
-        const int co = c - 2;
-        MDN_WAIT(go[s], (co >> 1) & 1);
-        if (lane == 0) {
-          const int n = min(C, sq.len - co * C);
-          const int tok = sq.tok0 + co * C;
-          const uint32_t src = st + kStOut;
-          if (!write_o) {
-            // Psi / Phi runs of the parallel scan produce states only
-          } else if (n == C) {
-            tma_store_2d(&map_o, h * kD + v0, tok, src);
-          } else {   // short chunk: rows >= n belong to another sequence; one bulk copy per valid row (an unswizzled tile)
-            for (int r = 0; r < n; ++r)
-              bulk_store(static_cast<uint8_t*>(a.o) + (((size_t)(tok + r) * H + h) * kD + v0) * sizeof(TO),
-                         src + r * kN * (uint32_t)sizeof(TO), kN * (uint32_t)sizeof(TO));
-          }
-          tma_store_commit();
-          tma_store_wait_read();
+      MDN_WAIT(go[s], (c >> 1) & 1);
+      if (lane == 0) {
+        const int n = min(C, sq.len - c * C);
+        const int tok = sq.tok0 + c * C;
+        const uint32_t src = s_base + kOffOut + s * kOutBytes;
+        if (n == C) {
+          tma_store_2d(&map_o, h * kD + v0, tok, src);
+        } else {   // short chunk: rows >= n belong to another sequence; one bulk copy per valid row (an unswizzled tile)
+#pragma unroll 1
+          for (int r = 0; r < n; ++r)
+            bulk_store(static_cast<uint8_t*>(a.o) + (((size_t)(tok + r) * H + h) * kD + v0) * sizeof(TO),
+                       src + r * kN * (uint32_t)sizeof(TO), kN * (uint32_t)sizeof(TO));
         }
-        __syncwarp();
-        MDN_MARK(co, kEvStored);
+        tma_store_commit();
+        tma_store_wait_read();
+        mbar_arrive(bar(bars.ofree[s]));
       }
-      if (c < nch) {
-        if (lane == 0) {
-          const uint32_t fb = bar(bars.full[s]);
-          const int mat = (sq.slot0 + c) * H + h;
-          mbar_arrive_expect_tx(fb, kTxT + (write_o ? kTxW : 0u) + (v_zero ? 0u : kTxV));
-          if (!v_zero) tma_load_2d(st + kStV, &map_v, h * kD + v0, sq.tok0 + c * C, fb);
-          tma_load_2d(st + kStT, &map_t, 0, mat * C, fb);
-          if (write_o) {
-            tma_load_2d(st + kStW, &map_w, 0, mat * C, fb);
-            tma_load_2d(st + kStW + 8192, &map_w, 32, mat * C, fb);
-          }
-        }
-        __syncwarp();
-        MDN_MARK(c, kEvTma);
-        issued = c + 1;
-      }
+      __syncwarp();
+      MDN_MARK(c, kEvStored);
     }
-    if (lane == 0) {
-      for (int c = max(0, issued - 2); c < issued && !ok; ++c)
-        for (uint32_t it = 0; it < (1u << 16) && !mbar_try_wait(bar(bars.full[c & 1]), (c >> 1) & 1); ++it) {}
-      tma_store_wait_all();
-    }
+    if (lane == 0) tma_store_wait_all();
   } else if (warp == kWarpMma) {
-    // ================================================================== MMA issuer
+    // ================================================================== products of the serial chain
     // The whole warp walks the loop and waits (warp-uniform control flow and operands); one elected lane issues the products and
-    // the commits.  A product that reads what the one just before it accumulates waits for that one's commit: MMA-1x issued
-    // right behind MMA-3 read masters that lacked part of the update (o off by 3e-4 of its RMS), and was no faster.
+    // the commits.  A product that reads what another one accumulates waits for that one's commit: MMA-1x issued right behind
+    // MMA-3 read masters that lacked part of the update (o off by 3e-4 of its RMS), and was no faster.
     const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
     const uint32_t sb = __shfl_sync(0xffffffffu, s_base, 0);
     const bool lead = elect_one();
@@ -335,95 +303,113 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
     const uint32_t id64 = idesc_bf16(128, 64, false, false, false);
     const uint32_t id128_mn = idesc_bf16(128, 128, false, true, false);
     const uint32_t id64_tf32 = idesc_tf32(128, 64, false, false, false);
-    const uint64_t dK_0 = smem_desc_sw128(sb + kOffK32, 16, 1024), dK_1 = dK_0 + (kK32Bytes >> 4);   // + (j >> 2) * 8192 + (j & 3) * 32 bytes per K step
-    const uint64_t dQ = smem_desc_sw128(sb + kOffQ32, 16, 1024);
+    const uint64_t dK = smem_desc_sw128(sb + kOffK32, 16, 1024);   // + (j >> 2) * 8192 + (j & 3) * 32 bytes per K step
     const uint64_t dT_0 = smem_desc_sw128(sb + kOffStage + kStT, 16, 1024), dT_1 = dT_0 + (kStageBytes >> 4);
-    const uint64_t dW_0 = smem_desc_sw128(sb + kOffStage + kStW, 16, 1024), dW_1 = dW_0 + (kStageBytes >> 4);
     const uint64_t dKmn_0 = smem_desc_sw128(sb + kOffStage + kStK, 8192, 1024), dKmn_1 = dKmn_0 + (kStageBytes >> 4);
-    // ---- MMA-1x: X = P K^T (K S and K M)
-    auto mma1x = [&](int c) {
-      const uint64_t dK = (c & 1) ? dK_1 : dK_0;
+#pragma unroll 1
+    for (int c = 0; c < nch; ++c) {
+      const int s = c & 1;
+      const uint32_t ph = c & 1;
+      const uint64_t dT = s ? dT_1 : dT_0, dKmn = s ? dKmn_1 : dKmn_0;
+      if (c == 0) {
+        MDN_WAIT(init, 0);
+        if (lane == 0) mbar_arrive(bar(bars.xr));   // (in the place of a previous chunk's commit)
+        __syncwarp();
+      }
+      // ---- MMA-1x: X = P K^T (K S and K M)
+      MDN_POLL(xr, ph);
+      tc_fence_after_sync();
+      if (c == 0) { MDN_NOW(2); }
+      MDN_MARK(c, kEvTop);
       if (lead) {
 #pragma unroll
         for (int j = 0; j < 16; ++j)
           umma_ts_tf32(tm + kColX, tm + kColP + 8 * j, dK + (uint64_t)((j >> 2) * 512 + (j & 3) * 2), id64_tf32, j > 0);
-        umma_commit(bar(bars.mx[c & 1]));
+        umma_commit(bar(bars.mx));
       }
       MDN_MARK(c, kEvXIssued);
-    };
-    for (int c = 0; c < nch; ++c) {
-      const int s = c & 1;
-      const uint32_t ph = c & 1;
-      if (c == 0) {
-        MDN_WAIT(k32[0], 0);
-        MDN_WAIT(init, 0);
-        __syncwarp();
-        tc_fence_after_sync();
-        MDN_NOW(2);
-        mma1x(0);
-      }
-      const uint64_t dT = s ? dT_1 : dT_0, dW = s ? dW_1 : dW_0, dKmn = s ? dKmn_1 : dKmn_0;
-      MDN_MARK(c, kEvTop);
-      // ---- MMA-1z: Z = P Q^T (Q S and Q M), once the previous chunk's output has been read out of Z
-      if (write_o) {
-        MDN_SPIN(q32, ph);
-        MDN_SPIN(zu, ph ^ 1);
-        tc_fence_after_sync();
-        if (lead) {
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            umma_ts_tf32(tm + kColZ, tm + kColP + 8 * j, dQ + (uint64_t)((j >> 2) * 512 + (j & 3) * 2), id64_tf32, j > 0);
-          umma_commit(bar(bars.mz));
-        }
-        MDN_MARK(c, kEvZIssued);
-      }
-      // (T, W and the K tile of the stage have landed: the epilogue waited for V, which came with T and W, the converters for K)
       // ---- MMA-2: Y = (R_hi + R_lo)^T T^T
-      MDN_SPIN(r, ph);
+      MDN_POLL(r, ph);
       tc_fence_after_sync();
       MDN_MARK(c, kEvRSeen);
       if (lead) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) umma_ts(tm + kColY, tm + kColX + a_col(k >> 2, k & 3), dT + 2 * (k & 3), id64, k > 0);
+        for (int j = 0; j < 8; ++j)
+          umma_ts(tm + kColY + 64 * s, tm + kColX + a_col(j >> 2, j & 3), dT + 2 * (j & 3), id64, j > 0);
         umma_commit(bar(bars.m2));
       }
       MDN_MARK(c, kEvM2Issued);
-      // ---- MMA-3': Z += V~^T W^T, V~ read as tf32 from the accumulator MMA-2 has just filled
-      if (write_o) {
-        MDN_SPIN(m2, ph);
-        MDN_SPIN(oi, ph);
-        tc_fence_after_sync();
-        if (lead) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            umma_ts_tf32(tm + kColZ, tm + kColY + 8 * j, dW + (uint64_t)((j >> 2) * 512 + (j & 3) * 2), id64_tf32, true);
-          umma_commit(bar(bars.mo));
-        }
-        MDN_MARK(c, kEvMoIssued);
-      }
       // ---- MMA-3: P += [wS V~ | -wM V~]^T K   (K tile read MN-major: N = dk, K = tokens)
-      MDN_SPIN(v, ph);
+      MDN_POLL(v, ph);
       tc_fence_after_sync();
       MDN_MARK(c, kEvVSeen);
       if (lead) {
 #pragma unroll
         for (int k = 0; k < 8; ++k)
           umma_ts(tm + kColP, tm + kColX + a_col(k >> 2, k & 3), dKmn + 128 * (k & 3), id128_mn, true);
+        umma_commit(bar(bars.xr));
         umma_commit(bar(bars.m3[s]));
       }
       MDN_MARK(c, kEvM3Issued);
       if (c == 0) { MDN_NOW(3); }
       if (c == nch - 1) { MDN_NOW(4); }
-      if (c + 1 < nch) {
-        MDN_SPIN(k32[s ^ 1], ((c + 1) >> 1) & 1);
-        MDN_SPIN(m3[s], (c >> 1) & 1);
+    }
+  } else if (warp == kWarpMmaOut) {
+    // ================================================================== products of the output
+    // In the gaps of the serial chain: behind MMA-1x the previous chunk's MMA-3' and the first half of MMA-1z, behind MMA-2 the second
+    // half (eager chunks: both halves first, the masters are rescaled under MMA-2).
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t sb = __shfl_sync(0xffffffffu, s_base, 0);
+    const bool lead = elect_one();
+    const uint32_t id64_tf32 = idesc_tf32(128, 64, false, false, false);
+    const uint64_t dQ = smem_desc_sw128(sb + kOffQ32, 16, 1024);
+    const uint64_t dW_0 = smem_desc_sw128(sb + kOffStage + kStW, 16, 1024), dW_1 = dW_0 + (kStageBytes >> 4);
+#pragma unroll 1
+    for (int c = 0; c <= (write_o ? nch : -1); ++c) {
+      const int s = c & 1;
+      const uint32_t ph = c & 1, ph2 = (c >> 1) & 1;
+      if (c < nch) MDN_POLL(mx, ph);
+      // ---- MMA-3' of the previous chunk: Z += V~^T W^T, V~ read as tf32 from the accumulator of MMA-2 (the epilogue has waited for
+      // that one's commit)
+      if (c > 0) {
+        const uint64_t dW = s ? dW_0 : dW_1;
+        MDN_POLL(oi, ph ^ 1);
         tc_fence_after_sync();
-        mma1x(c + 1);
+        if (lead) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            umma_ts_tf32(tm + kColZ + 64 * (s ^ 1), tm + kColY + 64 * (s ^ 1) + 8 * j, dW + (uint64_t)((j >> 2) * 512 + (j & 3) * 2), id64_tf32, true);
+          umma_commit(bar(bars.mo));
+        }
+        MDN_MARK(c, kEvMoIssued);
       }
+      if (c == nch) break;
+      // ---- MMA-1z: Z = P Q^T (Q S and Q M)
+      MDN_POLL(q32, ph);
+      MDN_POLL(adj[s], ph2);
+      const bool eager = reinterpret_cast<const float*>(smem + kOffAdj + s * kAdjBytes)[kLazy] == 0.f;
+      tc_fence_after_sync();
+#pragma unroll 1
+      for (uint32_t half = 0; half < 2; ++half) {
+        if (half == 1 && !eager) MDN_POLL(m2, ph);
+        if (lead) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            umma_ts_tf32(tm + kColZ + 64 * s, tm + kColP + 64 * half + 8 * j, dQ + (uint64_t)(1024 * half + (j >> 2) * 512 + (j & 3) * 2),
+                         id64_tf32, half + j > 0);
+          if (half == 1) umma_commit(bar(bars.mz));
+        }
+        MDN_MARK(c, kEvZIssued);
+      }
+      if (!ok) break;
+      // MMA-3 may overwrite the masters (and MMA-2 of the next chunk but one what MMA-3' above has read)
+      MDN_POLL(mz, ph);
+      if (lane == 0) mbar_arrive(bar(bars.v));
+      __syncwarp();
     }
   } else if (warp >= kWarpCvt && warp < kWarpOut) {
     // ================================================================== converter warps
-    // fp32 copies of the K tile (from the stage, into the buffer that the chunk before the previous one has left) and of the Q tile.
+    // fp32 copies of the K and Q tiles, each as soon as the previous chunk's product has read the one before.
     // A thread takes half a token row (rows across the lanes: minimal wavefronts in both swizzled layouts): the loads first.
     const uint32_t t128 = static_cast<uint32_t>(tid - kWarpCvt * 32), row = t128 & 63, half = t128 >> 6, sw = row & 7;
     auto load8 = [&](uint4 (&u)[8], uint32_t tile) {   // dk half `half`: [64 rows x 128 B]
@@ -446,17 +432,18 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
         store4(copy, i, 1, u[i].z << 16, u[i].z & 0xffff0000u, u[i].w << 16, u[i].w & 0xffff0000u);
       }
     };
+#pragma unroll 1
     for (int c = 0; c < nch; ++c) {
       const int s = c & 1;
       const uint32_t k_tile = s_base + kOffStage + s * kStageBytes + kStK;
       MDN_WAIT(kfull[s], (c >> 1) & 1);
-      if (c >= 2) MDN_WAIT(mx[s], ((c - 2) >> 1) & 1);   // chunk c - 2's product has read this copy
+      if (c > 0) MDN_WAIT(mx, (c - 1) & 1);              // the previous chunk's product has read the copy
       MDN_MARK(c, kEvCvtK);
       uint4 uk[8];
       load8(uk, k_tile);
-      store8(s_base + kOffK32 + s * kK32Bytes, uk);
+      store8(s_base + kOffK32, uk);
       fence_proxy_async_smem();
-      warp_arrive(bars.k32[s]);
+      warp_arrive(bars.xr);
       MDN_MARK(c, kEvCvtKDone);
       if (write_o) {
         MDN_WAIT(qfull, c & 1);
@@ -490,45 +477,46 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
   } else if (kLayer && warp >= kWarpOut) {
     // ================================================================== output warps
     // Fused output step, second half: y = sigmoid(g) * o / sqrt(mean_d o^2 + eps) * w_d, the mean over both CTAs' columns.  Two
-    // threads per token, 32 of its 64 values each, in eight 16-byte pieces whose places rotate with the token (no bank is
-    // touched twice by eight neighbouring lanes).  The whole fp32 tile is in registers before anything is written over it.
+    // threads per token, 32 neighbouring values each, in four pieces of eight whose order and halves rotate with the token and the
+    // thread (eight neighbouring lanes touch every bank once).  The whole fp32 tile is in registers before anything is written
+    // over it.  Sums of squares go to the other CTA by st.async, which completes its barrier's bytes: a plain remote store and a
+    // releasing arrival waited 2 k cycles for this thread's outstanding loads.
     if (post) {
       const int t128 = tid - kWarpOut * 32, row = t128 >> 1, part = t128 & 1;
-      const uint32_t peer_bar[2] = {map_to_cta(bar(bars.peer[0]), peer_rank), map_to_cta(bar(bars.peer[1]), peer_rank)};
-      const uint32_t peer_at = map_to_cta(smem_u32(&peer_ss[0][row]), peer_rank);
-      const int swz = ((row >> 1) & 3) * 2;   // (the epilogue's store rotates a row's 16-byte pieces by this)
-      int place[8], col[8];                   // a piece's place in the row, its first column
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        place[i] = 2 * ((i + row) & 7) + part;
-        col[i] = 4 * (place[i] ^ swz);
-      }
+      const uint32_t peer_bar = map_to_cta(bar(bars.peer[0]), peer_rank), peer_at = map_to_cta(smem_u32(&peer_ss[0][row]), peer_rank);
+      const int swz = (row >> 1) & 3;   // (the epilogue's store rotates a row's pieces by this)
+#pragma unroll 1
       for (int c = 0; c < nch; ++c) {
         const int s = c & 1;
         const uint32_t ph2 = (c >> 1) & 1;
-        uint8_t* const out = smem + kOffStage + s * kStageBytes + kStOut;
+        uint8_t* const out = smem + kOffOut + s * kOutBytes;
         const int n = min(C, sq.len - c * C);
-        const __nv_bfloat16* gp = static_cast<const __nv_bfloat16*>(a.post_g) + ((size_t)(sq.tok0 + c * C + row) * H + h) * kD + v0;
-        uint2 gate[8];   // before the wait
+        const __nv_bfloat16* gp = static_cast<const __nv_bfloat16*>(a.post_g) + ((size_t)(sq.tok0 + c * C + row) * H + h) * kD + v0 + 32 * part;
+        auto piece = [&](int i) { return (i + row) & 3; };   // place of the i-th piece among the thread's four; its columns: 8 (place ^ swz)
+        uint4 gate[4];   // before the wait
 #pragma unroll
-        for (int i = 0; i < 8; ++i) gate[i] = row < n ? __ldg(reinterpret_cast<const uint2*>(gp + col[i])) : make_uint2(0u, 0u);
-        uint32_t good = mbar_wait(bar(bars.pn[s]), ph2, abortp) ? 1u : 0u;
+        for (int i = 0; i < 4; ++i)
+          gate[i] = row < n ? __ldg(reinterpret_cast<const uint4*>(gp + 8 * (piece(i) ^ swz))) : make_uint4(0u, 0u, 0u, 0u);
+        if (t128 == 0) mbar_arrive_expect_tx(bar(bars.peer[s]), C * (uint32_t)sizeof(float));
+        uint32_t good = warp_wait(bar(bars.pn[s]), ph2, abortp) ? 1u : 0u;
         __syncwarp();
         MDN_MARK(c, kEvPn);
-        float4 ov[8];
+        float4 ov[8];   // piece i: values 0..3 in ov[2 i], 4..7 in ov[2 i + 1]
         float ss = 0.f;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          ov[i] = *reinterpret_cast<const float4*>(out + row * kN * 4 + place[i] * 16);
+        for (int i = 0; i < 4; ++i) {
+          const float4* at = reinterpret_cast<const float4*>(out + row * kN * 4 + part * 128 + piece(i) * 32);
+          const float4 x = at[part], y = at[part ^ 1];
+          ov[2 * i] = part ? y : x;
+          ov[2 * i + 1] = part ? x : y;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
           ss = fmaf(ov[i].x, ov[i].x, fmaf(ov[i].y, ov[i].y, fmaf(ov[i].z, ov[i].z, fmaf(ov[i].w, ov[i].w, ss))));
-        }
         ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-        if (part == 0) {
-          st_cluster_f32(peer_at + s * (uint32_t)sizeof(peer_ss[0]), ss);
-          mbar_arrive_cluster(peer_bar[s]);
-        }
+        if (part == 0) st_async_f32(peer_at + s * (uint32_t)sizeof(peer_ss[0]), ss, peer_bar + s * 8);
         MDN_MARK(c, kEvSsSent);
-        if (!mbar_wait_cluster(bar(bars.peer[s]), ph2, abortp)) good = 0;
+        if (!warp_wait(bar(bars.peer[s]), ph2, abortp)) good = 0;
         __syncwarp();
         MDN_MARK(c, kEvPeer);
         ss += *const_cast<volatile float*>(&peer_ss[s][row]);
@@ -544,19 +532,24 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
             : "memory");
         if (good == 0) { ok = false; break; }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float4 wv = *reinterpret_cast<const float4*>(w_sm + col[i]);
-          const float g0 = __uint_as_float(gate[i].x << 16), g1 = __uint_as_float(gate[i].x & 0xffff0000u);
-          const float g2 = __uint_as_float(gate[i].y << 16), g3 = __uint_as_float(gate[i].y & 0xffff0000u);
-          const float y0 = ov[i].x * rstd * wv.x * sigmoid_fast(g0), y1 = ov[i].y * rstd * wv.y * sigmoid_fast(g1);
-          const float y2 = ov[i].z * rstd * wv.z * sigmoid_fast(g2), y3 = ov[i].w * rstd * wv.w * sigmoid_fast(g3);
+        for (int i = 0; i < 4; ++i) {
+          const int col = 32 * part + 8 * (piece(i) ^ swz);
+          const uint32_t gw[4] = {gate[i].x, gate[i].y, gate[i].z, gate[i].w};
+          const float o8[8] = {ov[2 * i].x, ov[2 * i].y, ov[2 * i].z, ov[2 * i].w, ov[2 * i + 1].x, ov[2 * i + 1].y, ov[2 * i + 1].z, ov[2 * i + 1].w};
+          float y[8];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            y[2 * e] = o8[2 * e] * rstd * w_sm[col + 2 * e] * sigmoid_fast(__uint_as_float(gw[e] << 16));
+            y[2 * e + 1] = o8[2 * e + 1] * rstd * w_sm[col + 2 * e + 1] * sigmoid_fast(__uint_as_float(gw[e] & 0xffff0000u));
+          }
           if (sizeof(TO) == 4) {
-            *reinterpret_cast<float4*>(out + (row * kN + col[i]) * 4) = make_float4(y0, y1, y2, y3);
+            float4* to = reinterpret_cast<float4*>(out + (row * kN + col) * 4);
+            to[0] = make_float4(y[0], y[1], y[2], y[3]);
+            to[1] = make_float4(y[4], y[5], y[6], y[7]);
           } else {   // 128-byte rows, swizzled as the store's tensor map has it (short chunks: plain rows)
-            uint2 pk;
-            pk.x = pack_bf16(y0, y1); pk.y = pack_bf16(y2, y3);
-            const int ch = (col[i] >> 3) ^ (n == C ? row & 7 : 0);
-            *reinterpret_cast<uint2*>(out + row * 128 + ch * 16 + (col[i] & 4) * 2) = pk;
+            const int ch = (col >> 3) ^ (n == C ? row & 7 : 0);
+            *reinterpret_cast<uint4*>(out + row * 128 + ch * 16) =
+                make_uint4(pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]), pack_bf16(y[4], y[5]), pack_bf16(y[6], y[7]));
           }
         }
         fence_proxy_async_smem();
@@ -575,231 +568,251 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
     // whole states between global memory and the masters: one lane per row (lower sixteen: S, upper: M)
     const int dg = v0 + 16 * q4 + (lane & 15);
     const bool is_m = lane >= 16;
+    // a coefficient vector's values for this thread's four token pairs
+    auto coef4 = [&](float2 (&f)[4], const float* aj, int vec) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) f[j] = *reinterpret_cast<const float2*>(aj + vec + r0 + 8 * j + cp);
+    };
+    auto pair = [](const uint32_t (&x)[16], int j, int e) { return make_float2(__uint_as_float(x[4 * j + 2 * e]), __uint_as_float(x[4 * j + 2 * e + 1])); };
+    // ---------------- inter-chunk output terms cZ .* (Q S) + cU .* (Q M) into the lower lanes of Z, for MMA-3' to accumulate onto
+    // (the upper lanes accumulate onto Q M: nobody reads them); false: a wait ran out
+    auto inter = [&](int c) -> bool {
+      const float* aj = reinterpret_cast<const float*>(smem + kOffAdj + (c & 1) * kAdjBytes);
+      const uint32_t zc = tl + kColZ + 64 * (c & 1) + r0;
+      float2 cz[4], cu[4];
+      coef4(cz, aj, kCz);
+      coef4(cu, aj, kCu);
+      if (!warp_wait(bar(bars.mz), c & 1, abortp)) return false;
+      __syncwarp();
+      tc_fence_after_sync();
+      uint32_t zs[16], zm[16];
+      tmem_ld_16x256_x4(zc, zs);
+      tmem_ld_16x256_x4(zc + kUpper, zm);
+      tmem_wait_ld();
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float2 o2 = __ffma2_rn(cz[j], pair(zs, j, e), __fmul2_rn(cu[j], pair(zm, j, e)));
+          zs[4 * j + 2 * e] = __float_as_uint(o2.x);
+          zs[4 * j + 2 * e + 1] = __float_as_uint(o2.y);
+        }
+      tmem_st_16x256_x4(zc, zs);
+      tmem_wait_st();
+      tc_fence_before_sync();
+      warp_arrive(bars.oi);
+      MDN_MARK(c, kEvOiArrive);
+      return true;
+    };
+    // ---------------- a chunk's output: Z -> [64 tokens x 64 value columns] tile in shared memory
+    auto output = [&](int c) -> bool {
+      const int s = c & 1;
+      if (!warp_wait(bar(bars.mo), c & 1, abortp)) return false;
+      __syncwarp();
+      tc_fence_after_sync();
+      MDN_MARK(c, kEvMoSeen);
+      uint32_t u[16];
+      tmem_ld_16x256_x4(tl + kColZ + 64 * s + r0, u);
+      tmem_wait_ld();
+      tc_fence_before_sync();
+      warp_arrive(bars.zu[s]);
+      if (c >= 2 && !warp_wait(bar(bars.ofree[s]), ((c - 2) >> 1) & 1, abortp)) return false;
+      __syncwarp();
+      if (post || sizeof(TO) == 4) {
+        // an fp32 tile; for the output warps a row's pieces of eight values are rotated by its token pair (no bank is touched twice)
+        float* tile = reinterpret_cast<float*>(smem + kOffOut + s * kOutBytes);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int t = r0 + 8 * j + cp + (e & 1), d = 16 * q4 + row + 8 * (e >> 1);
+            tile[t * kN + (post ? d ^ (((t >> 1) & 3) << 3) : d)] = __uint_as_float(u[4 * j + e]);
+          }
+      } else {
+        uint32_t pk[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) pk[2 * j + e] = pack_bf16(__uint_as_float(u[4 * j + 2 * e]), __uint_as_float(u[4 * j + 2 * e + 1]));
+        const uint32_t swz = sq.len - c * C >= C ? m_tok & 7 : 0;   // (a short chunk leaves row by row)
+#pragma unroll
+        for (int g = 0; g < 2; ++g)
+          stmatrix_x4_trans(s_base + kOffOut + s * kOutBytes + (m_tok + 16 * g) * 128 + ((m_ch ^ swz) << 4), pk + 4 * g);
+      }
+      fence_proxy_async_smem();
+      if (post) warp_arrive(bars.pn[s]); else warp_arrive(bars.go[s]);
+      MDN_MARK(c, kEvOutDone);
+      return true;
+    };
+    {
+      // ---------------- the start state into the masters
+      const float* src = is_m ? rn.M0 : rn.S0;
+      const bool id = is_m ? rn.id_m : rn.id_s;
+#pragma unroll 1
+      for (int i = 0; i < 2; ++i) {
+        const int col0 = hf * 64 + i * 32;
+        uint32_t x[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+          x[j] = __float_as_uint(src ? __ldg(src + (size_t)(col0 + j) * kD + dg) : (id && col0 + j == dg ? 1.f : 0.f));
+        __syncwarp();
+        tmem_st32(tl + kColP + col0, x);
+      }
+      tmem_wait_st();
+      tc_fence_before_sync();
+      warp_arrive(bars.init);
+    }
+#pragma unroll 1
     for (int c = 0; c <= nch; ++c) {
       const int s = c & 1;
       const uint32_t ph = c & 1, ph2 = (c >> 1) & 1;
       const float* aj = reinterpret_cast<const float*>(smem + kOffAdj + s * kAdjBytes);
-      if (c == 0) {
-        // ---------------- the start state into the masters
-        const float* src = is_m ? rn.M0 : rn.S0;
-        const bool id = is_m ? rn.id_m : rn.id_s;
-#pragma unroll 1
-        for (int i = 0; i < 2; ++i) {
-          const int col0 = hf * 64 + i * 32;
-          uint32_t x[32];
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            x[j] = __float_as_uint(src ? __ldg(src + (size_t)(col0 + j) * kD + dg) : (id && col0 + j == dg ? 1.f : 0.f));
-          __syncwarp();
-          tmem_st32(tl + kColP + col0, x);
-        }
-        tmem_wait_st();
-        tc_fence_before_sync();
-        warp_arrive(bars.init);
-      }
-      if (c == nch) {
-        // ---------------- final states: [S; M] = G [Sh; Mh]  (the last chunk's MMA-3 was waited for below)
-        MDN_WAIT(fin, 0);
+      if (c < nch) {
+        MDN_WAIT(kfull[s], ph2);
+        MDN_WAIT(adj[s], ph2);
         __syncwarp();
-        const float g11 = g_final[0], g12 = g_final[1], g22 = g_final[2];
-        tc_fence_after_sync();
-        float* dst = is_m ? rn.Mf : rn.Sf;
-#pragma unroll 1
-        for (int i = 0; i < 2; ++i) {
-          const int col0 = hf * 64 + i * 32;
-          uint32_t x[32];
-          tmem_ld32(tl + kColP + col0, x);
+        // ---------------- EPI-1: R^T = V^T - cX .* (K S) + cY .* (K M)  -> bf16 hi, lo into X, in both halves of the lanes
+        {
+          // V and the coefficients are fetched before the wait
+          uint32_t vr[8];   // [pair of token groups][m]: token group 2 g + m / 2, value column half m % 2
+          if (!v_zero) {
+#pragma unroll
+            for (int g = 0; g < 2; ++g)
+              ldmatrix_x4_trans(s_base + kOffStage + s * kStageBytes + kStV + (m_tok + 16 * g) * 128 + ((m_ch ^ (m_tok & 7)) << 4), vr + 4 * g);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) vr[i] = 0u;
+          }
+          float2 cx[4], cy[4];
+          coef4(cx, aj, kCx);   // (-cX)
+          coef4(cy, aj, kCy);
+          MDN_POLL(mx, ph);
+          tc_fence_after_sync();
+          MDN_MARK(c, kEvMxSeen);
+          uint32_t xs[16], xm[16];
+          tmem_ld_16x256_x4(tl + kColX + r0, xs);
+          tmem_ld_16x256_x4(tl + kUpper + kColX + r0, xm);
           tmem_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float mine = __uint_as_float(x[j]), other = __shfl_xor_sync(0xffffffffu, mine, 16);
-            const float y = is_m ? g22 * mine : unscale_s(g11, mine, g12, other);
-            if (dst) dst[(size_t)(col0 + j) * kD + dg] = y;
-          }
-        }
-        break;
-      }
-      uint8_t* stg = smem + kOffStage + s * kStageBytes;
-      MDN_WAIT(full[s], ph2);
-      MDN_WAIT(adj[s], ph2);
-      __syncwarp();
-      // a vector's values for this thread's four token pairs
-      auto coef4 = [&](float2 (&f)[4], int vec) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) f[j] = *reinterpret_cast<const float2*>(aj + vec + r0 + 8 * j + cp);
-      };
-      auto pair = [](const uint32_t (&x)[16], int j, int e) { return make_float2(__uint_as_float(x[4 * j + 2 * e]), __uint_as_float(x[4 * j + 2 * e + 1])); };
-      // ---------------- EPI-1: R^T = V^T - cX .* (K S) + cY .* (K M)  -> bf16 hi, lo into X, in both halves of the lanes
-      {
-        // V and the coefficients are fetched before the wait
-        uint32_t vr[8];   // [pair of token groups][m]: token group 2 g + m / 2, value column half m % 2
-        if (!v_zero) {
-#pragma unroll
-          for (int g = 0; g < 2; ++g)
-            ldmatrix_x4_trans(s_base + kOffStage + s * kStageBytes + kStV + (m_tok + 16 * g) * 128 + ((m_ch ^ (m_tok & 7)) << 4), vr + 4 * g);
-        } else {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) vr[i] = 0u;
-        }
-        float2 cx[4], cy[4];
-        coef4(cx, kCx);   // (-cX)
-        coef4(cy, kCy);
-        MDN_WAIT(mx[s], ph2);
-        __syncwarp();
-        tc_fence_after_sync();
-        MDN_MARK(c, kEvMxSeen);
-        uint32_t xs[16], xm[16];
-        tmem_ld_16x256_x4(tl + kColX + r0, xs);
-        tmem_ld_16x256_x4(tl + kUpper + kColX + r0, xm);
-        tmem_wait_ld();
-        uint32_t hi[8], lo[8];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const uint32_t vw = vr[4 * (j >> 1) + 2 * (j & 1) + e];
-            float2 x = make_float2(__uint_as_float(vw << 16), __uint_as_float(vw & 0xffff0000u));
-            x = __ffma2_rn(cx[j], pair(xs, j, e), x);
-            x = __ffma2_rn(cy[j], pair(xm, j, e), x);
-            split_pack_bf16(x, hi[2 * j + e], lo[2 * j + e]);
-          }
-        // (the columns this warp has just read)
-        tmem_st_16x128_x4(tl + kColX + r0, hi);
-        tmem_st_16x128_x4(tl + kUpper + kColX + r0, hi);
-        tmem_st_16x128_x4(tl + kColX + r0 + kPk, lo);
-        tmem_st_16x128_x4(tl + kUpper + kColX + r0 + kPk, lo);
-        tmem_wait_st();
-      }
-      tc_fence_before_sync();
-      warp_arrive(bars.r);
-      MDN_MARK(c, kEvRArrive);
-      // ---------------- inter-chunk output terms cZ .* (Q S) + cU .* (Q M) into the lower lanes of Z, for MMA-3' to accumulate onto
-      // (the upper lanes accumulate onto Q M: nobody reads them)
-      if (write_o) {
-        float2 cz[4], cu[4];
-        coef4(cz, kCz);
-        coef4(cu, kCu);
-        MDN_WAIT(mz, ph);
-        __syncwarp();
-        tc_fence_after_sync();
-        uint32_t zs[16], zm[16];
-        tmem_ld_16x256_x4(tl + kColZ + r0, zs);
-        tmem_ld_16x256_x4(tl + kUpper + kColZ + r0, zm);
-        tmem_wait_ld();
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const float2 o2 = __ffma2_rn(cz[j], pair(zs, j, e), __fmul2_rn(cu[j], pair(zm, j, e)));
-            zs[4 * j + 2 * e] = __float_as_uint(o2.x);
-            zs[4 * j + 2 * e + 1] = __float_as_uint(o2.y);
-          }
-        tmem_st_16x256_x4(tl + kColZ + r0, zs);
-        tmem_wait_st();
-        tc_fence_before_sync();
-        warp_arrive(bars.oi);
-        MDN_MARK(c, kEvOiArrive);
-      }
-      // ---------------- EPI-2: wS .* V~ | -wM .* V~ -> X as bf16 hi, lo.  Eager chunks: the masters take G' = D_c G first (under MMA-2;
-      // MMA-1 of this chunk, their last reader, is done) and the update is added in true coordinates.
-      const bool eager = aj[kLazy] == 0.f;
-      const float n11 = aj[kN11], n12 = aj[kN12], n22 = aj[kN22];
-              if (eager) {   // Sh <- n11 Sh + n12 Mh, Mh <- n22 Mh
-      #pragma unroll 1
-                for (int i = 0; i < 2; ++i) {
-                  const uint32_t col0 = kColP + hf * 64 + i * 32;
-                  uint32_t ps[16], pm[16];
-                  tmem_ld_16x256_x4(tl + col0, ps);
-                  tmem_ld_16x256_x4(tl + kUpper + col0, pm);
-                  tmem_wait_ld();
-      #pragma unroll
-                  for (int j = 0; j < 16; ++j) {
-                    ps[j] = __float_as_uint(unscale_s(n11, __uint_as_float(ps[j]), n12, __uint_as_float(pm[j])));
-                    pm[j] = __float_as_uint(n22 * __uint_as_float(pm[j]));
-                  }
-                  tmem_st_16x256_x4(tl + col0, ps);
-                  tmem_st_16x256_x4(tl + kUpper + col0, pm);
-                }
-              }
-      {
-        float2 ws[4], wm[4];
-        coef4(ws, kWs);
-        coef4(wm, kWm);
-        MDN_WAIT(m2, ph);
-        __syncwarp();
-        tc_fence_after_sync();
-        MDN_MARK(c, kEvM2Seen);
-        uint32_t vt[16];
-        tmem_ld_16x256_x4(tl + kColY + r0, vt);
-        tmem_wait_ld();
-        uint32_t hi[8], lo[8];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-          for (int e = 0; e < 2; ++e) split_pack_bf16(__fmul2_rn(ws[j], pair(vt, j, e)), hi[2 * j + e], lo[2 * j + e]);
-        tmem_st_16x128_x4(tl + kColX + r0, hi);          // X is free: MMA-2 has consumed R
-        tmem_st_16x128_x4(tl + kColX + r0 + kPk, lo);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-          for (int e = 0; e < 2; ++e)
-            split_pack_bf16(__fmul2_rn(make_float2(-wm[j].x, -wm[j].y), pair(vt, j, e)), hi[2 * j + e], lo[2 * j + e]);
-        tmem_st_16x128_x4(tl + kUpper + kColX + r0, hi);
-        tmem_st_16x128_x4(tl + kUpper + kColX + r0 + kPk, lo);
-        tmem_wait_st();
-        tc_fence_before_sync();
-        warp_arrive(bars.v);
-        MDN_MARK(c, kEvVArrive);
-      }
-      // ---------------- the chunk's output tile (under MMA-3): Z -> [64 tokens x 64 value columns] over the stage's V (and T)
-      if (write_o) {
-        MDN_WAIT(mo, ph);
-        __syncwarp();
-        tc_fence_after_sync();
-        MDN_MARK(c, kEvMoSeen);
-        uint32_t u[16];
-        tmem_ld_16x256_x4(tl + kColZ + r0, u);
-        tmem_wait_ld();
-        tc_fence_before_sync();
-        warp_arrive(bars.zu);
-        if (post || sizeof(TO) == 4) {
-          // an fp32 tile; for the output warps a row's 16-byte pieces are rotated by its token pair (no bank is touched twice)
-          float* tile = reinterpret_cast<float*>(stg + kStOut);
+          uint32_t hi[8], lo[8];
 #pragma unroll
           for (int j = 0; j < 4; ++j)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int t = r0 + 8 * j + cp + (e & 1), d = 16 * q4 + row + 8 * (e >> 1);
-              tile[t * kN + (post ? d ^ (((t >> 1) & 3) << 3) : d)] = __uint_as_float(u[4 * j + e]);
+            for (int e = 0; e < 2; ++e) {
+              const uint32_t vw = vr[4 * (j >> 1) + 2 * (j & 1) + e];
+              float2 x = make_float2(__uint_as_float(vw << 16), __uint_as_float(vw & 0xffff0000u));
+              x = __ffma2_rn(cx[j], pair(xs, j, e), x);
+              x = __ffma2_rn(cy[j], pair(xm, j, e), x);
+              split_pack_bf16(x, hi[2 * j + e], lo[2 * j + e]);
             }
-        } else {
-          uint32_t pk[8];
+          // (the columns this warp has just read)
+          tmem_st_16x128_x4(tl + kColX + r0, hi);
+          tmem_st_16x128_x4(tl + kUpper + kColX + r0, hi);
+          tmem_st_16x128_x4(tl + kColX + r0 + kPk, lo);
+          tmem_st_16x128_x4(tl + kUpper + kColX + r0 + kPk, lo);
+          tmem_wait_st();
+        }
+        tc_fence_before_sync();
+        warp_arrive(bars.r);
+        MDN_MARK(c, kEvRArrive);
+      }
+      if (write_o && c > 0 && !output(c - 1)) { ok = false; break; }   // (under MMA-2)
+      if (c == nch) break;
+      // EPI-2, then the inter-chunk output terms.  Eager chunks the other way round: the masters take G' = D_c G (under MMA-2) behind
+      // MMA-1z, their last reader in this chunk, and the update is added in true coordinates.
+      const bool eager = aj[kLazy] == 0.f;
+#pragma unroll 1
+      for (int step = 0; step < 2; ++step) {
+        if ((step == 0) == eager) {
+          if (write_o && !inter(c)) { ok = false; break; }
+          continue;
+        }
+        if (eager) {
+            const float n11 = aj[kN11], n12 = aj[kN12], n22 = aj[kN22];   // Sh <- n11 Sh + n12 Mh, Mh <- n22 Mh
+#pragma unroll 1
+            for (int i = 0; i < 2; ++i) {
+              const uint32_t col0 = kColP + hf * 64 + i * 32;
+              uint32_t ps[16], pm[16];
+              tmem_ld_16x256_x4(tl + col0, ps);
+              tmem_ld_16x256_x4(tl + kUpper + col0, pm);
+              tmem_wait_ld();
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                ps[j] = __float_as_uint(unscale_s(n11, __uint_as_float(ps[j]), n12, __uint_as_float(pm[j])));
+                pm[j] = __float_as_uint(n22 * __uint_as_float(pm[j]));
+              }
+              tmem_st_16x256_x4(tl + col0, ps);
+              tmem_st_16x256_x4(tl + kUpper + col0, pm);
+            }
+          }
+        // ---------------- EPI-2: wS .* V~ | -wM .* V~ -> X as bf16 hi, lo
+        {
+          float2 ws[4], wm[4];
+          coef4(ws, aj, kWs);
+          coef4(wm, aj, kWm);
+          MDN_POLL(m2, ph);
+          tc_fence_after_sync();
+          MDN_MARK(c, kEvM2Seen);
+          uint32_t vt[16];
+          tmem_ld_16x256_x4(tl + kColY + 64 * s + r0, vt);
+          tmem_wait_ld();
+          uint32_t hi[8], lo[8];
 #pragma unroll
           for (int j = 0; j < 4; ++j)
 #pragma unroll
-            for (int e = 0; e < 2; ++e) pk[2 * j + e] = pack_bf16(__uint_as_float(u[4 * j + 2 * e]), __uint_as_float(u[4 * j + 2 * e + 1]));
-          const uint32_t swz = sq.len - c * C >= C ? m_tok & 7 : 0;   // (a short chunk leaves row by row)
+            for (int e = 0; e < 2; ++e) split_pack_bf16(__fmul2_rn(ws[j], pair(vt, j, e)), hi[2 * j + e], lo[2 * j + e]);
+          tmem_st_16x128_x4(tl + kColX + r0, hi);          // X is free: MMA-2 has consumed R
+          tmem_st_16x128_x4(tl + kColX + r0 + kPk, lo);
 #pragma unroll
-          for (int g = 0; g < 2; ++g)
-            stmatrix_x4_trans(s_base + kOffStage + s * kStageBytes + kStOut + (m_tok + 16 * g) * 128 + ((m_ch ^ swz) << 4), pk + 4 * g);
+          for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+              split_pack_bf16(__fmul2_rn(make_float2(-wm[j].x, -wm[j].y), pair(vt, j, e)), hi[2 * j + e], lo[2 * j + e]);
+          tmem_st_16x128_x4(tl + kUpper + kColX + r0, hi);
+          tmem_st_16x128_x4(tl + kUpper + kColX + r0 + kPk, lo);
+          tmem_wait_st();
+          tc_fence_before_sync();
+          warp_arrive(bars.v);
+          MDN_MARK(c, kEvVArrive);
         }
-        fence_proxy_async_smem();
-        if (post) warp_arrive(bars.pn[s]);
-        MDN_MARK(c, kEvOutDone);
       }
-      if (!post) warp_arrive(bars.go[s]);
-      if (c == nch - 1) MDN_WAIT(m3[s], ph2);   // the final states follow
+      if (!ok) break;
+    }
+    while (ok) {   // (once)
+      // ---------------- final states: [S; M] = G [Sh; Mh]  
+      if (nch > 0) MDN_WAIT(m3[(nch - 1) & 1], ((nch - 1) >> 1) & 1);
+      MDN_WAIT(fin, 0);
+      __syncwarp();
+      const float g11 = g_final[0], g12 = g_final[1], g22 = g_final[2];
+      tc_fence_after_sync();
+      float* dst = is_m ? rn.Mf : rn.Sf;
+#pragma unroll 1
+      for (int i = 0; i < 2; ++i) {
+        const int col0 = hf * 64 + i * 32;
+        uint32_t x[32];
+        tmem_ld32(tl + kColP + col0, x);
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          const float mine = __uint_as_float(x[j]), other = __shfl_xor_sync(0xffffffffu, mine, 16);
+          const float y = is_m ? g22 * mine : unscale_s(g11, mine, g12, other);
+          if (dst) dst[(size_t)(col0 + j) * kD + dg] = y;
+        }
+      }
+      break;
     }
   }
 #undef MDN_WAIT
-#undef MDN_SPIN
+#undef MDN_POLL
 #undef MDN_MARK
   if (warp == 0) { MDN_NOW(6); }
 
   if (!ok && lane == 0) atomicCAS(a.status, kDevOk, kDevTimeout);
   tc_fence_before_sync();
   __syncthreads();
-  if constexpr (kLayer) cluster_sync_all();   // neither CTA's shared memory goes while the other may still write to it
+  if constexpr (kLayer) {   // neither CTA's shared memory goes while the other may still write to it
+    if (!ok) __nanosleep(100000);   // (what was sent before a wait ran out lands)
+    cluster_sync_all();
+  }
 #ifdef MDN_DEBUG
   if (warp == 0) { MDN_NOW(5); }
   if (tline != nullptr && tid < 256) tline[(kTlFirst + (tid >> 5)) * 32 + (tid & 31)] = tl_sm[tid >> 5][tid & 31];

@@ -896,7 +896,7 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
 #endif
   const unsigned chains = (unsigned)pl.geom.num_seqs * p.H;
   auto launch = [&](unsigned grid) -> cudaError_t {
-    if (!layer && 2 * grid <= (unsigned)kSms) return launch_chain_half(pl, a, ChainTensors{q, k, v}, grid, launches);
+    if (2 * grid <= (unsigned)kSms) return launch_chain_half(pl, a, ChainTensors{q, k, v}, grid, launches);
     auto kern = layer ? (o_bf16 ? chain_tf32_kernel<__nv_bfloat16, true> : chain_tf32_kernel<float, true>)
                       : (o_bf16 ? chain_tf32_kernel<__nv_bfloat16, false> : chain_tf32_kernel<float, false>);
     cudaError_t e = allow_smem<(int)kSmemBytes>(kern);

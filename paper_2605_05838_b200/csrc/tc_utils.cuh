@@ -94,6 +94,22 @@ __device__ __forceinline__ bool mbar_wait_spin(uint32_t bar, uint32_t parity, vo
   return false;
 }
 
+// The same for whole warps: every lane gets the same answer, and the warp is together again behind it.  warp_wait is a function: a
+// kernel whose warps are in many roles has all their code in use at once, and what of it does not fit the instruction cache is
+// fetched again every chunk (see chain_half.cu).  Not for kernels that change their register count (setmaxnreg).
+static __device__ __noinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+}
+// ... in place, for the waits on a critical path (the call there costs 0.2 k cycles).
+__device__ __forceinline__ bool warp_poll(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
+  uint32_t left = kSpinLimit;
+#pragma unroll 1
+  while (!mbar_try_wait(bar, parity) && --left != 0) {}
+  if (left == 0) *abort_flag = 1;
+  return __all_sync(0xffffffffu, left != 0);
+}
+
 // ----------------------------------------------------------------------------- thread-block clusters
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -106,28 +122,11 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t smem_addr, uint32_t rank
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float x) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(x) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t mapped_bar) {   // releases this thread's stores to the cluster
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(mapped_bar) : "memory");
-}
-// mbar_wait for a barrier that another CTA of the cluster arrives at (and whose stores are to be read afterwards).
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  for (uint32_t it = 0; it < kSpinLimit; ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok != 0) return true;
-    if ((it & 255u) == 255u && *abort_flag != 0) return false;
-  }
-  *abort_flag = 1;
-  return false;
+// Asynchronous store of one word to another CTA of the cluster that counts as four of the bytes its barrier (in that CTA) expects.
+__device__ __forceinline__ void st_async_f32(uint32_t mapped_addr, float x, uint32_t mapped_bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+               ::"r"(mapped_addr), "r"(__float_as_uint(x)), "r"(mapped_bar)
+               : "memory");
 }
 __device__ __forceinline__ void cluster_sync_all() {   // every thread of every CTA of the cluster
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
