@@ -14,15 +14,16 @@
 //
 // Per chunk:  MMA-1x X = P K^T (P: both masters)  ->  EPI-1 R^T (bf16 hi + lo) into X  ->  MMA-2 Y = R^T T^T  ->  EPI-2 wS V~ | -wM V~
 //             (bf16 hi + lo) into X  ->  MMA-3 P += X K  ->  next chunk's MMA-1x.
-// The rest is cut to fit the two gaps in which the tensor pipe would wait for the epilogue: MMA-1z Z = P Q^T in two halves, the first
-// under EPI-1, the second under EPI-2 (whole under EPI-1 it delayed MMA-2 by 0.4 k cycles); o_inter into Z behind EPI-2; MMA-3'
-// Z += V~^T W^T behind the NEXT chunk's MMA-1x; output tile under that chunk's MMA-2.  Z is double-buffered for that.
+// The output runs beside it, on warps of its own, cut to fit the gaps in which the tensor pipe would wait for the epilogue: MMA-1z
+// Z = P Q^T partly under EPI-1, partly under EPI-2; o_inter into Z; MMA-3' Z += V~^T W^T behind the NEXT chunk's MMA-1x; output
+// tile.  Y and Z are double-buffered for that.
 //
 // What bounds a chunk: the serial chain of the three product groups (0.72 + 0.36 + 0.51 k cycles), their commit-to-wake latencies
-// and the two epilogue steps.  Registers, shared memory and tensor memory (448 of 512 columns) are not the limit here.
-// Two warps issue products: one those of the serial chain alone (three waits per chunk), one those of the output.  A wait in the
-// issuing warp costs 0.2 .. 0.4 k cycles even if its phase is long complete (one warp for all, with eight waits: 4.3 k cycles per
-// chunk).
+// and the two epilogue steps.  Registers, shared memory and tensor memory (448 of 512 columns) are not the limit; the instruction cache
+// is: the warps are in seven roles, all their code is in use at once, and what of it has to be fetched again every chunk is fetched
+// through a cache that the SMs of a cluster of SMs share.  So code is kept short: waits are calls (in place: + 23 KB), loops that
+// need not be are not unrolled.  A wait in a product-issuing warp costs 0.2 .. 0.4 k cycles even if its phase is long complete: the
+// serial chain's products have a warp of their own with three waits per chunk.
 //
 // With the layer operations the RMSNorm of the output step sums over all 128 value columns: the two CTAs of a chain are a
 // thread-block cluster and exchange each token's sum of squares through distributed shared memory.
@@ -37,11 +38,12 @@ using namespace tc;
 
 constexpr int kD = 128, kN = 64;   // key columns; value columns of a CTA
 // Warps 0..7 epilogue (lane quarter = warp % 4, token half = warp / 4), 8 the products of the state's serial chain, 9 loads and
-// coefficients, 10 the products of the output, 11 output stores, 12..15 converters, with the layer operations 16..19 output step.
+// coefficients, 10 the products of the output, 11 output stores, 12..15 converters, 16..19 output.
 constexpr int kEpiWarps = 8, kWarpMma = 8, kWarpLoad = 9, kWarpMmaOut = 10, kWarpStore = 11, kWarpCvt = 12, kCvtWarps = 4, kWarpOut = 16, kOutWarps = 4;
-constexpr int threads_of(bool layer) { return (kWarpOut + (layer ? kOutWarps : 0)) * 32; }
+constexpr int kThreads = (kWarpOut + kOutWarps) * 32;
 constexpr int kOutThreads = kOutWarps * 32;
 constexpr int kTok = 32, kPk = 16;   // tokens of an epilogue warp; their packed bf16 pairs
+constexpr int kZFirst = 4;           // products of MMA-1z that fit under EPI-1, behind MMA-3'
 
 // Shared memory (offsets from a 1024-byte aligned base)
 constexpr uint32_t kOffK32 = 0, kOffQ32 = 32768;     // fp32 K and Q [64 tokens x 128 dk]: four dk quarters x [64 rows x 128 B], swizzled
@@ -63,35 +65,35 @@ constexpr uint32_t kUpper = 16u << 16;               // the upper sixteen lanes 
 // A barrier that a waiter could fall a whole phase behind comes in pairs, by the chunk's parity.
 struct Bars {
   uint64_t kfull[2];  // bf16 K and V tiles of a stage landed                             (1 + tx bytes)
-  uint64_t full[2];   // T, W, coefficient vectors                                        (1 + tx bytes)
+  uint64_t full[2];   // T, coefficient vectors                                           (1 + tx bytes)
+  uint64_t wfull[2];  // W                                                                (1 + tx bytes)
   uint64_t qfull;     // bf16 Q tile landed                                               (1 + tx bytes)
   uint64_t qfree;     // ... and read                                                     (4 warps)
   uint64_t xr;        // MMA-1x may start: fp32 K copy written, masters updated           (4 warps + commit)
   uint64_t q32;       // fp32 Q copy written                                              (4 warps)
-  uint64_t adj[2];    // a chunk's coefficient block written, its T and W landed          (1)
+  uint64_t adj[2];    // a chunk's coefficient block written, its T landed                (1)
   uint64_t fin;       // G after the last chunk written                                   (1)
   uint64_t init;      // masters of chunk 0 stored                                        (8 warps)
   uint64_t mx;        // X done: the fp32 K copy is free too                              (commit)
   uint64_t mz;        // Z done: the fp32 Q copy is free too                              (commit)
   uint64_t r;         // EPI-1 done: R^T in X                                             (8 warps)
   uint64_t m2;        // V~ in Y                                                          (commit)
-  uint64_t oi;        // inter-chunk output terms in Z                                    (8 warps)
-  uint64_t v;         // MMA-3 may start: update operand in X (eager chunks: masters rescaled), MMA-1z done  (8 warps + 1)
+  uint64_t oi[2];     // inter-chunk output terms in Z                                    (4 warps)
+  uint64_t v;         // MMA-3 may start: update operand in X (eager chunks: masters rescaled), MMA-1z done  (8 warps + commit)
   uint64_t m3[2];     // masters updated: the stage's K, V, T are free too                (commit)
-  uint64_t mo;        // MMA-3' done                                                      (commit)
-  uint64_t zu[2];     // Z (the chunk's output) has been read: W and the coefficient block are free too  (8 warps)
-  uint64_t go[2];     // the output tile is staged                                        (8 warps; fused output step 4)
+  uint64_t mo[2];     // MMA-3' done                                                      (commit)
+  uint64_t zu[2];     // Z (the chunk's output) has been read: W is free too              (4 warps)
+  uint64_t go[2];     // the output tile is staged                                        (4 warps)
   uint64_t ofree[2];  // ... and read by its store                                        (1)
-  uint64_t pn[2];     // fused output step: the fp32 tile is staged                       (8 warps)
-  uint64_t peer[2];   // ... and the other CTA's sums of squares have arrived             (1 + 256 bytes)
+  uint64_t peer[2];   // fused output step: the other CTA's sums of squares have arrived             (1 + 256 bytes)
 };
 
 enum Ev : int { kEvTop = 0, kEvXIssued, kEvZIssued, kEvRSeen, kEvM2Issued, kEvMoIssued, kEvVSeen, kEvM3Issued,
                 kEvMxSeen, kEvRArrive, kEvOiArrive, kEvM2Seen, kEvVArrive, kEvMoSeen, kEvOutDone, kEvCvtK, kEvCvtKDone, kEvCvtQ,
-                kEvCvtQDone, kEvTma, kEvAdj, kEvStored, kEvPn, kEvSsSent, kEvPeer, kEvGo };
+                kEvCvtQDone, kEvTma, kEvAdj, kEvStored };
 
 template <typename TO, bool kLayer>
-__global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const ChainTf32Args a, const __grid_constant__ CUtensorMap map_q,
+__global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32Args a, const __grid_constant__ CUtensorMap map_q,
                                                                 const __grid_constant__ CUtensorMap map_k,
                                                                 const __grid_constant__ CUtensorMap map_v,
                                                                 const __grid_constant__ CUtensorMap map_t,
@@ -136,15 +138,15 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
     abort_flag = 0;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      mbar_init(bar(bars.kfull[i]), 1); mbar_init(bar(bars.full[i]), 1);
-      mbar_init(bar(bars.adj[i]), 1); mbar_init(bar(bars.m3[i]), 1); mbar_init(bar(bars.zu[i]), kEpiWarps);
-      mbar_init(bar(bars.go[i]), post ? kOutWarps : kEpiWarps); mbar_init(bar(bars.ofree[i]), 1);
-      mbar_init(bar(bars.pn[i]), kEpiWarps); mbar_init(bar(bars.peer[i]), 1);
+      mbar_init(bar(bars.kfull[i]), 1); mbar_init(bar(bars.full[i]), 1); mbar_init(bar(bars.wfull[i]), 1);
+      mbar_init(bar(bars.adj[i]), 1); mbar_init(bar(bars.m3[i]), 1); mbar_init(bar(bars.mo[i]), 1); mbar_init(bar(bars.oi[i]), kOutWarps);
+      mbar_init(bar(bars.zu[i]), kOutWarps); mbar_init(bar(bars.go[i]), kOutWarps); mbar_init(bar(bars.ofree[i]), 1);
+      mbar_init(bar(bars.peer[i]), 1);
     }
     mbar_init(bar(bars.qfull), 1); mbar_init(bar(bars.qfree), kCvtWarps); mbar_init(bar(bars.q32), kCvtWarps); mbar_init(bar(bars.xr), kCvtWarps + 1);
     mbar_init(bar(bars.fin), 1); mbar_init(bar(bars.init), kEpiWarps);
-    mbar_init(bar(bars.mx), 1); mbar_init(bar(bars.mz), 1); mbar_init(bar(bars.m2), 1); mbar_init(bar(bars.mo), 1);
-    mbar_init(bar(bars.r), kEpiWarps); mbar_init(bar(bars.oi), kEpiWarps); mbar_init(bar(bars.v), kEpiWarps + (write_o ? 1 : 0));
+    mbar_init(bar(bars.mx), 1); mbar_init(bar(bars.mz), 1); mbar_init(bar(bars.m2), 1);
+    mbar_init(bar(bars.r), kEpiWarps); mbar_init(bar(bars.v), kEpiWarps + (write_o ? 1 : 0));
     mbar_fence_init();
   }
   if (kLayer && tid < kN) w_sm[tid] = (a.post_on && a.post_w) ? __ldg(a.post_w + v0 + tid) : 1.f;
@@ -160,12 +162,12 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
   const uint32_t tmem = tmem_slot;
   bool ok = true;
   volatile int* abortp = &abort_flag;
-#define MDN_WAIT(b, par)                                                            \
-  if (!warp_wait(smem_u32(&bars.b), (par), abortp)) { \
-    ok = false;                                             \
-    break;                                                  \
+#define MDN_WAIT(b, par)                                            \
+  if (!warp_wait(smem_u32(&bars.b), (par), abortp)) {               \
+    ok = false;                                                     \
+    break;                                                          \
   }
-  // waits on the chain's critical path poll, in place (a call there costs 0.2 .. 0.4 k cycles)
+  // waits on the chain's critical path poll, in place (a call there costs 0.2 k cycles)
 #define MDN_POLL(b, par)                                            \
   if (!warp_poll(smem_u32(&bars.b), (par), abortp)) {               \
     ok = false;                                                     \
@@ -201,8 +203,7 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
   if (warp == kWarpLoad) {
     // ================================================================== loads, coefficients
     // A stage's K, V and T tiles are refilled (for chunk c + 2) as soon as MMA-3 has read K, the Q buffer as soon as it is converted, W
-    // when the output it belongs to has been read.  A chunk's coefficient block is published when its T and W have landed too and the
-    // output that its Z held has been read: who waits for the block need not wait for those.
+    // when the output it belongs to has been read.  Who waits for a chunk's coefficient block need not wait for its T.
     int issued = 0;
     float g11 = 1.f, g12 = 0.f, g22 = 1.f;
 #pragma unroll 1
@@ -225,26 +226,31 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
           tma_load_2d(s_base + kOffQb, &map_q, h * kD, tok0, bar(bars.qfull));
           tma_load_2d(s_base + kOffQb + 8192, &map_q, h * kD + 64, tok0, bar(bars.qfull));
         }
-        if (c >= 2) MDN_WAIT(zu[s], ph2 ^ 1);
       }
       if (early && c == 0) { grid_dependency_wait(); MDN_NOW(1); }
       if (lane == 0) {
         const uint32_t fb = bar(bars.full[s]);
-        mbar_arrive_expect_tx(fb, kCoefBytes + kTxT + (write_o ? kTxW : 0u));
+        mbar_arrive_expect_tx(fb, kCoefBytes + kTxT);
         bulk_load(st + kStCoef, a.coef + (size_t)mat * MDN_NUM_COEF * C, kCoefBytes, fb);
         tma_load_2d(st + kStT, &map_t, 0, mat * C, fb);
-        if (write_o) {
-          tma_load_2d(st + kStW, &map_w, 0, mat * C, fb);
-          tma_load_2d(st + kStW + 8192, &map_w, 32, mat * C, fb);
-        }
       }
       issued = c + 1;
       MDN_MARK(c, kEvTma);
       MDN_WAIT(full[s], ph2);
+      if (write_o && c >= 2) MDN_WAIT(oi[s], ph2 ^ 1);   // chunk c - 2's block has been read (MMA-3 of that chunk: by the epilogue)
       publish_coefs<kLayer>(reinterpret_cast<const float*>(smem + kOffStage + s * kStageBytes + kStCoef),
                             reinterpret_cast<float*>(smem + kOffAdj + s * kAdjBytes), a.scale, lane, g11, g12, g22);
       warp_arrive(bars.adj[s]);
       MDN_MARK(c, kEvAdj);
+      if (write_o) {
+        if (c >= 2) MDN_WAIT(zu[s], ph2 ^ 1);
+        if (lane == 0) {
+          mbar_arrive_expect_tx(bar(bars.wfull[s]), kTxW);
+          tma_load_2d(st + kStW, &map_w, 0, mat * C, bar(bars.wfull[s]));
+          tma_load_2d(st + kStW + 8192, &map_w, 32, mat * C, bar(bars.wfull[s]));
+        }
+        __syncwarp();
+      }
     }
     if (early && nch == 0) grid_dependency_wait();   // (every CTA ends after the previous kernel has)
     if (ok) {
@@ -258,7 +264,8 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
         uint32_t it = 0;
 #pragma unroll 1
         while (it < (1u << 18) && !(mbar_try_wait(bar(bars.kfull[c & 1]), (c >> 1) & 1) &&
-                                    mbar_try_wait(bar(bars.full[c & 1]), (c >> 1) & 1) && (!write_o || mbar_try_wait(bar(bars.qfull), c & 1)))) ++it;
+                                    mbar_try_wait(bar(bars.full[c & 1]), (c >> 1) & 1) &&
+                                    (!write_o || (mbar_try_wait(bar(bars.qfull), c & 1) && mbar_try_wait(bar(bars.wfull[c & 1]), (c >> 1) & 1))))) ++it;
       }
     }
   } else if (warp == kWarpStore) {
@@ -356,8 +363,8 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
     }
   } else if (warp == kWarpMmaOut) {
     // ================================================================== products of the output
-    // In the gaps of the serial chain: behind MMA-1x the previous chunk's MMA-3' and the first half of MMA-1z, behind MMA-2 the second
-    // half (eager chunks: both halves first, the masters are rescaled under MMA-2).
+    // In the gaps of the serial chain: behind MMA-1x the previous chunk's MMA-3' and some of the sixteen products of MMA-1z, behind MMA-2
+    // the others (eager chunks: all sixteen first, the masters are rescaled under MMA-2).
     const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
     const uint32_t sb = __shfl_sync(0xffffffffu, s_base, 0);
     const bool lead = elect_one();
@@ -368,44 +375,48 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
     for (int c = 0; c <= (write_o ? nch : -1); ++c) {
       const int s = c & 1;
       const uint32_t ph = c & 1, ph2 = (c >> 1) & 1;
-      if (c < nch) MDN_POLL(mx, ph);
-      // ---- MMA-3' of the previous chunk: Z += V~^T W^T, V~ read as tf32 from the accumulator of MMA-2 (the epilogue has waited for
-      // that one's commit)
+      // (waits that are mostly over first, where nothing waits for this warp)
+      bool eager = false;
+      if (c > 0) {
+        MDN_WAIT(wfull[s ^ 1], ((c - 1) >> 1) & 1);
+        MDN_WAIT(oi[s ^ 1], ((c - 1) >> 1) & 1);
+      }
+      if (c < nch) {
+        MDN_WAIT(q32, ph);
+        MDN_WAIT(adj[s], ph2);
+        if (c >= 2) MDN_WAIT(zu[s], ph2 ^ 1);   // the output that this chunk's Z held has been read
+        eager = reinterpret_cast<const float*>(smem + kOffAdj + s * kAdjBytes)[kLazy] == 0.f;
+        MDN_POLL(mx, ph);
+      }
+      tc_fence_after_sync();
+      // ---- MMA-3' of the previous chunk: Z += V~^T W^T, V~ read as tf32 from the accumulator of MMA-2 (MMA-3 has waited for it)
       if (c > 0) {
         const uint64_t dW = s ? dW_0 : dW_1;
-        MDN_POLL(oi, ph ^ 1);
-        tc_fence_after_sync();
         if (lead) {
 #pragma unroll
           for (int j = 0; j < 8; ++j)
             umma_ts_tf32(tm + kColZ + 64 * (s ^ 1), tm + kColY + 64 * (s ^ 1) + 8 * j, dW + (uint64_t)((j >> 2) * 512 + (j & 3) * 2), id64_tf32, true);
-          umma_commit(bar(bars.mo));
+          umma_commit(bar(bars.mo[s ^ 1]));
         }
         MDN_MARK(c, kEvMoIssued);
       }
       if (c == nch) break;
       // ---- MMA-1z: Z = P Q^T (Q S and Q M)
-      MDN_POLL(q32, ph);
-      MDN_POLL(adj[s], ph2);
-      const bool eager = reinterpret_cast<const float*>(smem + kOffAdj + s * kAdjBytes)[kLazy] == 0.f;
-      tc_fence_after_sync();
-#pragma unroll 1
-      for (uint32_t half = 0; half < 2; ++half) {
-        if (half == 1 && !eager) MDN_POLL(m2, ph);
-        if (lead) {
+      auto mma1z = [&](int j) {
+        umma_ts_tf32(tm + kColZ + 64 * s, tm + kColP + 8 * j, dQ + (uint64_t)((j >> 2) * 512 + (j & 3) * 2), id64_tf32, j > 0);
+      };
+      if (lead) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            umma_ts_tf32(tm + kColZ + 64 * s, tm + kColP + 64 * half + 8 * j, dQ + (uint64_t)(1024 * half + (j >> 2) * 512 + (j & 3) * 2),
-                         id64_tf32, half + j > 0);
-          if (half == 1) umma_commit(bar(bars.mz));
-        }
-        MDN_MARK(c, kEvZIssued);
+        for (int j = 0; j < kZFirst; ++j) mma1z(j);
       }
-      if (!ok) break;
-      // MMA-3 may overwrite the masters (and MMA-2 of the next chunk but one what MMA-3' above has read)
-      MDN_POLL(mz, ph);
-      if (lane == 0) mbar_arrive(bar(bars.v));
-      __syncwarp();
+      if (!eager) MDN_POLL(m2, ph);
+      if (lead) {
+#pragma unroll
+        for (int j = kZFirst; j < 16; ++j) mma1z(j);
+        umma_commit(bar(bars.mz));
+        umma_commit(bar(bars.v));   // MMA-3 may overwrite the masters (and MMA-2 of the next chunk but one what MMA-3' above has read)
+      }
+      MDN_MARK(c, kEvZIssued);
     }
   } else if (warp >= kWarpCvt && warp < kWarpOut) {
     // ================================================================== converter warps
@@ -474,89 +485,170 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
         MDN_MARK(c, kEvCvtQDone);
       }
     }
-  } else if (kLayer && warp >= kWarpOut) {
-    // ================================================================== output warps
-    // Fused output step, second half: y = sigmoid(g) * o / sqrt(mean_d o^2 + eps) * w_d, the mean over both CTAs' columns.  Two
-    // threads per token, 32 neighbouring values each, in four pieces of eight whose order and halves rotate with the token and the
-    // thread (eight neighbouring lanes touch every bank once).  The whole fp32 tile is in registers before anything is written
-    // over it.  Sums of squares go to the other CTA by st.async, which completes its barrier's bytes: a plain remote store and a
-    // releasing arrival waited 2 k cycles for this thread's outstanding loads.
-    if (post) {
-      const int t128 = tid - kWarpOut * 32, row = t128 >> 1, part = t128 & 1;
-      const uint32_t peer_bar = map_to_cta(bar(bars.peer[0]), peer_rank), peer_at = map_to_cta(smem_u32(&peer_ss[0][row]), peer_rank);
-      const int swz = (row >> 1) & 3;   // (the epilogue's store rotates a row's pieces by this)
+  } else if (warp >= kWarpOut) {
+    // ================================================================== output warps (one lane quarter each, all 64 tokens)
+    const int q4 = warp & 3, row = lane >> 2, cp = 2 * (lane & 3);   // value columns 16 q4 + row, + 8; tokens 32 hf + 8 j + cp, + 1
+    const uint32_t tl = tmem + (static_cast<uint32_t>(q4 * 32) << 16);
+    // fused output step: y = sigmoid(g) * o / sqrt(mean_d o^2 + eps) * w_d, the mean over both CTAs' columns.  Two threads per token, 32
+    // neighbouring values each, in four pieces of eight whose order and halves rotate with the token and the thread (eight neighbouring
+    // lanes touch every bank once).  The whole fp32 tile is in registers before anything is written over it.  Sums of squares go to
+    // the other CTA by st.async, which completes its barrier's bytes: a plain remote store and a releasing arrival waited 2 k
+    // cycles for this thread's outstanding loads.
+    const int t128 = tid - kWarpOut * 32, tok = t128 >> 1, part = t128 & 1, swz = (tok >> 1) & 3;
+    const uint32_t peer_bar = kLayer ? map_to_cta(bar(bars.peer[0]), peer_rank) : 0u;
+    const uint32_t peer_at = kLayer ? map_to_cta(smem_u32(&peer_ss[0][kLayer ? tok : 0]), peer_rank) : 0u;
+    auto piece = [&](int i) { return (i + tok) & 3; };   // place of the i-th piece among the thread's four; its columns: 8 (place ^ swz)
+    // With the fused step these warps meet at barriers: one whose wait runs out goes on to the next of those, which carries the vote
+    // whether every wait has ended, and they all leave together.
+    uint32_t good = 1;
+    auto out_vote = [&]() -> bool {
+      asm volatile(
+          "{\n\t.reg .pred p, q;\n\t"
+          "setp.ne.u32 q, %0, 0;\n\t"
+          "barrier.cta.red.and.pred p, 1, %1, q;\n\t"
+          "selp.u32 %0, 1, 0, p;\n\t}\n"
+          : "+r"(good)
+          : "n"(kOutThreads)
+          : "memory");
+      return good != 0;
+    };
+#define MDN_OUT_WAIT(b, par)                                        \
+  if (!warp_wait(smem_u32(&bars.b), (par), abortp)) {               \
+    good = 0;                                                       \
+    if (!post) { ok = false; break; }                               \
+  }
 #pragma unroll 1
-      for (int c = 0; c < nch; ++c) {
-        const int s = c & 1;
-        const uint32_t ph2 = (c >> 1) & 1;
+    for (int c = 0; c <= (write_o ? nch : -1); ++c) {
+      // ---------------- the previous chunk's output: Z -> [64 tokens x 64 value columns] tile in shared memory
+      if (c > 0) {
+        const int s = (c - 1) & 1, n = min(C, sq.len - (c - 1) * C);
+        const uint32_t ph2 = ((c - 1) >> 1) & 1;
         uint8_t* const out = smem + kOffOut + s * kOutBytes;
-        const int n = min(C, sq.len - c * C);
-        const __nv_bfloat16* gp = static_cast<const __nv_bfloat16*>(a.post_g) + ((size_t)(sq.tok0 + c * C + row) * H + h) * kD + v0 + 32 * part;
-        auto piece = [&](int i) { return (i + row) & 3; };   // place of the i-th piece among the thread's four; its columns: 8 (place ^ swz)
-        uint4 gate[4];   // before the wait
+        uint4 gate[kLayer ? 4 : 1];   // before the wait
+        if (kLayer && post) {
+          const __nv_bfloat16* gp = static_cast<const __nv_bfloat16*>(a.post_g) + ((size_t)(sq.tok0 + (c - 1) * C + tok) * H + h) * kD + v0 + 32 * part;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          gate[i] = row < n ? __ldg(reinterpret_cast<const uint4*>(gp + 8 * (piece(i) ^ swz))) : make_uint4(0u, 0u, 0u, 0u);
-        if (t128 == 0) mbar_arrive_expect_tx(bar(bars.peer[s]), C * (uint32_t)sizeof(float));
-        uint32_t good = warp_wait(bar(bars.pn[s]), ph2, abortp) ? 1u : 0u;
-        __syncwarp();
-        MDN_MARK(c, kEvPn);
-        float4 ov[8];   // piece i: values 0..3 in ov[2 i], 4..7 in ov[2 i + 1]
-        float ss = 0.f;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float4* at = reinterpret_cast<const float4*>(out + row * kN * 4 + part * 128 + piece(i) * 32);
-          const float4 x = at[part], y = at[part ^ 1];
-          ov[2 * i] = part ? y : x;
-          ov[2 * i + 1] = part ? x : y;
+          for (int i = 0; i < (kLayer ? 4 : 1); ++i)
+            gate[i] = tok < n ? __ldg(reinterpret_cast<const uint4*>(gp + 8 * (piece(i) ^ swz))) : make_uint4(0u, 0u, 0u, 0u);
+          if (t128 == 0) mbar_arrive_expect_tx(bar(bars.peer[s]), C * (uint32_t)sizeof(float));
         }
+        if (c >= 3) MDN_OUT_WAIT(ofree[s], ph2 ^ 1);
+        MDN_OUT_WAIT(mo[s], ph2);
+        tc_fence_after_sync();
+        MDN_MARK(c - 1, kEvMoSeen);
+#pragma unroll 1
+        for (int r0 = 0; r0 < C; r0 += 32) {
+          uint32_t u[16];
+          tmem_ld_16x256_x4(tl + kColZ + 64 * s + r0, u);
+          tmem_wait_ld();
+          if (post || sizeof(TO) == 4) {
+            // an fp32 tile; for the fused step a token's pieces of eight values are rotated by its pair (no bank is touched twice)
+            float* at = reinterpret_cast<float*>(out) + (r0 + cp) * kN;
+            const int turn = post ? (lane & 3) << 3 : 0, d0 = (16 * q4 + row) ^ turn, d1 = (16 * q4 + row + 8) ^ turn;
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-          ss = fmaf(ov[i].x, ov[i].x, fmaf(ov[i].y, ov[i].y, fmaf(ov[i].z, ov[i].z, fmaf(ov[i].w, ov[i].w, ss))));
-        ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-        if (part == 0) st_async_f32(peer_at + s * (uint32_t)sizeof(peer_ss[0]), ss, peer_bar + s * 8);
-        MDN_MARK(c, kEvSsSent);
-        if (!warp_wait(bar(bars.peer[s]), ph2, abortp)) good = 0;
-        __syncwarp();
-        MDN_MARK(c, kEvPeer);
-        ss += *const_cast<volatile float*>(&peer_ss[s][row]);
-        const float rstd = rsqrtf(ss * (1.f / kD) + a.post_eps);
-        // the tile has been read by all four warps (the barrier carries the vote whether every wait has ended)
-        asm volatile(
-            "{\n\t.reg .pred p, q;\n\t"
-            "setp.ne.u32 q, %0, 0;\n\t"
-            "barrier.cta.red.and.pred p, 1, %1, q;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}\n"
-            : "+r"(good)
-            : "n"(kOutThreads)
-            : "memory");
-        if (good == 0) { ok = false; break; }
+            for (int j = 0; j < 4; ++j)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int col = 32 * part + 8 * (piece(i) ^ swz);
-          const uint32_t gw[4] = {gate[i].x, gate[i].y, gate[i].z, gate[i].w};
-          const float o8[8] = {ov[2 * i].x, ov[2 * i].y, ov[2 * i].z, ov[2 * i].w, ov[2 * i + 1].x, ov[2 * i + 1].y, ov[2 * i + 1].z, ov[2 * i + 1].w};
-          float y[8];
+              for (int e = 0; e < 4; ++e) at[(8 * j + (e & 1)) * kN + (e < 2 ? d0 : d1)] = __uint_as_float(u[4 * j + e]);
+          } else {
+            uint32_t pk[8];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            y[2 * e] = o8[2 * e] * rstd * w_sm[col + 2 * e] * sigmoid_fast(__uint_as_float(gw[e] << 16));
-            y[2 * e + 1] = o8[2 * e + 1] * rstd * w_sm[col + 2 * e + 1] * sigmoid_fast(__uint_as_float(gw[e] & 0xffff0000u));
+            for (int j = 0; j < 8; ++j) pk[j] = pack_bf16(__uint_as_float(u[2 * j]), __uint_as_float(u[2 * j + 1]));
+            // lane's 16-byte row: token (lane & 7) + 8 (lane >> 4) of a pair of token groups, value columns 8 ((lane >> 3) & 1)
+            const uint32_t m_tok = r0 + (lane & 7) + 8 * (lane >> 4), m_ch = 2 * q4 + ((lane >> 3) & 1);
+            const uint32_t turn = n == C ? m_tok & 7 : 0;   // (a short chunk leaves row by row)
+#pragma unroll
+            for (int g = 0; g < 2; ++g)
+              stmatrix_x4_trans(s_base + kOffOut + s * kOutBytes + (m_tok + 16 * g) * 128 + ((m_ch ^ turn) << 4), pk + 4 * g);
           }
-          if (sizeof(TO) == 4) {
-            float4* to = reinterpret_cast<float4*>(out + (row * kN + col) * 4);
-            to[0] = make_float4(y[0], y[1], y[2], y[3]);
-            to[1] = make_float4(y[4], y[5], y[6], y[7]);
-          } else {   // 128-byte rows, swizzled as the store's tensor map has it (short chunks: plain rows)
-            const int ch = (col >> 3) ^ (n == C ? row & 7 : 0);
-            *reinterpret_cast<uint4*>(out + row * 128 + ch * 16) =
-                make_uint4(pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]), pack_bf16(y[4], y[5]), pack_bf16(y[6], y[7]));
+        }
+        tc_fence_before_sync();
+        warp_arrive(bars.zu[s]);
+        if constexpr (kLayer) if (post) {
+          if (!out_vote()) { ok = false; break; }   // the fp32 tile is complete
+          float4 ov[8];   // piece i: values 0..3 in ov[2 i], 4..7 in ov[2 i + 1]
+          float ss = 0.f;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4* at = reinterpret_cast<const float4*>(out + tok * kN * 4 + part * 128 + piece(i) * 32);
+            const float4 x = at[part], y = at[part ^ 1];
+            ov[2 * i] = part ? y : x;
+            ov[2 * i + 1] = part ? x : y;
+          }
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            ss = fmaf(ov[i].x, ov[i].x, fmaf(ov[i].y, ov[i].y, fmaf(ov[i].z, ov[i].z, fmaf(ov[i].w, ov[i].w, ss))));
+          ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+          if (part == 0) st_async_f32(peer_at + s * (uint32_t)sizeof(peer_ss[0]), ss, peer_bar + s * 8);
+          MDN_OUT_WAIT(peer[s], ph2);
+          ss += *const_cast<volatile float*>(&peer_ss[s][tok]);
+          const float rstd = rsqrtf(ss * (1.f / kD) + a.post_eps);
+          if (!out_vote()) { ok = false; break; }   // the tile has been read
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int col = 32 * part + 8 * (piece(i) ^ swz);
+            const uint32_t gw[4] = {gate[i].x, gate[i].y, gate[i].z, gate[i].w};
+            const float o8[8] = {ov[2 * i].x, ov[2 * i].y, ov[2 * i].z, ov[2 * i].w, ov[2 * i + 1].x, ov[2 * i + 1].y, ov[2 * i + 1].z, ov[2 * i + 1].w};
+            float y[8];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              y[2 * e] = o8[2 * e] * rstd * w_sm[col + 2 * e] * sigmoid_fast(__uint_as_float(gw[e] << 16));
+              y[2 * e + 1] = o8[2 * e + 1] * rstd * w_sm[col + 2 * e + 1] * sigmoid_fast(__uint_as_float(gw[e] & 0xffff0000u));
+            }
+            if (sizeof(TO) == 4) {
+              float4* to = reinterpret_cast<float4*>(out + (tok * kN + col) * 4);
+              to[0] = make_float4(y[0], y[1], y[2], y[3]);
+              to[1] = make_float4(y[4], y[5], y[6], y[7]);
+            } else {   // 128-byte rows, swizzled as the store's tensor map has it (short chunks: plain rows)
+              const int ch = (col >> 3) ^ (n == C ? tok & 7 : 0);
+              *reinterpret_cast<uint4*>(out + tok * 128 + ch * 16) =
+                  make_uint4(pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]), pack_bf16(y[4], y[5]), pack_bf16(y[6], y[7]));
+            }
           }
         }
         fence_proxy_async_smem();
         warp_arrive(bars.go[s]);
-        MDN_MARK(c, kEvGo);
+        MDN_MARK(c - 1, kEvOutDone);
       }
+      if (c == nch) break;
+      // ---------------- inter-chunk output terms cZ .* (Q S) + cU .* (Q M) into the lower lanes of Z, for MMA-3' to accumulate onto
+      // (the upper lanes accumulate onto Q M: nobody reads them)
+      const int s = c & 1;
+      const float* aj = reinterpret_cast<const float*>(smem + kOffAdj + s * kAdjBytes) + cp;
+      MDN_OUT_WAIT(adj[s], (c >> 1) & 1);
+      MDN_OUT_WAIT(mz, c & 1);
+      tc_fence_after_sync();
+#pragma unroll 1
+      for (int r0 = 0; r0 < C; r0 += 32) {
+        const uint32_t zc = tl + kColZ + 64 * s + r0;
+        uint32_t zs[16], zm[16];
+        tmem_ld_16x256_x4(zc, zs);
+        tmem_ld_16x256_x4(zc + kUpper, zm);
+        float2 cz[4], cu[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          cz[j] = *reinterpret_cast<const float2*>(aj + kCz + r0 + 8 * j);
+          cu[j] = *reinterpret_cast<const float2*>(aj + kCu + r0 + 8 * j);
+        }
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const int i = 4 * j + 2 * e;
+            const float2 o2 = __ffma2_rn(cz[j], make_float2(__uint_as_float(zs[i]), __uint_as_float(zs[i + 1])),
+                                         __fmul2_rn(cu[j], make_float2(__uint_as_float(zm[i]), __uint_as_float(zm[i + 1]))));
+            zs[i] = __float_as_uint(o2.x);
+            zs[i + 1] = __float_as_uint(o2.y);
+          }
+        tmem_st_16x256_x4(zc, zs);
+      }
+      tmem_wait_st();
+      tc_fence_before_sync();
+      warp_arrive(bars.oi[s]);
+      MDN_MARK(c, kEvOiArrive);
     }
+    if (good == 0) ok = false;
+#undef MDN_OUT_WAIT
   } else if (warp < kEpiWarps) {
     // ================================================================== epilogue warps
     const int q4 = warp & 3, hf = warp >> 2;
@@ -574,76 +666,6 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
       for (int j = 0; j < 4; ++j) f[j] = *reinterpret_cast<const float2*>(aj + vec + r0 + 8 * j + cp);
     };
     auto pair = [](const uint32_t (&x)[16], int j, int e) { return make_float2(__uint_as_float(x[4 * j + 2 * e]), __uint_as_float(x[4 * j + 2 * e + 1])); };
-    // ---------------- inter-chunk output terms cZ .* (Q S) + cU .* (Q M) into the lower lanes of Z, for MMA-3' to accumulate onto
-    // (the upper lanes accumulate onto Q M: nobody reads them); false: a wait ran out
-    auto inter = [&](int c) -> bool {
-      const float* aj = reinterpret_cast<const float*>(smem + kOffAdj + (c & 1) * kAdjBytes);
-      const uint32_t zc = tl + kColZ + 64 * (c & 1) + r0;
-      float2 cz[4], cu[4];
-      coef4(cz, aj, kCz);
-      coef4(cu, aj, kCu);
-      if (!warp_wait(bar(bars.mz), c & 1, abortp)) return false;
-      __syncwarp();
-      tc_fence_after_sync();
-      uint32_t zs[16], zm[16];
-      tmem_ld_16x256_x4(zc, zs);
-      tmem_ld_16x256_x4(zc + kUpper, zm);
-      tmem_wait_ld();
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const float2 o2 = __ffma2_rn(cz[j], pair(zs, j, e), __fmul2_rn(cu[j], pair(zm, j, e)));
-          zs[4 * j + 2 * e] = __float_as_uint(o2.x);
-          zs[4 * j + 2 * e + 1] = __float_as_uint(o2.y);
-        }
-      tmem_st_16x256_x4(zc, zs);
-      tmem_wait_st();
-      tc_fence_before_sync();
-      warp_arrive(bars.oi);
-      MDN_MARK(c, kEvOiArrive);
-      return true;
-    };
-    // ---------------- a chunk's output: Z -> [64 tokens x 64 value columns] tile in shared memory
-    auto output = [&](int c) -> bool {
-      const int s = c & 1;
-      if (!warp_wait(bar(bars.mo), c & 1, abortp)) return false;
-      __syncwarp();
-      tc_fence_after_sync();
-      MDN_MARK(c, kEvMoSeen);
-      uint32_t u[16];
-      tmem_ld_16x256_x4(tl + kColZ + 64 * s + r0, u);
-      tmem_wait_ld();
-      tc_fence_before_sync();
-      warp_arrive(bars.zu[s]);
-      if (c >= 2 && !warp_wait(bar(bars.ofree[s]), ((c - 2) >> 1) & 1, abortp)) return false;
-      __syncwarp();
-      if (post || sizeof(TO) == 4) {
-        // an fp32 tile; for the output warps a row's pieces of eight values are rotated by its token pair (no bank is touched twice)
-        float* tile = reinterpret_cast<float*>(smem + kOffOut + s * kOutBytes);
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int t = r0 + 8 * j + cp + (e & 1), d = 16 * q4 + row + 8 * (e >> 1);
-            tile[t * kN + (post ? d ^ (((t >> 1) & 3) << 3) : d)] = __uint_as_float(u[4 * j + e]);
-          }
-      } else {
-        uint32_t pk[8];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-          for (int e = 0; e < 2; ++e) pk[2 * j + e] = pack_bf16(__uint_as_float(u[4 * j + 2 * e]), __uint_as_float(u[4 * j + 2 * e + 1]));
-        const uint32_t swz = sq.len - c * C >= C ? m_tok & 7 : 0;   // (a short chunk leaves row by row)
-#pragma unroll
-        for (int g = 0; g < 2; ++g)
-          stmatrix_x4_trans(s_base + kOffOut + s * kOutBytes + (m_tok + 16 * g) * 128 + ((m_ch ^ swz) << 4), pk + 4 * g);
-      }
-      fence_proxy_async_smem();
-      if (post) warp_arrive(bars.pn[s]); else warp_arrive(bars.go[s]);
-      MDN_MARK(c, kEvOutDone);
-      return true;
-    };
     {
       // ---------------- the start state into the masters
       const float* src = is_m ? rn.M0 : rn.S0;
@@ -663,11 +685,11 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
       warp_arrive(bars.init);
     }
 #pragma unroll 1
-    for (int c = 0; c <= nch; ++c) {
+    for (int c = 0; c < nch; ++c) {
       const int s = c & 1;
       const uint32_t ph = c & 1, ph2 = (c >> 1) & 1;
       const float* aj = reinterpret_cast<const float*>(smem + kOffAdj + s * kAdjBytes);
-      if (c < nch) {
+      {
         MDN_WAIT(kfull[s], ph2);
         MDN_WAIT(adj[s], ph2);
         __syncwarp();
@@ -715,18 +737,12 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
         warp_arrive(bars.r);
         MDN_MARK(c, kEvRArrive);
       }
-      if (write_o && c > 0 && !output(c - 1)) { ok = false; break; }   // (under MMA-2)
-      if (c == nch) break;
-      // EPI-2, then the inter-chunk output terms.  Eager chunks the other way round: the masters take G' = D_c G (under MMA-2) behind
-      // MMA-1z, their last reader in this chunk, and the update is added in true coordinates.
-      const bool eager = aj[kLazy] == 0.f;
-#pragma unroll 1
-      for (int step = 0; step < 2; ++step) {
-        if ((step == 0) == eager) {
-          if (write_o && !inter(c)) { ok = false; break; }
-          continue;
-        }
-        if (eager) {
+      // Eager chunks: the masters take G' = D_c G (under MMA-2) behind MMA-1z, their last reader in this chunk, and the update is added in
+      // true coordinates.
+      {
+        if (aj[kLazy] == 0.f) {
+            if (write_o) MDN_WAIT(mz, ph);
+            tc_fence_after_sync();
             const float n11 = aj[kN11], n12 = aj[kN12], n22 = aj[kN22];   // Sh <- n11 Sh + n12 Mh, Mh <- n22 Mh
 #pragma unroll 1
             for (int i = 0; i < 2; ++i) {
@@ -775,7 +791,6 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_half_kernel(const
           MDN_MARK(c, kEvVArrive);
         }
       }
-      if (!ok) break;
     }
     while (ok) {   // (once)
       // ---------------- final states: [S; M] = G [Sh; Mh]  
@@ -842,7 +857,7 @@ cudaError_t launch_chain_half(const Plan& pl, const ChainTf32Args& a, const Chai
                     : (o_bf16 ? chain_half_kernel<__nv_bfloat16, false> : chain_half_kernel<float, false>);
   cudaError_t e = allow_smem<(int)kSmemBytes>(kern);
   if (e != cudaSuccess) return e;
-  e = launch_pdl_cluster(layer ? 2 : 1, kern, dim3(2 * items), dim3(threads_of(layer)), kSmemBytes, pl.stream, a, mq, mk, mv, mt, mw, mo);
+  e = launch_pdl_cluster(layer ? 2 : 1, kern, dim3(2 * items), dim3(kThreads), kSmemBytes, pl.stream, a, mq, mk, mv, mt, mw, mo);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e == cudaSuccess) ++*launches;
   return e;

@@ -105,7 +105,8 @@ __device__ __forceinline__ bool warp_poll(uint32_t bar, uint32_t parity, volatil
   if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
   uint32_t left = kSpinLimit;
 #pragma unroll 1
-  while (!mbar_try_wait(bar, parity) && --left != 0) {}
+  while (!mbar_try_wait(bar, parity) && --left != 0)
+    if ((left & 255u) == 0 && *abort_flag != 0) left = 1;
   if (left == 0) *abort_flag = 1;
   return __all_sync(0xffffffffu, left != 0);
 }
