@@ -25,8 +25,14 @@
 // need not be are not unrolled.  A wait in a product-issuing warp costs 0.2 .. 0.4 k cycles even if its phase is long complete: the
 // serial chain's products have a warp of their own with three waits per chunk.
 //
-// With the layer operations the RMSNorm of the output step sums over all 128 value columns: the two CTAs of a chain are a
-// thread-block cluster and exchange each token's sum of squares through distributed shared memory.
+// Measured: 3.9 .. 4.2 k cycles per chunk against 6.3 k of chain_tf32.cu.  4 x 2048 tokens x 8 heads, whole call: 131.7 -> 96.5 us;
+// 200 tokens x 16 heads with a start state: 24.5 -> 19.5.
+//
+// The layer operations stay with chain_tf32.cu: their output step (a norm over all value columns, so an exchange between the two
+// CTAs) kept four output warps busy for longer than a chunk lasts here, and its code made every warp wait for instructions (4 x 3001
+// tokens x 16 heads: 252 .. 292 us in four arrangements, 265 there).
+#include <cstddef>
+
 #include "chain_tf32.cuh"
 #include "mdn_common.cuh"
 #include "tc_utils.cuh"
@@ -37,11 +43,10 @@ namespace {
 using namespace tc;
 
 constexpr int kD = 128, kN = 64;   // key columns; value columns of a CTA
-// Warps 0..7 epilogue (lane quarter = warp % 4, token half = warp / 4), 8 the products of the state's serial chain, 9 loads and
-// coefficients, 10 the products of the output, 11 output stores, 12..15 converters, 16..19 output.
+// Warps 0..7 epilogue (lane quarter = warp % 4, token half = warp / 4), 8 the products of the state's serial chain, 9 loads of K, V, Q,
+// coefficients, 10 the products of the output, 11 loads of T, W, output stores, 12..15 converters, 16..19 output.
 constexpr int kEpiWarps = 8, kWarpMma = 8, kWarpLoad = 9, kWarpMmaOut = 10, kWarpStore = 11, kWarpCvt = 12, kCvtWarps = 4, kWarpOut = 16, kOutWarps = 4;
 constexpr int kThreads = (kWarpOut + kOutWarps) * 32;
-constexpr int kOutThreads = kOutWarps * 32;
 constexpr int kTok = 32, kPk = 16;   // tokens of an epilogue warp; their packed bf16 pairs
 constexpr int kZFirst = 4;           // products of MMA-1z that fit under EPI-1, behind MMA-3'
 
@@ -62,37 +67,43 @@ static_assert(kStCoef + kCoefBytes <= kStageBytes && kSmemBytes <= kSmemOptin - 
 constexpr uint32_t kColP = 0, kColX = 128, kColY = 192, kColZ = 320;
 constexpr uint32_t kUpper = 16u << 16;               // the upper sixteen lanes of a warp's quarter: M
 
-// A barrier that a waiter could fall a whole phase behind comes in pairs, by the chunk's parity.
+// A barrier that a waiter could fall a whole phase behind comes in pairs, by the chunk's parity.  Grouped by their counts: the block's
+// first threads set up one each.
 struct Bars {
-  uint64_t kfull[2];  // bf16 K and V tiles of a stage landed                             (1 + tx bytes)
-  uint64_t full[2];   // T, coefficient vectors                                           (1 + tx bytes)
-  uint64_t wfull[2];  // W                                                                (1 + tx bytes)
-  uint64_t qfull;     // bf16 Q tile landed                                               (1 + tx bytes)
-  uint64_t qfree;     // ... and read                                                     (4 warps)
-  uint64_t xr;        // MMA-1x may start: fp32 K copy written, masters updated           (4 warps + commit)
-  uint64_t q32;       // fp32 Q copy written                                              (4 warps)
-  uint64_t adj[2];    // a chunk's coefficient block written, its T landed                (1)
-  uint64_t fin;       // G after the last chunk written                                   (1)
-  uint64_t init;      // masters of chunk 0 stored                                        (8 warps)
-  uint64_t mx;        // X done: the fp32 K copy is free too                              (commit)
-  uint64_t mz;        // Z done: the fp32 Q copy is free too                              (commit)
-  uint64_t r;         // EPI-1 done: R^T in X                                             (8 warps)
-  uint64_t m2;        // V~ in Y                                                          (commit)
-  uint64_t oi[2];     // inter-chunk output terms in Z                                    (4 warps)
-  uint64_t v;         // MMA-3 may start: update operand in X (eager chunks: masters rescaled), MMA-1z done  (8 warps + commit)
-  uint64_t m3[2];     // masters updated: the stage's K, V, T are free too                (commit)
-  uint64_t mo[2];     // MMA-3' done                                                      (commit)
-  uint64_t zu[2];     // Z (the chunk's output) has been read: W is free too              (4 warps)
-  uint64_t go[2];     // the output tile is staged                                        (4 warps)
-  uint64_t ofree[2];  // ... and read by its store                                        (1)
-  uint64_t peer[2];   // fused output step: the other CTA's sums of squares have arrived             (1 + 256 bytes)
+  // one arrival (a commit, or a thread; loads: and their bytes)
+  uint64_t kfull[2];  // bf16 K and V tiles of a stage landed
+  uint64_t full[2];   // coefficient vectors landed
+  uint64_t tfull[2];  // T landed
+  uint64_t wfull[2];  // W landed
+  uint64_t adj[2];    // a chunk's coefficient block written, its T landed
+  uint64_t m3[2];     // masters updated: the stage's K, V, T are free too
+  uint64_t mo[2];     // MMA-3' done
+  uint64_t ofree[2];  // the output tile has been read by its store
+  uint64_t qfull;     // bf16 Q tile landed
+  uint64_t mx;        // X done: the fp32 K copy is free too
+  uint64_t mz;        // Z done: the fp32 Q copy is free too
+  uint64_t m2;        // V~ in Y
+  uint64_t fin;       // G after the last chunk written
+  // four warps
+  uint64_t qfree;     // the bf16 Q tile has been read
+  uint64_t q32;       // fp32 Q copy written
+  uint64_t oi[2];     // inter-chunk output terms in Z
+  uint64_t zu[2];     // Z (the chunk's output) has been read: W is free too
+  uint64_t go[2];     // the output tile is staged
+  // eight warps
+  uint64_t init;      // masters of chunk 0 stored
+  uint64_t r;         // EPI-1 done: R^T in X
+  uint64_t v;         // MMA-3 may start: update operand in X (eager chunks: masters rescaled)   (+ commit: MMA-1z done)
+  uint64_t xr;        // MMA-1x may start: fp32 K copy written (four warps), masters updated (commit)
 };
+constexpr int kBars1 = 21, kBars4 = kBars1 + 8, kBars8 = kBars4 + 3;
+static_assert(offsetof(Bars, qfree) == kBars1 * 8 && offsetof(Bars, init) == kBars4 * 8 && offsetof(Bars, xr) == kBars8 * 8, "barrier groups");
 
 enum Ev : int { kEvTop = 0, kEvXIssued, kEvZIssued, kEvRSeen, kEvM2Issued, kEvMoIssued, kEvVSeen, kEvM3Issued,
                 kEvMxSeen, kEvRArrive, kEvOiArrive, kEvM2Seen, kEvVArrive, kEvMoSeen, kEvOutDone, kEvCvtK, kEvCvtKDone, kEvCvtQ,
                 kEvCvtQDone, kEvTma, kEvAdj, kEvStored };
 
-template <typename TO, bool kLayer>
+template <typename TO>
 __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32Args a, const __grid_constant__ CUtensorMap map_q,
                                                                 const __grid_constant__ CUtensorMap map_k,
                                                                 const __grid_constant__ CUtensorMap map_v,
@@ -105,13 +116,11 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
   __shared__ float g_final[4];   // G after the last chunk: what the final states are read through
-  __shared__ __align__(16) float w_sm[kLayer ? kN : 4];        // RMSNorm weight of the fused output step
-  __shared__ float peer_ss[2][kLayer ? C : 1];                 // the other CTA's sums of squares, by chunk parity
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int H = a.g.H;
   // Coefficients, T and W come from the previous kernel, which lets this one in before it has finished (intra_mma.cu): only
-  // the warp that loads those waits.  Everything else read here (the call's inputs, the chunk
+  // the warps that load those wait.  Everything else read here (the call's inputs, the chunk
   // map) was complete before that kernel could let anybody in.  Segment states come from the kernel just before this one.
   const bool early = a.seg_G == 0;
   if (!early) grid_dependency_wait();
@@ -129,27 +138,14 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
     __syncwarp();
     if (lane == 0) mbar_arrive(smem_u32(&b));
   };
-  const bool qk_on = kLayer && a.qk_on;
-  const float qk_dh = (qk_on && a.qk_d) ? __ldg(a.qk_d + h) : 0.f;
-  const bool post = kLayer && a.post_on && write_o;
-  const uint32_t peer_rank = kLayer ? cluster_rank() ^ 1u : 0u;
 
-  if (tid == 0) {
-    abort_flag = 0;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(bar(bars.kfull[i]), 1); mbar_init(bar(bars.full[i]), 1); mbar_init(bar(bars.wfull[i]), 1);
-      mbar_init(bar(bars.adj[i]), 1); mbar_init(bar(bars.m3[i]), 1); mbar_init(bar(bars.mo[i]), 1); mbar_init(bar(bars.oi[i]), kOutWarps);
-      mbar_init(bar(bars.zu[i]), kOutWarps); mbar_init(bar(bars.go[i]), kOutWarps); mbar_init(bar(bars.ofree[i]), 1);
-      mbar_init(bar(bars.peer[i]), 1);
-    }
-    mbar_init(bar(bars.qfull), 1); mbar_init(bar(bars.qfree), kCvtWarps); mbar_init(bar(bars.q32), kCvtWarps); mbar_init(bar(bars.xr), kCvtWarps + 1);
-    mbar_init(bar(bars.fin), 1); mbar_init(bar(bars.init), kEpiWarps);
-    mbar_init(bar(bars.mx), 1); mbar_init(bar(bars.mz), 1); mbar_init(bar(bars.m2), 1);
-    mbar_init(bar(bars.r), kEpiWarps); mbar_init(bar(bars.v), kEpiWarps + (write_o ? 1 : 0));
+  if (tid == 0) abort_flag = 0;
+  if (tid <= kBars8) {
+    const bool is_v = tid == kBars8 - 1;
+    mbar_init(smem_u32(&bars) + 8 * tid, tid < kBars1 ? 1 : tid < kBars4 ? 4 : tid < kBars8 ? kEpiWarps + (is_v && write_o ? 1 : 0) : kCvtWarps + 1);
     mbar_fence_init();
   }
-  if (kLayer && tid < kN) w_sm[tid] = (a.post_on && a.post_w) ? __ldg(a.post_w + v0 + tid) : 1.f;
+  static_assert(kCvtWarps == 4 && kOutWarps == 4, "barrier counts");
   if (warp == kWarpMma) tmem_alloc(smem_u32(&tmem_slot), 512);
   if (warp == kWarpLoad && lane == 0) {
     prefetch_tensormap(&map_q); prefetch_tensormap(&map_k); prefetch_tensormap(&map_v);
@@ -157,7 +153,6 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
   }
   tc_fence_before_sync();
   __syncthreads();
-  if constexpr (kLayer) cluster_sync_all();   // the other CTA's barriers are set up before anything arrives at them
   tc_fence_after_sync();
   const uint32_t tmem = tmem_slot;
   bool ok = true;
@@ -202,8 +197,8 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
 #endif
   if (warp == kWarpLoad) {
     // ================================================================== loads, coefficients
-    // A stage's K, V and T tiles are refilled (for chunk c + 2) as soon as MMA-3 has read K, the Q buffer as soon as it is converted, W
-    // when the output it belongs to has been read.  Who waits for a chunk's coefficient block need not wait for its T.
+    // A stage's K and V tiles are refilled (for chunk c + 2) as soon as MMA-3 has read K, the Q buffer as soon as it is converted.  Who
+    // waits for a chunk's coefficient block need not wait for its T.
     int issued = 0;
     float g11 = 1.f, g12 = 0.f, g22 = 1.f;
 #pragma unroll 1
@@ -230,27 +225,18 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
       if (early && c == 0) { grid_dependency_wait(); MDN_NOW(1); }
       if (lane == 0) {
         const uint32_t fb = bar(bars.full[s]);
-        mbar_arrive_expect_tx(fb, kCoefBytes + kTxT);
+        mbar_arrive_expect_tx(fb, kCoefBytes);
         bulk_load(st + kStCoef, a.coef + (size_t)mat * MDN_NUM_COEF * C, kCoefBytes, fb);
-        tma_load_2d(st + kStT, &map_t, 0, mat * C, fb);
       }
       issued = c + 1;
       MDN_MARK(c, kEvTma);
       MDN_WAIT(full[s], ph2);
+      MDN_WAIT(tfull[s], ph2);
       if (write_o && c >= 2) MDN_WAIT(oi[s], ph2 ^ 1);   // chunk c - 2's block has been read (MMA-3 of that chunk: by the epilogue)
-      publish_coefs<kLayer>(reinterpret_cast<const float*>(smem + kOffStage + s * kStageBytes + kStCoef),
+      publish_coefs<false>(reinterpret_cast<const float*>(smem + kOffStage + s * kStageBytes + kStCoef),
                             reinterpret_cast<float*>(smem + kOffAdj + s * kAdjBytes), a.scale, lane, g11, g12, g22);
       warp_arrive(bars.adj[s]);
       MDN_MARK(c, kEvAdj);
-      if (write_o) {
-        if (c >= 2) MDN_WAIT(zu[s], ph2 ^ 1);
-        if (lane == 0) {
-          mbar_arrive_expect_tx(bar(bars.wfull[s]), kTxW);
-          tma_load_2d(st + kStW, &map_w, 0, mat * C, bar(bars.wfull[s]));
-          tma_load_2d(st + kStW + 8192, &map_w, 32, mat * C, bar(bars.wfull[s]));
-        }
-        __syncwarp();
-      }
     }
     if (early && nch == 0) grid_dependency_wait();   // (every CTA ends after the previous kernel has)
     if (ok) {
@@ -265,33 +251,65 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
 #pragma unroll 1
         while (it < (1u << 18) && !(mbar_try_wait(bar(bars.kfull[c & 1]), (c >> 1) & 1) &&
                                     mbar_try_wait(bar(bars.full[c & 1]), (c >> 1) & 1) &&
-                                    (!write_o || (mbar_try_wait(bar(bars.qfull), c & 1) && mbar_try_wait(bar(bars.wfull[c & 1]), (c >> 1) & 1))))) ++it;
+                                    (!write_o || mbar_try_wait(bar(bars.qfull), c & 1)))) ++it;
       }
     }
   } else if (warp == kWarpStore) {
-    // ================================================================== output stores
+    // ================================================================== T and W tiles, output stores
+    // (A warp of its own: a copy takes the issuing warp 0.1 .. 0.2 k cycles, and nine a chunk in one warp made the K tile 2 k late.)
+    int issued = 0;
+    if (early) grid_dependency_wait();
 #pragma unroll 1
-    for (int c = 0; c < (write_o ? nch : 0); ++c) {
-      const int s = c & 1;
-      MDN_WAIT(go[s], (c >> 1) & 1);
-      if (lane == 0) {
-        const int n = min(C, sq.len - c * C);
-        const int tok = sq.tok0 + c * C;
-        const uint32_t src = s_base + kOffOut + s * kOutBytes;
-        if (n == C) {
-          tma_store_2d(&map_o, h * kD + v0, tok, src);
-        } else {   // short chunk: rows >= n belong to another sequence; one bulk copy per valid row (an unswizzled tile)
-#pragma unroll 1
-          for (int r = 0; r < n; ++r)
-            bulk_store(static_cast<uint8_t*>(a.o) + (((size_t)(tok + r) * H + h) * kD + v0) * sizeof(TO),
-                       src + r * kN * (uint32_t)sizeof(TO), kN * (uint32_t)sizeof(TO));
+    for (int c = 0; c < nch + (write_o ? 2 : 0); ++c) {
+      const int s = c & 1, mat = (sq.slot0 + c) * H + h;
+      const uint32_t ph2 = (c >> 1) & 1;
+      const uint32_t st = s_base + kOffStage + s * kStageBytes;
+      if (c < nch) {
+        if (c >= 2) MDN_WAIT(m3[s], ph2 ^ 1);
+        if (lane == 0) {
+          mbar_arrive_expect_tx(bar(bars.tfull[s]), kTxT);
+          tma_load_2d(st + kStT, &map_t, 0, mat * C, bar(bars.tfull[s]));
         }
-        tma_store_commit();
-        tma_store_wait_read();
-        mbar_arrive(bar(bars.ofree[s]));
+        issued = c + 1;
+        if (write_o) {
+          if (c >= 2) MDN_WAIT(zu[s], ph2 ^ 1);
+          if (lane == 0) {
+            mbar_arrive_expect_tx(bar(bars.wfull[s]), kTxW);
+            tma_load_2d(st + kStW, &map_w, 0, mat * C, bar(bars.wfull[s]));
+            tma_load_2d(st + kStW + 8192, &map_w, 32, mat * C, bar(bars.wfull[s]));
+          }
+        }
+      }
+      if (c >= 2 && write_o) {
+        const int co = c - 2;
+        MDN_WAIT(go[s], ph2 ^ 1);
+        if (lane == 0) {
+          const int n = min(C, sq.len - co * C), tok = sq.tok0 + co * C;
+          const uint32_t src = s_base + kOffOut + s * kOutBytes;
+          if (n == C) {
+            tma_store_2d(&map_o, h * kD + v0, tok, src);
+          } else {   // short chunk: rows >= n belong to another sequence; one bulk copy per valid row (an unswizzled tile)
+#pragma unroll 1
+            for (int r = 0; r < n; ++r)
+              bulk_store(static_cast<uint8_t*>(a.o) + (((size_t)(tok + r) * H + h) * kD + v0) * sizeof(TO),
+                         src + r * kN * (uint32_t)sizeof(TO), kN * (uint32_t)sizeof(TO));
+          }
+          tma_store_commit();
+          tma_store_wait_read();
+          mbar_arrive(bar(bars.ofree[s]));
+        }
+        MDN_MARK(co, kEvStored);
       }
       __syncwarp();
-      MDN_MARK(c, kEvStored);
+    }
+    if (!ok && lane == 0) {
+#pragma unroll 1
+      for (int c = max(0, issued - 2); c < issued; ++c) {
+        uint32_t it = 0;
+#pragma unroll 1
+        while (it < (1u << 18) && !(mbar_try_wait(bar(bars.tfull[c & 1]), (c >> 1) & 1) &&
+                                    (!write_o || mbar_try_wait(bar(bars.wfull[c & 1]), (c >> 1) & 1)))) ++it;
+      }
     }
     if (lane == 0) tma_store_wait_all();
   } else if (warp == kWarpMma) {
@@ -382,10 +400,10 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
         MDN_WAIT(oi[s ^ 1], ((c - 1) >> 1) & 1);
       }
       if (c < nch) {
-        MDN_WAIT(q32, ph);
-        MDN_WAIT(adj[s], ph2);
         if (c >= 2) MDN_WAIT(zu[s], ph2 ^ 1);   // the output that this chunk's Z held has been read
+        MDN_WAIT(adj[s], ph2);
         eager = reinterpret_cast<const float*>(smem + kOffAdj + s * kAdjBytes)[kLazy] == 0.f;
+        MDN_WAIT(q32, ph);
         MDN_POLL(mx, ph);
       }
       tc_fence_after_sync();
@@ -463,23 +481,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
         warp_arrive(bars.qfree);
         if (c > 0) MDN_WAIT(mz, (c - 1) & 1);             // the previous chunk's product has read the copy
         MDN_MARK(c, kEvCvtQ);
-        if constexpr (kLayer) {
-          // fused q/k norm: the copy is q - d k (its 1/|q - d k| rides on the output terms' coefficients)
-#pragma unroll
-          for (uint32_t i = 0; i < 8; ++i) {
-            const uint32_t wk[4] = {uk[i].x, uk[i].y, uk[i].z, uk[i].w}, wq[4] = {uq[i].x, uq[i].y, uq[i].z, uq[i].w};
-            uint32_t f[8];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              f[2 * e] = __float_as_uint(fmaf(-qk_dh, __uint_as_float(wk[e] << 16), __uint_as_float(wq[e] << 16)));
-              f[2 * e + 1] = __float_as_uint(fmaf(-qk_dh, __uint_as_float(wk[e] & 0xffff0000u), __uint_as_float(wq[e] & 0xffff0000u)));
-            }
-            store4(s_base + kOffQ32, i, 0, f[0], f[1], f[2], f[3]);
-            store4(s_base + kOffQ32, i, 1, f[4], f[5], f[6], f[7]);
-          }
-        } else {
-          store8(s_base + kOffQ32, uq);
-        }
+        store8(s_base + kOffQ32, uq);
         fence_proxy_async_smem();
         warp_arrive(bars.q32);
         MDN_MARK(c, kEvCvtQDone);
@@ -489,51 +491,14 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
     // ================================================================== output warps (one lane quarter each, all 64 tokens)
     const int q4 = warp & 3, row = lane >> 2, cp = 2 * (lane & 3);   // value columns 16 q4 + row, + 8; tokens 32 hf + 8 j + cp, + 1
     const uint32_t tl = tmem + (static_cast<uint32_t>(q4 * 32) << 16);
-    // fused output step: y = sigmoid(g) * o / sqrt(mean_d o^2 + eps) * w_d, the mean over both CTAs' columns.  Two threads per token, 32
-    // neighbouring values each, in four pieces of eight whose order and halves rotate with the token and the thread (eight neighbouring
-    // lanes touch every bank once).  The whole fp32 tile is in registers before anything is written over it.  Sums of squares go to
-    // the other CTA by st.async, which completes its barrier's bytes: a plain remote store and a releasing arrival waited 2 k
-    // cycles for this thread's outstanding loads.
-    const int t128 = tid - kWarpOut * 32, tok = t128 >> 1, part = t128 & 1, swz = (tok >> 1) & 3;
-    const uint32_t peer_bar = kLayer ? map_to_cta(bar(bars.peer[0]), peer_rank) : 0u;
-    const uint32_t peer_at = kLayer ? map_to_cta(smem_u32(&peer_ss[0][kLayer ? tok : 0]), peer_rank) : 0u;
-    auto piece = [&](int i) { return (i + tok) & 3; };   // place of the i-th piece among the thread's four; its columns: 8 (place ^ swz)
-    // With the fused step these warps meet at barriers: one whose wait runs out goes on to the next of those, which carries the vote
-    // whether every wait has ended, and they all leave together.
-    uint32_t good = 1;
-    auto out_vote = [&]() -> bool {
-      asm volatile(
-          "{\n\t.reg .pred p, q;\n\t"
-          "setp.ne.u32 q, %0, 0;\n\t"
-          "barrier.cta.red.and.pred p, 1, %1, q;\n\t"
-          "selp.u32 %0, 1, 0, p;\n\t}\n"
-          : "+r"(good)
-          : "n"(kOutThreads)
-          : "memory");
-      return good != 0;
-    };
-#define MDN_OUT_WAIT(b, par)                                        \
-  if (!warp_wait(smem_u32(&bars.b), (par), abortp)) {               \
-    good = 0;                                                       \
-    if (!post) { ok = false; break; }                               \
-  }
 #pragma unroll 1
     for (int c = 0; c <= (write_o ? nch : -1); ++c) {
       // ---------------- the previous chunk's output: Z -> [64 tokens x 64 value columns] tile in shared memory
       if (c > 0) {
         const int s = (c - 1) & 1, n = min(C, sq.len - (c - 1) * C);
         const uint32_t ph2 = ((c - 1) >> 1) & 1;
-        uint8_t* const out = smem + kOffOut + s * kOutBytes;
-        uint4 gate[kLayer ? 4 : 1];   // before the wait
-        if (kLayer && post) {
-          const __nv_bfloat16* gp = static_cast<const __nv_bfloat16*>(a.post_g) + ((size_t)(sq.tok0 + (c - 1) * C + tok) * H + h) * kD + v0 + 32 * part;
-#pragma unroll
-          for (int i = 0; i < (kLayer ? 4 : 1); ++i)
-            gate[i] = tok < n ? __ldg(reinterpret_cast<const uint4*>(gp + 8 * (piece(i) ^ swz))) : make_uint4(0u, 0u, 0u, 0u);
-          if (t128 == 0) mbar_arrive_expect_tx(bar(bars.peer[s]), C * (uint32_t)sizeof(float));
-        }
-        if (c >= 3) MDN_OUT_WAIT(ofree[s], ph2 ^ 1);
-        MDN_OUT_WAIT(mo[s], ph2);
+        if (c >= 3) MDN_WAIT(ofree[s], ph2 ^ 1);
+        MDN_WAIT(mo[s], ph2);
         tc_fence_after_sync();
         MDN_MARK(c - 1, kEvMoSeen);
 #pragma unroll 1
@@ -541,14 +506,12 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
           uint32_t u[16];
           tmem_ld_16x256_x4(tl + kColZ + 64 * s + r0, u);
           tmem_wait_ld();
-          if (post || sizeof(TO) == 4) {
-            // an fp32 tile; for the fused step a token's pieces of eight values are rotated by its pair (no bank is touched twice)
-            float* at = reinterpret_cast<float*>(out) + (r0 + cp) * kN;
-            const int turn = post ? (lane & 3) << 3 : 0, d0 = (16 * q4 + row) ^ turn, d1 = (16 * q4 + row + 8) ^ turn;
+          if (sizeof(TO) == 4) {
+            float* at = reinterpret_cast<float*>(smem + kOffOut + s * kOutBytes) + (r0 + cp) * kN + 16 * q4 + row;
 #pragma unroll
             for (int j = 0; j < 4; ++j)
 #pragma unroll
-              for (int e = 0; e < 4; ++e) at[(8 * j + (e & 1)) * kN + (e < 2 ? d0 : d1)] = __uint_as_float(u[4 * j + e]);
+              for (int e = 0; e < 4; ++e) at[(8 * j + (e & 1)) * kN + 8 * (e >> 1)] = __uint_as_float(u[4 * j + e]);
           } else {
             uint32_t pk[8];
 #pragma unroll
@@ -563,48 +526,6 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
         }
         tc_fence_before_sync();
         warp_arrive(bars.zu[s]);
-        if constexpr (kLayer) if (post) {
-          if (!out_vote()) { ok = false; break; }   // the fp32 tile is complete
-          float4 ov[8];   // piece i: values 0..3 in ov[2 i], 4..7 in ov[2 i + 1]
-          float ss = 0.f;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float4* at = reinterpret_cast<const float4*>(out + tok * kN * 4 + part * 128 + piece(i) * 32);
-            const float4 x = at[part], y = at[part ^ 1];
-            ov[2 * i] = part ? y : x;
-            ov[2 * i + 1] = part ? x : y;
-          }
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            ss = fmaf(ov[i].x, ov[i].x, fmaf(ov[i].y, ov[i].y, fmaf(ov[i].z, ov[i].z, fmaf(ov[i].w, ov[i].w, ss))));
-          ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-          if (part == 0) st_async_f32(peer_at + s * (uint32_t)sizeof(peer_ss[0]), ss, peer_bar + s * 8);
-          MDN_OUT_WAIT(peer[s], ph2);
-          ss += *const_cast<volatile float*>(&peer_ss[s][tok]);
-          const float rstd = rsqrtf(ss * (1.f / kD) + a.post_eps);
-          if (!out_vote()) { ok = false; break; }   // the tile has been read
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int col = 32 * part + 8 * (piece(i) ^ swz);
-            const uint32_t gw[4] = {gate[i].x, gate[i].y, gate[i].z, gate[i].w};
-            const float o8[8] = {ov[2 * i].x, ov[2 * i].y, ov[2 * i].z, ov[2 * i].w, ov[2 * i + 1].x, ov[2 * i + 1].y, ov[2 * i + 1].z, ov[2 * i + 1].w};
-            float y[8];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              y[2 * e] = o8[2 * e] * rstd * w_sm[col + 2 * e] * sigmoid_fast(__uint_as_float(gw[e] << 16));
-              y[2 * e + 1] = o8[2 * e + 1] * rstd * w_sm[col + 2 * e + 1] * sigmoid_fast(__uint_as_float(gw[e] & 0xffff0000u));
-            }
-            if (sizeof(TO) == 4) {
-              float4* to = reinterpret_cast<float4*>(out + (tok * kN + col) * 4);
-              to[0] = make_float4(y[0], y[1], y[2], y[3]);
-              to[1] = make_float4(y[4], y[5], y[6], y[7]);
-            } else {   // 128-byte rows, swizzled as the store's tensor map has it (short chunks: plain rows)
-              const int ch = (col >> 3) ^ (n == C ? tok & 7 : 0);
-              *reinterpret_cast<uint4*>(out + tok * 128 + ch * 16) =
-                  make_uint4(pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]), pack_bf16(y[4], y[5]), pack_bf16(y[6], y[7]));
-            }
-          }
-        }
         fence_proxy_async_smem();
         warp_arrive(bars.go[s]);
         MDN_MARK(c - 1, kEvOutDone);
@@ -614,8 +535,8 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
       // (the upper lanes accumulate onto Q M: nobody reads them)
       const int s = c & 1;
       const float* aj = reinterpret_cast<const float*>(smem + kOffAdj + s * kAdjBytes) + cp;
-      MDN_OUT_WAIT(adj[s], (c >> 1) & 1);
-      MDN_OUT_WAIT(mz, c & 1);
+      MDN_WAIT(adj[s], (c >> 1) & 1);
+      MDN_WAIT(mz, c & 1);
       tc_fence_after_sync();
 #pragma unroll 1
       for (int r0 = 0; r0 < C; r0 += 32) {
@@ -647,8 +568,6 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
       warp_arrive(bars.oi[s]);
       MDN_MARK(c, kEvOiArrive);
     }
-    if (good == 0) ok = false;
-#undef MDN_OUT_WAIT
   } else if (warp < kEpiWarps) {
     // ================================================================== epilogue warps
     const int q4 = warp & 3, hf = warp >> 2;
@@ -689,111 +608,107 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
       const int s = c & 1;
       const uint32_t ph = c & 1, ph2 = (c >> 1) & 1;
       const float* aj = reinterpret_cast<const float*>(smem + kOffAdj + s * kAdjBytes);
+      MDN_WAIT(kfull[s], ph2);
+      MDN_WAIT(adj[s], ph2);
+      __syncwarp();
+      // ---------------- EPI-1: R^T = V^T - cX .* (K S) + cY .* (K M)  -> bf16 hi, lo into X, in both halves of the lanes
       {
-        MDN_WAIT(kfull[s], ph2);
-        MDN_WAIT(adj[s], ph2);
-        __syncwarp();
-        // ---------------- EPI-1: R^T = V^T - cX .* (K S) + cY .* (K M)  -> bf16 hi, lo into X, in both halves of the lanes
-        {
-          // V and the coefficients are fetched before the wait
-          uint32_t vr[8];   // [pair of token groups][m]: token group 2 g + m / 2, value column half m % 2
-          if (!v_zero) {
+        // V and the coefficients are fetched before the wait
+        uint32_t vr[8];   // [pair of token groups][m]: token group 2 g + m / 2, value column half m % 2
+        if (!v_zero) {
 #pragma unroll
-            for (int g = 0; g < 2; ++g)
-              ldmatrix_x4_trans(s_base + kOffStage + s * kStageBytes + kStV + (m_tok + 16 * g) * 128 + ((m_ch ^ (m_tok & 7)) << 4), vr + 4 * g);
-          } else {
+          for (int g = 0; g < 2; ++g)
+            ldmatrix_x4_trans(s_base + kOffStage + s * kStageBytes + kStV + (m_tok + 16 * g) * 128 + ((m_ch ^ (m_tok & 7)) << 4), vr + 4 * g);
+        } else {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) vr[i] = 0u;
-          }
-          float2 cx[4], cy[4];
-          coef4(cx, aj, kCx);   // (-cX)
-          coef4(cy, aj, kCy);
-          MDN_POLL(mx, ph);
-          tc_fence_after_sync();
-          MDN_MARK(c, kEvMxSeen);
-          uint32_t xs[16], xm[16];
-          tmem_ld_16x256_x4(tl + kColX + r0, xs);
-          tmem_ld_16x256_x4(tl + kUpper + kColX + r0, xm);
-          tmem_wait_ld();
-          uint32_t hi[8], lo[8];
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const uint32_t vw = vr[4 * (j >> 1) + 2 * (j & 1) + e];
-              float2 x = make_float2(__uint_as_float(vw << 16), __uint_as_float(vw & 0xffff0000u));
-              x = __ffma2_rn(cx[j], pair(xs, j, e), x);
-              x = __ffma2_rn(cy[j], pair(xm, j, e), x);
-              split_pack_bf16(x, hi[2 * j + e], lo[2 * j + e]);
-            }
-          // (the columns this warp has just read)
-          tmem_st_16x128_x4(tl + kColX + r0, hi);
-          tmem_st_16x128_x4(tl + kUpper + kColX + r0, hi);
-          tmem_st_16x128_x4(tl + kColX + r0 + kPk, lo);
-          tmem_st_16x128_x4(tl + kUpper + kColX + r0 + kPk, lo);
-          tmem_wait_st();
+          for (int i = 0; i < 8; ++i) vr[i] = 0u;
         }
-        tc_fence_before_sync();
-        warp_arrive(bars.r);
-        MDN_MARK(c, kEvRArrive);
+        float2 cx[4], cy[4];
+        coef4(cx, aj, kCx);   // (-cX)
+        coef4(cy, aj, kCy);
+        MDN_POLL(mx, ph);
+        tc_fence_after_sync();
+        MDN_MARK(c, kEvMxSeen);
+        uint32_t xs[16], xm[16];
+        tmem_ld_16x256_x4(tl + kColX + r0, xs);
+        tmem_ld_16x256_x4(tl + kUpper + kColX + r0, xm);
+        tmem_wait_ld();
+        uint32_t hi[8], lo[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const uint32_t vw = vr[4 * (j >> 1) + 2 * (j & 1) + e];
+            float2 x = make_float2(__uint_as_float(vw << 16), __uint_as_float(vw & 0xffff0000u));
+            x = __ffma2_rn(cx[j], pair(xs, j, e), x);
+            x = __ffma2_rn(cy[j], pair(xm, j, e), x);
+            split_pack_bf16(x, hi[2 * j + e], lo[2 * j + e]);
+          }
+        // (the columns this warp has just read)
+        tmem_st_16x128_x4(tl + kColX + r0, hi);
+        tmem_st_16x128_x4(tl + kUpper + kColX + r0, hi);
+        tmem_st_16x128_x4(tl + kColX + r0 + kPk, lo);
+        tmem_st_16x128_x4(tl + kUpper + kColX + r0 + kPk, lo);
+        tmem_wait_st();
       }
-      // Eager chunks: the masters take G' = D_c G (under MMA-2) behind MMA-1z, their last reader in this chunk, and the update is added in
-      // true coordinates.
-      {
-        if (aj[kLazy] == 0.f) {
-            if (write_o) MDN_WAIT(mz, ph);
-            tc_fence_after_sync();
-            const float n11 = aj[kN11], n12 = aj[kN12], n22 = aj[kN22];   // Sh <- n11 Sh + n12 Mh, Mh <- n22 Mh
+      tc_fence_before_sync();
+      warp_arrive(bars.r);
+      MDN_MARK(c, kEvRArrive);
+      // ---------------- eager chunks: the masters take G' = D_c G (under MMA-2) behind MMA-1z, their last reader in this chunk, and the
+      // update is added in true coordinates:  Sh <- n11 Sh + n12 Mh, Mh <- n22 Mh
+      if (aj[kLazy] == 0.f) {
+        if (write_o) MDN_WAIT(mz, ph);
+        tc_fence_after_sync();
+        const float n11 = aj[kN11], n12 = aj[kN12], n22 = aj[kN22];
 #pragma unroll 1
-            for (int i = 0; i < 2; ++i) {
-              const uint32_t col0 = kColP + hf * 64 + i * 32;
-              uint32_t ps[16], pm[16];
-              tmem_ld_16x256_x4(tl + col0, ps);
-              tmem_ld_16x256_x4(tl + kUpper + col0, pm);
-              tmem_wait_ld();
-#pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                ps[j] = __float_as_uint(unscale_s(n11, __uint_as_float(ps[j]), n12, __uint_as_float(pm[j])));
-                pm[j] = __float_as_uint(n22 * __uint_as_float(pm[j]));
-              }
-              tmem_st_16x256_x4(tl + col0, ps);
-              tmem_st_16x256_x4(tl + kUpper + col0, pm);
-            }
-          }
-        // ---------------- EPI-2: wS .* V~ | -wM .* V~ -> X as bf16 hi, lo
-        {
-          float2 ws[4], wm[4];
-          coef4(ws, aj, kWs);
-          coef4(wm, aj, kWm);
-          MDN_POLL(m2, ph);
-          tc_fence_after_sync();
-          MDN_MARK(c, kEvM2Seen);
-          uint32_t vt[16];
-          tmem_ld_16x256_x4(tl + kColY + 64 * s + r0, vt);
+        for (int i = 0; i < 2; ++i) {
+          const uint32_t col0 = kColP + hf * 64 + i * 32;
+          uint32_t ps[16], pm[16];
+          tmem_ld_16x256_x4(tl + col0, ps);
+          tmem_ld_16x256_x4(tl + kUpper + col0, pm);
           tmem_wait_ld();
-          uint32_t hi[8], lo[8];
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) split_pack_bf16(__fmul2_rn(ws[j], pair(vt, j, e)), hi[2 * j + e], lo[2 * j + e]);
-          tmem_st_16x128_x4(tl + kColX + r0, hi);          // X is free: MMA-2 has consumed R
-          tmem_st_16x128_x4(tl + kColX + r0 + kPk, lo);
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int e = 0; e < 2; ++e)
-              split_pack_bf16(__fmul2_rn(make_float2(-wm[j].x, -wm[j].y), pair(vt, j, e)), hi[2 * j + e], lo[2 * j + e]);
-          tmem_st_16x128_x4(tl + kUpper + kColX + r0, hi);
-          tmem_st_16x128_x4(tl + kUpper + kColX + r0 + kPk, lo);
-          tmem_wait_st();
-          tc_fence_before_sync();
-          warp_arrive(bars.v);
-          MDN_MARK(c, kEvVArrive);
+          for (int j = 0; j < 16; ++j) {
+            ps[j] = __float_as_uint(unscale_s(n11, __uint_as_float(ps[j]), n12, __uint_as_float(pm[j])));
+            pm[j] = __float_as_uint(n22 * __uint_as_float(pm[j]));
+          }
+          tmem_st_16x256_x4(tl + col0, ps);
+          tmem_st_16x256_x4(tl + kUpper + col0, pm);
         }
+      }
+      // ---------------- EPI-2: wS .* V~ | -wM .* V~ -> X as bf16 hi, lo
+      {
+        float2 ws[4], wm[4];
+        coef4(ws, aj, kWs);
+        coef4(wm, aj, kWm);
+        MDN_POLL(m2, ph);
+        tc_fence_after_sync();
+        MDN_MARK(c, kEvM2Seen);
+        uint32_t vt[16];
+        tmem_ld_16x256_x4(tl + kColY + 64 * s + r0, vt);
+        tmem_wait_ld();
+        uint32_t hi[8], lo[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) split_pack_bf16(__fmul2_rn(ws[j], pair(vt, j, e)), hi[2 * j + e], lo[2 * j + e]);
+        tmem_st_16x128_x4(tl + kColX + r0, hi);          // X is free: MMA-2 has consumed R
+        tmem_st_16x128_x4(tl + kColX + r0 + kPk, lo);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int e = 0; e < 2; ++e)
+            split_pack_bf16(__fmul2_rn(make_float2(-wm[j].x, -wm[j].y), pair(vt, j, e)), hi[2 * j + e], lo[2 * j + e]);
+        tmem_st_16x128_x4(tl + kUpper + kColX + r0, hi);
+        tmem_st_16x128_x4(tl + kUpper + kColX + r0 + kPk, lo);
+        tmem_wait_st();
+        tc_fence_before_sync();
+        warp_arrive(bars.v);
+        MDN_MARK(c, kEvVArrive);
       }
     }
     while (ok) {   // (once)
-      // ---------------- final states: [S; M] = G [Sh; Mh]  
+      // ---------------- final states: [S; M] = G [Sh; Mh]
       if (nch > 0) MDN_WAIT(m3[(nch - 1) & 1], ((nch - 1) >> 1) & 1);
       MDN_WAIT(fin, 0);
       __syncwarp();
@@ -824,10 +739,6 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
   if (!ok && lane == 0) atomicCAS(a.status, kDevOk, kDevTimeout);
   tc_fence_before_sync();
   __syncthreads();
-  if constexpr (kLayer) {   // neither CTA's shared memory goes while the other may still write to it
-    if (!ok) __nanosleep(100000);   // (what was sent before a wait ran out lands)
-    cluster_sync_all();
-  }
 #ifdef MDN_DEBUG
   if (warp == 0) { MDN_NOW(5); }
   if (tline != nullptr && tid < 256) tline[(kTlFirst + (tid >> 5)) * 32 + (tid & 31)] = tl_sm[tid >> 5][tid & 31];
@@ -852,12 +763,10 @@ cudaError_t launch_chain_half(const Plan& pl, const ChainTf32Args& a, const Chai
       !encode_tma_2d(&mw, TmaMap2D{pl.ws + pl.lay.off_W, 64, mats * C, 256, 32, 64, true}, true) ||
       !encode_tma_2d(&mo, TmaMap2D{a.o, row, tokens, row * (o_bf16 ? 2u : 4u), kN, 64, o_bf16}, !o_bf16))
     return cudaErrorInvalidValue;
-  const bool layer = a.qk_on || a.post_on;
-  auto kern = layer ? (o_bf16 ? chain_half_kernel<__nv_bfloat16, true> : chain_half_kernel<float, true>)
-                    : (o_bf16 ? chain_half_kernel<__nv_bfloat16, false> : chain_half_kernel<float, false>);
+  auto kern = o_bf16 ? chain_half_kernel<__nv_bfloat16> : chain_half_kernel<float>;
   cudaError_t e = allow_smem<(int)kSmemBytes>(kern);
   if (e != cudaSuccess) return e;
-  e = launch_pdl_cluster(layer ? 2 : 1, kern, dim3(2 * items), dim3(kThreads), kSmemBytes, pl.stream, a, mq, mk, mv, mt, mw, mo);
+  e = launch_pdl(kern, dim3(2 * items), dim3(kThreads), kSmemBytes, pl.stream, a, mq, mk, mv, mt, mw, mo);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e == cudaSuccess) ++*launches;
   return e;

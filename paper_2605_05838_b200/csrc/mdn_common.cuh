@@ -125,21 +125,15 @@ template <int kBytes, typename... A> inline cudaError_t allow_smem(void (*kern)(
 // before its own wait is over: so whatever was complete when the PREVIOUS kernel began its work (a call's inputs, whoever
 // made them and however early that kernel let its dependents in) is complete here before the wait, and may be read there.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl_cluster(unsigned cluster, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                                      cudaStream_t stream, Args&&... args) {   // `cluster` CTAs form a thread-block cluster
+inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                              Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
-}
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args&&... args) {
-  return launch_pdl_cluster(1, kern, grid, block, smem, stream, static_cast<KArgs>(args)...);
 }
 
 template <typename T> __device__ __forceinline__ float to_f32(T x);
