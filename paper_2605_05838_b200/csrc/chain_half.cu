@@ -132,12 +132,6 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
 
   const uint32_t s_base = smem_u32(smem);
   auto bar = [](uint64_t& b) { return smem_u32(&b); };
-  // One arrival per warp, for what its lanes have done before (tensor memory: behind the wait for it and the fence).  An arrival
-  // per thread is 256 shared-memory operations per hand-over: 3.9 -> 3.65 k cycles per chunk.
-  auto warp_arrive = [&](uint64_t& b) {
-    __syncwarp();
-    if (lane == 0) mbar_arrive(smem_u32(&b));
-  };
 
   if (tid == 0) abort_flag = 0;
   if (tid <= kBars8) {
@@ -235,7 +229,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
       if (write_o && c >= 2) MDN_WAIT(oi[s], ph2 ^ 1);   // chunk c - 2's block has been read (MMA-3 of that chunk: by the epilogue)
       publish_coefs<false>(reinterpret_cast<const float*>(smem + kOffStage + s * kStageBytes + kStCoef),
                             reinterpret_cast<float*>(smem + kOffAdj + s * kAdjBytes), a.scale, lane, g11, g12, g22);
-      warp_arrive(bars.adj[s]);
+      warp_arrive(bar(bars.adj[s]));
       MDN_MARK(c, kEvAdj);
     }
     if (early && nch == 0) grid_dependency_wait();   // (every CTA ends after the previous kernel has)
@@ -472,18 +466,18 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
       load8(uk, k_tile);
       store8(s_base + kOffK32, uk);
       fence_proxy_async_smem();
-      warp_arrive(bars.xr);
+      warp_arrive(bar(bars.xr));
       MDN_MARK(c, kEvCvtKDone);
       if (write_o) {
         MDN_WAIT(qfull, c & 1);
         uint4 uq[8];
         load8(uq, s_base + kOffQb);
-        warp_arrive(bars.qfree);
+        warp_arrive(bar(bars.qfree));
         if (c > 0) MDN_WAIT(mz, (c - 1) & 1);             // the previous chunk's product has read the copy
         MDN_MARK(c, kEvCvtQ);
         store8(s_base + kOffQ32, uq);
         fence_proxy_async_smem();
-        warp_arrive(bars.q32);
+        warp_arrive(bar(bars.q32));
         MDN_MARK(c, kEvCvtQDone);
       }
     }
@@ -525,9 +519,9 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
           }
         }
         tc_fence_before_sync();
-        warp_arrive(bars.zu[s]);
+        warp_arrive(bar(bars.zu[s]));
         fence_proxy_async_smem();
-        warp_arrive(bars.go[s]);
+        warp_arrive(bar(bars.go[s]));
         MDN_MARK(c - 1, kEvOutDone);
       }
       if (c == nch) break;
@@ -565,7 +559,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
       }
       tmem_wait_st();
       tc_fence_before_sync();
-      warp_arrive(bars.oi[s]);
+      warp_arrive(bar(bars.oi[s]));
       MDN_MARK(c, kEvOiArrive);
     }
   } else if (warp < kEpiWarps) {
@@ -601,7 +595,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
       }
       tmem_wait_st();
       tc_fence_before_sync();
-      warp_arrive(bars.init);
+      warp_arrive(bar(bars.init));
     }
 #pragma unroll 1
     for (int c = 0; c < nch; ++c) {
@@ -652,7 +646,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
         tmem_wait_st();
       }
       tc_fence_before_sync();
-      warp_arrive(bars.r);
+      warp_arrive(bar(bars.r));
       MDN_MARK(c, kEvRArrive);
       // ---------------- eager chunks: the masters take G' = D_c G (under MMA-2) behind MMA-1z, their last reader in this chunk, and the
       // update is added in true coordinates:  Sh <- n11 Sh + n12 Mh, Mh <- n22 Mh
@@ -703,7 +697,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
         tmem_st_16x128_x4(tl + kUpper + kColX + r0 + kPk, lo);
         tmem_wait_st();
         tc_fence_before_sync();
-        warp_arrive(bars.v);
+        warp_arrive(bar(bars.v));
         MDN_MARK(c, kEvVArrive);
       }
     }

@@ -898,7 +898,7 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
   auto launch = [&](unsigned grid) -> cudaError_t {
     // two CTAs per run while all of them are resident at once (measured at 32 chains: 131.7 -> 96.5 us; above, a second wave of
     // halves would cost 2 x 4.1 k cycles per chunk against 6.3 k)
-    if (!layer && 2 * grid <= (unsigned)kSms) return launch_chain_half(pl, a, ChainTensors{q, k, v}, grid, launches);
+    if (!layer && half_runs(grid)) return launch_chain_half(pl, a, ChainTensors{q, k, v}, grid, launches);
     auto kern = layer ? (o_bf16 ? chain_tf32_kernel<__nv_bfloat16, true> : chain_tf32_kernel<float, true>)
                       : (o_bf16 ? chain_tf32_kernel<__nv_bfloat16, false> : chain_tf32_kernel<float, false>);
     cudaError_t e = allow_smem<(int)kSmemBytes>(kern);
@@ -910,11 +910,14 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
   };
   const int G = pl.lay.segments;
   if (G <= 1) return launch(chains);
+  const SegSplit split = choose_segments(p);
+  // The split is chosen (and its scratch sized) by the pace of one CTA per chain; where two make the whole chain faster than the
+  // scan is expected to be, it runs serially all the same.
+  if (!layer && p.segments == 0 && p.num_seqs == 0 && half_runs(chains) && kHalfChunk * pl.geom.chunks_per_seq <= split.cost) return launch(chains);
 
   // ---- parallel inter-chunk scan: Psi / Phi of the middle segments, serial combine, then all segments for real
   constexpr size_t kMat = (size_t)kD * kD;
   float* seg = reinterpret_cast<float*>(pl.seg);
-  const SegSplit split = choose_segments(p);
   a.seg_G = G;
   a.seg_first = split.first; a.seg_mid = split.mid; a.seg_least = p.segments ? 1 : kSegLeast;
   a.seg_E = seg;

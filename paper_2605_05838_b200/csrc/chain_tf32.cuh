@@ -122,7 +122,7 @@ __device__ __forceinline__ void publish_coefs(const float* cf, float* aj, float 
   const float aC = cf[kAbar * C + C - 1], bC = cf[kB * C + C - 1], mC = cf[kMubar * C + C - 1];
   const float n11 = __fmul_rn(aC, g11), n12 = __fsub_rn(__fmul_rn(aC, g12), __fmul_rn(bC, g22)), n22 = __fmul_rn(mC, g22);
   const bool lazy = n11 >= kLazyMin && n22 >= kLazyMin && fabsf(n12) <= kLazyMix * n22;
-#pragma unroll 1   // (two divisions less in the instruction cache)
+#pragma unroll
   for (int e = 0; e < 2; ++e) {
     const int t = 2 * lane + e;
     const float ab = cf[kAbar * C + t], bb = cf[kB * C + t], pp = cf[kAlphaBPrev * C + t];
