@@ -580,19 +580,17 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
     };
     auto pair = [](const uint32_t (&x)[16], int j, int e) { return make_float2(__uint_as_float(x[4 * j + 2 * e]), __uint_as_float(x[4 * j + 2 * e + 1])); };
     {
-      // ---------------- the start state into the masters
+      // ---------------- the start state into the masters (all loads in flight at once)
       const float* src = is_m ? rn.M0 : rn.S0;
       const bool id = is_m ? rn.id_m : rn.id_s;
-#pragma unroll 1
-      for (int i = 0; i < 2; ++i) {
-        const int col0 = hf * 64 + i * 32;
-        uint32_t x[32];
+      const int col0 = hf * 64;
+      uint32_t x[2][32];
 #pragma unroll
-        for (int j = 0; j < 32; ++j)
-          x[j] = __float_as_uint(src ? __ldg(src + (size_t)(col0 + j) * kD + dg) : (id && col0 + j == dg ? 1.f : 0.f));
-        __syncwarp();
-        tmem_st32(tl + kColP + col0, x);
-      }
+      for (int j = 0; j < 64; ++j)
+        x[j >> 5][j & 31] = __float_as_uint(src ? __ldg(src + (size_t)(col0 + j) * kD + dg) : (id && col0 + j == dg ? 1.f : 0.f));
+      __syncwarp();
+      tmem_st32(tl + kColP + col0, x[0]);
+      tmem_st32(tl + kColP + col0 + 32, x[1]);
       tmem_wait_st();
       tc_fence_before_sync();
       warp_arrive(bar(bars.init));

@@ -869,14 +869,14 @@ size_t seg_scratch_bytes(const mdn_params& p, int segments) {
 // Packed input: the lengths are known on the device only.  The model takes the mean; every sequence is then split in the same
 // proportions by its own length, so that what the longest one takes falls by the factor the model saw, and the shorter ones
 // only leave SMs free earlier.  The mean says less than a length: 0.7 there.
-SegSplit choose_segments(const mdn_params& p) {
-  const SegSplit off{1, 0, 0, 0.};
+static SegSplit choose_split(const mdn_params& p, double* expected) {
+  const SegSplit off{1, 0, 0};
   if (!tensor_path_supported(p) || p.segments == 1) return off;
   const long seqs = p.num_seqs > 0 ? p.num_seqs : p.B, tokens = p.num_seqs > 0 ? p.T / seqs : p.T;
   const long nch = (tokens + C - 1) / C, chains = seqs * p.H;
   if (p.segments >= 3) {   // forced: equal segments (at least a chunk: packed input can have fewer tokens than sequences)
     const int per = nch > 0 ? (int)((nch + p.segments - 1) / p.segments) : 1;
-    return SegSplit{p.segments, per, per, 0.};
+    return SegSplit{p.segments, per, per};
   }
   auto waves = [](long ctas, long sms) { return (ctas + sms - 1) / sms; };
   const double serial = (double)(waves(chains, kSms) * nch);
@@ -896,11 +896,21 @@ SegSplit choose_segments(const mdn_params& p) {
         best = cost;
         // with the phases that chain_half.cu runs at its pace
         const double h1 = half_runs(chains * (1 + 3 * m)) ? kHalfChunk : 1., h3 = half_runs(chains * (m + 1)) ? kHalfChunk : 1.;
-        r = SegSplit{(int)m + 2, (int)first, (int)L, (p1 > p0 ? p1 : p0) * h1 + w3 * (L + kRun) * h3 + step * m + kFix};
+        r = SegSplit{(int)m + 2, (int)first, (int)L};
+        *expected = (p1 > p0 ? p1 : p0) * h1 + w3 * (L + kRun) * h3 + step * m + kFix;
       }
     }
   }
   return r;
+}
+SegSplit choose_segments(const mdn_params& p) {
+  double expected = 0.;
+  return choose_split(p, &expected);
+}
+double expected_scan_cost(const mdn_params& p) {
+  double expected = 0.;
+  choose_split(p, &expected);
+  return expected;
 }
 
 }  // namespace mdn

@@ -238,13 +238,13 @@ bool chain_uses_tf32_kernel(const Plan& pl);
 size_t seg_scratch_bytes(const mdn_params& p, int segments);
 // The parallel inter-chunk scan's split of a sequence of nch chunks: G segments, the first `first` chunks long, the others
 // `mid` (the last one what is left).
-// `cost` is what the model expects of it, in chunk-times of chain_tf32.cu.
-struct SegSplit { int G, first, mid; double cost; };
+struct SegSplit { int G, first, mid; };
 // Whether so many runs at once get two CTAs each (chain_half.cu), and what a chunk costs there (4.1 k against 6.3 k cycles).
 inline bool half_runs(long runs) { return 2 * runs <= kSms; }
 constexpr double kHalfChunk = 0.66;
 constexpr int kSegLeast = 4;   // chunks: below that a run's start and end outweigh what running it in parallel saves
 SegSplit choose_segments(const mdn_params& p);
+double expected_scan_cost(const mdn_params& p);   // what the model expects of that split (chosen, not forced), in chunk-times of chain_tf32.cu
 cudaError_t launch_seg_combine(const Plan& pl, int G, float* E, const float* Psi, const float* PhiS,
                                const float* PhiM, int* launches);
 
