@@ -115,8 +115,7 @@ __device__ __forceinline__ ChainRun chain_run(const ChainTf32Args& a, int item) 
 }
 
 // The scalar recurrence of G = [[g11, g12], [0, g22]] over one chunk and the chunk's six coefficient vectors (two tokens per lane
-// of the calling warp), from its coefficient vectors cf to the published block aj.  Contractions are spelled out: both kernels round
-// alike.
+// of the calling warp), from its coefficient vectors cf to the published block aj.
 template <bool kLayer>
 __device__ __forceinline__ void publish_coefs(const float* cf, float* aj, float scale, int lane, float& g11, float& g12, float& g22) {
   const float aC = cf[kAbar * C + C - 1], bC = cf[kB * C + C - 1], mC = cf[kMubar * C + C - 1];
@@ -132,17 +131,17 @@ __device__ __forceinline__ void publish_coefs(const float* cf, float* aj, float 
     float cx, cy, cz, cu;
     if constexpr (kLayer) {
       const float rk = cf[kRk * C + t], sq_ = scale * cf[kRq * C + t];
-      cx = ab * rk * g11; cy = fmaf(pp, g22, -__fmul_rn(ab * rk, g12));
-      cz = sq_ * (ab * g11); cu = sq_ * fmaf(ab, g12, -__fmul_rn(bb, g22));
+      cx = ab * rk * g11; cy = pp * g22 - ab * rk * g12;
+      cz = sq_ * (ab * g11); cu = sq_ * (ab * g12 - bb * g22);
     } else {
-      cx = ab * g11; cy = fmaf(pp, g22, -__fmul_rn(ab, g12));
-      cz = scale * cx; cu = scale * fmaf(ab, g12, -__fmul_rn(bb, g22));
+      cx = ab * g11; cy = pp * g22 - ab * g12;
+      cz = scale * cx; cu = scale * (ab * g12 - bb * g22);
     }
     aj[kCx + t] = -cx;     // stored negated: the epilogue's first step is one packed FMA per token pair
     aj[kCy + t] = cy;
     aj[kCz + t] = cz;
     aj[kCu + t] = cu;
-    aj[kWs + t] = lazy ? fmaf(n12 / n22, gm, gs) / n11 : gs;
+    aj[kWs + t] = lazy ? (gs + (n12 / n22) * gm) / n11 : gs;
     aj[kWm + t] = lazy ? gm / n22 : gm;
   }
   if (lane == 0) { aj[kN11] = n11; aj[kN12] = n12; aj[kN22] = n22; aj[kLazy] = lazy ? 1.f : 0.f; }
@@ -150,7 +149,7 @@ __device__ __forceinline__ void publish_coefs(const float* cf, float* aj, float 
 }
 
 // S = g11 Sh + g12 Mh, one element.
-__device__ __forceinline__ float unscale_s(float g11, float s, float g12, float m) { return fmaf(g11, s, __fmul_rn(g12, m)); }
+__device__ __forceinline__ float unscale_s(float g11, float s, float g12, float m) { return fmaf(g12, m, __fmul_rn(g11, s)); }
 
 // chain_half.cu: `items` runs (of a launch described by a), two CTAs each.
 struct ChainTensors { const void* q; const void* k; const void* v; };
