@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
           const float mine = __uint_as_float(x[j]), other = __shfl_xor_sync(0xffffffffu, mine, 16);
-          const float y = is_m ? g22 * mine : unscale_s(g11, mine, g12, other);
+          const float y = is_m ? g22 * mine : final_s(g11, mine, g12, other);
           if (dst) dst[(size_t)(col0 + j) * kD + dg] = y;
         }
       }

@@ -633,7 +633,7 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             const float sv = __uint_as_float(sr[j]), mv = __uint_as_float(mr[j]);
-            if (Sfp) Sfp[(size_t)(col0 + j) * kD + d] = unscale_s(g11, sv, g12, mv);
+            if (Sfp) Sfp[(size_t)(col0 + j) * kD + d] = final_s(g11, sv, g12, mv);
             if (Mfp) Mfp[(size_t)(col0 + j) * kD + d] = g22 * mv;
           }
         }

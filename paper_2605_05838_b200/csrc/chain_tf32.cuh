@@ -148,8 +148,9 @@ __device__ __forceinline__ void publish_coefs(const float* cf, float* aj, float 
   if (lazy) { g11 = n11; g12 = n12; g22 = n22; } else { g11 = 1.f; g12 = 0.f; g22 = 1.f; }
 }
 
-// S = g11 Sh + g12 Mh, one element.
-__device__ __forceinline__ float unscale_s(float g11, float s, float g12, float m) { return fmaf(g12, m, __fmul_rn(g11, s)); }
+// S = g11 Sh + g12 Mh, one element: of the masters that an eager chunk rescales, and of a final state.
+__device__ __forceinline__ float unscale_s(float g11, float s, float g12, float m) { return fmaf(g11, s, __fmul_rn(g12, m)); }
+__device__ __forceinline__ float final_s(float g11, float s, float g12, float m) { return fmaf(g12, m, __fmul_rn(g11, s)); }
 
 // chain_half.cu: `items` runs (of a launch described by a), two CTAs each.
 struct ChainTensors { const void* q; const void* k; const void* v; };
