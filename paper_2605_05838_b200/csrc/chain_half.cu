@@ -25,8 +25,8 @@
 // need not be are not unrolled.  A wait in a product-issuing warp costs 0.2 .. 0.4 k cycles even if its phase is long complete: the
 // serial chain's products have a warp of their own with three waits per chunk.
 //
-// Measured: 3.9 .. 4.2 k cycles per chunk against 6.3 k of chain_tf32.cu.  4 x 2048 tokens x 8 heads, whole call: 131.7 -> 96.5 us;
-// 200 tokens x 16 heads with a start state: 24.5 -> 19.5.
+// Measured: 3.9 .. 4.2 k cycles per chunk against 6.3 k of chain_tf32.cu.  4 x 2048 tokens x 8 heads, whole call: 131.5 -> 94.4 us;
+// 200 tokens x 16 heads with a start state: 23.9 -> 18.3.
 //
 // The layer operations stay with chain_tf32.cu: their output step (a norm over all value columns, so an exchange between the two
 // CTAs) kept four output warps busy for longer than a chunk lasts here, and its code made every warp wait for instructions (4 x 3001

@@ -897,7 +897,7 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
 #endif
   const unsigned chains = (unsigned)pl.geom.num_seqs * p.H;
   auto launch = [&](unsigned grid) -> cudaError_t {
-    // two CTAs per run while all of them are resident at once (measured at 32 chains: 131.7 -> 96.5 us; above, a second wave of
+    // two CTAs per run while all of them are resident at once (measured at 32 chains: 131.5 -> 94.4 us; above, a second wave of
     // halves would cost 2 x 4.1 k cycles per chunk against 6.3 k)
     if (!layer && half_runs(grid)) return launch_chain_half(pl, a, ChainTensors{q, k, v}, grid, launches);
     auto kern = layer ? (o_bf16 ? chain_tf32_kernel<__nv_bfloat16, true> : chain_tf32_kernel<float, true>)
