@@ -91,27 +91,24 @@ struct Bars {
   uint64_t go[2];     // a stage's output tile is staged and nothing reads the stage any more (256; with the fused output step + 128)
   uint64_t cfull;     // bf16 K, Q of a chunk landed in their buffer                         (1 + tx bytes)
   uint64_t cfree;     // ... and read: the next chunk's may be loaded                       (64)
-  uint64_t kq;        // fp32 [K; Q] of a chunk written                                   (64)
+  uint64_t kq;        // fp32 [K; Q] of a chunk written, the chunk before's Sh update done   (64 + commit)
   uint64_t adj[2];    // a chunk's coefficient block written                              (32)
   uint64_t fin;       // G after the last chunk written                                   (32)
   uint64_t init;      // masters of chunk 0 stored                                        (256)
   uint64_t mx;        // first half of MMA-1 done: X, Z                                    (commit)
   uint64_t m1;        // MMA-1 done: X, Z, Y, U                                            (commit)
   uint64_t r;         // EPI-1 done: R^T hi/lo in X                                        (256)
-  uint64_t m2;        // MMA-2 done                                                       (commit)
-  uint64_t oi;        // inter-chunk output terms stored in U                             (256)
+  uint64_t m2;        // MMA-2 done, inter-chunk output terms stored in U                 (commit + 256; state-only runs: commit)
   uint64_t v1a;       // EPI-2, first part: wS V~ in X (eager chunks: Sh rescaled)         (256)
   uint64_t v1b;       // EPI-2, second part: wM V~ in Y (eager chunks: Mh rescaled)        (256)
-  uint64_t m3s;       // MMA-3, Sh part done                                              (commit)
-  uint64_t m3;        // MMA-3 done                                                       (commit)
+  uint64_t m3;        // MMA-3 done, U (the chunk's output) has been read                 (commit + 256; state-only runs: commit)
   uint64_t mo;        // MMA-3' done                                                      (commit)
-  uint64_t zu;        // U (the chunk's output) has been read                              (256)
   uint64_t pn[2];     // fused output step: a stage's fp32 tile is staged                     (256)
 };
 
 enum Ev : int { kEvMma1 = 0, kEvM1Seen, kEvRArrive, kEvOiArrive, kEvM2Seen, kEvV1Arrive, kEvOutDone, kEvM3Seen, kEvRSeen,
                 kEvV1Seen, kEvCvtStart, kEvCvtDone, kEvTmaIssued, kEvStoresDone, kEvM2Own, kEvEager,
-                kEvXzIssued, kEvYuIssued, kEvM2Issued, kEvSIssued, kEvMIssued, kEvV1bSeen, kEvV1bArrive, kEvZuArrive, kEvMoIssued, kEvM3sOwn, kEvKqSeen, kEvLoopTop, kEvRArrive2, kEvV1Arrive2 };
+                kEvXzIssued, kEvYuIssued, kEvM2Issued, kEvSIssued, kEvMIssued, kEvV1bSeen, kEvV1bArrive, kEvZuArrive, kEvMoIssued, kEvKqSeen, kEvLoopTop, kEvRArrive2, kEvV1Arrive2 };
 
 template <typename TO> __device__ __forceinline__ void stage_o(uint8_t* tile, int r, int d, float x);
 template <> __device__ __forceinline__ void stage_o<float>(uint8_t* tile, int r, int d, float x) {
@@ -157,9 +154,9 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
   const uint32_t b_go0 = smem_u32(&bars.go[0]), b_go1 = smem_u32(&bars.go[1]);
   const uint32_t b_kq = smem_u32(&bars.kq), b_adj0 = smem_u32(&bars.adj[0]), b_adj1 = smem_u32(&bars.adj[1]);
   const uint32_t b_init = smem_u32(&bars.init), b_m1 = smem_u32(&bars.m1), b_r = smem_u32(&bars.r);
-  const uint32_t b_m2 = smem_u32(&bars.m2), b_oi = smem_u32(&bars.oi), b_v1a = smem_u32(&bars.v1a);
-  const uint32_t b_v1b = smem_u32(&bars.v1b), b_mx = smem_u32(&bars.mx), b_m3s = smem_u32(&bars.m3s);
-  const uint32_t b_m3 = smem_u32(&bars.m3), b_mo = smem_u32(&bars.mo), b_zu = smem_u32(&bars.zu);
+  const uint32_t b_m2 = smem_u32(&bars.m2), b_v1a = smem_u32(&bars.v1a);
+  const uint32_t b_v1b = smem_u32(&bars.v1b), b_mx = smem_u32(&bars.mx);
+  const uint32_t b_m3 = smem_u32(&bars.m3), b_mo = smem_u32(&bars.mo);
   const uint32_t b_fin = smem_u32(&bars.fin), b_cfull = smem_u32(&bars.cfull), b_cfree = smem_u32(&bars.cfree);
   const uint32_t b_pn0 = smem_u32(&bars.pn[0]), b_pn1 = smem_u32(&bars.pn[1]);
   // kLayer = false compiles the layer operations out
@@ -171,13 +168,15 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
     mbar_init(b_full0, 1); mbar_init(b_full1, 1);
     const uint32_t n_go = kEpiThreads + (kLayer && a.post_on && write_o ? kOutThreads : 0);
     mbar_init(b_go0, n_go); mbar_init(b_go1, n_go);
-    mbar_init(b_kq, kCvtThreads); mbar_init(b_adj0, 32); mbar_init(b_adj1, 32);
+    mbar_init(b_kq, kCvtThreads + 1); mbar_init(b_adj0, 32); mbar_init(b_adj1, 32);
     mbar_init(b_fin, 32); mbar_init(b_cfull, 1); mbar_init(b_cfree, kCvtThreads);
-    mbar_init(b_init, kEpiThreads); mbar_init(b_r, kEpiThreads); mbar_init(b_oi, kEpiThreads);
-    mbar_init(b_v1a, kEpiThreads); mbar_init(b_v1b, kEpiThreads); mbar_init(b_zu, kEpiThreads);
+    mbar_init(b_init, kEpiThreads); mbar_init(b_r, kEpiThreads);
+    mbar_init(b_v1a, kEpiThreads); mbar_init(b_v1b, kEpiThreads);
     if constexpr (kLayer) { mbar_init(b_pn0, kEpiThreads); mbar_init(b_pn1, kEpiThreads); }
-    mbar_init(b_m1, 1); mbar_init(b_m2, 1); mbar_init(b_m3, 1); mbar_init(b_mo, 1); mbar_init(b_mx, 1); mbar_init(b_m3s, 1);
+    const uint32_t n_out = 1 + (write_o ? kEpiThreads : 0);
+    mbar_init(b_m1, 1); mbar_init(b_m2, n_out); mbar_init(b_m3, n_out); mbar_init(b_mo, 1); mbar_init(b_mx, 1);
     mbar_fence_init();
+    mbar_arrive(b_kq);   // (the first chunk has no update before it)
   }
   if (kLayer && tid < kD) w_sm[tid] = (a.post_on && a.post_w) ? __ldg(a.post_w + tid) : 1.f;
   if (warp == kWarpMma) tmem_alloc(smem_u32(&tmem_slot), 512);
@@ -347,13 +346,16 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
         MDN_SPIN(b_kq, ph);
         MDN_MARK(c, kEvKqSeen);
         if (c == 0) MDN_WAIT(b_init, 0);
+        // ---- MMA-1: [X | Z] = Sh [K; Q]^T, [Y | U] = Mh [K; Q]^T  (state-only runs: X, Y against K alone).  Each half behind
+        // the commit of the update of the master it reads and of the operand it overwrites: products with different
+        // accumulators have no order among themselves (one issued right behind another was seen to miss part of what
+        // that one accumulates: chain_half.cu).  The tensor pipe stays busy: the Sh update's commit comes while the Mh
+        // update runs, that one's while X, Z are made.  Each commit arrives on a barrier that this warp waits for anyway:
+        // a wait more costs it 0.15 .. 0.2 k cycles, complete or not, a commit more 0.05 .. 0.1, and it issues for half of
+        // the chunk.  (8 x 4096 tokens x 16 heads, 32768 packed x 16: 394.3 -> 394.0, 490.2 -> 491.3 us with this order enforced;
+        // with three waits of its own for it 396.7 -> 403.4, 520.7 -> 538.8 on another box.)
         tc_fence_after_sync();
         MDN_MARK(c, kEvMma1);
-        // ---- MMA-1: [X | Z] = Sh [K; Q]^T, [Y | U] = Mh [K; Q]^T  (state-only runs: X, Y against K alone).  Issued right
-        // behind the previous chunk's updates of Sh, Mh, without waiting for their commits: the tensor pipe runs this
-        // thread's products in issue order, a product that overwrites another's operand included - the probe library's
-        // chained-product tests show it - and at least eight products lie between an update and the first product that reads
-        // it here.  (With none between, a product can miss part of what it reads: chain_half.cu.)  Commits are for the epilogue.
         if (lead) {
 #pragma unroll
           for (int j = 0; j < 16; ++j)
@@ -361,7 +363,7 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
           umma_commit(b_mx);
         }
         MDN_MARK(c, kEvXzIssued);
-        if (write_o) MDN_SPIN(b_zu, ph ^ 1);   // the previous chunk's output has been read out of U
+        MDN_SPIN(b_m3, ph ^ 1);   // Mh updated, and the previous chunk's output has been read out of U
         tc_fence_after_sync();
         if (lead) {
 #pragma unroll
@@ -384,10 +386,10 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
           umma_commit(b_m2);
         }
         MDN_MARK(c, kEvM2Issued);
-        // ---- MMA-3': U += V~^T W^T, V~ read as tf32 from the accumulator MMA-2 has just filled, W an fp32 tile;
-        // U holds the inter-chunk terms.  Runs while the epilogue makes the state-update operands.
+        // ---- MMA-3': U += V~^T W^T, V~ read as tf32 from the accumulator of MMA-2 (b_m2: its commit, and U holds the
+        // inter-chunk terms), W an fp32 tile.  Runs while the epilogue makes the state-update operands.
         if (write_o) {
-          MDN_SPIN(b_oi, ph);
+          MDN_SPIN(b_m2, ph);
           tc_fence_after_sync();
           MDN_MARK(c, kEvM2Own);
           if (lead) {
@@ -407,7 +409,7 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
 #pragma unroll
           for (int k = 0; k < 8; ++k)
             umma_ts(tm + kColS, tm + kColX + a_col(k >> 2, k & 3), dKmn + 128 * (k & 3), id128_mn, true);
-          umma_commit(b_m3s);
+          umma_commit(b_kq);
         }
         MDN_MARK(c, kEvSIssued);
         MDN_SPIN(b_v1b, ph);
@@ -721,7 +723,7 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
         tmem_st32(tl + kColU + r0, u);
         tmem_wait_st();
         tc_fence_before_sync();
-        mbar_arrive(b_oi);
+        mbar_arrive(b_m2);
         MDN_MARK(c, kEvOiArrive);
       }
       // ---------------- EPI-2: wS .* V~ -> X (handed over first), wM .* V~ -> Y, each as bf16 hi, lo.  V~ itself stays
@@ -815,7 +817,7 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
         tmem_ld32(tl + kColU + r0, u);
         tmem_wait_ld();
         tc_fence_before_sync();
-        mbar_arrive(b_zu);
+        mbar_arrive(b_m3);
         MDN_MARK(c, kEvZuArrive);
         bool plain_out = true;
         if constexpr (kLayer) plain_out = !post;
