@@ -399,9 +399,13 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
         eager = reinterpret_cast<const float*>(smem + kOffAdj + s * kAdjBytes)[kLazy] == 0.f;
         MDN_WAIT(q32, ph);
         MDN_POLL(mx, ph);
+      } else if (c > 0) {
+        MDN_WAIT(m2, ph ^ 1);
       }
       tc_fence_after_sync();
-      // ---- MMA-3' of the previous chunk: Z += V~^T W^T, V~ read as tf32 from the accumulator of MMA-2 (MMA-3 has waited for it)
+      // ---- MMA-3' of the previous chunk: Z += V~^T W^T, V~ read as tf32 from the accumulator of MMA-2, which another warp issued
+      // and whose commit this one has seen: through mx (MMA-1x follows the previous chunk's MMA-3, that its epilogue's wait for
+      // m2), behind the last chunk by the wait for m2 itself
       if (c > 0) {
         const uint64_t dW = s ? dW_0 : dW_1;
         if (lead) {

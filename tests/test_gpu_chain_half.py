@@ -52,3 +52,50 @@ def test_two_ctas_per_chain_packed(mdn):
     import torch
     got, ref = run_gpu(mdn, inp, o_dtype=torch.float32), run_oracle(inp)
     assert max(rel_err(x, y) for x, y in zip(got, ref)) <= 2e-2
+
+
+def eager_chunks(inp, h):
+    """Which chunks of head h rescale the masters: the rule of the lazily scaled state (limits 2^-64 and 1), on G in 64 bits."""
+    g11, g12, g22, out = 1.0, 0.0, 1.0, []
+    for c in range(0, inp["beta"].shape[1], 64):
+        al, mu, be = (inp[n][0, c:c + 64, h].astype(np.float64) for n in ("log_alpha", "log_mu", "beta"))
+        for a, m, b in zip(np.exp(al), np.exp(mu), be):
+            g22 *= m
+            g11, g12 = a * g11, a * g12 - b * g22
+        out.append(not (g11 >= 2.0 ** -64 and g22 >= 2.0 ** -64 and abs(g12) <= g22))
+        if out[-1]:
+            g11, g12, g22 = 1.0, 0.0, 1.0
+    return out
+
+
+# (tokens, constant gates alpha, mu, beta or None for preset S, mu = 0 at the last token, which chunks are eager)
+EAGER_ENDS = [(1, (0.99, 0.9, 0.05), True, [1]), (17, (0.999, 0.5, 0.05), False, [1]), (64, (0.999, 0.8, 0.01), False, [1]),
+              (64, (0.3, 0.5, 0.3), False, [1]), (65, None, True, [0, 1]), (128, (0.3, 0.5, 0.3), False, [1, 1]),
+              (64 * 4, None, True, [0, 0, 0, 1]), (64 * 4 + 9, None, True, [0, 0, 0, 0, 1])]
+
+
+@pytest.mark.parametrize("T,gates,cut,eager", EAGER_ENDS)
+def test_last_chunk_rescales(mdn, T, gates, cut, eager):
+    """A run that ends in a chunk that rescales the masters: its output product is the only one with no later product of the state
+    in front of it.  The same bits as the kernel with one CTA per chain, every time."""
+    import torch
+    w = wl.Workload("half_eager", B=1, T=T, H=2, dk=128, dv=128, dtype="bf16", init_state_std=0.2, seed=T)
+    inp = wl.make_inputs(w)
+    if gates:
+        for n, x in zip(("log_alpha", "log_mu", "beta"), (np.log(gates[0]), np.log(gates[1]), gates[2])):
+            inp[n][:] = np.float32(x)
+    if cut:
+        inp["log_mu"][:, -1] = -np.inf
+    assert eager_chunks(inp, 0) == eager_chunks(inp, 1) == [bool(e) for e in eager]
+    ref, t = run_oracle(inp), to_torch(inp)
+    names = ("q", "k", "v", "beta", "log_alpha", "log_mu", "eta")
+    copies = lambda x: x.expand(38, *x.shape[1:]).contiguous()
+    for o_dtype in (torch.float32, torch.bfloat16):
+        many = mdn.chunk_fwd(*(copies(t[n]) for n in names), initial_S=copies(t["initial_S"]), initial_M=copies(t["initial_M"]),
+                             scale=inp["scale"], o_dtype=o_dtype)
+        want = [x[0].double().cpu().numpy() for x in many]
+        for _ in range(10):
+            got = run_gpu(mdn, inp, o_dtype=o_dtype)
+            assert all(np.array_equal(x[0], y) for x, y in zip(got, want))
+        if o_dtype == torch.float32:
+            assert max(rel_err(x, y) for x, y in zip(got, ref)) <= 2e-2
