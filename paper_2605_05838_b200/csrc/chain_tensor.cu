@@ -363,8 +363,13 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tensor_kernel(const ChainAr
         umma_commit(b_m1);
         // ---- MMA-1b (output terms, off the critical path).  The tensor pipe runs its MMAs in issue order, so a group
         // issued here delays MMA-2 by whatever of it is still running when EPI-1 is done: only Z = S_b Q^T is issued
-        // here (it fits under EPI-1) ...
+        // here (it fits under EPI-1) ...  It overwrites the V~ that the previous chunk's MMA-3' has read: behind that product's
+        // commit, which the epilogue has waited for before it read U (products with different accumulators have no order
+        // among themselves).  That was under MMA-1a, so nothing waits here: 8 x 4096 tokens x 16 heads, a training step
+        // 1753.8 -> 1752.9 us with the wait for U moved here.
         if (write_o) {
+          MDN_WAIT(b_zu, ph ^ 1);
+          tc_fence_after_sync();
 #pragma unroll
           for (int k = 0; k < 8; ++k)
             umma_ss(tmem + kColZ, ((k >> 2) ? dSb1 : dSb0) + 2 * (k & 3), ((k >> 2) ? dQ1 : dQ0) + 2 * (k & 3), id64, k > 0);
@@ -389,8 +394,6 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tensor_kernel(const ChainAr
         umma_commit(b_m2);
         // ... and U = M_b Q^T here: it fits under EPI-2 and is done before MMA-3 can start
         if (write_o) {
-          MDN_WAIT(b_zu, ph ^ 1);
-          tc_fence_after_sync();
 #pragma unroll
           for (int k = 0; k < 8; ++k)
             umma_ss(tmem + kColU, ((k >> 2) ? dMb1 : dMb0) + 2 * (k & 3), ((k >> 2) ? dQ1 : dQ0) + 2 * (k & 3), id64, k > 0);

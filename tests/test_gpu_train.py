@@ -94,6 +94,25 @@ def test_keep_chunk_states(mdn, name, kw):
     assert ev <= 2e-2
 
 
+@pytest.mark.parametrize("T", [64 * 2, 64 * 7 + 9])
+def test_keep_chunk_states_overwrites_no_operand_in_use(mdn, T):
+    """Q S of a chunk goes where the previous chunk's output product reads V~ from.  A full GPU of chains, ten times: the same bits
+    in every copy of the two chains that the oracle walks, and its o within the path's bound."""
+    import torch
+    w = wl.Workload("keep_war", B=1, T=T, H=2, dk=128, dv=128, dtype="bf16", seed=T, init_state_std=0.1)
+    inp = wl.make_inputs(w)
+    t = to_torch(inp)
+    many = lambda x: x.expand(70, *x.shape[1:]).contiguous()
+    args = [many(t[n]) for n in ("q", "k", "v", "beta", "log_alpha", "log_mu", "eta")]
+    ref, first = run_oracle(inp), None
+    for _ in range(10):
+        got = mdn.chunk_fwd(*args, initial_S=many(t["initial_S"]), initial_M=many(t["initial_M"]), scale=inp["scale"],
+                            path="tensor", o_dtype=torch.float32, keep_chunk_states=True)[:3]
+        first = first or [x[:1].clone() for x in got]
+        assert all(torch.equal(x, y.expand_as(x)) for x, y in zip(got, first))
+    assert max(rel_err(x.double().cpu().numpy(), y) for x, y in zip(first, ref)) <= 2e-2
+
+
 @pytest.mark.parametrize("T, with_final", [(64 * 4 + 20, True), (64 * 3, False)])
 def test_bwd_state_chain(mdn, T, with_final):
     """Adjoint of the inter-chunk state recurrence (stage 1 of the chunk-parallel backward) against the fp64 chunk-form
