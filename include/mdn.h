@@ -91,12 +91,15 @@ typedef struct {
  *   2. a short serial combine over segments (fp32) giving every segment's true start state;
  *   3. in parallel: segments 1.. as usual from those start states (outputs and final state).
  * The result is the same recurrence; only rounding differs.  Chosen automatically when the call has
- * too few chains to fill the GPU and the sequences are long (e.g. B=1, H=16, T=65536; packed input: on average).
+ * too few chains to fill the GPU and the sequences are long (e.g. B=1, H=16, T=65536; packed input: on average);
+ * a forward of fixed length without q/k norm and output step that keeps no states still runs its chains serially
+ * where that is faster for it (few enough chains for two CTAs each, not too long: e.g. B=2, H=16, T=4000).
  */
 
 /* Bytes of device workspace mdn_chunk_fwd needs for these parameters (0 on invalid
  * parameters).  Holds the chunk map, the per-chunk coefficient vectors, the
- * per-chunk T and W matrices and the parallel inter-chunk scan's segment states;
+ * per-chunk T and W matrices and the parallel inter-chunk scan's segment states (one
+ * workspace serves every forward with these parameters, also where one of them uses no scan);
  * contents are scratch.  The scan makes the size of a shorter call the larger one at
  * times: with segments = 0, every call with a workspace (or arena) argument also takes one
  * that suffices for segments = 1, and runs that way. */
@@ -464,7 +467,7 @@ typedef struct {
   uint64_t off_W;           /* [num_slots][H][64][64]  (tensor path: bf16 hi part, lo part follows; or fp32) */
   uint64_t total_bytes;
   uint64_t off_seg;         /* segment states, Psi and Phi matrices of the parallel scan (fp32)          */
-  int32_t segments;         /* segments per sequence the call will use (1 = plain serial chain)          */
+  int32_t segments;         /* segments per sequence that the workspace has room for (1 = no scan)       */
   int32_t reserved;
 } mdn_ws_layout;
 

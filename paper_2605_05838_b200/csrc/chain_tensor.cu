@@ -872,6 +872,7 @@ size_t seg_scratch_bytes(const mdn_params& p, int segments) {
 // Packed input: the lengths are known on the device only.  The model takes the mean; every sequence is then split in the same
 // proportions by its own length, so that what the longest one takes falls by the factor the model saw, and the shorter ones
 // only leave SMs free earlier.  The mean says less than a length: 0.7 there.
+// *expected: what the model expects of that split (chosen, not forced), in chunk-times of chain_tf32.cu.
 static SegSplit choose_split(const mdn_params& p, double* expected) {
   const SegSplit off{1, 0, 0};
   if (!tensor_path_supported(p) || p.segments == 1) return off;
@@ -910,10 +911,12 @@ SegSplit choose_segments(const mdn_params& p) {
   double expected = 0.;
   return choose_split(p, &expected);
 }
-double expected_scan_cost(const mdn_params& p) {
+bool serial_beats_scan(const Plan& pl) {
+  const mdn_params& p = pl.p;
+  if (pl.lay.segments <= 1 || p.segments != 0 || p.num_seqs > 0 || pl.qk.on || pl.post.on || !chain_uses_tf32_kernel(pl)) return false;
   double expected = 0.;
   choose_split(p, &expected);
-  return expected;
+  return half_runs((long)p.B * p.H) && kHalfChunk * pl.geom.chunks_per_seq <= expected;
 }
 
 }  // namespace mdn

@@ -913,10 +913,6 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
   };
   const int G = pl.lay.segments;
   if (G <= 1) return launch(chains);
-  // The split is chosen (and its scratch sized) by the pace of one CTA per chain; where two make the whole chain faster than the
-  // scan is expected to be, it runs serially all the same.
-  if (!layer && p.segments == 0 && p.num_seqs == 0 && half_runs(chains) && kHalfChunk * pl.geom.chunks_per_seq <= expected_scan_cost(p))
-    return launch(chains);
 
   // ---- parallel inter-chunk scan: Psi / Phi of the middle segments, serial combine, then all segments for real
   constexpr size_t kMat = (size_t)kD * kD;

@@ -185,6 +185,7 @@ static mdn_status run_forward(const Plan& plan, const void* q, const void* k, co
                               const float* initial_M, void* o, float* final_S, float* final_M) {
   Plan pl = plan;
   pl.w_f32 = chain_uses_tf32_kernel(pl);   // the plain forward's chain kernel reads W as fp32
+  if (serial_beats_scan(pl)) pl.lay.segments = 1;
   if (!q || !k || !v || !o) return MDN_ERR_INVALID_ARG;
   if (!aligned(q, 16) || !aligned(k, 16) || !aligned(v, 16) || !aligned(o, 16)) return MDN_ERR_INVALID_ARG;
   if ((initial_S && !aligned(initial_S, 16)) || (initial_M && !aligned(initial_M, 16)) ||

@@ -244,7 +244,9 @@ inline bool half_runs(long runs) { return 2 * runs <= kSms; }
 constexpr double kHalfChunk = 0.66;
 constexpr int kSegLeast = 4;   // chunks: below that a run's start and end outweigh what running it in parallel saves
 SegSplit choose_segments(const mdn_params& p);
-double expected_scan_cost(const mdn_params& p);   // what the model expects of that split (chosen, not forced), in chunk-times of chain_tf32.cu
+// The split is chosen (and its scratch sized) for every kind of call by the pace of one CTA per chain.  True for a plain forward
+// whose whole chains, two CTAs each, are expected to be faster than that: it runs serially (2 x 4000 tokens x 16 heads: 225 -> 188 us).
+bool serial_beats_scan(const Plan& pl);
 cudaError_t launch_seg_combine(const Plan& pl, int G, float* E, const float* Psi, const float* PhiS,
                                const float* PhiM, int* launches);
 

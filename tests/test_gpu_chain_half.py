@@ -99,3 +99,24 @@ def test_last_chunk_rescales(mdn, T, gates, cut, eager):
             assert all(np.array_equal(x[0], y) for x, y in zip(got, want))
         if o_dtype == torch.float32:
             assert max(rel_err(x, y) for x, y in zip(got, ref)) <= 2e-2
+
+
+@pytest.mark.parametrize("T,H,launches", [(64 * 29, 1, 2), (64 * 48 - 3, 16, 2), (64 * 51, 16, 5)])
+def test_serial_chain_where_it_beats_the_scan(mdn, T, H, launches):
+    """Both sides of the rule: a workspace with room for the scan, and the serial chain's kernels (intra-chunk, chain) and bits
+    where two CTAs per chain are the faster way, the scan's five kernels otherwise.  A call that keeps its states is always split."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(T)
+    unit = lambda x: (x / x.norm(dim=-1, keepdim=True)).bfloat16()
+    q, k, v = (torch.randn((1, T, H, 128), device="cuda", generator=g) for _ in range(3))
+    gates = [s * torch.rand((1, T, H), device="cuda", generator=g) for s in (0.05, -0.05, -0.05, 1.0)]
+    args = (unit(q), unit(k), v.bfloat16(), *gates)
+    assert mdn.workspace_layout(mdn.make_params(args[0], args[2], path="tensor")).segments > 1
+    got = mdn.chunk_fwd(*args, path="tensor")
+    assert mdn.last_launch_count() == launches
+    one = mdn.chunk_fwd(*args, path="tensor", segments=1)
+    assert mdn.last_launch_count() == 2
+    if launches == 2:
+        assert all(torch.equal(x, y) for x, y in zip(got, one))
+    mdn.chunk_fwd(*args, path="tensor", keep_chunk_states=True)
+    assert mdn.last_launch_count() == 5
