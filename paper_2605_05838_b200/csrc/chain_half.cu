@@ -164,11 +164,10 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
   }
 #ifdef MDN_DEBUG
   // Stamps go to shared memory for the chunks kTlFirst .. kTlFirst + 7 and are copied out when the kernel ends.
-  long long* const tline = a.timeline != nullptr ? a.timeline + 1024 * (size_t)blockIdx.x : nullptr;   // (1024 words per CTA)
-  constexpr int kTlFirst = 16;
-  __shared__ long long tl_sm[8][32];
+  long long* const tline = (blockIdx.x == 0) ? a.timeline : nullptr;
+  __shared__ long long tl_sm[kTlChunks][32];
 #define MDN_MARK(c, ev) \
-  if (tline != nullptr && lane == 0 && (c) >= kTlFirst && (c) < kTlFirst + 8 && \
+  if (tline != nullptr && lane == 0 && (c) >= kTlFirst && (c) < kTlFirst + kTlChunks && \
       ((warp >= kWarpMma && warp <= kWarpCvt) || warp == 2 || warp == kWarpOut)) tl_sm[(c) - kTlFirst][(ev)] = clock64();
   auto now = [&](int i) {   // ... and the nanosecond stamps of the run as a whole in the words before them
     unsigned long long ns;
@@ -737,7 +736,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
   __syncthreads();
 #ifdef MDN_DEBUG
   if (warp == 0) { MDN_NOW(5); }
-  if (tline != nullptr && tid < 256) tline[(kTlFirst + (tid >> 5)) * 32 + (tid & 31)] = tl_sm[tid >> 5][tid & 31];
+  if (tline != nullptr && tid < kTlChunks * 32) tline[(kTlFirst + (tid >> 5)) * 32 + (tid & 31)] = tl_sm[tid >> 5][tid & 31];
 #endif
   if (warp == kWarpMma) {
     __syncwarp();

@@ -205,13 +205,12 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
   // Stamps go to shared memory (a global store per stamp slows the stamping thread by hundreds of cycles) for the
   // chunks kTlFirst .. kTlFirst + 7 and are copied out when the kernel ends.
   long long* const tline = (blockIdx.x == 0) ? a.timeline : nullptr;
-  constexpr int kTlFirst = 16;
-  __shared__ long long tl_sm[8][32];
+  __shared__ long long tl_sm[kTlChunks][32];
 #define MDN_MARK(c, ev) \
-  if (tline != nullptr && lane == 0 && (c) >= kTlFirst && (c) < kTlFirst + 8 && \
+  if (tline != nullptr && lane == 0 && (c) >= kTlFirst && (c) < kTlFirst + kTlChunks && \
       (warp >= kWarpMma || warp == kWarpEpi + 2)) tl_sm[(c) - kTlFirst][(ev)] = clock64();
 #define MDN_MARK2(c, ev) \
-  if (tline != nullptr && lane == 0 && (c) >= kTlFirst && (c) < kTlFirst + 8 && warp == 5) tl_sm[(c) - kTlFirst][(ev)] = clock64();
+  if (tline != nullptr && lane == 0 && (c) >= kTlFirst && (c) < kTlFirst + kTlChunks && warp == 5) tl_sm[(c) - kTlFirst][(ev)] = clock64();
 #else
 #define MDN_MARK(c, ev)
 #define MDN_MARK2(c, ev)
@@ -855,7 +854,7 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns));
     tline[62] = clock64(); tline[63] = (long long)ns;
   }
-  if (tline != nullptr && tid < 256) tline[(kTlFirst + (tid >> 5)) * 32 + (tid & 31)] = (tid & 31) < 30 ? tl_sm[tid >> 5][tid & 31] : 0;
+  if (tline != nullptr && tid < kTlChunks * 32) tline[(kTlFirst + (tid >> 5)) * 32 + (tid & 31)] = (tid & 31) < 30 ? tl_sm[tid >> 5][tid & 31] : 0;
 #endif
   if (warp == kWarpMma) {
     __syncwarp();
@@ -894,7 +893,7 @@ cudaError_t launch_chain_tf32(const Plan& pl, const void* q, const void* k, cons
   const bool layer = a.qk_on || a.post_on;
   a.timeline = nullptr;
 #ifdef MDN_DEBUG   // debug builds only (-DMDN_DEBUG): the product library reads nothing from the environment
-  const char* tl = getenv("MDN_DEBUG_TIMELINE");   // device address of an int64 buffer, [chunks][32]
+  const char* tl = getenv("MDN_DEBUG_TIMELINE");   // device address of an int64 buffer, [24][32]
   a.timeline = tl ? reinterpret_cast<long long*>(strtoull(tl, nullptr, 0)) : nullptr;
 #endif
   const unsigned chains = (unsigned)pl.geom.num_seqs * p.H;

@@ -12,6 +12,11 @@ constexpr uint32_t kAdjBytes = 2048;
 constexpr float kLazyMin = 5.421010862427522e-20f;   // 2^-64: smallest g11', g22' a lazy chunk may leave
 constexpr float kLazyMix = 1.f;                      // largest |g12'| / g22' (beyond it the two hat terms of S cancel too much)
 
+// Debug builds: the chunks that are stamped.  The buffer holds 24 rows of 32 words; the words before the first stamped chunk's row
+// take the run's own stamps.
+constexpr int kTlFirst = 16, kTlChunks = 8;
+static_assert((kTlFirst + kTlChunks) * 32 <= 24 * 32, "the documented size of the buffer");
+
 struct ChainTf32Args {
   ChunkGeom g;
   const float* coef;
@@ -30,7 +35,7 @@ struct ChainTf32Args {
   float* seg_Psi;
   float* seg_PhiS;
   float* seg_PhiM;
-  long long* timeline;   // debug builds: CTA 0 writes clock64() at [chunk * 32 + event]
+  long long* timeline;   // debug builds: CTA 0 writes clock64() at [chunk * 32 + event], chunks kTlFirst .. kTlFirst + 7
   // layer operations (Section 3.3), kLayer instantiation only
   int qk_on;             // q <- L2Norm(q - d k), k <- L2Norm(k): 1/|k|, 1/|q - d k| arrive as coefficient vectors 6, 7
   const float* qk_d;     // [H] or NULL
