@@ -39,6 +39,13 @@ CASES = [
     ("packed bf16", dict(B=1, T=70 + 1 + 129 + 300 + 64, H=2, dk=128, dv=128, dtype="bf16", varlen=True, seed=33),
      [70, 1, 129, 300, 64], 0, "tensor"),
     ("segments forced", dict(B=1, T=64 * 40, H=2, dk=128, dv=128, dtype="bf16", seed=34, init_state_std=0.1), None, 4, "tensor"),
+    # the same with more than 74 runs at once: one CTA each instead of two
+    ("one CTA per chain, ragged T", dict(B=25, T=200, H=3, dk=128, dv=128, dtype="bf16", seed=37), None, 0, "tensor"),
+    ("one CTA per chain, one short chunk", dict(B=1, T=5, H=75, dk=128, dv=128, dtype="bf16", seed=38), None, 0, "tensor"),
+    ("one CTA per chain, packed", dict(B=1, T=70 + 1 + 129 + 300 + 64, H=16, dk=128, dv=128, dtype="bf16", varlen=True, seed=39),
+     [70, 1, 129, 300, 64], 0, "tensor"),
+    ("one CTA per chain, segments forced", dict(B=1, T=64 * 12 + 3, H=38, dk=128, dv=128, dtype="bf16", seed=40, init_state_std=0.1), None, 4,
+     "tensor"),
     ("fp32 SIMT", dict(B=2, T=130, H=2, dk=64, dv=64, dtype="f32", seed=35), None, 0, "simt"),
     ("packed fp32 SIMT", dict(B=1, T=63 + 65 + 2, H=2, dk=64, dv=64, dtype="f32", varlen=True, seed=36), [63, 65, 2], 0, "simt"),
 ]

@@ -28,7 +28,8 @@ def run_copies(mdn, t, inp, **kw):
     return [x[:1] for x in got]
 
 
-REGIMES = [(0.999, 0.8, 0.001), (0.97, 0.98, 0.015), (0.999, 0.999, 0.0002), (0.95, 0.999, 0.015), (0.3, 0.5, 0.3)]
+REGIMES = [(0.999, 0.8, 0.001), (0.99, 0.9, 0.01), (0.98, 0.97, 0.01), (0.97, 0.98, 0.015), (0.9, 0.95, 0.1), (0.995, 0.6, 0.01),
+           (0.999, 0.999, 0.0002), (0.95, 0.999, 0.015), (0.3, 0.5, 0.3)]
 
 
 @pytest.mark.parametrize("T,alpha,mu,beta", [(t, *r) for r in REGIMES for t in (64 * 6 + 9, 64)])
@@ -49,3 +50,20 @@ def test_products_that_read_an_accumulator_wait_for_it(mdn, T, alpha, mu, beta):
         first = first or got
         assert all(np.array_equal(x, y) for x, y in zip(got, first))
     assert max(rel_err(x, y) for x, y in zip(first, ref)) <= 2e-2
+
+
+@pytest.mark.parametrize("segments,T", [(3, 64 * 9), (4, 64 * 13 + 17), (5, 64 * 3 + 5)])
+def test_forced_scan(mdn, segments, T):
+    """38 chains: every phase of the scan has more than 74 runs, the serial chain two CTAs for each.  The first segment's tokens are
+    the same bits on both kernels; a ragged tail, and more segments than chunks."""
+    import torch
+    from helpers import run_gpu
+    w = wl.Workload("tf32_scan", B=1, T=T, H=38, dk=128, dv=128, dtype="bf16", init_state_std=0.3, seed=50 + segments)
+    inp = wl.make_inputs(w)
+    ref = run_oracle(inp)
+    got = run_gpu(mdn, inp, path="tensor", o_dtype=torch.float32, segments=segments)
+    assert mdn.last_launch_count() == 5
+    assert max(rel_err(x, y) for x, y in zip(got, ref)) <= 2e-2
+    per = ((T + 63) // 64 + segments - 1) // segments * 64
+    one = run_gpu(mdn, inp, path="tensor", o_dtype=torch.float32, segments=1)
+    assert np.array_equal(got[0][:, :per], one[0][:, :per])

@@ -160,8 +160,10 @@ def test_tf32_tmem_a_mnmajor_b(probe):
 
 def test_tf32_product_reading_the_previous_accumulator(probe):
     """Y = (A B^T) C^T with the second product's A operand = the first one's accumulator in tensor memory.
-    With a commit + wait in between (mode 3) the result must be right; issued back to back (mode 2) it must be the
-    same bit for bit: the tensor pipe runs one thread's products in issue order."""
+    With a commit + wait in between (mode 3) the result must be right; issued back to back (mode 2) it has been the
+    same bit for bit for this pair of shapes.  That is an observation, not an order: products with different accumulators
+    have none (one that read a 128-column update issued right before it missed part of it), and the library's kernels
+    wait for the commit of what they read."""
     rng = np.random.default_rng(9)
     a, b, c = rng.standard_normal((128, 128)), rng.standard_normal((64, 128)), rng.standard_normal((64, 64))
     x = a.astype(np.float32).astype(np.float64) @ b.astype(np.float32).astype(np.float64).T
@@ -172,13 +174,13 @@ def test_tf32_product_reading_the_previous_accumulator(probe):
     chained = run_tf32(probe, 2, a, b, c, (128, 64))
     print("back-to-back dependent products: max |chained - waited| %.3e (0 = the pipe ordered them)"
           % np.abs(chained - waited).max())
-    assert np.array_equal(chained, waited)          # the chain kernel relies on it (chain_tf32.cu, MMA issuer)
+    assert np.array_equal(chained, waited)          # (no kernel relies on it)
 
 
 def test_product_overwriting_the_previous_products_operand(probe):
     """Write-after-read through the pipe: a product issued right behind another one overwrites the columns that one
-    reads its A operand from; the first result must still be the product of the ORIGINAL operand (the chain kernel
-    issues dependent products back to back and relies on the pipe running them in issue order)."""
+    reads its A operand from; the first result has been the product of the ORIGINAL operand for this pair of shapes (no
+    kernel relies on it: what overwrites an operand waits for the commit of the product that reads it)."""
     rng = np.random.default_rng(10)
     a, b = rng.standard_normal((128, 128)), rng.standard_normal((64, 128))
     plain = run_tf32(probe, 0, a, b, None, (128, 64))
