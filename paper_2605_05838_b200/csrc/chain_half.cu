@@ -382,12 +382,12 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
     const uint32_t id64_tf32 = idesc_tf32(128, 64, false, false, false);
     const uint64_t dQ = smem_desc_sw128(sb + kOffQ32, 16, 1024);
     const uint64_t dW_0 = smem_desc_sw128(sb + kOffStage + kStW, 16, 1024), dW_1 = dW_0 + (kStageBytes >> 4);
+    bool eager = false;
 #pragma unroll 1
     for (int c = 0; c <= (write_o ? nch : -1); ++c) {
       const int s = c & 1;
       const uint32_t ph = c & 1, ph2 = (c >> 1) & 1;
       // (waits that are mostly over first, where nothing waits for this warp)
-      bool eager = false;
       if (c > 0) {
         MDN_WAIT(wfull[s ^ 1], ((c - 1) >> 1) & 1);
         MDN_WAIT(oi[s ^ 1], ((c - 1) >> 1) & 1);
@@ -398,13 +398,13 @@ __global__ void __launch_bounds__(kThreads, 1) chain_half_kernel(const ChainTf32
         eager = reinterpret_cast<const float*>(smem + kOffAdj + s * kAdjBytes)[kLazy] == 0.f;
         MDN_WAIT(q32, ph);
         MDN_POLL(mx, ph);
-      } else if (c > 0) {
+      } else if (eager) {
         MDN_WAIT(m2, ph ^ 1);
       }
       tc_fence_after_sync();
       // ---- MMA-3' of the previous chunk: Z += V~^T W^T, V~ read as tf32 from the accumulator of MMA-2, which another warp issued
       // and whose commit this one has seen: through mx (MMA-1x follows the previous chunk's MMA-3, that its epilogue's wait for
-      // m2), behind the last chunk by the wait for m2 itself
+      // m2); behind the last chunk through its own wait for m2, in the middle of MMA-1z or (eager) just above
       if (c > 0) {
         const uint64_t dW = s ? dW_0 : dW_1;
         if (lead) {

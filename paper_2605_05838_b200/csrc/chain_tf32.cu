@@ -352,7 +352,8 @@ __global__ void __launch_bounds__(threads_of(kLayer), 1) chain_tf32_kernel(const
         // update runs, that one's while X, Z are made.  Each commit arrives on a barrier that this warp waits for anyway:
         // a wait more costs it 0.15 .. 0.2 k cycles, complete or not, a commit more 0.05 .. 0.1, and it issues for half of
         // the chunk.  (8 x 4096 tokens x 16 heads, 32768 packed x 16: 394.3 -> 394.0, 490.2 -> 491.3 us with this order enforced;
-        // with three waits of its own for it 396.7 -> 403.4, 520.7 -> 538.8 on another box.)
+        // with three waits of its own for it 396.7 -> 403.4, 520.7 -> 538.8 on another box.  State-only runs do have a wait more:
+        // calls split for the scan take 0 .. 1 % longer, 1 x 30000 x 8 484.5 -> 489.6.)
         tc_fence_after_sync();
         MDN_MARK(c, kEvMma1);
         if (lead) {
