@@ -361,12 +361,11 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tensor_kernel(const ChainAr
         for (int k = 0; k < 8; ++k)
           umma_ss(tmem + kColY, ((k >> 2) ? dMb1 : dMb0) + 2 * (k & 3), ((k >> 2) ? dK1 : dK0) + 2 * (k & 3), id64, k > 0);
         umma_commit(b_m1);
-        // ---- MMA-1b (output terms, off the critical path).  The tensor pipe runs its MMAs in issue order, so a group
-        // issued here delays MMA-2 by whatever of it is still running when EPI-1 is done: only Z = S_b Q^T is issued
-        // here (it fits under EPI-1) ...  It overwrites the V~ that the previous chunk's MMA-3' has read: behind that product's
-        // commit, which the epilogue has waited for before it read U (products with different accumulators have no order
-        // among themselves).  That was under MMA-1a, so nothing waits here: 8 x 4096 tokens x 16 heads, a training step
-        // 1753.8 -> 1752.9 us with the wait for U moved here.
+        // ---- MMA-1b (output terms, off the critical path).  A group issued here delays MMA-2 by whatever of it is still
+        // running when EPI-1 is done: only Z = S_b Q^T is issued here (it fits under EPI-1) ...  It overwrites the V~ that
+        // the previous chunk's MMA-3' reads: behind that product's commit, which the epilogue has waited for before it read
+        // U (products with different accumulators have no order among themselves).  U is read under MMA-1a, so that nothing
+        // waits here: 8 x 4096 tokens x 16 heads, a training step 1753.8 -> 1752.9 us with the wait moved up from Q M.
         if (write_o) {
           MDN_WAIT(b_zu, ph ^ 1);
           tc_fence_after_sync();
